@@ -452,74 +452,4 @@ cudaError_t launch_advance_step(int* step, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// ---- image build: W_P = bf16(W P), fp32 accumulation -------------------------
-namespace {
-constexpr int IT = 64;   // tile of output rows / columns
-constexpr int IK = 16;   // depth step
-
-template <bool PF32>
-__global__ void __launch_bounds__(256)
-k_build_image(const uint16_t* __restrict__ W, const void* __restrict__ P, int o, int d, int k,
-              uint16_t* __restrict__ WP) {
-  __shared__ float As[IK][IT + 1];
-  __shared__ float Bs[IK][IT];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int o0 = blockIdx.y * IT, k0 = blockIdx.x * IT;
-  float acc[4][4] = {};
-  for (int d0 = 0; d0 < d; d0 += IK) {
-    for (int idx = threadIdx.x; idx < IT * IK; idx += 256) {
-      const int m = idx / IK, kk = idx % IK;
-      float v = 0.f;
-      if (o0 + m < o && d0 + kk < d)
-        v = __uint_as_float(((uint32_t)W[(size_t)(o0 + m) * d + d0 + kk]) << 16);
-      As[kk][m] = v;
-    }
-    for (int idx = threadIdx.x; idx < IT * IK; idx += 256) {
-      const int kk = idx / IT, n = idx % IT;
-      float v = 0.f;
-      if (d0 + kk < d && k0 + n < k) {
-        const size_t at = (size_t)(d0 + kk) * k + k0 + n;
-        if constexpr (PF32) v = reinterpret_cast<const float*>(P)[at];
-        else v = __uint_as_float(((uint32_t) reinterpret_cast<const uint16_t*>(P)[at]) << 16);
-      }
-      Bs[kk][n] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < IK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int m = o0 + ty * 4 + i, n = k0 + tx * 4 + j;
-      if (m < o && n < k) {
-        __nv_bfloat16 h = __float2bfloat16_rn(acc[i][j]);
-        WP[(size_t)m * k + n] = *reinterpret_cast<uint16_t*>(&h);
-      }
-    }
-}
-}  // namespace
-
-cudaError_t launch_build_image(const void* W, const void* P, int o, int d, int k, bool p_f32,
-                               void* WP, cudaStream_t st) {
-  dim3 grid((k + IT - 1) / IT, (o + IT - 1) / IT);
-  if (p_f32)
-    k_build_image<true><<<grid, 256, 0, st>>>((const uint16_t*)W, P, o, d, k, (uint16_t*)WP);
-  else
-    k_build_image<false><<<grid, 256, 0, st>>>((const uint16_t*)W, P, o, d, k, (uint16_t*)WP);
-  return cudaGetLastError();
-}
-
 }  // namespace gsi

@@ -41,6 +41,10 @@ bool encode(CUtensorMap* m, const void* base, size_t rows, size_t cols, unsigned
 
 }  // namespace
 
+bool encode_bf16_map(CUtensorMap* m, const void* base, size_t rows, size_t cols, unsigned box_rows) {
+  return encode(m, base, rows, cols, box_rows);
+}
+
 bool build_tma_maps(const GroupParams& g, bool front, int max_tokens, TmaMaps* out) {
   std::memset(out, 0, sizeof *out);
   for (int j = 0; j < g.n_maps; ++j)

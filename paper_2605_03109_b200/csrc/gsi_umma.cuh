@@ -280,6 +280,10 @@ __device__ __forceinline__ void tile_release(uint32_t tmem) {
 
 }  // namespace umma
 
+// Tensor map of a row-major bf16 matrix [rows][cols]: boxes of box_rows x 64 elements, 128-byte
+// swizzle.  False when the driver's encoder is unavailable or rejects the shape.
+bool encode_bf16_map(CUtensorMap* m, const void* base, size_t rows, size_t cols, unsigned box_rows);
+
 // Tensor maps of one layer (host-encoded at set-up, passed to the kernels by value as a
 // __grid_constant__ parameter).  A operands use boxes of 128 rows, B operands of 16 rows;
 // every box is 64 K-elements wide with the 128-byte swizzle.

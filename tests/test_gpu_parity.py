@@ -191,6 +191,23 @@ def test_build_image_entry_point_matches_bf16_of_fp64_product():
         image_ulp_check(W, P, wp.cpu())
 
 
+@pytest.mark.parametrize("o,d,k,p_dtype", [
+    (8, 8, 8, "bf16"), (136, 72, 24, "bf16"),          # less than one tile, ragged edges
+    (128, 64, 64, "bf16"), (264, 4096, 72, "bf16"),    # exact tile; three row tiles, split depth
+    (1000, 3000, 200, "bf16"), (520, 1032, 1024, "bf16"),
+    (24, 40, 8, "f32"), (264, 2056, 136, "f32"),       # fp32 basis: one block; split depth
+])
+def test_image_tiles_and_edges(o, d, k, p_dtype):
+    g = G()
+    q = S.gen_basis(max(d, k), k, 3 + o)[:d]
+    P, W = S.store_basis(q, p_dtype), S.gen_weight(o, d, 4 + k)
+    out = torch.full((o + 1, k), 7.0, dtype=torch.bfloat16, device="cuda")   # one guard row
+    g.gsi_build_image(W.cuda(), P.cuda(), out=out)
+    assert torch.all(out[o] == 7.0)
+    # fp32 sums in another order than the oracle's: a rounding boundary is crossed by well under 5 %
+    assert image_ulp_check(W, P, out[:o].cpu()) < 0.05
+
+
 def test_forward_host_variant():
     x, P, Ws = make_small(768, 64, (3072,), 4, seed=81, outlier_every=2)
     g = G()
