@@ -141,11 +141,11 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W_host_array,
  * max_tokens tokens (gsi_forward_n).  x [n][d] fp32; y [n][sum d_out] fp32;
  * gate_mask_out [n] bytes (1 = slow path, W r added); rho_out [n] fp32 or NULL.
  * Each token is processed independently of the others in the call (Algorithm 1
- * is per token); its rounding can depend on the size of the call: calls of 2 or
- * more tokens (bf16 basis; k, d and every d_out multiples of 128) run the
- * contractions on the tensor cores with exactly split operands and another
- * summation order and add W r from r rounded to bf16 (|dy| <= 3e-3 max|y|);
- * with other shapes that rounding applies from 5 gated tokens per call on.
+ * is per token); its rounding can depend on the size of the call: calls of 5 or
+ * more tokens (bf16 basis; k, d and every d_out multiples of 128) sum in another
+ * order and add W r from r rounded to bf16 (|dy| <= 3e-3 max|y|); with other
+ * shapes that rounding applies only from 33 gated tokens per call on, where
+ * sum d_out * d is 2^25 or more, d a multiple of 64 and every d_out of 128.
  * Results of a given call are reproducible bit for bit.
  * Enqueues on `stream` and returns; n_tokens = 0 is a no-op.
  */
@@ -172,10 +172,10 @@ gsi_status_t gsi_forward_host(gsi_handle_t h, const float* x_host, int n_tokens,
  * a host application that owns all device memory, a library called while
  * someone else's stream capture is open, a latency-critical path that may not
  * enter the allocator.  Such a caller cannot provide the workspace gsi_create
- * wants.  Here the scratch (coefficients, residual, partial sums, fired-token
- * list) lives in a fixed array inside the library: about 1.5 MB that every GPU
- * which loads the library holds until the process exits.  No device status word can
- * be read back for this entry point (its kernels contain no bounded wait).
+ * wants.  Here the scratch (the words its CTAs exchange) lives in a fixed array
+ * inside the library: about 0.7 MB that every GPU which loads the library holds
+ * until the process exits.  No device status word can be read back for this entry
+ * point.
  *
  * The caller passes everything else: W_host_array (HOST array of n_maps DEVICE
  * pointers, W_j [d_out_j][d] bf16), d_out (HOST array), P [d][k], and W_P, the
@@ -189,8 +189,8 @@ gsi_status_t gsi_forward_host(gsi_handle_t h, const float* x_host, int n_tokens,
  * The first call on each device resolves the array's device address (with that
  * device current); make that first call before any stream capture begins.  The
  * call allocates nothing and frees nothing.  All calls on a device share the one
- * array, which keeps the previous call's contents: the counters that must start
- * at zero are cleared on `stream` at the start of every call.  Two calls whose
+ * array, which keeps the previous call's contents; every word carries the number of
+ * the call that wrote it, so nothing is cleared between calls.  Two calls whose
  * kernels overlap on the GPU (different streams, or one stream per thread) race
  * on the array - serialise them.
  */

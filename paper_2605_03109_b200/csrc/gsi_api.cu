@@ -21,7 +21,7 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 struct Layout {
   size_t wp, c, cpart, r, normpart, ctrl, fired, rho, x_stage, y_stage, gate_stage, rho_stage,
-      pk_acc, pk_slot, tc_rb, tc_ypart, f_pt, f_xb, f_cb, f_cpart, f_normpart, pk_pp, pk_wpp, total;
+      pk_acc, pk_slot, tc_rb, tc_ypart, f_pt, f_xb, f_cb, f_cpart, f_normpart, pk_pp, pk_wpp, fused, total;
   int O, n_slabs, slab_rows;
   bool tc, front, dense_tc, packed;
 };
@@ -106,6 +106,7 @@ Layout make_layout_ws(const gsi_desc_t* d) {
   L.pk_pp = take(packed ? (size_t)((d->d + 15) / 16 * 16) * k * 2 : 0);
   L.pk_wpp = take(packed ? (size_t)((O + 15) / 16) * persist_image_row_bytes(d->k, d->flags & GSI_FLAG_FP8_IMAGE) : 0);
   L.packed = packed;
+  L.fused = take(dense ? 0 : fused_words_bytes(d->d, d->k, d->max_tokens));
   L.total = at;
   return L;
 }
@@ -281,6 +282,8 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W, const void
   g.cb = reinterpret_cast<uint16_t*>(h->ws + L.f_cb);
   g.cpart3 = reinterpret_cast<float*>(h->ws + L.f_cpart);
   g.normpart3 = reinterpret_cast<float*>(h->ws + L.f_normpart);
+  g.fused_words = reinterpret_cast<unsigned long long*>(h->ws + L.fused);
+  g.fused_call = reinterpret_cast<unsigned*>(ctrl + 32);
 
   if (L.tc || L.dense_tc) {
     if (!build_tma_maps(g, L.front, desc->max_tokens, &h->tm)) {
@@ -775,7 +778,7 @@ static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t 
     io.log_step_stride = (long long)G * s->B;
     h->last_stream = stream;   // the joins below put all of the step's work in the caller's stream order
     return launch_generic_forward(h->gp, h->has_tm ? &h->tm : nullptr, io, s->B, st, nullptr,
-                                  s->front_stream ? &lane : nullptr) == cudaSuccess;
+                                  s->front_stream ? &lane : nullptr, s->mode == 1) == cudaSuccess;
   };
   for (int i = 0; i < G; ++i) {
     if (s->aux && i + 1 < G && s->pair_first[i]) {
@@ -815,7 +818,7 @@ gsi_status_t gsi_stack_launches_per_step(gsi_stack_t s, int* n_out) {
   }
   int n = 0;
   for (gsi_layer* h : s->groups) {
-    n += generic_launch_count(h->gp, s->B);
+    n += generic_launch_count(h->gp, s->B, s->mode == 1);
   }
   *n_out = n + 1;
   return GSI_OK;

@@ -118,7 +118,11 @@ struct GroupParams {
   uint16_t* cb;           // [3B rounded up to 16][k] bf16 terms of c
   float* cpart3;          // [proj_splits][B][k] split-K partial sums of c
   float* normpart3;       // [d/128][B][2] per-tile partial sums of ||r||^2, ||x||^2
+  // calls in one launch (gsi_fused.cu)
+  unsigned long long* fused_words;   // exchange words: fp32 value and call number
+  unsigned* fused_call;              // calls so far
 };
+constexpr int kFusedMaxGrid = 160;
 
 // The block that arrives last (of n_blocks) sums the per-part norm partials in part
 // order in double precision, writes gate / rho (Eq. (3.3)) and the ascending list of
@@ -221,8 +225,13 @@ struct ResidualLane {
 
 cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, const IoRef& io,
                                    int n_tokens, cudaStream_t stream, int* n_launches,
-                                   ResidualLane* lane = nullptr);
+                                   ResidualLane* lane = nullptr, bool per_stage = false);
 cudaError_t launch_advance_step(int* step, cudaStream_t stream);
+// A whole call in one cooperative launch, any supported shape.  leave_from > 0: from that many
+// gated tokens on their W r is left to a contraction that follows (g.r, g.fired, *g.n_fired).
+cudaError_t launch_forward_fused(const GroupParams& g, const IoRef& io, int n_tokens, int leave_from,
+                                 cudaStream_t stream);
+size_t fused_words_bytes(int d, int k, int max_tokens);
 // One token on CUDA cores: c, r = x - P c into g.r (x may be g.r itself), rho into
 // g.rho_scratch[0] (or io.rho), gate byte, fired list.  No image product.
 cudaError_t launch_project_residual(const GroupParams& g, const IoRef& io, cudaStream_t stream);
@@ -266,7 +275,7 @@ cudaError_t launch_transpose_bf16(const void* P, int d, int k, void* PT, cudaStr
 int front_proj_splits(int d, int k);
 int front_rows(int max_tokens);   // rows of the three-term operands
 // Kernel launches one generic forward of n_tokens tokens makes.
-int generic_launch_count(const GroupParams& g, int n_tokens);
+int generic_launch_count(const GroupParams& g, int n_tokens, bool per_stage);
 cudaError_t launch_build_image(const void* W, const void* P, int o, int d, int k, bool p_f32,
                                void* WP, cudaStream_t stream);
 

@@ -377,10 +377,24 @@ cudaError_t dispatch_vpl(const GroupParams& g, const IoRef& io, int n_tokens, cu
   }
 }
 
+// Which calls run as the one cooperative launch: those whose shape the tensor-core front end does
+// not take, and the small ones of the others.
+constexpr int kFusedFewTokens = 4;
+bool takes_fused(const GroupParams& g, bool front, int n_tokens) { return !front || n_tokens <= kFusedFewTokens; }
+
+// Gated tokens from which the fused launch leaves W r to the tensor-core contraction, 0 = never.
+// The fused launch reads W once for 32 tokens; the contraction reads it once for 64 but costs
+// three launches whether it has work or not.
+int leave_to_contraction(const GroupParams& g, bool tc, int n_tokens) {
+  if (!tc || g.tc_min_fired <= 0 || n_tokens <= 32 || (g.flags & GSI_FLAG_STATIC_PROJECTION)) return 0;
+  return (double)g.O * g.d >= 33554432.0 ? 33 : 0;
+}
+
 }  // namespace
 
 cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, const IoRef& io,
-                                   int n_tokens, cudaStream_t st, int* n_launches, ResidualLane* lane) {
+                                   int n_tokens, cudaStream_t st, int* n_launches, ResidualLane* lane,
+                                   bool per_stage) {
   int dummy = 0;
   if (!n_launches) n_launches = &dummy;
   int grid = (g.O + kWarps - 1) / kWarps;
@@ -394,6 +408,12 @@ cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, cons
   }
   cudaError_t e;
   const bool front = tm && g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens;
+  if (!per_stage && takes_fused(g, front, n_tokens)) {
+    const int leave = leave_to_contraction(g, tm != nullptr, n_tokens);
+    if ((e = launch_forward_fused(g, io, n_tokens, leave, st)) != cudaSuccess) return e;
+    *n_launches += 1;
+    return leave ? launch_residual_gemm_tc(g, *tm, io, leave, false, n_tokens, st, n_launches) : cudaSuccess;
+  }
   if (front) {
     e = launch_front_tc(g, *tm, io, n_tokens, st, n_launches);
   } else {
@@ -437,11 +457,13 @@ cudaError_t launch_gated_gemv(const GroupParams& g, const IoRef& io, cudaStream_
   return cudaGetLastError();
 }
 
-int generic_launch_count(const GroupParams& g, int n_tokens) {
+int generic_launch_count(const GroupParams& g, int n_tokens, bool per_stage) {
   // (a tensor-core contraction with one split over the depth writes y itself: no kernel that adds partial sums)
   const int add = tc_splits(g.O, g.d) > 1 ? 1 : 0;
   if (g.flags & GSI_FLAG_DENSE)
     return (g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens) ? 2 + add : 1;
+  if (!per_stage && takes_fused(g, g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens, n_tokens))
+    return 1 + (leave_to_contraction(g, g.tc_min_fired > 0, n_tokens) ? 2 + add : 0);
   const bool stat = g.flags & GSI_FLAG_STATIC_PROJECTION;
   if (g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens) return stat ? 4 : 5 + add;
   return 4 + (stat ? 0 : 1 + (g.tc_min_fired > 0 ? 2 + add : 0));

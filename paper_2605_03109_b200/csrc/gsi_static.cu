@@ -14,21 +14,15 @@ namespace {
 constexpr int kStaticMaxTokens = 4;
 constexpr int kStaticMaxK = 512;
 constexpr int kStaticMaxD = 16384;
-constexpr int kStaticMaxSlabs = 148;
 constexpr int kMaxDevices = 64;
 
-// layout of the scratch array (bytes, each block 256-aligned)
-constexpr size_t kOffCtrl = 0;                                                    // 256 B
-constexpr size_t kOffFired = 256;                                                 // 256 B
-constexpr size_t kOffRho = 512;                                                   // 256 B
-constexpr size_t kOffC = 768;                                                     // tokens*k floats
-constexpr size_t kOffNorm = kOffC + (size_t)kStaticMaxTokens * kStaticMaxK * 4;
-constexpr size_t kOffR = kOffNorm + 8192;
-constexpr size_t kOffCpart = kOffR + (size_t)kStaticMaxTokens * kStaticMaxD * 4;
+// layout of the scratch array (bytes)
+constexpr size_t kOffCtrl = 0;     // call counter, status word
+constexpr size_t kOffRho = 256;
+constexpr size_t kOffWords = 512;  // exchange words
 constexpr size_t kStaticScratchBytes =
-    kOffCpart + (size_t)kStaticMaxSlabs * kStaticMaxTokens * kStaticMaxK * 4;
-static_assert((size_t)kStaticMaxSlabs * kStaticMaxTokens * 2 * 4 <= 8192, "norm partials");
-static_assert(kOffNorm % 256 == 0 && kOffR % 256 == 0 && kOffCpart % 256 == 0, "alignment");
+    kOffWords + 8 * ((size_t)gsi::kFusedMaxGrid * kStaticMaxTokens * 34 +
+                     (size_t)kStaticMaxTokens * (kStaticMaxK + kStaticMaxD));
 
 // The scratch itself.  In host code this name is only a stand-in for the
 // symbol: it is NOT a device address and must never be handed to a kernel.
@@ -97,28 +91,17 @@ extern "C" gsi_status_t gsi_forward_static(const void* const* W_host_array, cons
   }
   g.off[n_maps] = off;
   g.O = off;
-  int slab = (d + kStaticMaxSlabs - 1) / kStaticMaxSlabs;
-  if (slab < 8) slab = 8;
-  g.slab_rows = slab;
-  g.n_slabs = (d + slab - 1) / slab;
-
   unsigned char* base = nullptr;
   gsi_status_t st = scratch_for_current_device(&base);
   if (st != GSI_OK) return st;
-  int* ctrl = reinterpret_cast<int*>(base + kOffCtrl);
-  g.n_fired = ctrl + 0;
-  g.counter = reinterpret_cast<unsigned*>(ctrl + 1);
-  g.status = ctrl + 2;
-  g.fired = reinterpret_cast<int*>(base + kOffFired);
+  if (fused_words_bytes(d, k, n_tokens) > kStaticScratchBytes - kOffWords) return GSI_ERR_UNSUPPORTED;
+  unsigned* ctrl = reinterpret_cast<unsigned*>(base + kOffCtrl);
+  g.fused_call = ctrl;
+  g.status = reinterpret_cast<int*>(ctrl + 1);
   g.rho_scratch = reinterpret_cast<float*>(base + kOffRho);
-  g.c = reinterpret_cast<float*>(base + kOffC);
-  g.normpart = reinterpret_cast<float*>(base + kOffNorm);
-  g.r = reinterpret_cast<float*>(base + kOffR);
-  g.cpart = reinterpret_cast<float*>(base + kOffCpart);
-
-  // The array keeps whatever the last call left.  The arrival counter and the
-  // fired count must start at zero; everything else is written before it is read.
-  if (cudaMemsetAsync(ctrl, 0, 256, stream) != cudaSuccess) return GSI_ERR_CUDA;
+  g.fused_words = reinterpret_cast<unsigned long long*>(base + kOffWords);
+  // The array keeps whatever the last call left; its exchange words carry that call's number,
+  // which is not this call's, so nothing has to be cleared.
 
   IoRef io{};
   io.x = x;
@@ -127,6 +110,5 @@ extern "C" gsi_status_t gsi_forward_static(const void* const* W_host_array, cons
   io.rho = rho_out;
   io.step = nullptr;
   io.n_steps = 1;
-  return launch_generic_forward(g, nullptr, io, n_tokens, stream, nullptr) == cudaSuccess ? GSI_OK
-                                                                                  : GSI_ERR_CUDA;
+  return launch_forward_fused(g, io, n_tokens, 0, stream) == cudaSuccess ? GSI_OK : GSI_ERR_CUDA;
 }

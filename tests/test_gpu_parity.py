@@ -69,6 +69,46 @@ def test_small_and_odd_shapes(d, k, d_out, T, batch):
         assert 0 < st["gate_rate"] <= 1.0
 
 
+@pytest.mark.parametrize("d,k,d_out,n,p_dtype", [
+    (8, 8, (8,), 1, "f32"), (40, 40, (8, 24), 4, "bf16"),         # fewer rows than CTAs
+    (264, 24, (2408,), 5, "bf16"), (4104, 248, (48,), 8, "f32"),  # a few tokens; 17 rows of W per CTA
+    (6400, 16, (4744, 8), 9, "bf16"), (1000, 1000, (136,), 16, "bf16"),
+    (2056, 200, (5000,), 17, "f32"), (16384, 40, (200,), 32, "bf16"),   # W r in parts of the width
+    (1032, 520, (72, 1160), 33, "bf16"), (3000, 72, (504,), 64, "f32"),
+    (4096, 64, (8192,), 40, "bf16"),                              # W r left to the contraction
+])
+def test_one_launch_forward_edges(d, k, d_out, n, p_dtype):
+    """Calls that run as one cooperative launch, against the oracle; a token's result does not
+    depend on the tokens it travels with (unless W r goes through bf16 in the contraction)."""
+    x, P, Ws = make_small(d, k, d_out, n, seed=d + n, noise=0.02, p_dtype=p_dtype,
+                          outlier_every=1 if n == 40 else 3)
+    _, y, gate, rho = run_layer(x, P, Ws, 0.3, n)
+    compare_group(x, P, Ws, 0.3, y, gate, rho)
+    if n > 4 and n != 40:
+        _, y1, gate1, rho1 = run_layer(x, P, Ws, 0.3, 3)
+        assert np.array_equal(y, y1) and np.array_equal(gate, gate1) and np.array_equal(rho, rho1)
+
+
+def test_one_launch_forward_on_two_streams_at_once():
+    """Two handles on two streams: cooperative launches that compete for the SMs all complete."""
+    g = G()
+    handles = []
+    for i in range(2):
+        x, P, Ws = make_small(1024, 64, (2048,), 2, seed=60 + i, outlier_every=2)
+        lay = g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=2)
+        handles.append((lay, x.cuda(), torch.cuda.Stream()))
+    refs = [lay.forward(x)[0].clone() for lay, x, _ in handles]
+    torch.cuda.synchronize()
+    outs = []
+    for _ in range(100):
+        for i, (lay, x, st) in enumerate(handles):
+            with torch.cuda.stream(st):
+                outs.append((i, lay.forward(x, stream=st)[0]))
+    torch.cuda.synchronize()
+    assert all(lay.status() == 0 for lay, _, _ in handles)
+    assert all(torch.equal(y, refs[i]) for i, y in outs)
+
+
 def test_config1_literal_batch1_all_tokens():
     st = S.config1()
     m = S.materialize_group(st, 0, 0, st.steps)
