@@ -27,6 +27,7 @@ struct Layout {
 };
 
 constexpr int kTcMinFired = 5;  // fewer fired tokens: one pass of the CUDA-core GEMV
+constexpr double kOwnStreamBytes = 262144.0;   // W rows of a CTA up to which a gated residual stays on its group's share
 constexpr int kFrontMinTokens = 2;  // single-token calls: the CUDA-core front end
 
 bool tc_shapes_ok(const gsi_desc_t* d) {
@@ -130,7 +131,7 @@ struct gsi_stack {
   int mode;                 // 0 auto, 1 generic kernels, 2 persistent kernel required
   bool persistent;          // the persistent kernel is in use
   int grid;                 // CTAs of the persistent kernel (= SMs)
-  bool has_pairs;           // some phase of the persistent schedule holds two groups
+  bool has_pairs;           // some phase of the persistent schedule holds several groups
   int common_k;             // rank shared by every gated group of the persistent schedule, or 0
   PersistGroup* dev_groups; // device table
   int* dev_phase_first;     // device: first group of every phase of the persistent schedule
@@ -493,16 +494,15 @@ gsi_status_t gsi_stack_create(int n_groups, const gsi_handle_t* groups, void* wo
 }
 
 // The basis rows and the image rows are dealt to the CTAs of a group's share in units of 16
-// rows.  One CTA's share fits its buffers, and the 16 KB chunks of its basis slab, and of its
-// image slab, each fit the ring together (pass 1 and the image rows run with every chunk of
-// their slab resident; one chunk per lane is waited for).
+// rows: the least share whose rows fit a CTA's buffers.
+static int least_share(const gsi_layer* h) {
+  const int pt = (h->desc.d + 15) / 16, ot = (h->lay.O + 15) / 16;
+  return std::max((pt + kPersistMaxPRows / 16 - 1) / (kPersistMaxPRows / 16),
+                  (ot + kPersistMaxORows / 16 - 1) / (kPersistMaxORows / 16));
+}
 static bool rows_fit(const gsi_layer* h, int ctas) {
-  if (ctas <= 0) return false;
   if ((h->desc.flags & GSI_FLAG_DENSE) || h->desc.k <= 0) return true;
-  const int pg = ((h->desc.d + 15) / 16 + ctas - 1) / ctas, og = ((h->lay.O + 15) / 16 + ctas - 1) / ctas;
-  if (pg * 16 > kPersistMaxPRows || og * 16 > kPersistMaxORows) return false;
-  const int gc = std::max(1, 16384 / (h->desc.k * 32));   // groups per chunk
-  return (pg + gc - 1) / gc <= 10 && (og + gc - 1) / gc <= 10;
+  return least_share(h) <= ctas;
 }
 
 // W stream geometry of a group: whole rows per contiguous piece of at most 32 KB.
@@ -533,17 +533,66 @@ static bool persistent_eligible(const gsi_stack* s, int grid) {
   return true;
 }
 
-// CTAs given to the first group of a pair: in proportion to the bytes its fast path
-// streams, between a quarter and three quarters of the grid; 0 if the rows of either
-// group do not fit its share (the pair then runs one group after the other).
-static int pair_split(const gsi_layer* a, const gsi_layer* b, int grid) {
-  if ((a->desc.flags | b->desc.flags) & GSI_FLAG_DENSE) return 0;
-  const double wa = (double)(a->desc.d + a->lay.O) * a->desc.k;
-  const double wb = (double)(b->desc.d + b->lay.O) * b->desc.k;
-  int na = (int)(grid * wa / (wa + wb) + 0.5);
-  na = std::max(grid / 4, std::min(grid - grid / 4, na));
-  if (!rows_fit(a, na) || !rows_fit(b, grid - na)) return 0;
-  return na;
+// Time of a phase of groups [i, i + len) in microseconds as the shares in `ncta` (filled in) leave
+// it, or a negative number when the rows do not fit.  A tick costs about 4 us whatever it carries
+// (the barriers, the scalar code and the latency of its sections); on top of that either the memory
+// system (6 bytes per picosecond) or the CTA with the longest row passes: rounds of fifteen 16-row
+// units, 0.85 us each at k = 256, and pass 1, 0.1 us per unit (per-warp timeline at the GPT-J
+// shapes).  The CTAs go one by one to the group whose rows take longest, basis rows counting
+// twice (pass 1 and residual).
+static double phase_cost(const gsi_stack* s, int i, int len, int* ncta) {
+  double bytes = 0.0, load[kPersistMaxLen];
+  int left = s->grid;
+  for (int j = 0; j < len; ++j) {
+    const gsi_layer* h = s->groups[i + j];
+    ncta[j] = least_share(h);
+    left -= ncta[j];
+    load[j] = (2.0 * h->desc.d + h->lay.O) * h->desc.k;
+    bytes += 2.0 * ((double)h->desc.d + h->lay.O) * h->desc.k;
+  }
+  if (left < 0) return -1.0;
+  for (; left > 0; --left) {
+    int at = 0;
+    for (int j = 1; j < len; ++j)
+      if (load[j] / ncta[j] > load[at] / ncta[at]) at = j;
+    ++ncta[at];
+  }
+  double rows = 0.0;
+  for (int j = 0; j < len; ++j) {
+    const gsi_layer* h = s->groups[i + j];
+    const int pt = ((h->desc.d + 15) / 16 + ncta[j] - 1) / ncta[j], ot = ((h->lay.O + 15) / 16 + ncta[j] - 1) / ncta[j];
+    const int rounds = (pt + ot + kPersistConsumerWarps - 1) / kPersistConsumerWarps;
+    rows = std::max(rows, (0.85 * rounds + 0.1 * pt) * h->desc.k / 256.0);
+  }
+  return 4.0 + std::max(bytes / 6.0e6, rows);
+}
+
+// The phases of the persistent schedule: consecutive groups in one phase as far as that shortens
+// the step (inputs are staged before it), chosen over all partitions of the order.
+static void plan_phases(gsi_stack* s, std::vector<int>* first, std::vector<int>* share) {
+  const int G = (int)s->groups.size();
+  std::vector<double> best(G + 1, 0.0);   // cost of groups [i, G)
+  std::vector<int> len(G, 1);
+  int ncta[kPersistMaxLen];
+  auto dense = [&](int i) { return (s->groups[i]->desc.flags & GSI_FLAG_DENSE) != 0; };
+  for (int i = G - 1; i >= 0; --i) {
+    best[i] = -1.0;
+    for (int l = 1; l <= kPersistMaxLen && i + l <= G; ++l) {
+      if (l > 1 && (dense(i) || dense(i + l - 1))) break;   // a dense group is a phase of its own
+      const double c = dense(i) ? 4.0 : phase_cost(s, i, l, ncta);
+      if (c < 0.0) break;
+      if (best[i] < 0.0 || c + best[i + l] < best[i]) {
+        best[i] = c + best[i + l];
+        len[i] = l;
+      }
+    }
+  }
+  first->clear();
+  share->assign(G, s->grid);
+  for (int i = 0; i < G; i += len[i]) {
+    first->push_back(i);
+    if (!dense(i)) (void)phase_cost(s, i, len[i], share->data() + i);
+  }
 }
 
 gsi_status_t gsi_stack_set_concurrent(gsi_stack_t s, int first_group, int enable) {
@@ -635,10 +684,7 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
       const GroupParams& gp = h->gp;
       pg.P = reinterpret_cast<const uint16_t*>(h->ws + h->lay.pk_pp);
       pg.WP = reinterpret_cast<const uint16_t*>(h->ws + h->lay.pk_wpp);
-      for (int j = 0; j < gp.n_maps; ++j) {
-        pg.W[j] = gp.W[j];
-        pg.w_rows[j] = (short)((gp.d_out[j] + s->grid - 1) / s->grid);
-      }
+      for (int j = 0; j < gp.n_maps; ++j) pg.W[j] = gp.W[j];
       pg.w_pr = w_piece_rows(gp.d);
       for (int j = 0; j <= gp.n_maps; ++j) pg.off[j] = gp.off[j];
       pg.n_maps = gp.n_maps;
@@ -657,48 +703,42 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
       pg.xmax = reinterpret_cast<unsigned*>(h->ws + h->lay.pk_slot);
       pg.pub = reinterpret_cast<unsigned long long*>(h->ws + h->lay.pk_slot + (size_t)kPersistMaxGrid * 4);
       pg.bar = h->bar;
-      pg.cta0 = 0;
-      pg.ncta = s->grid;
-      pg.phase_len = 1;
       pg.x_step_stride = (long long)s->B * gp.d;
     }
-    // pairs of independent groups split the grid
-    for (int i = 0; i + 1 < G; ++i) {
-      if (!s->pair_first[i]) continue;
-      const int na = pair_split(s->groups[i], s->groups[i + 1], s->grid);
-      if (na == 0) continue;
-      PersistGroup &a = s->host_groups[i], &b = s->host_groups[i + 1];
-      a.ncta = na;
-      b.cta0 = na;
-      b.ncta = s->grid - na;
-      a.phase_len = b.phase_len = 2;
-    }
-    for (int i = 0; i < G; ++i) {
-      PersistGroup& pg = s->host_groups[i];
-      // rows are dealt in groups of 16: CTA c of the share owns groups [c n / ncta, (c + 1) n / ncta)
-      // (the first n CTAs one group each when there are fewer groups than CTAs)
-      const int pgroups = (pg.d + 15) / 16, ogroups = (pg.O + 15) / 16;
-      pg.p_rows = 16 * ((pgroups + pg.ncta - 1) / pg.ncta);
-      pg.o_rows = 16 * ((ogroups + pg.ncta - 1) / pg.ncta);
-      pg.n_contrib = std::min(pg.ncta, pgroups);
-    }
+    std::vector<int> share;
+    plan_phases(s, &s->host_phase_first, &share);
     s->has_pairs = false;
     s->common_k = -1;
-    for (int i = 0; i < G; ++i) {
-      if (s->host_groups[i].flags & GSI_FLAG_DENSE) continue;
-      const int k = s->host_groups[i].k;
-      s->common_k = s->common_k < 0 || s->common_k == k ? k : 0;
+    for (size_t ph = 0; ph < s->host_phase_first.size(); ++ph) {
+      const int i0 = s->host_phase_first[ph];
+      const int i1 = ph + 1 < s->host_phase_first.size() ? s->host_phase_first[ph + 1] : G;
+      if (i1 - i0 > 1) s->has_pairs = true;
+      int at = 0;
+      for (int i = i0; i < i1; ++i) {
+        PersistGroup& pg = s->host_groups[i];
+        const gsi_layer* h = s->groups[i];
+        pg.cta0 = at;
+        pg.ncta = share[i];
+        pg.phase_len = i1 - i0;
+        at += share[i];
+        // rows are dealt in groups of 16: CTA c of the share owns groups [c n / ncta, (c + 1) n / ncta)
+        // (the first n CTAs one group each when there are fewer groups than CTAs)
+        const int pgroups = (pg.d + 15) / 16, ogroups = (pg.O + 15) / 16;
+        pg.p_rows = 16 * ((pgroups + pg.ncta - 1) / pg.ncta);
+        pg.o_rows = 16 * ((ogroups + pg.ncta - 1) / pg.ncta);
+        pg.n_contrib = std::min(pg.ncta, pgroups);
+        // W r on the group's own share where a CTA's rows are few pieces: such a stream is a chain
+        // of latencies (2.5 us whatever its size), and those of a phase then run side by side
+        const bool own = !(pg.flags & GSI_FLAG_DENSE) && w_rows_fit(h, pg.ncta) &&
+                         (double)((pg.O + pg.ncta - 1) / pg.ncta) * pg.d * 2 <= kOwnStreamBytes;
+        pg.w_cta0 = (short)(own ? pg.cta0 : 0);
+        pg.w_ncta = (short)(own ? pg.ncta : s->grid);
+        for (int j = 0; j < h->gp.n_maps; ++j)
+          pg.w_rows[j] = (short)((h->gp.d_out[j] + pg.w_ncta - 1) / pg.w_ncta);
+        if (!(pg.flags & GSI_FLAG_DENSE)) s->common_k = s->common_k < 0 || s->common_k == pg.k ? pg.k : 0;
+      }
     }
     if (s->common_k < 0) s->common_k = 0;
-    s->host_phase_first.clear();
-    for (int i = 0; i < G;) {   // length of the phase after each group's
-      const int len = s->host_groups[i].phase_len;
-      s->host_phase_first.push_back(i);
-      const int nxt = i + len < G ? s->host_groups[i + len].phase_len : 0;
-      for (int j = 0; j < len; ++j) s->host_groups[i + j].next_len = nxt;
-      if (len == 2) s->has_pairs = true;
-      i += len;
-    }
     s->n_phases = (int)s->host_phase_first.size();
     const float** dev_ptrs = reinterpret_cast<const float**>(
         reinterpret_cast<char*>(s->dev_groups) + (size_t)G * 512);

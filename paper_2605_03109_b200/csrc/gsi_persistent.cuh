@@ -6,7 +6,8 @@
 namespace gsi {
 
 constexpr int kPersistConsumerWarps = 15;  // + 1 producer warp = 16 warps: registers are allotted per 4 warps
-constexpr int kPersistMaxPRows = 256;   // basis rows one CTA may own
+constexpr int kPersistMaxPRows = 320;   // basis rows one CTA may own
+constexpr int kPersistMaxLen = 7;       // groups of one phase (lanes of the warp that polls their scalars)
 constexpr int kPersistMaxORows = 512;   // output rows one CTA may own
 constexpr int kPersistMaxGrid = 160;    // CTAs (tagged words per group)
 constexpr int kPersistMaxTokens = 2;    // tokens per step served by one launch per token (more: batched kernels)
@@ -49,15 +50,15 @@ struct PersistGroup {
   float pmax;                        // max |P| (patched in on the device at bind time)
   int p_rows, o_rows;                // most rows one CTA owns of P and of the images (multiples of 16)
   int n_contrib;                     // CTAs that own basis rows: the first min(ncta, ceil(d / 16)) of the share
-  // Two consecutive groups whose inputs do not depend on each other's outputs may form one
-  // phase: CTAs [cta0, cta0 + ncta) run this group's projection, residual and image while the
-  // rest of the grid runs its partner's.  A gated residual always streams W with the whole grid.
+  // Consecutive groups form a phase (their inputs are staged before the step): CTAs
+  // [cta0, cta0 + ncta) run this group's projection, residual and image.
   int cta0, ncta;                    // this group's share of the grid (0, grid when alone)
-  int phase_len;                     // groups in this group's phase: 1, or 2 for both of a pair
-  int next_len;                      // groups in the phase after this group's (0 at the end)
-  // W stream (gated residual, dense baseline): every CTA owns w_rows[j] consecutive rows of
-  // every map j (one contiguous run of memory), copied as contiguous pieces of w_pr whole rows
-  // (at most 32 KB).
+  int phase_len;                     // groups in this group's phase
+  // W stream (gated residual, dense baseline): CTA w_cta0 + i, i < w_ncta, owns rows
+  // [i w_rows[j], (i + 1) w_rows[j]) of every map j (one contiguous run of memory), copied as
+  // contiguous pieces of w_pr whole rows (at most 32 KB).  Large maps use the whole grid, small
+  // ones the group's own share, so that the streams of a phase run side by side.
+  short w_cta0, w_ncta;
   short w_rows[GSI_MAX_MAPS];
   int w_pr;
 };

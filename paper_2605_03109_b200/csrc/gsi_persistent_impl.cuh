@@ -63,6 +63,7 @@ constexpr int kChunk = 16384;               // largest chunk
 static_assert(kPersistMaxWRows <= kPersistConsumerWarps * 32, "one thread per row of a W stream");
 constexpr int kWVecMax = 5;                 // 16-byte vectors of a row one lane may own in the W stream (d <= 16384)
 constexpr unsigned kLocalSpinLimit = 1u << 20;   // waits inside the CTA (ring, producer hand-off)
+constexpr int kP1Chunks = 7;                // chunks of a basis slab that pass 1 waits for at a time
 constexpr int kCountShift = 54;
 constexpr unsigned long long kOne = 1ull << kCountShift;
 
@@ -71,16 +72,26 @@ constexpr unsigned long long kOne = 1ull << kCountShift;
 struct Plan {
   short gi;        // the group whose fast path (or dense stream) this CTA runs in this tick
   short gi0;       // first group of the tick's phase
-  unsigned char len, next_len;   // groups in this phase and in the next
+  unsigned char len;             // groups in this phase
   unsigned char kind;            // 0 nothing (closing ticks), 1 gated subspace group, 2 dense group
   unsigned char zeroer;          // this CTA clears the group's counters for the next launch
   short pg, og;                  // 16-row groups of the basis slab and of the image slab
   short pchunks, ochunks;        // ... and their ring chunks
   int p0, o0;                    // first rows
   short lc, n_contrib;           // index within the group's share of the grid; CTAs that own basis rows
-  short gc_log2, pad;            // log2 of the 16-row groups per 16 KB chunk
+  short gc_log2;                 // log2 of the 16-row groups per 16 KB chunk
 };
 static_assert(sizeof(Plan) == 32, "one plan record");
+
+// What every CTA needs of a group that it did not run: its gate and the arrivals of its r.
+struct Settle {
+  unsigned long long* r2;    // accumulator of ||r||^2 of this launch
+  unsigned long long* pub;   // published ||x||^2 and threshold
+  unsigned* bar;             // arrival counter before its gated residual
+  short n_contrib;
+  short mode;                // 0 gated, 1 static projection, 2 dense
+};
+static_assert(sizeof(Settle) == 32, "one record");
 
 // Groups [a, b) of n that part i of `parts` owns: an even split, or one group each for the
 // first n parts when there are fewer groups than parts.
@@ -101,19 +112,21 @@ constexpr int kOffOff = 1280;       // offset of every chunk in flight within th
 constexpr int kOffMisc = 1536;      // scalars
 constexpr int kOffTrace = 1792;     // cycle counters of the trace (16 words)
 constexpr int kOffProd = 1920;      // state of the producer thread (16 bytes)
-constexpr int kOffX = 2048;         // x of this CTA's basis rows, two buffers (kPersistMaxPRows floats each)
-constexpr int kOffXt = kOffX + 3 * kPersistMaxPRows * 4;  // ... as three bf16 terms in A-operand order, two buffers (16 tile rows x 256 B each)
-constexpr int kOffCb = kOffXt + 2 * 4096;                 // c as three bf16 terms in B-operand order (32 tile columns x 256 B)
+constexpr int kOffX = 2048;         // x of this CTA's basis rows, three buffers (kPersistMaxPRows floats each)
+constexpr int kOffXt = kOffX + 3 * kPersistMaxPRows * 4;  // ... as three bf16 terms in A-operand order, two buffers
+constexpr int kXtBytes = kPersistMaxPRows / 16 * 256;     // (256 B per tile row)
+constexpr int kOffCb = kOffXt + 2 * kXtBytes;                 // c as three bf16 terms in B-operand order (32 tile columns x 256 B)
 constexpr int kOffFx = kOffCb + 8192;                     // fixed-point partial c and ||x||^2, source of the bulk reduction (514 words)
 constexpr int kOffPlan = kOffFx + 4224;                   // the launch's plan (kPersistMaxTicks records)
-constexpr int kOffDesc = kOffPlan + kPersistMaxTicks * 32;   // 8 group descriptors, 256 B each
-constexpr int kDescSlots = 16;
+constexpr int kOffSettle = kOffPlan + kPersistMaxTicks * 32;   // one record per group
+constexpr int kOffDesc = kOffSettle + kPersistMaxTicks * 32;   // descriptors of this CTA's groups, by phase
+constexpr int kDescSlots = 8;
 constexpr int kOffYacc = kOffDesc + kDescSlots * 512;     // W stream: per-warp partial results (kNW x kPersistMaxWRows floats)
 constexpr int kOffRing = ((kOffYacc + kNW * kPersistMaxWRows * 4 + 1023) / 1024) * 1024;
 constexpr int kRingBytes = (232448 - kOffRing) / 1024 * 1024;
 constexpr int kSmemBytes = kOffRing + kRingBytes;
 static_assert(kSmemBytes <= 232448, "shared memory budget of one sm_100 CTA");
-static_assert(kOffXt % 16 == 0 && kOffCb % 16 == 0 && kOffFx % 16 == 0 && kOffPlan % 16 == 0 && kOffDesc % 16 == 0, "alignment");
+static_assert(kOffXt % 16 == 0 && kOffCb % 16 == 0 && kOffFx % 16 == 0 && kOffSettle % 16 == 0 && kOffPlan % 16 == 0 && kOffDesc % 16 == 0, "alignment");
 static_assert(sizeof(PersistGroup) <= 512 && sizeof(PersistGroup) % 4 == 0, "descriptor slot");
 constexpr int kDescWords = (int)(sizeof(PersistGroup) / 4);
 
@@ -121,7 +134,7 @@ struct Misc {
   int abort;
   unsigned amax_bits[2];    // by tick parity: max |x| of the phase's group (>= 0x7f800000: a non-finite token)
   float x2_part[2];         // this CTA's sum of x^2 over its rows, by tick parity
-  int fire[4];              // decisions on the previous phase's groups, by tick parity: 1 = stream W
+  unsigned fire[2];         // decisions on the previous phase's groups, by tick parity: bit u = stream W of group u
   double x2;                // ||x||^2 of this phase's group
   unsigned long long r2_acc;   // this CTA's ||r||^2 of the tick's phase in fixed point; the upper bits count the warps
   volatile unsigned decision[4];   // hand-off to the producer: (phase + 1) << 8 | fire mask
@@ -316,8 +329,9 @@ __device__ __forceinline__ bool produce_w(const PersistGroup& g, unsigned char* 
   // few hundred cycles: the out-of-line acquire with its state in shared memory is too slow)
   unsigned n = prs.n, lin = prs.lin, tail_n = prs.tail_n, tail_lin = prs.tail_lin;
   bool ok = true;
-  const int cta = blockIdx.x;
+  const int cta = (int)blockIdx.x - g.w_cta0;
   const int d = g.d, pr = g.w_pr;
+  if (cta < 0 || cta >= g.w_ncta) return true;
   for (int j = 0; j < g.n_maps && ok; ++j) {
     const int dout = g.off[j + 1] - g.off[j], rows = g.w_rows[j];
     const int row0 = cta * rows;
@@ -425,19 +439,17 @@ __device__ void producer(const PersistParams& p, unsigned char* smem, Misc* misc
           break;
         }
       }
-      wmask = v & 3u;
+      wmask = v & 0xffu;
     }
     // one call site for every W stream of the tick: the gated groups, then a dense group
     if (wmask || pl.kind == 2) {
 #pragma unroll 1
-      for (int u = 0; ok && u < 3; ++u) {
-        const PersistGroup* gw = nullptr;
-        if (u < 2) {
-          if (u < len_pp && (wmask & (1u << u))) gw = &p.groups[g_pp + u];
-        } else if (pl.kind == 2) {
-          gw = g;
-        }
-        if (gw) ok = produce_w(*gw, smem);
+      for (; ok && (wmask || pl.kind == 2);) {
+        const PersistGroup* gw = g;
+        if (wmask) gw = &p.groups[g_pp + __ffs(wmask) - 1];
+        ok = produce_w(*gw, smem);
+        if (!wmask) break;
+        wmask &= wmask - 1;
       }
     }
   }
@@ -708,7 +720,7 @@ __device__ __forceinline__ unsigned w_run(const PersistGroup* gp, const WGeo& q,
   Misc* misc = reinterpret_cast<Misc*>(smem + kOffMisc);
   volatile int* abort = &misc->abort;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int cta = blockIdx.x;
+  const int cta = (int)blockIdx.x - gp->w_cta0;   // (within the group's share of the stream)
   Trace tr;
   tr.acc = (traced && tid == 0) ? reinterpret_cast<unsigned long long*>(smem + kOffTrace) : nullptr;
   tr.t = clock64();
@@ -800,7 +812,7 @@ __device__ __noinline__ void xmax_collect(unsigned char* smem, int tt, unsigned 
   const Plan& pn = reinterpret_cast<const Plan*>(smem + kOffPlan)[tt];
   Misc* misc = reinterpret_cast<Misc*>(smem + kOffMisc);
   const PersistGroup& gn =
-      *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (pn.gi & (kDescSlots - 1)) * 512);
+      *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (tt & (kDescSlots - 1)) * 512);
   const int lane = threadIdx.x & 31;
   unsigned w[kXmaxWords] = {w0, w1, w2, w3, w4};
   unsigned m = 0, it = 0;
@@ -836,7 +848,7 @@ __device__ __noinline__ void stat_warp_step(unsigned char* smem, int tt, bool re
   if (pn.kind != 1) return;
   const int lane = threadIdx.x & 31;
   const PersistGroup& gn =
-      *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (pn.gi & (kDescSlots - 1)) * 512);
+      *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (tt & (kDescSlots - 1)) * 512);
   float* sx = reinterpret_cast<float*>(smem + kOffX) + (tt % 3) * kPersistMaxPRows;
   const int rows = pn.pg * 16;
   if (request) {
@@ -854,7 +866,7 @@ __device__ __noinline__ void stat_warp_step(unsigned char* smem, int tt, bool re
   }
   cp_async_wait_all();
   __syncwarp();
-  unsigned short* xt = reinterpret_cast<unsigned short*>(smem + kOffXt) + (tt & 1) * 2048;
+  unsigned short* xt = reinterpret_cast<unsigned short*>(smem + kOffXt) + (tt & 1) * (kXtBytes / 2);
   Misc* misc = reinterpret_cast<Misc*>(smem + kOffMisc);
   float amax = 0.f, s2 = 0.f;
 #pragma unroll 1
@@ -887,6 +899,21 @@ __device__ __noinline__ void stat_warp_step(unsigned char* smem, int tt, bool re
 // the producer and the consumers part).
 template <bool kPairs, int kK>
 __device__ __forceinline__ void make_plan(const PersistParams& p, unsigned char* smem) {
+  Settle* settle = reinterpret_cast<Settle*>(smem + kOffSettle);
+  const unsigned parity = (unsigned)*p.epoch & 1u;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < p.n_groups; i += kThreadsP) {
+    const PersistGroup* g = p.groups + i;
+    const int k = __ldg(&g->k);
+    const unsigned flags = __ldg(&g->flags);
+    Settle s;
+    s.r2 = g->acc + (size_t)parity * (k + 4) + k + 2;
+    s.pub = g->pub;
+    s.bar = g->bar + 2 + parity;
+    s.n_contrib = (short)__ldg(&g->n_contrib);
+    s.mode = (flags & GSI_FLAG_DENSE) ? 2 : (flags & GSI_FLAG_STATIC_PROJECTION) ? 1 : 0;
+    settle[i] = s;
+  }
   Plan* plan = reinterpret_cast<Plan*>(smem + kOffPlan);
   const int cta = blockIdx.x, n_ticks = p.n_phases + 2;
 #pragma unroll 1
@@ -898,13 +925,13 @@ __device__ __forceinline__ void make_plan(const PersistParams& p, unsigned char*
       const PersistGroup* ga = p.groups + gi0;
       const int len = kPairs ? __ldg(&ga->phase_len) : 1;
       int gi = gi0;
-      if (kPairs && len == 2 && cta >= __ldg(&ga->cta0) + __ldg(&ga->ncta)) gi = gi0 + 1;
+      if (kPairs)
+        while (gi + 1 < gi0 + len && cta >= __ldg(&p.groups[gi + 1].cta0)) ++gi;
       const PersistGroup* g = p.groups + gi;
       const bool dense = __ldg(&g->flags) & GSI_FLAG_DENSE;
       pl.gi = (short)gi;
       pl.gi0 = (short)gi0;
       pl.len = (unsigned char)len;
-      pl.next_len = (unsigned char)(kPairs ? __ldg(&ga->next_len) : min(__ldg(&ga->next_len), 1));
       pl.kind = dense ? 2 : 1;
       const int lc = cta - __ldg(&g->cta0), ncta = __ldg(&g->ncta);
       pl.lc = (short)lc;
@@ -963,26 +990,28 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
   Trace tr;
   tr.start(p, smem);
 
-  auto desc = [&](int i) -> const PersistGroup& {
-    return *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (i & (kDescSlots - 1)) * 512);
+  const Settle* settle = reinterpret_cast<const Settle*>(smem + kOffSettle);
+  // the descriptor of the group this CTA runs in phase ph (read only when there is one)
+  auto desc = [&](int ph) -> const PersistGroup& {
+    return *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (ph & (kDescSlots - 1)) * 512);
   };
-  // groups [g0, g0 + cnt) from the device table into their slots (threads 0 .. cnt*kDescWords-1)
-  auto desc_load = [&](int g0, int cnt) -> uint32_t {
-    return tid < cnt * kDescWords ? __ldg(reinterpret_cast<const uint32_t*>(p.groups + g0) + tid) : 0u;
+  // ... from the device table into its slot (threads 0 .. kDescWords - 1)
+  auto desc_load = [&](int ph) -> uint32_t {
+    return ph < p.n_phases && tid < kDescWords ? __ldg(reinterpret_cast<const uint32_t*>(p.groups + plan[ph].gi) + tid)
+                                               : 0u;
   };
-  auto desc_store = [&](int g0, int cnt, uint32_t w) {
-    if (tid < cnt * kDescWords) {
-      const int j = tid / kDescWords;
-      reinterpret_cast<uint32_t*>(smem + kOffDesc + ((g0 + j) & (kDescSlots - 1)) * 512)[tid - j * kDescWords] = w;
-    }
+  auto desc_store = [&](int ph, uint32_t w) {
+    if (ph < p.n_phases && tid < kDescWords)
+      reinterpret_cast<uint32_t*>(smem + kOffDesc + (ph & (kDescSlots - 1)) * 512)[tid] = w;
   };
   // the operand rows / columns beyond the three terms stay zero for the whole launch
-  for (int i = tid; i < (2 * 4096 + 8192) / 4; i += kNC) reinterpret_cast<uint32_t*>(smem + kOffXt)[i] = 0u;
+  for (int i = tid; i < (2 * kXtBytes + 8192) / 4; i += kNC) reinterpret_cast<uint32_t*>(smem + kOffXt)[i] = 0u;
   // the descriptors of the first two phases (descriptors are staged three phases ahead; the
   // tick before the first phase stages the third)
   {
-    const int cnt = plan[0].len + (p.n_phases > 1 ? plan[1].len : 0);
-    desc_store(0, cnt, desc_load(0, cnt));
+    const uint32_t w0 = desc_load(0), w1 = desc_load(1);
+    desc_store(0, w0);
+    desc_store(1, w1);
   }
   csync();
   if (warp == kStatWarp) {   // the first phase's rows of x: nothing ran ahead of them
@@ -990,7 +1019,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     stat_warp_step(smem, 0, false, slot_io, p.token, tag);
     if (plan[0].kind == 1) {
       unsigned xw[kXmaxWords];
-      xmax_issue(desc(plan[0].gi).xmax, plan[0].n_contrib, xw);
+      xmax_issue(desc(0).xmax, plan[0].n_contrib, xw);
       xmax_collect(smem, 0, tag, p.spin_limit, p.status, xw[0], xw[1], xw[2], xw[3], xw[4]);
     }
   }
@@ -1005,7 +1034,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     const Plan pl = t >= 0 ? plan[t] : Plan{};
     const Plan pf = t + 1 < p.n_phases ? plan[t + 1] : Plan{};   // the phase whose pass 1 runs in this tick
     const bool gsi = pl.kind == 1, dense = pl.kind == 2, gsi_f = pf.kind == 1;
-    const PersistGroup& g = desc(pl.gi);        // read only when the tick has a group
+    const PersistGroup& g = desc(t);            // read only when the tick has a group
     const int k = gsi ? (kK ? kK : g.k) : 0;
     const int KT = k >> 4;                      // tile columns
     const int pg = pl.pg, og = pl.og, pchunks = pl.pchunks, ochunks = pl.ochunks, gcl = pl.gc_log2;
@@ -1013,16 +1042,9 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     const int len_p = t >= 1 ? plan[t - 1].len : 0, g_p = t >= 1 ? plan[t - 1].gi0 : 0;
     const float* s_x = s_xb + ((t + 3) % 3) * kPersistMaxPRows;
     unsigned long long* acc = gsi ? g.acc + (size_t)parity * (k + 4) : nullptr;
-    const int tp = (t & 1) * 2;
 
-    // the descriptors of the phase three ahead: requested now, stored before the barrier that ends the exchange
-    const int g_stage = t + 3 < p.n_phases ? plan[t + 3].gi0 : 0, n_stage = t + 3 < p.n_phases ? plan[t + 3].len : 0;
-    const uint32_t desc_word = desc_load(g_stage, n_stage);
-    // (warp 1, lanes 7 and 8) the arrival counter that guards this tick's gated residual of
-    // group lane - 7 of phase t - 2: the address now, the wait with the exchange
-    const unsigned* bar_pp = nullptr;
-    if (warp == 1 && (lane == 7 || lane == 8) && t >= 2 && (mask_pp & (1u << (lane - 7))))
-      bar_pp = p.groups[plan[t - 2].gi0 + (lane - 7)].bar + 2 + parity;
+    // the descriptor of the phase three ahead: requested now, stored before the barrier that ends the exchange
+    const uint32_t desc_word = desc_load(t + 3);
 
     // ---- a run of dense groups (the dense baseline): nothing of the exchange machinery has
     //      work in these ticks.  Per tick: post the (empty) decision on the previous phase for
@@ -1044,27 +1066,26 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
       int tt = t;
       for (;;) {
         const Plan plc = plan[tt];
-        const PersistGroup& gc = desc(plc.gi);
-        const int gs = tt + 3 < p.n_phases ? plan[tt + 3].gi0 : 0, ns = tt + 3 < p.n_phases ? plan[tt + 3].len : 0;
-        if (tt != t) dword = desc_load(gs, ns);
+        const PersistGroup& gc = desc(tt);
+        if (tt != t) dword = desc_load(tt + 3);
         if (plc.zeroer && tid < 2) gc.bar[2 * tid + (parity ^ 1u)] = 0u;
         if (tid == 0 && tt >= 1) misc->decision[(tt - 1) & 3] = (unsigned)tt << 8;
         const bool more = tt + 1 < n_ticks && plan[tt + 1].kind == 2 && not_gated(tt + 2) && not_gated(tt + 3);
         if (warp == kStatWarp && tt + 1 < n_ticks) {
           const Plan& pn = plan[tt + 1];
           if (pn.kind == 2) {
-            const char* xn = reinterpret_cast<const char*>(x_of(desc(pn.gi)));
-            for (int i = lane * 128; i < desc(pn.gi).d * 4; i += 32 * 128)
+            const char* xn = reinterpret_cast<const char*>(x_of(desc(tt + 1)));
+            for (int i = lane * 128; i < desc(tt + 1).d * 4; i += 32 * 128)
               asm volatile("prefetch.global.L2 [%0];" ::"l"(xn + i));
           }
         }
         tr.mark(0);
         n = w_run(&gc, q, in, gc.y + (size_t)p.token * gc.O, true, smem, n, p.status, p.trace != nullptr);
         if (tr.acc) tr.t = clock64();
-        desc_store(gs, ns, dword);   // (their latency ran under the stream)
+        desc_store(tt + 3, dword);   // (its latency ran under the stream)
         if (tid == 0) red_relaxed_u32(gc.bar + parity, 1u);
         if (more) {   // in flight while the barrier is waited for
-          const PersistGroup& gn = desc(plan[tt + 1].gi);
+          const PersistGroup& gn = desc(tt + 1);
           q = w_geometry(&gn);
           w_load_in(q, x_of(gn), in);
         }
@@ -1088,7 +1109,6 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     } else {
     // ---- A. the bulk reduction of the previous tick has read its source
     if (lane == 0 || tid == kNC - 1) bulk_reduce_wait_read();   // the lanes that issue bulk reductions
-    if (tid == 0) misc->fire[tp] = misc->fire[tp + 1] = 0;
     if (t >= 0 && pl.zeroer) {  // this CTA clears the group's counters for the next launch
       if (gsi) {
 #pragma unroll 1
@@ -1123,7 +1143,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     const unsigned n_pr = n;
     if (gsi) n += pchunks;
     if (gsi_f && warp >= kP1First && warp < kStatWarp) {
-      const PersistGroup& gf = desc(pf.gi);
+      const PersistGroup& gf = desc(t + 1);
       const int kf = kK ? kK : gf.k, KTf = kf >> 4, gclf = pf.gc_log2, wp1 = warp - kP1First;
       // partial c of this warp's tile columns kt = wp1 * tpw + s: lanes 0..3 hold, after the
       // folds below, columns 16 kt + 8 m + 2 lane + v in cacc[s][m][v]
@@ -1133,17 +1153,23 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
       // the warps that own tile columns wait for the slab and, between them, give it back
       const int nf = min(kP1, (KTf + tpw - 1) / tpw);
       const bool p1_active = wp1 < nf && pf.pg > 0;
-      bool okf = !p1_active || chunks_landed(smem, n_pf, pf.pchunks, abort);
+      bool okf = true;
 #pragma unroll
       for (int s3 = 0; s3 < kTpwMax; ++s3)
 #pragma unroll
         for (int m = 0; m < 2; ++m)
 #pragma unroll
           for (int v = 0; v < 4; ++v) cacc[s3][m][v] = 0.f;
-      const unsigned short* xt = s_xt + ((t + 1) & 1) * 2048;
-      if (okf) {
+      const unsigned short* xt = s_xt + ((t + 1) & 1) * (kXtBytes / 2);
+      // (a slab of few chunks is waited for as a whole; a larger one streams through the ring)
 #pragma unroll 1
-        for (int R = 0; R < pf.pg; ++R) {
+      for (int cb = 0; p1_active && okf && cb < pf.pchunks; cb += kP1Chunks) {
+        const int cn = min(kP1Chunks, pf.pchunks - cb);
+        okf = chunks_landed(smem, n_pf + cb, cn, abort);
+        if (!okf) break;
+        const int R1 = min((int)pf.pg, (cb + cn) << gclf);
+#pragma unroll 1
+        for (int R = cb << gclf; R < R1; ++R) {
           const uint2 ax = *reinterpret_cast<const uint2*>(xt + (R * 32 + lane) * 4);
           const uint4 a = make_uint4(ax.x, 0u, ax.y, 0u);
           const int ci = R >> gclf, rr = R - (ci << gclf);
@@ -1158,11 +1184,11 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
             }
           }
         }
-      }
-      if (okf && p1_active && lane == 0) {   // (every tile of the slab is in registers: the last mma has issued)
-        const uint32_t share = unit_share(wp1, nf);
+        if (lane == 0) {   // (every tile of the chunks is in registers: the last mma has issued)
+          const uint32_t share = unit_share(wp1, nf);
 #pragma unroll 1
-        for (int c = 0; c < pf.pchunks; ++c) mbar_arrive_n(&empty[(n_pf + c) % kNB], share);
+          for (int c = cb; c < cb + cn; ++c) mbar_arrive_n(&empty[(n_pf + c) % kNB], share);
+        }
       }
       // the three terms of x sit in rows 0..2 = lanes 0-3, 4-7, 8-11: fold them onto lanes 0-3
 #pragma unroll
@@ -1207,7 +1233,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
       }
     }
     if (gsi_f && tid == kNC - 1 && pf.pg > 0) {   // ||x||^2 of phase t + 1 over this CTA's rows
-      const PersistGroup& gf = desc(pf.gi);
+      const PersistGroup& gf = desc(t + 1);
       const int kf = kK ? kK : gf.k;
       const unsigned amax_f = misc->amax_bits[(t + 1) & 1];
       const double amax = (double)__uint_as_float(amax_f);
@@ -1236,8 +1262,8 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     // ---- E. wait until every contributing CTA has been added: four warps poll a quarter of
     //      the accumulators of c each (contiguous words, all loads of a lane in flight together,
     //      one round trip per attempt) and leave c as three bf16 terms in operand order;
-    //      warp 1 polls the scalars: lane 0 this phase's ||x||^2, lanes 1+2u / 2+2u the
-    //      previous phase's ||r||^2 and published ||x||^2 of its group u.
+    //      warp 1 polls the scalars: the previous phase's ||r||^2 of its group u on lane u, the
+    //      threshold on lane 8 + u, and on lane 7 this phase's ||x||^2.
     if (gsi && (warp == 0 || (warp >= 2 && warp <= 4))) {
       constexpr int kWpl = kK ? (kK + 127) / 128 : 4;   // words per lane
       const int q4 = warp == 0 ? 0 : warp - 1;          // this warp's quarter of the words
@@ -1275,22 +1301,20 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
       }
     }
     if (warp == 1) {
-      // lane 0: this phase's ||x||^2 (an accumulator: arrivals in the upper bits); lanes
-      // 1 + 2u / 2 + 2u: the previous phase's ||r||^2 (accumulator) and its gate threshold
-      // (tagged word) of group u
-      // (on CTA 0, which writes the logs, lanes 5 + u also fetch the group's published ||x||^2)
-      const int u = lane <= 4 ? (lane - 1) >> 1 : lane - 5;
-      const bool live_u = u >= 0 && u < len_p && !(desc(g_p + u).flags & GSI_FLAG_DENSE);
-      const bool settle = lane >= 1 && lane <= 4 && live_u;
-      const PersistGroup& gs = desc(g_p + (u & 1));   // read only when `live_u`
-      const bool w_x2 = gsi && lane == 0, w_r2 = settle && (lane & 1);
-      const bool w_thr = (settle && !(lane & 1)) || (cta == 0 && lane >= 5 && lane <= 6 && live_u);
-      // lanes 7, 8: the arrivals before the gated residual this tick streams (phase t - 2, group
-      // lane - 7): every CTA has made its r and image rows visible (they arrived a tick ago)
-      const bool w_bar = bar_pp != nullptr;
-      const unsigned long long* wp = w_x2   ? acc + k
-                                     : w_r2 ? gs.acc + (size_t)parity * (gs.k + 4) + gs.k + 2
-                                            : gs.pub + (lane <= 4 ? 1 : 0);
+      // eight lanes a role, group u of a phase on lane u of each: the previous phase's ||r||^2
+      // (accumulator: arrivals in the upper bits), its gate threshold (tagged word), on CTA 0,
+      // which writes the logs, its published ||x||^2; the arrivals before the gated residuals
+      // this tick streams (phase t - 2: every CTA has made its r and image rows visible, they
+      // arrived a tick ago).  Lane 7: this phase's ||x||^2.
+      static_assert(kPersistMaxLen <= 7, "lanes");
+      const int role = lane >> 3, u = lane & 7;
+      const bool exists = u < 7 && (role == 3 ? (mask_pp >> u) & 1u : u < len_p);
+      const Settle& gs = settle[exists ? (role == 3 ? plan[t - 2].gi0 : g_p) + u : 0];
+      const bool live = exists && gs.mode != 2;
+      const bool w_x2 = gsi && lane == 7, w_r2 = role == 0 && live;
+      const bool w_thr = live && (role == 1 || (role == 2 && cta == 0));
+      const bool w_bar = role == 3 && exists;
+      const unsigned long long* wp = w_x2 ? acc + k : w_r2 ? gs.r2 : gs.pub + (role == 1 ? 1 : 0);
       const unsigned want = w_x2 ? (unsigned)n_contrib : (unsigned)gs.n_contrib;
       unsigned long long w = 0;
       unsigned it = 0;
@@ -1302,7 +1326,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
           mine = w_thr ? (unsigned)(w >> 63) == tag
                        : (unsigned)((w + (kOne >> 1)) >> kCountShift) == want;
         } else if (w_bar) {
-          mine = ld_relaxed_u32(bar_pp) >= (unsigned)G;
+          mine = ld_relaxed_u32(gs.bar) >= (unsigned)G;
         }
         done = __all_sync(0xffffffffu, mine);
         if (!done && (++it > p.spin_limit || ((it & 1023u) == 0 && *abort))) {
@@ -1331,14 +1355,15 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
                                     ((unsigned long long)tag << 63));
         }
       }
-      // the lane that holds ||r||^2 of group u takes the threshold from its neighbour
-      const unsigned long long w_nb = __shfl_down_sync(0xffffffffu, w, 1);
-      const unsigned long long wx = __shfl_sync(0xffffffffu, w, 5 + (u & 1));
+      // the lane that holds ||r||^2 of group u takes the threshold from lane 8 + u
+      const unsigned long long w_nb = __shfl_down_sync(0xffffffffu, w, 8);
+      const unsigned long long wx = __shfl_down_sync(0xffffffffu, w, 16);
+      bool fires = false;
       if (w_r2) {
         const unsigned long long val = w - ((unsigned long long)want << kCountShift);
         const bool finite = !(w_nb & (1ull << 62));
         const bool fast = finite && val < (w_nb & ((1ull << 62) - 1));
-        misc->fire[tp + u] = (!fast && finite && !(gs.flags & GSI_FLAG_STATIC_PROJECTION)) ? 1 : 0;
+        fires = !fast && finite && gs.mode == 0;
         if (cta == 0) {   // the logs: rho from ||r||^2 2^-e and ||x||^2 2^-e, both in the float range
           const double x2 = __longlong_as_double((long long)(wx & ~(1ull << 63)));
           const int ex = x2 > 0.0 ? exp_above(x2) : 0;
@@ -1350,8 +1375,10 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
                                    : __int_as_float(0x7fc00000);
         }
       }
+      const unsigned fired = __ballot_sync(0xffffffffu, fires);
+      if (lane == 0) misc->fire[t & 1] = fired;
     }
-    desc_store(g_stage, n_stage, desc_word);
+    desc_store(t + 3, desc_word);
     if (tid == 0) misc->stop[1] = *abort;
     csync();
     tr.mark(4);
@@ -1363,15 +1390,14 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     // ---- F. hand the decision to the producer; a gated group's r and image rows must be
     //      visible grid-wide before its W rows are streamed in the next tick: release fence
     //      and arrival now, the wait comes then
-    const unsigned mask_p = (unsigned)misc->fire[tp] | ((unsigned)misc->fire[tp + 1] << 1);
+    const unsigned mask_p = misc->fire[t & 1];
     if (tid == 0 && t >= 1) {
       misc->decision[(t - 1) & 3] = ((unsigned)t << 8) | mask_p;
 #pragma unroll 1
-      for (int u = 0; u < len_p; ++u)
-        if (mask_p & (1u << u)) {
-          __threadfence();
-          red_relaxed_u32(desc(g_p + u).bar + 2 + parity, 1u);
-        }
+      for (unsigned m = mask_p; m; m &= m - 1) {
+        __threadfence();
+        red_relaxed_u32(settle[g_p + __ffs(m) - 1].bar, 1u);
+      }
     }
     const double x2_own = gsi ? misc->x2 : 0.0;
     // ... and their statistics are published a row pass ahead of the next phase's exchange
@@ -1379,7 +1405,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     // during its row units, the check comes after them)
     unsigned xw[kXmaxWords];
     const bool xmax_next = warp == kStatWarp && t + 2 < n_ticks && plan[t + 2].kind == 1;
-    if (xmax_next) xmax_issue(desc(plan[t + 2].gi).xmax, plan[t + 2].n_contrib, xw);
+    if (xmax_next) xmax_issue(desc(t + 2).xmax, plan[t + 2].n_contrib, xw);
 
     // ---- G / I. the row passes on the tensor cores, one copy of the code for both: part 0 the
     //      residual rows of the basis slab (still in the ring), part 1 the image rows.  A unit
@@ -1508,24 +1534,22 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     //      one, then this phase's own stream if it is a dense group (followed by a grid barrier
     //      that keeps a dense stack in model order).
     if (mask_stream || dense) {
-      const int len_pp = plan[t - 2 >= 0 ? t - 2 : 0].len, g_pp = plan[t - 2 >= 0 ? t - 2 : 0].gi0;
+      const int g_pp = plan[t - 2 >= 0 ? t - 2 : 0].gi0;
+      unsigned left = mask_stream;
 #pragma unroll 1
-      for (int u = 0; u < 3; ++u) {
-        const PersistGroup* gw = nullptr;
-        if (u < 2) {
-          if (u < len_pp && (mask_stream & (1u << u))) gw = p.groups + g_pp + u;
-        } else if (dense) {
-          gw = &desc(plan[t].gi);
-        }
-        if (!gw) continue;
+      while (left || dense) {
+        const bool own = !left;   // the dense group of this tick
+        const PersistGroup* gw = own ? &desc(t) : p.groups + g_pp + __ffs(left) - 1;
+        left &= left - 1;
+        if (!own && (cta < gw->w_cta0 || cta >= gw->w_cta0 + gw->w_ncta)) continue;
         // (a gated group's r and image rows are visible: warp 1 waited for every CTA's arrival
         // during this tick's exchange)
-        const float* src = u < 2 ? gw->r
-                                 : gw->x + (long long)slot_io * gw->x_step_stride + (size_t)p.token * gw->d;
+        const float* src = !own ? gw->r
+                                : gw->x + (long long)slot_io * gw->x_step_stride + (size_t)p.token * gw->d;
         tr.mark(9);
-        n = w_stream(gw, src, gw->y + (size_t)p.token * gw->O, u == 2, smem, n, p.status, p.trace != nullptr);
+        n = w_stream(gw, src, gw->y + (size_t)p.token * gw->O, own, smem, n, p.status, p.trace != nullptr);
         if (tr.acc) tr.t = clock64();
-        if (u == 2) {
+        if (own) {
           if (tid == 0) {
             red_relaxed_u32(gw->bar + parity, 1u);
             grid_wait(gw->bar + parity, (unsigned)G, p, misc);
@@ -1533,6 +1557,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
               p.gate_log[((size_t)slot_io * p.log_step_stride + plan[t].gi) * p.n_tokens + p.token] = 1;
           }
           csync();
+          break;
         }
       }
       tr.mark(6);
@@ -1563,7 +1588,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_decode_step(const __grid_const
     misc->r2_acc = 0ull;
     // shared memory keeps what the previous launch on this SM left: the producer must not
     // mistake an old decision for this launch's
-    misc->fire[0] = misc->fire[1] = misc->fire[2] = misc->fire[3] = 0;
+    misc->fire[0] = misc->fire[1] = 0u;
     misc->decision[0] = misc->decision[1] = misc->decision[2] = misc->decision[3] = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }

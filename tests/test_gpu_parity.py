@@ -808,6 +808,46 @@ def test_persistent_trace_counters_do_not_change_results():
     assert torch.equal(before, tr)
 
 
+@pytest.mark.parametrize("shapes", [
+    # more groups than a phase holds, streams on the groups' own shares
+    [(256, 64, (136, 24))] * 9,
+    # ranks side by side in one phase, a basis slab that streams through the ring in parts
+    [(256, 64, (264,)), (16384, 512, (64,)), (1024, 128, (8, 2056)), (2048, 512, (4096,))],
+    # a dense group between phases of several
+    [(512, 128, (512,)), (768, 128, (256,)), "dense", (512, 128, (128,)), (512, 128, (640,))],
+])
+def test_persistent_phases_of_several_groups(shapes):
+    """Consecutive groups share a phase (its CTAs split between them): every group's gates and
+    outputs against the oracle, over steps in which none, some and all of them are gated."""
+    g = G()
+    n_steps = 5
+    groups, layers = [], []
+    for i, shape in enumerate(shapes):
+        d, k, d_out = shape if shape != "dense" else (512, 64, (264,))
+        x, P, Ws = make_small(d, k, d_out, n_steps, seed=7000 + i, noise=0.001, outlier_every=1)
+        live = [True, i % 2 == 0, False, i % 3 == 0, True]   # gated in this step
+        x2, _, _ = make_small(d, k, d_out, n_steps, seed=7000 + i, noise=0.001)
+        x = torch.stack([x[s] if live[s] else x2[s] for s in range(n_steps)]).contiguous()
+        dense = shape == "dense"
+        layers.append(g.Layer([W.cuda() for W in Ws], None if dense else P.cuda(), 0.05, max_tokens=1,
+                              flags=g.GSI_FLAG_DENSE if dense else 0))
+        groups.append((x, P, Ws, 0.0 if dense else 0.05, live))
+    stack = g.Stack(layers, mode=2)
+    stack.bind([x.cuda() for x, *_ in groups], n_steps=n_steps)
+    ys = [[] for _ in groups]
+    for s in range(n_steps):
+        stack.step()
+        torch.cuda.synchronize()
+        for i, y in enumerate(stack.ys):
+            ys[i].append(y.cpu().clone())
+    assert stack.status() == 0
+    gate = stack.gate_log.cpu().numpy()[:, :, 0]
+    for i, (x, P, Ws, eps, live) in enumerate(groups):
+        rho = None if eps == 0.0 else stack.rho_log.cpu().numpy()[:, i, 0]
+        compare_group(x, P, Ws, eps, torch.cat(ys[i]).numpy(), gate[:, i], rho)
+        assert eps == 0.0 or gate[:, i].tolist() == [int(v) for v in live]
+
+
 def test_persistent_nonfinite_token():
     g = G()
     x, P, Ws = make_small(256, 64, (64,), 3, seed=41)
