@@ -228,8 +228,8 @@ class Layer:
         Returns (appended, rho) as device tensors.  Writes the basis tensor given at creation."""
         assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous() and x.numel() == self.d
         assert k_active.is_cuda and k_active.dtype == torch.int32 and k_active.numel() == 1
-        appended = torch.zeros(1, dtype=torch.int32, device=x.device)
-        rho = torch.zeros(1, dtype=torch.float32, device=x.device)
+        appended = torch.empty(1, dtype=torch.int32, device=x.device)
+        rho = torch.empty(1, dtype=torch.float32, device=x.device)
         _check(lib.gsi_extend_basis(self.handle, x.data_ptr(), float(tau), k_active.data_ptr(),
                                     appended.data_ptr(), rho.data_ptr(), _stream_ptr(stream)),
                "gsi_extend_basis")

@@ -391,7 +391,7 @@ gsi_status_t gsi_extend_basis(gsi_handle_t h, const float* x, float tau, int* k_
   if (!h || !x || !k_active || !aligned16(x) || !(tau >= 0.f)) return GSI_ERR_INVALID_ARG;
   if (h->desc.flags & GSI_FLAG_DENSE) return GSI_ERR_UNSUPPORTED;
   const Layout& L = h->lay;
-  int* ctrl = reinterpret_cast<int*>(h->ws + L.ctrl);
+  const bool fp8 = h->desc.flags & GSI_FLAG_FP8_IMAGE;
   ExtendArgs a{};
   a.x = x;
   a.tau = tau;
@@ -399,16 +399,15 @@ gsi_status_t gsi_extend_basis(gsi_handle_t h, const float* x, float tau, int* k_
   a.appended_out = appended_out;
   a.rho_out = rho_out;
   a.y_scratch = reinterpret_cast<float*>(h->ws + L.y_stage);
-  a.gate_scratch = reinterpret_cast<unsigned char*>(h->ws + L.gate_stage);
-  a.ctrl = ctrl + 24;                                       // words 24..27 of the control block
-  a.inv_norm = reinterpret_cast<float*>(ctrl + 28);         // words 28..29
-  a.x_scratch = reinterpret_cast<float*>(h->ws + L.x_stage);
   a.pmax = h->gp.p_f32 ? nullptr : h->pmax;
   a.PT = L.front ? const_cast<uint16_t*>(h->gp.PT) : nullptr;
+  if (L.packed) {
+    a.P16 = reinterpret_cast<uint16_t*>(h->ws + L.pk_pp);
+    if (fp8) a.WP8 = reinterpret_cast<unsigned char*>(h->ws + L.pk_wpp);
+    else a.WP16 = reinterpret_cast<uint16_t*>(h->ws + L.pk_wpp);
+  }
   h->last_stream = stream;
-  if (launch_extend_basis(h->gp, a, stream) != cudaSuccess) return GSI_ERR_CUDA;
-  if (L.packed && !repack(h, stream)) return GSI_ERR_CUDA;   // the tiled copies follow the new column
-  return GSI_OK;
+  return launch_extend_basis(h->gp, a, stream) == cudaSuccess ? GSI_OK : GSI_ERR_CUDA;
 }
 
 gsi_status_t gsi_get_image(gsi_handle_t h, int map, const void** out) {

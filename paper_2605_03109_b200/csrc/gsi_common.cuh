@@ -232,11 +232,6 @@ cudaError_t launch_advance_step(int* step, cudaStream_t stream);
 cudaError_t launch_forward_fused(const GroupParams& g, const IoRef& io, int n_tokens, int leave_from,
                                  cudaStream_t stream);
 size_t fused_words_bytes(int d, int k, int max_tokens);
-// One token on CUDA cores: c, r = x - P c into g.r (x may be g.r itself), rho into
-// g.rho_scratch[0] (or io.rho), gate byte, fired list.  No image product.
-cudaError_t launch_project_residual(const GroupParams& g, const IoRef& io, cudaStream_t stream);
-// io.y[0][:] += W g.r for the token in the fired list (nothing if the list is empty).
-cudaError_t launch_gated_gemv(const GroupParams& g, const IoRef& io, cudaStream_t stream);
 // Online basis extension by one vector (see gsi_extend_basis).
 struct ExtendArgs {
   const float* x;        // [d] the token
@@ -245,12 +240,12 @@ struct ExtendArgs {
   int* appended_out;     // device or null
   float* rho_out;        // device or null
   float* y_scratch;      // [O] device
-  unsigned char* gate_scratch;  // [1] device
-  int* ctrl;             // [4] device: appended, column, spare, spare
-  float* inv_norm;       // [2] device: 1/||r2||, rho of the token
-  float* x_scratch;      // [d] device: r1, the input of the second pass
   float* pmax;           // [1] device: max |P| of the handle (bf16 basis) or null
-  uint16_t* PT;          // [k][d] transposed copy to keep in step, or null
+  // copies to keep in step, or null
+  uint16_t* PT;          // [k][d] transposed basis
+  uint16_t* P16;         // tiled basis
+  uint16_t* WP16;        // tiled image
+  unsigned char* WP8;    // tiled FP8 image
 };
 cudaError_t launch_extend_basis(const GroupParams& g, const ExtendArgs& a, cudaStream_t stream);
 // mapped: rb holds every token's residual (row = token) and the fired list selects the

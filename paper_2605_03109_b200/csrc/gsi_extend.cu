@@ -6,123 +6,307 @@
 // column k_active of every cached image.  Columns [k_active, k) of P are zero before, so
 // every other kernel of the library keeps working on the full width k.
 //
-// A rare, set-up-like operation: it reuses the CUDA-core projection / residual kernels
-// (twice) and the gated W r GEMV (once, for the image column) and adds three small
-// kernels of its own.  Everything stays on the device: no host synchronisation.
-#include "gsi_common.cuh"
+// ONE cooperative launch (every CTA resident), CUDA-core FMAs in fp32, no host
+// synchronisation; nearly every token ends after the first pass.
+//
+//   pass 1   c = P^T x, r1 = x - P c, rho
+//   (rho <= tau, no free column or a non-finite token: done)
+//   pass 2   c = P^T r1, r2 = r1 - P c, ||r2||
+//   store    v = r2 / ||r2|| rounded to the basis type: column of P, of its transposed copy and
+//            of the tiled copy; max|P|
+//   image    W v for this CTA's rows: column of the image and of its tiled copy (FP8: the
+//            sixteen-row blocks are quantised again, their scales may change)
+//
+// What bounds it: the chain of two exchanges per pass (words that carry their validity,
+// gsi_exchange.cuh) and 2 MB of basis.  Before, fourteen launches whether a column was appended
+// or not: 107 us for a token inside the subspace at 4096 x 256 and 28672 image rows, now 12.9 us;
+// with a column appended (235 MB of W) 168 us, now 78 us.
+#include "gsi_exchange.cuh"
+#include "gsi_pack.cuh"
 
 namespace gsi {
 
 namespace {
 
-constexpr int kExtThreads = 1024;
+using namespace exchange;
+
+constexpr int kT = 512, kW = kT / 32;
+constexpr int kStage = 4096;   // floats of x, r1 or v in shared memory at a time
 
 __device__ __forceinline__ uint16_t to_bf16_bits(float v) {
   const __nv_bfloat16 h = __float2bfloat16_rn(v);
   return *reinterpret_cast<const uint16_t*>(&h);
 }
 
-// After the first pass: keep rho of the token (it is the quantity the threshold tests).
-__global__ void k_ext_keep_rho(GroupParams g, ExtendArgs a) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    a.inv_norm[1] = g.rho_scratch[0];
-    if (a.rho_out) *a.rho_out = g.rho_scratch[0];
-  }
-}
-
-// After the second pass: ||r2||^2 in a fixed order, the decision, and the list of "fired"
-// tokens the W r GEMV works from (token 0 if a column is appended, nobody otherwise).
-__global__ void __launch_bounds__(kExtThreads) k_ext_decide(GroupParams g, ExtendArgs a) {
-  __shared__ double s_part[kExtThreads / 32];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < g.d; i += kExtThreads) s += (double)g.r[i] * (double)g.r[i];
+// Elements [i0, i0 + n) of a vector into shared memory, from plain floats or from tagged words.
+__device__ __forceinline__ bool stage(float* s, const float* x, const unsigned long long* words, unsigned tag, int i0,
+                                      int n) {
+  bool ok = true;
+  for (int ib = 0; ib < n; ib += 8 * kT) {
+    if (x) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < kExtThreads / 32; ++w) t += s_part[w];
-    const int col = *a.k_active;
-    const float rho = a.inv_norm[1];
-    // rho > tau is false for NaN: a non-finite token never extends the basis
-    const bool go = rho > a.tau && col >= 0 && col < g.k && t > 0.0 && t < 1e300;
-    a.ctrl[0] = go ? 1 : 0;
-    a.ctrl[1] = col;
-    a.inv_norm[0] = go ? (float)(1.0 / sqrt(t)) : 0.f;
-    *g.n_fired = go ? 1 : 0;
-    g.fired[0] = 0;
-    if (a.appended_out) *a.appended_out = go ? 1 : 0;
+      for (int u = 0; u < 8; ++u) {
+        const int i = ib + (int)threadIdx.x + u * kT;
+        if (i < n) s[i] = __ldg(x + i0 + i);
+      }
+    } else {
+      const int first = ib + (int)threadIdx.x;
+      const int cnt = n > first ? min(8, (n - first + kT - 1) / kT) : 0;
+      ok = gather(words + i0 + first, kT, cnt, tag, [&](int u, float v) { s[first + u * kT] = v; }) && ok;
+    }
   }
+  return ok;
 }
 
-// v = r2 / ||r2|| rounded to the basis type goes into column `col` of P (and row `col` of
-// the transposed copy); g.r receives the STORED value, so the image column is W times
-// what the basis really holds.
-__global__ void __launch_bounds__(256) k_ext_store_vector(GroupParams g, ExtendArgs a) {
-  if (!a.ctrl[0]) return;
-  const int col = a.ctrl[1];
-  const float inv = a.inv_norm[0];
+template <int VPL, bool PF32>
+__global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, int n_slabs) {
+  __shared__ float s_v[kStage];
+  __shared__ float s_part[kW * kCols];
+  __shared__ float s_c[1024];
+  __shared__ float s_scale[16];
+  __shared__ double s_norm[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = gridDim.x, cta = blockIdx.x, d = g.d, k = g.k, KV = k / 8;
+  const unsigned call = *g.fused_call;
+  const int col = *a.k_active;
+  const Words words = words_of(g);
+  const int p0 = (int)((long long)d * cta / G), p1 = (int)((long long)d * (cta + 1) / G);
+  const int n_cb = (k + kCols - 1) / kCols;
+  int lpr = 1;
+  while (lpr < KV && lpr < 32) lpr <<= 1;
+  const int rpp = 32 / lpr, rsub = lane / lpr, cl = lane % lpr;
+  auto give_up = [&](bool ok) -> bool {   // the same answer for every thread
+    if (!__syncthreads_or(!ok)) return false;
+    if (tid == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
+    if (tid == 0 && cta == 0) *g.fused_call = call + 3u;
+    return true;
+  };
+
+  float inv = 0.f;
+#pragma unroll 1
+  for (int pass = 1; pass <= 2; ++pass) {
+    const unsigned tag = call + (unsigned)pass;
+    bool ok = true;
+    // partial c of a slab of rows x 32 columns
+    if (cta < n_slabs * n_cb) {
+      const int slab = cta / n_cb, cb = cta % n_cb;
+      const int r0 = (int)((long long)d * slab / n_slabs), r1 = (int)((long long)d * (slab + 1) / n_slabs);
+      const int sub = lane >> 2, c = cb * kCols + (lane & 3) * 8;
+      float acc[8], sx = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+      for (int rb = r0; rb < r1; rb += kStage) {
+        const int n = min(kStage, r1 - rb);
+        __syncthreads();
+        ok = stage(s_v, pass == 1 ? a.x : nullptr, words.r, tag - 1u, rb, n) && ok;
+        __syncthreads();
+        for (int base = warp * 8 + sub; base < n; base += kW * 8 * 4) {
+          float p[4][8];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = base + u * kW * 8;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) p[u][e] = 0.f;
+            if (i < n && c < k) load8<PF32>(g.P, (size_t)(rb + i) * KV + c / 8, p[u]);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = base + u * kW * 8;
+            const float v = i < n ? s_v[i] : 0.f;
+            sx = fmaf(v, v, sx);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] = fmaf(p[u][e], v, acc[e]);
+          }
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) sx += __shfl_xor_sync(0xffffffffu, sx, o);
+      if (lane < 4)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s_part[warp * kCols + lane * 8 + e] = acc[e];
+      if (lane == 0) s_c[warp] = sx;
+      __syncthreads();
+      if (tid < kCols) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kW; ++w) s += s_part[w * kCols + tid];
+        if (cb * kCols + tid < k) put(words.c + (size_t)slab * k + cb * kCols + tid, s, tag);
+      } else if (tid == kCols && cb == 0) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kW; ++w) s += s_c[w];
+        put(words.x2 + slab, s, tag);
+      }
+      __syncthreads();
+    }
+    // c: every CTA adds all partials in slab order
+    for (int j = tid; j < k; j += kT) {
+      float s = 0.f;
+      ok = gather(words.c + j, k, n_slabs, tag, [&](int, float v) { s += v; }) && ok;
+      s_c[j] = s;
+    }
+    if (give_up(ok)) return;
+    // this CTA's rows of the residual
+    float c8[VPL][8], sr = 0.f;
+#pragma unroll
+    for (int v = 0; v < VPL; ++v)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) c8[v][e] = cl + v * lpr < KV ? s_c[(cl + v * lpr) * 8 + e] : 0.f;
+    for (int base = p0 + warp * rpp; base < p1; base += kW * rpp) {
+      const int row = base + rsub;
+      float dot = 0.f;
+      if (row < p1) {
+#pragma unroll
+        for (int v = 0; v < VPL; ++v)
+          if (cl + v * lpr < KV) {
+            float p8[8];
+            load8<PF32>(g.P, (size_t)row * KV + cl + v * lpr, p8);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) dot = fmaf(p8[e], c8[v][e], dot);
+          }
+      }
+      for (int o = lpr >> 1; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+      if (row < p1 && cl == 0) {
+        const float rv = (pass == 1 ? __ldg(a.x + row) : g.r[row]) - dot;   // (g.r: written here in pass 1)
+        g.r[row] = rv;
+        if (pass == 1) put(words.r + row, rv, tag);
+        sr = fmaf(rv, rv, sr);
+      }
+    }
+    sr = warp_sum(sr);
+    if (lane == 0) s_part[warp] = sr;
+    __syncthreads();
+    if (tid == 0) {
+      float s = 0.f;
+#pragma unroll
+      for (int w = 0; w < kW; ++w) s += s_part[w];
+      put(words.r2 + cta, s, tag);
+    }
+    if (warp < 2) {
+      double s = 0.0;
+      ok = warp ? warp_gather_sum(words.x2, 1, n_slabs, tag, s) : warp_gather_sum(words.r2, 1, G, tag, s);
+      if (lane == 0) s_norm[warp] = s;
+    }
+    if (give_up(ok)) return;
+    // the same sums in the same order on every CTA: the same decision
+    bool go;
+    if (pass == 1) {
+      const float rho = (float)(sqrt(s_norm[0]) / sqrt(s_norm[1]));
+      // rho > tau is false for NaN: a non-finite token never extends the basis
+      go = rho > a.tau && col >= 0 && col < k;
+      if (cta == 0 && tid == 0 && a.rho_out) *a.rho_out = rho;
+    } else {
+      go = s_norm[0] > 0.0 && s_norm[0] < 1e300;
+      inv = go ? (float)(1.0 / sqrt(s_norm[0])) : 0.f;
+    }
+    if (!go || pass == 2) {
+      if (cta == 0 && tid == 0) {
+        if (a.appended_out) *a.appended_out = go ? 1 : 0;
+        if (go) *a.k_active = col + 1;   // (every CTA has read it: its norms are here)
+        *g.fused_call = call + 3u;
+      }
+      if (!go) return;
+    }
+    __syncthreads();
+  }
+
+  // ---- store: the image column is W times what the basis really holds
+  const unsigned tag = call + 3u;
   float m = 0.f;
-  for (int i = blockIdx.x * 256 + threadIdx.x; i < g.d; i += gridDim.x * 256) {
+  for (int i = p0 + tid; i < p1; i += kT) {
     const float v = g.r[i] * inv;
-    float stored;
-    if (g.p_f32) {
-      const_cast<float*>(static_cast<const float*>(g.P))[(size_t)i * g.k + col] = v;
-      stored = v;
+    float stored = v;
+    if constexpr (PF32) {
+      const_cast<float*>(static_cast<const float*>(g.P))[(size_t)i * k + col] = v;
     } else {
       const uint16_t b = to_bf16_bits(v);
-      const_cast<uint16_t*>(static_cast<const uint16_t*>(g.P))[(size_t)i * g.k + col] = b;
-      if (a.PT) a.PT[(size_t)col * g.d + i] = b;
+      const_cast<uint16_t*>(static_cast<const uint16_t*>(g.P))[(size_t)i * k + col] = b;
+      if (a.PT) a.PT[(size_t)col * d + i] = b;
+      if (a.P16) a.P16[pack::t16_slot(i, col, k)] = b;
       stored = __uint_as_float((uint32_t)b << 16);
     }
-    g.r[i] = stored;
+    put(words.r + i, stored, tag);
     m = fmaxf(m, fabsf(stored));
   }
-  if (a.pmax) {   // max |P| of the handle: non-negative floats order like their bit patterns
+  if (a.pmax) {   // non-negative floats order like their bit patterns
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(a.pmax), __float_as_int(m));
+    if (lane == 0 && m > 0.f) atomicMax(reinterpret_cast<int*>(a.pmax), __float_as_int(m));
+  }
+
+  // ---- image: blocks of sixteen rows, a row per warp, four 16-byte loads of W in flight per lane
+  const int blocks = (g.O + 15) / 16;
+  const int o0 = (int)((long long)blocks * cta / G) * 16;
+  const int o1 = min(g.O, (int)((long long)blocks * (cta + 1) / G) * 16);
+  uint16_t* WP = const_cast<uint16_t*>(g.WP);
+  for (int c0 = 0; c0 < d; c0 += kStage) {
+    const int n = min(kStage, d - c0);
+    const bool last = c0 + n == d;
+    __syncthreads();
+    if (give_up(stage(s_v, nullptr, words.r, tag, c0, n))) return;
+    for (int row = o0 + warp; row < o1; row += kW) {
+      int j = 0;
+      while (j + 1 < g.n_maps && row >= g.off[j + 1]) ++j;
+      const uint4* w = reinterpret_cast<const uint4*>(g.W[j] + (size_t)(row - g.off[j]) * d + c0);
+      float s = 0.f;
+      for (int v0 = lane; v0 < n / 8; v0 += 4 * 32) {
+        uint4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          q[u] = v0 + 32 * u < n / 8 ? ld_stream(w + v0 + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (v0 + 32 * u < n / 8) {
+            float f[8];
+            unpack_bf16x8(q[u], f);
+            const float4* x4 = reinterpret_cast<const float4*>(s_v + (v0 + 32 * u) * 8);
+            const float4 lo = x4[0], hi = x4[1];
+            s = fmaf(f[0], lo.x, s); s = fmaf(f[1], lo.y, s); s = fmaf(f[2], lo.z, s); s = fmaf(f[3], lo.w, s);
+            s = fmaf(f[4], hi.x, s); s = fmaf(f[5], hi.y, s); s = fmaf(f[6], hi.z, s); s = fmaf(f[7], hi.w, s);
+          }
+      }
+      s = warp_sum(s);
+      if (lane == 0) {
+        if (c0 > 0) s += a.y_scratch[row];
+        if (!last) {
+          a.y_scratch[row] = s;
+        } else {
+          const uint16_t b = to_bf16_bits(s);
+          WP[(size_t)row * k + col] = b;
+          if (a.WP16) a.WP16[pack::t16_slot(row, col, k)] = b;
+        }
+      }
+    }
+  }
+  if (a.WP8) {
+    __syncthreads();   // the column is in this CTA's rows
+    for (int R = o0 / 16; R * 16 < o1; ++R) {
+      pack::fp8_rows16(WP, g.O, k, a.WP8, R, s_scale);
+      __syncthreads();
+    }
   }
 }
 
-// Column `col` of the concatenated images = bf16(W v); then the basis is one column wider.
-__global__ void __launch_bounds__(256) k_ext_store_image(GroupParams g, ExtendArgs a) {
-  if (!a.ctrl[0]) return;
-  const int col = a.ctrl[1];
-  uint16_t* WP = const_cast<uint16_t*>(g.WP);
-  for (int r = blockIdx.x * 256 + threadIdx.x; r < g.O; r += gridDim.x * 256)
-    WP[(size_t)r * g.k + col] = to_bf16_bits(a.y_scratch[r]);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *a.k_active = col + 1;
+template <int VPL>
+cudaError_t launch_t(GroupParams g, ExtendArgs a, int slabs, int grid, cudaStream_t st) {
+  void* args[] = {&g, &a, &slabs};
+  return g.p_f32 ? cudaLaunchCooperativeKernel((void*)k_extend<VPL, true>, dim3(grid), dim3(kT), args, 0, st)
+                 : cudaLaunchCooperativeKernel((void*)k_extend<VPL, false>, dim3(grid), dim3(kT), args, 0, st);
 }
 
 }  // namespace
 
 cudaError_t launch_extend_basis(const GroupParams& g, const ExtendArgs& a, cudaStream_t st) {
-  IoRef io{};
-  io.x = a.x;
-  io.y = a.y_scratch;
-  io.gate = a.gate_scratch;
-  io.rho = nullptr;          // rho goes to g.rho_scratch[0]
-  io.step = nullptr;
-  io.n_steps = 1;
-  cudaError_t e;
-  // pass 1: r1 = x - P (P^T x), rho
-  if ((e = launch_project_residual(g, io, st)) != cudaSuccess) return e;
-  k_ext_keep_rho<<<1, 32, 0, st>>>(g, a);
-  // pass 2: r2 = r1 - P (P^T r1)
-  if ((e = cudaMemcpyAsync(a.x_scratch, g.r, (size_t)g.d * sizeof(float), cudaMemcpyDeviceToDevice,
-                           st)) != cudaSuccess)
-    return e;
-  io.x = a.x_scratch;
-  if ((e = launch_project_residual(g, io, st)) != cudaSuccess) return e;
-  k_ext_decide<<<1, kExtThreads, 0, st>>>(g, a);
-  k_ext_store_vector<<<(g.d + 255) / 256, 256, 0, st>>>(g, a);
-  // image column: y_scratch = W v through the gated-residual GEMV (one pass over W)
-  if ((e = cudaMemsetAsync(a.y_scratch, 0, (size_t)g.O * sizeof(float), st)) != cudaSuccess) return e;
-  if ((e = launch_gated_gemv(g, io, st)) != cudaSuccess) return e;
-  k_ext_store_image<<<(g.O + 255) / 256, 256, 0, st>>>(g, a);
-  return cudaGetLastError();
+  const int grid = fused_grid();
+  if (!grid) return cudaErrorInvalidDevice;
+  const int slabs = fused_slabs(g.d, g.k, grid);
+  return g.k <= 256   ? launch_t<1>(g, a, slabs, grid, st)
+         : g.k <= 512 ? launch_t<2>(g, a, slabs, grid, st)
+                      : launch_t<4>(g, a, slabs, grid, st);
 }
 
 }  // namespace gsi

@@ -20,77 +20,26 @@
 // at 4096 x 256 -> 28672 41.7 -> 16.0 us; 21 tokens at 3000 x 200 -> 1576 84 -> 46 us (on CUDA-core
 // FMAs this kernel took 112 us there); 16 tokens, fp32 basis, 768 x 128 -> 2304 48.5 -> 23.7 us.
 //
-// The exchanges carry no fence and no counter: every word is 64 bits, the fp32 value in the lower
-// half and the call's number (the device-side call counter + 1) in the upper half, written and
-// read whole, so a reader that sees this call's number has the value (one L2 round trip; a
-// release / acquire barrier costs two and a fence).  Words of earlier calls carry other numbers,
-// so nothing is cleared between calls.  Every token's sums run in an order that depends on the
-// shape alone: results are reproducible, and a token's are the same in a call of any size.
+// The exchanges are words that carry the call's number (gsi_exchange.cuh): a release / acquire
+// barrier would cost two L2 round trips and a fence where these cost one.  Every token's sums run
+// in an order that depends on the shape alone: results are reproducible, and a token's are the
+// same in a call of any size.
 // Every wait is bounded; a wait that gives up sets GSI_ERR_TIMEOUT and the CTA returns.
-#include "gsi_common.cuh"
+#include "gsi_exchange.cuh"
 
 namespace gsi {
 
 namespace {
 
+using namespace exchange;
+
 constexpr int kT = 512, kW = kT / 32;
-constexpr int kCols = 32;              // columns of c per CTA in phase A: 64-byte pieces of a basis row
 constexpr int kTileRows = 16 * kW;     // rows of a basis slab (and of W) per pass: 16 per warp
 constexpr int kPitch = 80;             // bytes between the staged 64-byte pieces: conflict-free ldmatrix
 constexpr int kDirectTokens = 4;       // calls of so few tokens gather the slabs' partials themselves
-constexpr unsigned kSpinF = 1u << 20;
 // dynamic shared memory: operand terms (phase A: the slab), then partial sums
 constexpr int kOpBytes = 131072, kAuxBytes = 32768;
 constexpr int kSmemFused = kOpBytes + kAuxBytes;
-
-__device__ __forceinline__ void put(unsigned long long* p, float v, unsigned tag) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p),
-               "l"(((unsigned long long)tag << 32) | __float_as_uint(v))
-               : "memory");
-}
-__device__ __forceinline__ unsigned long long get(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ bool is(unsigned long long w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
-__device__ __forceinline__ float val(unsigned long long w) { return __uint_as_float((unsigned)w); }
-
-// `count` words p[i * stride] in order, eight in flight; false when a wait ran out.
-template <typename F>
-__device__ __forceinline__ bool gather(const unsigned long long* p, size_t stride, int count, unsigned tag, F&& take) {
-  for (int i0 = 0; i0 < count; i0 += 8) {
-    unsigned long long w[8];
-    for (unsigned it = 0;; ++it) {
-      bool all = true;
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (i0 + u < count) w[u] = get(p + (size_t)(i0 + u) * stride);
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (i0 + u < count) all = all && is(w[u], tag);
-      if (all) break;
-      if (it > kSpinF) return false;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (i0 + u < count) take(i0 + u, val(w[u]));
-  }
-  return true;
-}
-
-// Sum of `count` words by one warp in double (lane l: words l, l + 32, ...; fixed order).
-__device__ __forceinline__ bool warp_gather_sum(const unsigned long long* p, size_t stride, int count, unsigned tag,
-                                                double& sum) {
-  const int lane = threadIdx.x & 31;
-  double s = 0.0;
-  const int mine = count > lane ? (count - lane + 31) / 32 : 0;
-  const bool ok = gather(p + (size_t)lane * stride, 32 * stride, mine, tag, [&](int, float v) { s += (double)v; });
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  sum = s;
-  return __all_sync(0xffffffffu, ok);
-}
 
 __device__ __forceinline__ void mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                     uint32_t b1) {
@@ -325,11 +274,8 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
   const int G = gridDim.x, cta = blockIdx.x;
   const int d = g.d, k = g.k, n = n_tokens;
   const unsigned tag = *g.fused_call + 1u;
-  unsigned long long* cw = g.fused_words;                               // [slab][token][k]
-  unsigned long long* xw = cw + (size_t)kFusedMaxGrid * g.B * kCols;    // [slab][token]
-  unsigned long long* nw = xw + (size_t)kFusedMaxGrid * g.B;            // [cta][token]
-  unsigned long long* cf = nw + (size_t)kFusedMaxGrid * g.B;            // [token][k]
-  unsigned long long* rw = cf + (size_t)g.B * k;                        // [token][d]
+  const Words words = words_of(g);
+  unsigned long long *cw = words.c, *xw = words.x2, *nw = words.r2, *cf = words.cf, *rw = words.r;
   const int slot = io_slot(io);
   const float* x = io.x + (long long)slot * io.x_step_stride;
   const int o0 = (int)((long long)g.O * cta / G), o1 = (int)((long long)g.O * (cta + 1) / G);
@@ -662,23 +608,29 @@ size_t fused_words_bytes(int d, int k, int max_tokens) {
   return 8 * ((size_t)kFusedMaxGrid * max_tokens * (kCols + 2) + (size_t)max_tokens * (k + d));
 }
 
-cudaError_t launch_forward_fused(const GroupParams& g, const IoRef& io, int n_tokens, int leave_from,
-                                 cudaStream_t st) {
+int fused_grid() {
   static int sms_of[64] = {};
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   int grid = dev < 64 ? sms_of[dev] : 0;
   if (!grid) {
-    if ((e = cudaDeviceGetAttribute(&grid, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if (cudaDeviceGetAttribute(&grid, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     if (dev < 64) sms_of[dev] = grid;
   }
-  if (grid > kFusedMaxGrid) grid = kFusedMaxGrid;
-  // slabs x column blocks of phase A over the grid; slabs of at least 32 rows
-  const int n_cb = (g.k + kCols - 1) / kCols;
-  int slabs = grid / n_cb;
-  if (slabs > (g.d + 31) / 32) slabs = (g.d + 31) / 32;
-  if (slabs < 1) slabs = 1;
+  return grid > kFusedMaxGrid ? kFusedMaxGrid : grid;
+}
+
+int fused_slabs(int d, int k, int grid) {
+  int slabs = grid / ((k + kCols - 1) / kCols);
+  if (slabs > (d + 31) / 32) slabs = (d + 31) / 32;
+  return slabs < 1 ? 1 : slabs;
+}
+
+cudaError_t launch_forward_fused(const GroupParams& g, const IoRef& io, int n_tokens, int leave_from,
+                                 cudaStream_t st) {
+  const int grid = fused_grid();
+  if (!grid) return cudaErrorInvalidDevice;
+  const int slabs = fused_slabs(g.d, g.k, grid);
   // eight-token blocks at a time: those of the call, as far as their c fits (6 bytes per
   // coefficient, padded to 32) and the sums fit the registers (four)
   int nb = 1;

@@ -1161,6 +1161,44 @@ def test_extend_basis_single_token_matches_oracle(p_dtype, kind):
         assert np.all(np.abs(got - want_col) <= 2.0 ** -8 * np.abs(want_col) + 3e-3 * np.max(np.abs(want_col)))
 
 
+@pytest.mark.parametrize("d,k_act,k_cap,d_out,fp8", [
+    (2064, 30, 128, (264, 1000), True),     # ragged sixteen-row blocks of the FP8 image
+    (16400, 16, 1024, (72,), False),        # slabs longer than the staging buffer, widest basis
+    (40, 0, 8, (8,), False),                # fewer rows than CTAs
+])
+def test_extend_basis_edges_and_copies(d, k_act, k_cap, d_out, fp8):
+    g = G()
+    q, P, Ws = _extend_case(d, max(k_act, 1), k_cap, d_out, 760)
+    if k_act == 0:
+        P.zero_()
+    x = torch.randn(d, generator=torch.Generator().manual_seed(761))
+    ref = O.extend(_bits(P), k_act, x.double().numpy(), 0.05)
+    Pd = P.cuda()
+    lay = g.Layer([W.cuda() for W in Ws], Pd, 0.05, max_tokens=1, flags=g.GSI_FLAG_FP8_IMAGE if fp8 else 0)
+    ka = torch.tensor([k_act], dtype=torch.int32, device="cuda")
+    appended, rho = lay.extend_basis(x.cuda(), 0.05, ka)
+    torch.cuda.synchronize()
+    assert lay.status() == 0 and appended.item() == 1 and ka.item() == k_act + 1
+    assert abs(rho.item() - ref["rho"]) <= 1e-4 * ref["rho"]
+    want = O.bf16_to_f64(ref["v_bits"])
+    col = Pd[:, k_act].double().cpu().numpy()
+    # entries across a rounding boundary are one bf16 spacing apart: at most 2^-7 of the value (one
+    # of sixteen thousand in the longest case)
+    assert np.all(np.abs(col - want) <= 2.0 ** -7 * np.abs(want) + 1e-9) and np.mean(col == want) > 0.99
+    imgs = [lay.image(j).cpu() for j in range(len(Ws))]
+    for W, img in zip(Ws, imgs):
+        w = O.image(S.bits_of(W), ref["v_bits"].reshape(d, 1))[:, 0]
+        got = img[:, k_act].double().numpy()
+        assert np.all(np.abs(got - w) <= 2.0 ** -8 * np.abs(w) + 3e-3 * np.max(np.abs(w)))
+    if fp8:   # the codes are those of the image as it is now
+        want8 = O.quantise_image_e4m3(O.bf16_to_f64(S.to_bf16_bits(torch.cat(imgs))))
+        codes, scales = lay.image_fp8()
+        assert np.array_equal(scales.cpu().numpy(), want8["scales"])
+        # (-0 and +0 are one number)
+        cg = codes.cpu().numpy()
+        assert np.all((cg == want8["codes"]) | ((cg | want8["codes"]) == 0x80))
+
+
 def test_extend_basis_sequence_then_forward_sees_the_new_columns():
     """A stream of tokens, some in the span, some not: the GPU basis and the oracle's evolve
     independently from the same start and stay together (same decisions, same columns to
