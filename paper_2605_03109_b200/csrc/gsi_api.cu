@@ -285,6 +285,9 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W, const void
   g.normpart3 = reinterpret_cast<float*>(h->ws + L.f_normpart);
   g.fused_words = reinterpret_cast<unsigned long long*>(h->ws + L.fused);
   g.fused_call = reinterpret_cast<unsigned*>(ctrl + 32);
+  g.area_B = g.B;
+  g.area_k = g.k;
+  g.area_d = g.d;
 
   if (L.tc || L.dense_tc) {
     if (!build_tma_maps(g, L.front, desc->max_tokens, &h->tm)) {

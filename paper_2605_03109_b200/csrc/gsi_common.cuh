@@ -119,7 +119,8 @@ struct GroupParams {
   float* cpart3;          // [proj_splits][B][k] split-K partial sums of c
   float* normpart3;       // [d/128][B][2] per-tile partial sums of ||r||^2, ||x||^2
   // calls in one launch (gsi_fused.cu)
-  unsigned long long* fused_words;   // exchange words: fp32 value and call number
+  unsigned long long* fused_words;   // exchange area, laid out for ...
+  int area_B, area_k, area_d;        // ... the largest call that uses it
   unsigned* fused_call;              // calls so far
 };
 constexpr int kFusedMaxGrid = 160;

@@ -25,24 +25,47 @@ __device__ __forceinline__ unsigned long long get(const unsigned long long* p) {
 __device__ __forceinline__ bool is(unsigned long long w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
 __device__ __forceinline__ float val(unsigned long long w) { return __uint_as_float((unsigned)w); }
 
-// `count` words p[i * stride] in order, eight in flight; false when a wait ran out.
-template <typename F>
+// Wider words: 96 bits of payload and the call's number, written and read as one 128-bit access.
+struct Word128 {
+  uint32_t a, b, c, tag;
+};
+__device__ __forceinline__ void put128(Word128* p, uint32_t a, uint32_t b, uint32_t c, unsigned tag) {
+  asm volatile("{\n .reg .b128 v;\n mov.b128 v, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], v;\n}" ::"l"(p),
+               "l"(((unsigned long long)b << 32) | a), "l"(((unsigned long long)tag << 32) | c)
+               : "memory");
+}
+__device__ __forceinline__ Word128 get128(const Word128* p) {
+  unsigned long long lo, hi;
+  asm volatile("{\n .reg .b128 v;\n ld.relaxed.gpu.global.b128 v, [%2];\n mov.b128 {%0, %1}, v;\n}"
+               : "=l"(lo), "=l"(hi)
+               : "l"(p)
+               : "memory");
+  Word128 w;
+  w.a = (uint32_t)lo;
+  w.b = (uint32_t)(lo >> 32);
+  w.c = (uint32_t)hi;
+  w.tag = (uint32_t)(hi >> 32);
+  return w;
+}
+
+// `count` words p[i * stride] in order, kIn in flight; false when a wait ran out.
+template <int kIn = 8, typename F>
 __device__ __forceinline__ bool gather(const unsigned long long* p, size_t stride, int count, unsigned tag, F&& take) {
-  for (int i0 = 0; i0 < count; i0 += 8) {
-    unsigned long long w[8];
+  for (int i0 = 0; i0 < count; i0 += kIn) {
+    unsigned long long w[kIn];
     for (unsigned it = 0;; ++it) {
       bool all = true;
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
+      for (int u = 0; u < kIn; ++u)
         if (i0 + u < count) w[u] = get(p + (size_t)(i0 + u) * stride);
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
+      for (int u = 0; u < kIn; ++u)
         if (i0 + u < count) all = all && is(w[u], tag);
       if (all) break;
       if (it > kSpinF) return false;
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < kIn; ++u)
       if (i0 + u < count) take(i0 + u, val(w[u]));
   }
   return true;
@@ -61,18 +84,31 @@ __device__ __forceinline__ bool warp_gather_sum(const unsigned long long* p, siz
   return __all_sync(0xffffffffu, ok);
 }
 
-// The words of a handle of B tokens: partial c [slab][token][k], partial ||x||^2 [slab][token],
-// partial ||r||^2 [cta][token], c [token][k], r [token][d].
-struct Words {
-  unsigned long long *c, *x2, *r2, *cf, *r;
+// The exchange area of a handle (or of the allocation-free entry point).  A location holds words
+// of one kind only, so a stale payload is never taken for a call's number.  Words are read at the
+// point of coherence (16 KB per microsecond and SM, whoever else reads them): what every CTA reads
+// in bulk (cb, rb) is plain memory, ordered by a fence before a word and one after it.
+struct Area {
+  unsigned long long* c;      // partial c [slab][token][k]
+  Word128* norm;              // [cta][token]: ||r||^2 and ||x||^2 of the CTA's rows
+  Word128* gate;              // [token]: rho, fired
+  unsigned char *cb, *rb;     // c and r as three bf16 terms, in operand order: [token][term_bytes(k or d)]
+  unsigned long long* flag;   // [cta]: its part of cb is written
+  unsigned long long *ext_r, *ext_x2, *ext_r2;   // basis extension: [d], [slab], [cta]
 };
-__device__ __forceinline__ Words words_of(const GroupParams& g) {
-  Words w;
+// Operand bytes of one column: 192 for every 32 elements (zeros past the end).
+__host__ __device__ __forceinline__ int term_bytes(int n) { return (n + 31) / 32 * 192; }
+__device__ __forceinline__ Area area_of(const GroupParams& g) {
+  Area w;
   w.c = g.fused_words;
-  w.x2 = w.c + (size_t)kFusedMaxGrid * g.B * kCols;
-  w.r2 = w.x2 + (size_t)kFusedMaxGrid * g.B;
-  w.cf = w.r2 + (size_t)kFusedMaxGrid * g.B;
-  w.r = w.cf + (size_t)g.B * g.k;
+  w.norm = reinterpret_cast<Word128*>(w.c + (size_t)kFusedMaxGrid * g.area_B * kCols);
+  w.gate = w.norm + (size_t)kFusedMaxGrid * g.area_B;
+  w.cb = reinterpret_cast<unsigned char*>(w.gate + g.area_B);
+  w.rb = w.cb + (size_t)g.area_B * term_bytes(g.area_k);
+  w.flag = reinterpret_cast<unsigned long long*>(w.rb + (size_t)g.area_B * term_bytes(g.area_d));
+  w.ext_x2 = w.flag + kFusedMaxGrid;
+  w.ext_r2 = w.ext_x2 + kFusedMaxGrid;
+  w.ext_r = w.ext_r2 + kFusedMaxGrid;
   return w;
 }
 

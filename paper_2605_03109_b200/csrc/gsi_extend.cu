@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
   const int G = gridDim.x, cta = blockIdx.x, d = g.d, k = g.k, KV = k / 8;
   const unsigned call = *g.fused_call;
   const int col = *a.k_active;
-  const Words words = words_of(g);
+  const Area words = area_of(g);
   const int p0 = (int)((long long)d * cta / G), p1 = (int)((long long)d * (cta + 1) / G);
   const int n_cb = (k + kCols - 1) / kCols;
   int lpr = 1;
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       for (int rb = r0; rb < r1; rb += kStage) {
         const int n = min(kStage, r1 - rb);
         __syncthreads();
-        ok = stage(s_v, pass == 1 ? a.x : nullptr, words.r, tag - 1u, rb, n) && ok;
+        ok = stage(s_v, pass == 1 ? a.x : nullptr, words.ext_r, tag - 1u, rb, n) && ok;
         __syncthreads();
         for (int base = warp * 8 + sub; base < n; base += kW * 8 * 4) {
           float p[4][8];
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
         float s = 0.f;
 #pragma unroll
         for (int w = 0; w < kW; ++w) s += s_c[w];
-        put(words.x2 + slab, s, tag);
+        put(words.ext_x2 + slab, s, tag);
       }
       __syncthreads();
     }
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       if (row < p1 && cl == 0) {
         const float rv = (pass == 1 ? __ldg(a.x + row) : g.r[row]) - dot;   // (g.r: written here in pass 1)
         g.r[row] = rv;
-        if (pass == 1) put(words.r + row, rv, tag);
+        if (pass == 1) put(words.ext_r + row, rv, tag);
         sr = fmaf(rv, rv, sr);
       }
     }
@@ -184,11 +184,11 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       float s = 0.f;
 #pragma unroll
       for (int w = 0; w < kW; ++w) s += s_part[w];
-      put(words.r2 + cta, s, tag);
+      put(words.ext_r2 + cta, s, tag);
     }
     if (warp < 2) {
       double s = 0.0;
-      ok = warp ? warp_gather_sum(words.x2, 1, n_slabs, tag, s) : warp_gather_sum(words.r2, 1, G, tag, s);
+      ok = warp ? warp_gather_sum(words.ext_x2, 1, n_slabs, tag, s) : warp_gather_sum(words.ext_r2, 1, G, tag, s);
       if (lane == 0) s_norm[warp] = s;
     }
     if (give_up(ok)) return;
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       if (a.P16) a.P16[pack::t16_slot(i, col, k)] = b;
       stored = __uint_as_float((uint32_t)b << 16);
     }
-    put(words.r + i, stored, tag);
+    put(words.ext_r + i, stored, tag);
     m = fmaxf(m, fabsf(stored));
   }
   if (a.pmax) {   // non-negative floats order like their bit patterns
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
     const int n = min(kStage, d - c0);
     const bool last = c0 + n == d;
     __syncthreads();
-    if (give_up(stage(s_v, nullptr, words.r, tag, c0, n))) return;
+    if (give_up(stage(s_v, nullptr, words.ext_r, tag, c0, n))) return;
     for (int row = o0 + warp; row < o1; row += kW) {
       int j = 0;
       while (j + 1 < g.n_maps && row >= g.off[j + 1]) ++j;

@@ -2,8 +2,8 @@
 // cooperative kernel (every CTA resident).
 //
 //   A   partial c of a slab of basis rows x 32 columns per CTA              (line 1)
-//   x1  the partials are added in slab order: by every CTA for itself in calls of a few tokens,
-//       else each coefficient by one CTA, which passes the sum on to all
+//   x1  the partials are added in a fixed order: by every CTA for itself in calls of one or two
+//       tokens, else each coefficient by one CTA, which passes its terms on to all
 //   B   r of its rows of the basis, then y = W_P c of its image rows        (lines 2, 5)
 //   x2  every CTA gathers all partial norms and takes the gate decision     (lines 3-4, Eq. (3.3))
 //   C   gated tokens: y += W r over its rows of W                           (Eq. (3.2))
@@ -25,6 +25,8 @@
 // in an order that depends on the shape alone: results are reproducible, and a token's are the
 // same in a call of any size.
 // Every wait is bounded; a wait that gives up sets GSI_ERR_TIMEOUT and the CTA returns.
+#include <type_traits>
+
 #include "gsi_exchange.cuh"
 
 namespace gsi {
@@ -36,7 +38,10 @@ using namespace exchange;
 constexpr int kT = 512, kW = kT / 32;
 constexpr int kTileRows = 16 * kW;     // rows of a basis slab (and of W) per pass: 16 per warp
 constexpr int kPitch = 80;             // bytes between the staged 64-byte pieces: conflict-free ldmatrix
-constexpr int kDirectTokens = 4;       // calls of so few tokens gather the slabs' partials themselves
+constexpr int kDirectTokens = 2;       // calls of so few tokens gather the slabs' partials themselves
+constexpr int kDecideTokens = 4;       // calls of so few tokens decide the gates on every CTA
+constexpr int kSegs = 8;               // the slabs' partials are added in eight runs, these by a tree
+constexpr int kSlots = 16;             // 16-row units of the basis whose norms wait in shared memory
 // dynamic shared memory: operand terms (phase A: the slab), then partial sums
 constexpr int kOpBytes = 131072, kAuxBytes = 32768;
 constexpr int kSmemFused = kOpBytes + kAuxBytes;
@@ -70,10 +75,23 @@ __device__ __forceinline__ void split3_x8(const float (&v)[8], uint4 (&t)[3]) {
   for (int q = 0; q < 3; ++q) t[q] = make_uint4(w[0][q], w[1][q], w[2][q], w[3][q]);
 }
 
-// Operand of eight-token blocks: 16 bytes (eight neighbours of the contraction) of term q of
-// column (token) c at step s (32 of the contraction), lane quarter t.  Only the NC columns that
-// exist are stored.
-__device__ __forceinline__ int op_at(int s, int q, int c, int t, int NC) { return ((s * 3 + q) * NC + c) * 4 + t; }
+// Operand, per column (token) a run of `stride` bytes: for every step (32 of the contraction) and
+// term 64 bytes, the elements in order.  A stride of 64 modulo 128 bytes makes the reads (eight
+// columns x four lane quarters of 16 bytes) free of bank conflicts.
+__host__ __device__ __forceinline__ int op_stride(int steps) { return steps * 192 + ((steps & 1) ? 0 : 64); }
+// Byte offset of elements j, j + 1 (j even) of term q within a column.
+__device__ __forceinline__ int op_pair(int j, int q) { return ((j >> 5) * 3 + q) * 64 + (j & 31) * 2; }
+__device__ __forceinline__ void op_store_pair(unsigned char* column, int j, uint32_t hi, uint32_t mid, uint32_t lo) {
+  *reinterpret_cast<uint32_t*>(column + op_pair(j, 0)) = hi;
+  *reinterpret_cast<uint32_t*>(column + op_pair(j, 1)) = mid;
+  *reinterpret_cast<uint32_t*>(column + op_pair(j, 2)) = lo;
+}
+// ... of a column of `len` elements in global memory; the last pair brings the zeros past the end.
+__device__ __forceinline__ void terms_store_pair(unsigned char* column, int j, int len, const uint32_t (&t)[3]) {
+  op_store_pair(column, j, t[0], t[1], t[2]);
+  if (j + 2 == len)
+    for (j += 2; j & 31; j += 2) op_store_pair(column, j, 0u, 0u, 0u);
+}
 
 template <int NB>
 __device__ __forceinline__ void clear(float (&v)[NB][4]) {
@@ -84,16 +102,17 @@ __device__ __forceinline__ void clear(float (&v)[NB][4]) {
 }
 
 // sum[nb] += rows g and g + 8 (p0, p1: this lane's pointers to element 8 t of each row, null when
-// the row does not exist) x columns 8 nb .. 8 nb + 7 over steps s0, s0 + ds, .. < s1.  `op` holds
-// the operand from step op0 on; K: length of the contraction.  The tensor core's own accumulation
+// the row does not exist) x columns 8 nb .. 8 nb + 7 over steps s0, s0 + ds, .. < s1.  `op`: the
+// operand from step op0 on, NC columns; K: length of the contraction.  The tensor core's own accumulation
 // truncates (a chain of 48 instructions is 2e-6 off, ten times an FMA chain), so the products of
 // the leading terms start from zero in every step and are added in fp32; those of the lower
 // terms, 2^-8 of the value, go through one accumulator of their own (low).
 template <int NB, bool AF32, bool kStream>
 __device__ __forceinline__ void dot_steps(const void* p0, const void* p1, int K, int s0, int ds, int s1,
-                                          const uint4* op, int op0, int NC, float (&low)[NB][4], float (&sum)[NB][4]) {
+                                          const unsigned char* op, int stride, int op0, int NC, float (&low)[NB][4],
+                                          float (&sum)[NB][4]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  constexpr int U = AF32 ? 2 : 4;   // steps in flight
+  constexpr int U = AF32 || NB >= 4 ? 2 : 4;   // steps in flight
   constexpr int kTerms = AF32 ? 3 : 1;
 #pragma unroll 1
   for (int sb = s0; sb < s1; sb += U * ds) {
@@ -144,7 +163,8 @@ __device__ __forceinline__ void dot_steps(const void* p0, const void* p1, int K,
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
           uint4 b = make_uint4(0u, 0u, 0u, 0u);
-          if (nb * 8 + g < NC) b = op[op_at(s - op0, q, nb * 8 + g, t, NC)];
+          if (nb * 8 + g < NC)
+            b = *reinterpret_cast<const uint4*>(op + (nb * 8 + g) * stride + ((s - op0) * 3 + q) * 64 + t * 16);
 #pragma unroll
           for (int r = 0; r < kTerms; ++r) {
             float(&to)[4] = (q == 0 && r == 0) ? hi : low[nb];
@@ -166,21 +186,33 @@ __device__ __forceinline__ void add_low(const float (&low)[NB][4], float (&sum)[
     for (int i = 0; i < 4; ++i) sum[nb][i] += low[nb][i];
 }
 
+// `units` 16-byte units of NC operand columns from global to shared memory, all copies in flight.
+template <typename F>
+__device__ __forceinline__ void copy_columns(unsigned char* op, int stride, int units, int NC, F&& column) {
+  for (int c = 0; c < NC; ++c) {
+    const unsigned char* src = column(c);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(op + c * stride);
+    for (int i = threadIdx.x; i < units; i += kT)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 16), "l"(src + i * 16) : "memory");
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // y += W r for the fired tokens, 8 NB at a time.  A warp owns 16 of this CTA's rows of W and every
 // ks-th step of the contraction (narrow maps: several warps share 16 rows and their sums meet in
-// shared memory); r comes from the exchange words into operand form as much of the width at a
-// time as fits.
+// shared memory); r comes in operand form, as much of the width at a time as fits.
 template <int NB>
-__device__ __forceinline__ void stream_w(const GroupParams& g, const IoRef& io, const unsigned long long* rw,
-                                         unsigned tag, const int* s_fired, unsigned char* smem, int o0, int o1) {
+__device__ __forceinline__ void stream_w(const GroupParams& g, const IoRef& io, const unsigned char* rb,
+                                         const int* s_fired, unsigned char* smem, int o0, int o1) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lg = lane >> 2, lt = lane & 3;
   const int d = g.d, n_fired = s_fired[0], steps = (d + 31) / 32;
-  uint4* op = reinterpret_cast<uint4*>(smem);
+  unsigned char* op = smem;
   float* part = reinterpret_cast<float*>(smem + kOpBytes);   // [warp][16 rows][8 NB]
   static_assert(kW * 16 * 8 * NB * 4 <= kAuxBytes, "partial sums of the warps");
   for (int f0 = 0; f0 < n_fired; f0 += 8 * NB) {
     const int NC = min(8 * NB, n_fired - f0);
-    const int span = min(steps, kOpBytes / (192 * NC));   // steps whose operand fits (192 bytes per column)
+    const int span = min(steps, (kOpBytes / NC - 64) / 192);   // steps whose operand fits
+    const int stride = op_stride(span);
     for (int b0 = o0; b0 < o1; b0 += kTileRows) {
       const int rows = min(kTileRows, o1 - b0), tiles = (rows + 15) / 16;
       int ks = 1;
@@ -204,26 +236,13 @@ __device__ __forceinline__ void stream_w(const GroupParams& g, const IoRef& io, 
         const int s1 = min(steps, s0 + span);
         if (s0 > 0 || b0 == o0 || span < steps) {
           __syncthreads();   // the operand before is read
-          bool ok = true;
-          const int octets = (s1 - s0) * 4;   // eight elements each
-          for (int i = tid; i < octets * NC; i += kT) {
-            const int c = i / octets, o8 = i % octets, e = s0 * 32 + o8 * 8;
-            uint4 tm[3];
-            float v[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = 0.f;
-            if (e < d) ok = gather(rw + (size_t)s_fired[1 + f0 + c] * d + e, 1, 8, tag, [&](int q, float x) { v[q] = x; }) && ok;
-            split3_x8(v, tm);
-#pragma unroll
-            for (int q = 0; q < 3; ++q) op[op_at(o8 >> 2, q, c, o8 & 3, NC)] = tm[q];
-          }
-          if (__syncthreads_or(!ok)) {
-            if (tid == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
-            return;
-          }
+          copy_columns(op, stride, (s1 - s0) * 12, NC,
+                       [&](int c) { return rb + (size_t)s_fired[1 + f0 + c] * term_bytes(d) + s0 * 192; });
+          __syncthreads();
         }
         // step s belongs to warp s % ks (ks a power of two)
-        if (active) dot_steps<NB, false, true>(p[0], p[1], d, s0 + ((kq - s0) & (ks - 1)), ks, s1, op, s0, NC, low, sum);
+        if (active) dot_steps<NB, false, true>(p[0], p[1], d, s0 + ((kq - s0) & (ks - 1)), ks, s1, op, stride, s0,
+                                                NC, low, sum);
       }
       add_low<NB>(low, sum);
       auto add = [&](int tile_, int r16, int col, float v) {
@@ -258,29 +277,34 @@ __device__ __forceinline__ void stream_w(const GroupParams& g, const IoRef& io, 
   }
 }
 
-// 8 NB tokens at a time.  leave_from > 0: with that many gated tokens or more W r is left to the
-// tensor-core contraction that follows (r goes to g.r, the gated tokens to g.fired).
+// NB: eight-token blocks at a time in the projection.  leave_from > 0: with that many gated tokens or
+// more W r is left to the tensor-core contraction that follows (r goes to g.r, the gated tokens to
+// g.fired).
 template <int NB, bool PF32>
 __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io, int n_tokens, int n_slabs,
                                                          int leave_from) {
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ float s_x2[kW][8 * NB];                  // the warps' partial norms
-  __shared__ double s_norm[GSI_MAX_TOKENS][2];
+  __shared__ float2 s_unit[kSlots][GSI_MAX_TOKENS];    // ||r||^2, ||x||^2 of a 16-row unit of the basis
+  __shared__ float2 s_run[GSI_MAX_TOKENS];             // ... of the units before
+  __shared__ float s_rho[GSI_MAX_TOKENS];
+  __shared__ bool s_fast[GSI_MAX_TOKENS];
   __shared__ int s_fired[GSI_MAX_TOKENS + 1];
+  __shared__ int s_done;
   constexpr int kTerms = PF32 ? 3 : 1, kTok = 8 * NB;
   float* s_aux = reinterpret_cast<float*>(smem + kOpBytes);
-  uint4* op = reinterpret_cast<uint4*>(smem);
+  unsigned char* op = smem;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lg = lane >> 2, lt = lane & 3;
   const int G = gridDim.x, cta = blockIdx.x;
   const int d = g.d, k = g.k, n = n_tokens;
   const unsigned tag = *g.fused_call + 1u;
-  const Words words = words_of(g);
-  unsigned long long *cw = words.c, *xw = words.x2, *nw = words.r2, *cf = words.cf, *rw = words.r;
+  const Area words = area_of(g);
+  unsigned long long* cw = words.c;
   const int slot = io_slot(io);
   const float* x = io.x + (long long)slot * io.x_step_stride;
   const int o0 = (int)((long long)g.O * cta / G), o1 = (int)((long long)g.O * (cta + 1) / G);
-  const int p0 = (int)((long long)d * cta / G), p1 = (int)((long long)d * (cta + 1) / G);
+  const int p0 = (int)((long long)(d / 2) * cta / G) * 2, p1 = (int)((long long)(d / 2) * (cta + 1) / G) * 2;
 
+  if (tid == 0) s_done = 0;
   if (tid == 0 && o1 > o0) {   // the image rows are asked into the L2 while c is on its way
     const char* p = reinterpret_cast<const char*>(g.WP + (size_t)o0 * k);
     const size_t bytes = (size_t)(o1 - o0) * k * 2;
@@ -296,9 +320,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
     const int slab = cta / n_cb, cb = cta % n_cb;
     const int r0 = (int)((long long)d * slab / n_slabs), r1 = (int)((long long)d * (slab + 1) / n_slabs);
     for (int tb = 0; tb < n; tb += kTok) {
-      float acc[2][NB][4], sx[NB];
-#pragma unroll
-      for (int nb = 0; nb < NB; ++nb) sx[nb] = 0.f;
+      float acc[2][NB][4];
       clear<NB>(acc[0]);
       clear<NB>(acc[1]);
       for (int rb = r0; rb < r1; rb += kTileRows) {
@@ -339,11 +361,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
 #pragma unroll
           for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              split3_pair(xv[nb][2 * h], xv[nb][2 * h + 1], xt[nb][h]);
-              sx[nb] = fmaf(xv[nb][2 * h], xv[nb][2 * h], sx[nb]);
-              sx[nb] = fmaf(xv[nb][2 * h + 1], xv[nb][2 * h + 1], sx[nb]);
-            }
+            for (int h = 0; h < 2; ++h) split3_pair(xv[nb][2 * h], xv[nb][2 * h + 1], xt[nb][h]);
           // 8 x 8 blocks of the tile, transposed by the load: rows (k) 0-7 | 8-15 by columns (m) 0-7 | 8-15
           const int tr = 16 * warp + (lane & 7) + ((lane >> 4) << 3), tc = ((lane >> 3) & 1) * 16;
 #pragma unroll
@@ -370,15 +388,6 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
         }
       }
       // over the warps: 16 tokens at a time
-      if (cb == 0) {
-#pragma unroll
-        for (int nb = 0; nb < NB; ++nb) {
-          float s = sx[nb];
-          s += __shfl_xor_sync(0xffffffffu, s, 1);
-          s += __shfl_xor_sync(0xffffffffu, s, 2);
-          if (lt == 0) s_x2[warp][nb * 8 + lg] = s;
-        }
-      }
 #pragma unroll
       for (int nq = 0; nq < NB; nq += 2) {
         if (tb + nq * 8 >= n) break;
@@ -402,169 +411,263 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
         }
         __syncthreads();
       }
-      if (cb == 0 && tid < kTok && tb + tid < n) {
-        float s = 0.f;
-#pragma unroll
-        for (int w = 0; w < kW; ++w) s += s_x2[w][tid];
-        put(xw + (size_t)slab * n + tb + tid, s, tag);
-      }
       __syncthreads();
     }
   }
 
-  // ---- x1.  Sum of a coefficient over the slabs: Q threads, each its slabs in order
+  // ---- x1.  Coefficient i (= token * k + column) summed over the slabs by Q adjacent lanes: each
+  // adds kSegs / Q runs of slabs in order, the runs are added by a tree: the same sums for every Q
   bool ok = true;
-  int Q = 1;
-  while (2 * Q * k <= kT && Q < 8) Q *= 2;
-  auto slab_sum = [&](int i, bool live) -> float {   // i = token * k + j; all lanes of a group of Q
-    const int q = tid % Q;
-    float s = 0.f;
-    if (live) {
-      const int a = n_slabs * q / Q, b = n_slabs * (q + 1) / Q;
-      ok = gather(cw + (size_t)a * n * k + i, (size_t)n * k, b - a, tag, [&](int, float v) { s += v; }) && ok;
+  auto slab_sum = [&](int i, bool live, auto lanes) -> float {
+    constexpr int Q = decltype(lanes)::value, R = kSegs / Q;
+    float run[R];
+    int end[R];   // of the runs, from the first slab of this lane on
+    const int q = tid % Q, a = n_slabs * (q * R) / kSegs;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      run[r] = 0.f;
+      end[r] = n_slabs * (q * R + r + 1) / kSegs - a;
     }
+    if (live)
+      ok = gather<Q == 2 ? 12 : 4>(cw + (size_t)a * n * k + i, (size_t)n * k, end[R - 1], tag, [&](int u, float v) {
+#pragma unroll
+             for (int r = 0; r < R; ++r)
+               if (u < end[r] && (r == 0 || u >= end[r - 1])) run[r] += v;
+           }) && ok;
+#pragma unroll
+    for (int h = 1; h < R; h *= 2)
+#pragma unroll
+      for (int r = 0; r < R; r += 2 * h) run[r] += run[r + h];
+    float s = run[0];
+#pragma unroll
     for (int o = 1; o < Q; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
   };
-  const bool direct = n <= kDirectTokens;
-  if (!direct) {
-    const int i0 = (int)((long long)n * k * cta / G), i1 = (int)((long long)n * k * (cta + 1) / G);
-    for (int ib = i0; ib < i1; ib += kT / Q) {
-      const int i = ib + tid / Q;
-      const float s = slab_sum(i, i < i1);
-      if (i < i1 && tid % Q == 0) put(cf + i, s, tag);
-    }
-  }
-
-  // ---- x1 (end) and B
-  const int ksteps = (k + 31) / 32;
-  for (int tb = 0; tb < n; tb += kTok) {
-    const int NC = min(kTok, n - tb), items = NC * k;
-    unsigned short* op16 = reinterpret_cast<unsigned short*>(op);
-    auto store_c = [&](int i, float v) {   // i = column * k + j: the three terms of a coefficient
-      const int c = i / k, j = i - c * k;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        op16[op_at(j >> 5, q, c, (j >> 3) & 3, NC) * 8 + (j & 7)] = __bfloat16_as_ushort(h);
-        v -= __bfloat162float(h);
-      }
-    };
-    if (tb > 0) __syncthreads();
-    for (int i = tid; i < (ksteps * 32 - k) * NC; i += kT) {   // the operand beyond k
-      const int c = i % NC, j = k + i / NC;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) op16[op_at(j >> 5, q, c, (j >> 3) & 3, NC) * 8 + (j & 7)] = 0;
-    }
-    if (direct) {
-      for (int ib = 0; ib < items; ib += kT / Q) {
-        const int i = ib + tid / Q;
-        const float s = slab_sum(tb * k + i, i < items);
-        if (i < items && tid % Q == 0) store_c(i, s);
-      }
-    } else {
-      for (int ib = 0; ib < items; ib += 8 * kT) {
-        const int cnt = items > ib + tid ? min(8, (items - ib - tid + kT - 1) / kT) : 0;
-        ok = gather(cf + (size_t)tb * k + ib + tid, kT, cnt, tag, [&](int u, float v) { store_c(ib + tid + u * kT, v); }) && ok;
-      }
-    }
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
-      if (tid == 0 && cta == 0) *g.fused_call = tag;
-      return;
-    }
-    // units of 16 rows: first the basis rows, then (their norms travel meanwhile) the image rows
-    const int pt = (p1 - p0 + 15) / 16, ot = (o1 - o0 + 15) / 16;
-    float sr[NB][2];
-#pragma unroll
-    for (int nb = 0; nb < NB; ++nb) sr[nb][0] = sr[nb][1] = 0.f;
-    for (int u = warp; u < pt; u += kW) {
-      const int row = p0 + 16 * u + lg;
-      const void* pr[2];
-      float low[NB][4], sum[NB][4];
-      clear<NB>(low);
-      clear<NB>(sum);
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-        pr[h] = row + 8 * h < p1 ? static_cast<const char*>(g.P) + ((size_t)(row + 8 * h) * k + lt * 8) * (PF32 ? 4 : 2)
-                                 : nullptr;
-      dot_steps<NB, PF32, false>(pr[0], pr[1], k, 0, 1, ksteps, op, 0, NC, low, sum);
-      add_low<NB>(low, sum);
-#pragma unroll
-      for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int t = tb + nb * 8 + 2 * lt + (i & 1), r = row + 8 * (i >> 1);
-          if (t < n && r < p1) {
-            const float rv = __ldg(x + (size_t)t * d + r) - sum[nb][i];
-            put(rw + (size_t)t * d + r, rv, tag);
-            if (leave_from) g.r[(size_t)t * d + r] = rv;
-            sr[nb][i & 1] = fmaf(rv, rv, sr[nb][i & 1]);
-          }
-        }
-    }
-#pragma unroll
-    for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        float s = sr[nb][i];
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lg == 0) s_x2[warp][nb * 8 + 2 * lt + i] = s;
-      }
-    __syncthreads();
-    if (tid < NC) {
-      float s = 0.f;
-#pragma unroll
-      for (int w = 0; w < kW; ++w) s += s_x2[w][tid];
-      put(nw + (size_t)cta * n + tb + tid, s, tag);
-    }
-    // (warps without basis rows go first: units are dealt from the last warp down)
-    for (int u = kW - 1 - warp; u < ot; u += kW) {
-      const int row = o0 + 16 * u + lg;
-      const void* pr[2];
-      float low[NB][4], sum[NB][4];
-      clear<NB>(low);
-      clear<NB>(sum);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) pr[h] = row + 8 * h < o1 ? g.WP + (size_t)(row + 8 * h) * k + lt * 8 : nullptr;
-      dot_steps<NB, false, false>(pr[0], pr[1], k, 0, 1, ksteps, op, 0, NC, low, sum);
-      add_low<NB>(low, sum);
-#pragma unroll
-      for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int t = tb + nb * 8 + 2 * lt + (i & 1), r = row + 8 * (i >> 1);
-          if (t < n && r < o1) io.y[(size_t)t * g.O + r] = sum[nb][i];
-        }
-    }
-  }
-
-  // ---- x2: norms, gate (the same sums in the same order on every CTA)
-  for (int i = warp; i < 2 * n; i += kW) {
-    const int t = i >> 1;
-    double s = 0.0;
-    ok = ((i & 1) ? warp_gather_sum(xw + t, n, n_slabs, tag, s) : warp_gather_sum(nw + t, n, G, tag, s)) && ok;
-    if (lane == 0) s_norm[t][i & 1] = s;
-  }
-  if (__syncthreads_or(!ok)) {
+  auto timed_out = [&](bool good) -> bool {   // the same answer for every thread
+    if (!__syncthreads_or(!good)) return false;
     if (tid == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
     if (tid == 0 && cta == 0) *g.fused_call = tag;
-    return;
+    return true;
+  };
+  const bool direct = n <= kDirectTokens;
+  if (!direct) {
+    const int i0 = (int)((long long)n * (k / 2) * cta / G) * 2, i1 = (int)((long long)n * (k / 2) * (cta + 1) / G) * 2;
+    for (int ib = i0; ib < i1; ib += kT / 8) {
+      const int i = ib + tid / 8;
+      const float s = slab_sum(i, i < i1, std::integral_constant<int, 8>());
+      const float nx = __shfl_down_sync(0xffffffffu, s, 8);
+      if (i < i1 && tid % 16 == 0) {   // (i0, i1 and ib are even)
+        uint32_t t[3];
+        split3_pair(s, nx, t);
+        const int c = i / k;
+        terms_store_pair(words.cb + (size_t)c * term_bytes(k), i - c * k, k, t);
+        __threadfence();
+      }
+    }
+    if (timed_out(ok)) return;
+    if (tid == 0) put(words.flag + cta, 0.f, tag);
+    if (warp == 0) {
+      double unused;
+      ok = warp_gather_sum(words.flag, 1, G, tag, unused);
+      __threadfence();
+    }
   }
+
+  // ---- x1 (end) and B, as many tokens at a time as have their c in shared memory
+  const int ksteps = (k + 31) / 32, stride = op_stride(ksteps);
+  const int pt = (p1 - p0 + 15) / 16, ot = (o1 - o0 + 15) / 16;   // units of 16 rows
+  const int per_block = min(n, max(8, kOpBytes / stride / 8 * 8));
+  for (int tb = 0; tb < n; tb += per_block) {
+    const int NC = min(per_block, n - tb), ncb = (NC + 7) / 8;
+    if (tb > 0) __syncthreads();
+    if (tid < NC) s_run[tid] = make_float2(0.f, 0.f);
+    if (direct) {
+      const int tail = ksteps * 16 - k / 2;   // pairs of the operand beyond k
+      for (int i = tid; i < tail * NC; i += kT) op_store_pair(op + (i / tail) * stride, k + 2 * (i % tail), 0u, 0u, 0u);
+      for (int ib = 0; ib < NC * k; ib += kT / 2) {
+        const int i = ib + tid / 2;
+        const float s = slab_sum(tb * k + i, i < NC * k, std::integral_constant<int, 2>());
+        const float nx = __shfl_down_sync(0xffffffffu, s, 2);
+        if (i < NC * k && tid % 4 == 0) {
+          uint32_t t[3];
+          split3_pair(s, nx, t);
+          const int c = i >= k ? 1 : 0;
+          op_store_pair(op + c * stride, i - c * k, t[0], t[1], t[2]);
+        }
+      }
+      if (timed_out(ok)) return;
+    } else {
+      if (tb == 0 && timed_out(ok)) return;   // (every CTA's part of cb is there)
+      copy_columns(op, stride, ksteps * 12, NC, [&](int c) { return words.cb + (size_t)(tb + c) * term_bytes(k); });
+      __syncthreads();
+    }
+    // basis rows: a unit x eight tokens per warp.  The units' norms wait in shared memory and are
+    // added in order by the warp that hands in last; it sends them off while the image rows run.
+    for (int uc = 0; uc == 0 || uc < pt; uc += kSlots) {
+      const int nu = min(kSlots, pt - uc);
+      for (int it = warp; it < nu * ncb; it += kW) {
+        const int u = it / ncb, nb = it - u * ncb, t = tb + nb * 8 + 2 * lt;
+        const int row = p0 + 16 * (uc + u) + lg;
+        const void* pr[2];
+        float low[1][4], sum[1][4], xv[4];
+        clear<1>(low);
+        clear<1>(sum);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          xv[i] = (t + (i & 1) < tb + NC && row + 8 * (i >> 1) < p1) ? __ldg(x + (size_t)(t + (i & 1)) * d + row + 8 * (i >> 1)) : 0.f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          pr[h] = row + 8 * h < p1 ? static_cast<const char*>(g.P) + ((size_t)(row + 8 * h) * k + lt * 8) * (PF32 ? 4 : 2)
+                                   : nullptr;
+        dot_steps<1, PF32, false>(pr[0], pr[1], k, 0, 1, ksteps, op + nb * 8 * stride, stride, 0, NC - nb * 8, low, sum);
+        add_low<1>(low, sum);
+        float sr[2] = {0.f, 0.f}, sx[2] = {0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int tt = t + (i & 1), r = row + 8 * (i >> 1);
+          const bool live = tt < tb + NC && r < p1;
+          const float rv = live ? xv[i] - sum[0][i] : 0.f;
+          // two rows of a token are written together (p0 is even) by the lane of the even row
+          const float nx = __shfl_down_sync(0xffffffffu, rv, 4);
+          if (live && !(lg & 1)) {
+            uint32_t w[3];
+            split3_pair(rv, nx, w);
+            terms_store_pair(words.rb + (size_t)tt * term_bytes(d), r, d, w);
+          }
+          if (live && leave_from) g.r[(size_t)tt * d + r] = rv;
+          sr[i & 1] = fmaf(rv, rv, sr[i & 1]);
+          sx[i & 1] = fmaf(xv[i], xv[i], sx[i & 1]);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+#pragma unroll
+          for (int o = 4; o < 32; o <<= 1) {
+            sr[i] += __shfl_xor_sync(0xffffffffu, sr[i], o);
+            sx[i] += __shfl_xor_sync(0xffffffffu, sx[i], o);
+          }
+          if (lg == 0) s_unit[u][nb * 8 + 2 * lt + i] = make_float2(sr[i], sx[i]);
+        }
+      }
+      auto add_units = [&](int t) -> float2 {
+        float2 v = s_run[t];
+        for (int u = 0; u < nu; ++u) {
+          v.x += s_unit[u][t].x;
+          v.y += s_unit[u][t].y;
+        }
+        return v;
+      };
+      if (warp < nu * ncb) __threadfence();   // r before the word that announces it
+      if (uc + nu >= pt) {
+        __syncwarp();
+        int before = 0;
+        if (lane == 0) {
+          __threadfence_block();
+          before = atomicAdd(&s_done, 1);
+          __threadfence_block();
+        }
+        before = __shfl_sync(0xffffffffu, before, 0);
+        __syncwarp();
+        if (before == kW - 1) {
+          for (int t = lane; t < NC; t += 32) {
+            const float2 v = add_units(t);
+            put128(words.norm + (size_t)cta * n + tb + t, __float_as_uint(v.x), __float_as_uint(v.y), 0u, tag);
+          }
+          if (lane == 0) s_done = 0;
+        }
+      } else {
+        __syncthreads();
+        if (tid < NC) s_run[tid] = add_units(tid);
+        __syncthreads();
+      }
+    }
+    // image rows (the last warps, which have no basis rows in small calls, go first)
+    for (int it = kW - 1 - warp; it < ot * ncb; it += kW) {
+      const int u = it / ncb, nb = it - u * ncb, row = o0 + 16 * u + lg;
+      const void* pr[2];
+      float low[1][4], sum[1][4];
+      clear<1>(low);
+      clear<1>(sum);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) pr[h] = row + 8 * h < o1 ? g.WP + (size_t)(row + 8 * h) * k + lt * 8 : nullptr;
+      dot_steps<1, false, false>(pr[0], pr[1], k, 0, 1, ksteps, op + nb * 8 * stride, stride, 0, NC - nb * 8, low, sum);
+      add_low<1>(low, sum);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int t = tb + nb * 8 + 2 * lt + (i & 1), r = row + 8 * (i >> 1);
+        if (t < tb + NC && r < o1) io.y[(size_t)t * g.O + r] = sum[0][i];
+      }
+    }
+  }
+
+  // ---- x2: the norms of a token, every CTA's share, by one warp, added in double in a fixed order;
+  // the gate.  In small calls every CTA takes every decision (the same sums: the same decision),
+  // else token t's is taken by one CTA, which passes it on.
+  auto decide = [&](int t) -> bool {
+    constexpr int kPer = kFusedMaxGrid / 32;
+    Word128 w[kPer];
+    bool all = false;
+    for (unsigned it = 0; !all && it <= kSpinF; ++it) {
+      all = true;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int c = lane + 32 * i;
+        w[i] = Word128{0u, 0u, 0u, tag};
+        if (c < G) w[i] = get128(words.norm + (size_t)c * n + t);
+      }
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) all = all && w[i].tag == tag;
+      all = __all_sync(0xffffffffu, all);
+    }
+    ok = ok && all;
+    __threadfence();
+    double sr = 0.0, sx = 0.0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      sr += (double)__uint_as_float(w[i].a);
+      sx += (double)__uint_as_float(w[i].b);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      sr += __shfl_xor_sync(0xffffffffu, sr, o);
+      sx += __shfl_xor_sync(0xffffffffu, sx, o);
+    }
+    const double nr = sqrt(sr), nx = sqrt(sx);
+    if (lane == 0) s_rho[t] = (float)(nr / nx);
+    return nr < (double)g.eps * nx;   // false for NaN and for x = 0
+  };
+  if (n <= kDecideTokens) {
+    if (warp < n) {
+      const bool fast = decide(warp);
+      if (lane == 0) s_fast[warp] = fast;
+    }
+  } else {
+    for (int t = cta + warp * G; t < n; t += kW * G) {
+      const bool fast = decide(t);
+      if (lane == 0 && ok) put128(words.gate + t, __float_as_uint(s_rho[t]), fast ? 1u : 0u, 0u, tag);
+    }
+    __syncwarp();
+    if (warp < 2 && warp * 32 + lane < n) {
+      Word128 w = get128(words.gate + warp * 32 + lane);
+      for (unsigned it = 0; w.tag != tag && it <= kSpinF; ++it) w = get128(words.gate + warp * 32 + lane);
+      ok = ok && w.tag == tag;
+      s_fast[warp * 32 + lane] = w.b != 0u;
+      s_rho[warp * 32 + lane] = __uint_as_float(w.a);
+      __threadfence();
+    }
+  }
+  if (timed_out(ok)) return;
   if (warp == 0) {
     int f = 0;
     for (int t0 = 0; t0 < n; t0 += 32) {
       const int t = t0 + lane;
       bool fired = false;
       if (t < n) {
-        const double nr = sqrt(s_norm[t][0]), nx = sqrt(s_norm[t][1]);
-        const bool fast = nr < (double)g.eps * nx;   // false for NaN and for x = 0
+        const bool fast = s_fast[t];
         fired = !fast && !(g.flags & GSI_FLAG_STATIC_PROJECTION);
         if (cta == 0) {
           io.gate[(long long)slot * io.log_step_stride + t] = fast ? 0 : 1;
           float* rho = io.rho ? io.rho + (long long)slot * io.log_step_stride : g.rho_scratch;
-          rho[t] = (float)(nr / nx);
+          rho[t] = s_rho[t];
         }
       }
       const unsigned m = __ballot_sync(0xffffffffu, fired);
@@ -585,7 +688,9 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
   if (s_fired[0] == 0 || (leave_from && s_fired[0] >= leave_from)) return;
 
   // ---- C
-  stream_w<NB>(g, io, rw, tag, s_fired, smem, o0, o1);
+  if (s_fired[0] <= 8) stream_w<1>(g, io, words.rb, s_fired, smem, o0, o1);
+  else if (s_fired[0] <= 16) stream_w<2>(g, io, words.rb, s_fired, smem, o0, o1);
+  else stream_w<4>(g, io, words.rb, s_fired, smem, o0, o1);
 }
 
 template <int NB, bool PF32>
@@ -605,7 +710,8 @@ cudaError_t launch_fused_p(const GroupParams& g, const IoRef& io, int n, int sla
 }  // namespace
 
 size_t fused_words_bytes(int d, int k, int max_tokens) {
-  return 8 * ((size_t)kFusedMaxGrid * max_tokens * (kCols + 2) + (size_t)max_tokens * (k + d));
+  return 8 * ((size_t)kFusedMaxGrid * (max_tokens * (kCols + 2) + 3) + 2 * (size_t)max_tokens + d) +
+         (size_t)max_tokens * (term_bytes(k) + term_bytes(d));
 }
 
 int fused_grid() {
@@ -631,15 +737,9 @@ cudaError_t launch_forward_fused(const GroupParams& g, const IoRef& io, int n_to
   const int grid = fused_grid();
   if (!grid) return cudaErrorInvalidDevice;
   const int slabs = fused_slabs(g.d, g.k, grid);
-  // eight-token blocks at a time: those of the call, as far as their c fits (6 bytes per
-  // coefficient, padded to 32) and the sums fit the registers (four)
-  int nb = 1;
-  while (8 * nb < n_tokens && nb < 4 && 2 * nb * 48 * ((g.k + 31) / 32 * 32) <= kOpBytes) nb *= 2;
-  switch (nb) {
-    case 1: return launch_fused_p<1>(g, io, n_tokens, slabs, leave_from, grid, st);
-    case 2: return launch_fused_p<2>(g, io, n_tokens, slabs, leave_from, grid, st);
-    default: return launch_fused_p<4>(g, io, n_tokens, slabs, leave_from, grid, st);
-  }
+  return n_tokens <= 8    ? launch_fused_p<1>(g, io, n_tokens, slabs, leave_from, grid, st)
+         : n_tokens <= 16 ? launch_fused_p<2>(g, io, n_tokens, slabs, leave_from, grid, st)
+                          : launch_fused_p<4>(g, io, n_tokens, slabs, leave_from, grid, st);
 }
 
 }  // namespace gsi

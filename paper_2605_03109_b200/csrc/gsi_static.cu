@@ -20,9 +20,7 @@ constexpr int kMaxDevices = 64;
 constexpr size_t kOffCtrl = 0;     // call counter, status word
 constexpr size_t kOffRho = 256;
 constexpr size_t kOffWords = 512;  // exchange words
-constexpr size_t kStaticScratchBytes =
-    kOffWords + 8 * ((size_t)gsi::kFusedMaxGrid * kStaticMaxTokens * 34 +
-                     (size_t)kStaticMaxTokens * (kStaticMaxK + kStaticMaxD));
+constexpr size_t kStaticScratchBytes = 768 * 1024;   // fused_words_bytes of the largest call, checked below
 
 // The scratch itself.  In host code this name is only a stand-in for the
 // symbol: it is NOT a device address and must never be handed to a kernel.
@@ -94,7 +92,11 @@ extern "C" gsi_status_t gsi_forward_static(const void* const* W_host_array, cons
   unsigned char* base = nullptr;
   gsi_status_t st = scratch_for_current_device(&base);
   if (st != GSI_OK) return st;
-  if (fused_words_bytes(d, k, n_tokens) > kStaticScratchBytes - kOffWords) return GSI_ERR_UNSUPPORTED;
+  if (fused_words_bytes(kStaticMaxD, kStaticMaxK, kStaticMaxTokens) > kStaticScratchBytes - kOffWords)
+    return GSI_ERR_UNSUPPORTED;
+  g.area_B = kStaticMaxTokens;
+  g.area_k = kStaticMaxK;
+  g.area_d = kStaticMaxD;
   unsigned* ctrl = reinterpret_cast<unsigned*>(base + kOffCtrl);
   g.fused_call = ctrl;
   g.status = reinterpret_cast<int*>(ctrl + 1);
