@@ -100,8 +100,8 @@ def _check(code, where):
 
 
 def _stream_ptr(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:   # (the raw handle: building a Stream object costs 3 us a call)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -151,11 +151,11 @@ def gsi_forward_static(Ws, P, W_P, eps, x, y=None, gate=None, rho=None, stream=N
     d, k = int(P.shape[0]), int(P.shape[1])
     d_out = [int(W.shape[0]) for W in Ws]
     if y is None:
-        y = torch.empty((n, sum(d_out)), dtype=torch.float32, device=x.device)
+        y = x.new_empty((n, sum(d_out)))
     if gate is None:
-        gate = torch.empty(n, dtype=torch.uint8, device=x.device)
+        gate = x.new_empty(n, dtype=torch.uint8)
     if rho is None:
-        rho = torch.empty(n, dtype=torch.float32, device=x.device)
+        rho = x.new_empty(n)
     warr = (C.c_void_p * len(Ws))(*[W.data_ptr() for W in Ws])
     darr = (C.c_int * len(Ws))(*d_out)
     _check(lib.gsi_forward_static(warr, darr, len(Ws), P.data_ptr(), _dtype_code(P),
@@ -203,11 +203,11 @@ class Layer:
         assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous()
         n = int(x.shape[0])
         if y is None:
-            y = torch.empty((n, self.O), dtype=torch.float32, device=x.device)
+            y = x.new_empty((n, self.O))
         if gate is None:
-            gate = torch.empty(n, dtype=torch.uint8, device=x.device)
+            gate = x.new_empty(n, dtype=torch.uint8)
         if rho is None:
-            rho = torch.empty(n, dtype=torch.float32, device=x.device)
+            rho = x.new_empty(n)
         _check(lib.gsi_forward_n(self.handle, x.data_ptr(), n, y.data_ptr(), gate.data_ptr(),
                                  rho.data_ptr(), _stream_ptr(stream)), "gsi_forward_n")
         return y, gate, rho
@@ -228,8 +228,7 @@ class Layer:
         Returns (appended, rho) as device tensors.  Writes the basis tensor given at creation."""
         assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous() and x.numel() == self.d
         assert k_active.is_cuda and k_active.dtype == torch.int32 and k_active.numel() == 1
-        appended = torch.empty(1, dtype=torch.int32, device=x.device)
-        rho = torch.empty(1, dtype=torch.float32, device=x.device)
+        appended, rho = x.new_empty(1, dtype=torch.int32), x.new_empty(1)
         _check(lib.gsi_extend_basis(self.handle, x.data_ptr(), float(tau), k_active.data_ptr(),
                                     appended.data_ptr(), rho.data_ptr(), _stream_ptr(stream)),
                "gsi_extend_basis")

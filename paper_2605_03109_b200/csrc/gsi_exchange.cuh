@@ -48,6 +48,29 @@ __device__ __forceinline__ Word128 get128(const Word128* p) {
   return w;
 }
 
+// Words at(0) .. at(count - 1), four in flight; false when a wait ran out.
+template <typename P, typename F>
+__device__ __forceinline__ bool gather128(P&& at, int count, unsigned tag, F&& take) {
+  for (int i0 = 0; i0 < count; i0 += 4) {
+    Word128 w[4];
+    for (unsigned it = 0;; ++it) {
+      bool all = true;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u < count) w[u] = get128(at(i0 + u));
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u < count) all = all && w[u].tag == tag;
+      if (all) break;
+      if (it > kSpinF) return false;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u < count) take(i0 + u, w[u]);
+  }
+  return true;
+}
+
 // `count` words p[i * stride] in order, kIn in flight; false when a wait ran out.
 template <int kIn = 8, typename F>
 __device__ __forceinline__ bool gather(const unsigned long long* p, size_t stride, int count, unsigned tag, F&& take) {
@@ -85,15 +108,17 @@ __device__ __forceinline__ bool warp_gather_sum(const unsigned long long* p, siz
 }
 
 // The exchange area of a handle (or of the allocation-free entry point).  A location holds words
-// of one kind only, so a stale payload is never taken for a call's number.  Words are read at the
-// point of coherence (16 KB per microsecond and SM, whoever else reads them): what every CTA reads
-// in bulk (cb, rb) is plain memory, ordered by a fence before a word and one after it.
+// of one kind only, so a stale payload is never taken for a call's number.  What every CTA reads in
+// bulk only when some token is gated (rb) is plain memory, ordered by a fence before the norm words
+// and one after them; a barrier of its own for c, with its fences, took 6 us where the words take 2.
+// Every CTA starts a bulk read at another place: 148 readers in step at one place get 13 KB per
+// microsecond and SM, spread out 50.
 struct Area {
   unsigned long long* c;      // partial c [slab][token][k]
   Word128* norm;              // [cta][token]: ||r||^2 and ||x||^2 of the CTA's rows
   Word128* gate;              // [token]: rho, fired
-  unsigned char *cb, *rb;     // c and r as three bf16 terms, in operand order: [token][term_bytes(k or d)]
-  unsigned long long* flag;   // [cta]: its part of cb is written
+  Word128* cf;                // [token][k / 2]: two coefficients as three bf16 terms each
+  unsigned char* rb;          // r as three bf16 terms, in operand order: [token][term_bytes(d)]
   unsigned long long *ext_r, *ext_x2, *ext_r2;   // basis extension: [d], [slab], [cta]
 };
 // Operand bytes of one column: 192 for every 32 elements (zeros past the end).
@@ -103,10 +128,9 @@ __device__ __forceinline__ Area area_of(const GroupParams& g) {
   w.c = g.fused_words;
   w.norm = reinterpret_cast<Word128*>(w.c + (size_t)kFusedMaxGrid * g.area_B * kCols);
   w.gate = w.norm + (size_t)kFusedMaxGrid * g.area_B;
-  w.cb = reinterpret_cast<unsigned char*>(w.gate + g.area_B);
-  w.rb = w.cb + (size_t)g.area_B * term_bytes(g.area_k);
-  w.flag = reinterpret_cast<unsigned long long*>(w.rb + (size_t)g.area_B * term_bytes(g.area_d));
-  w.ext_x2 = w.flag + kFusedMaxGrid;
+  w.cf = w.gate + g.area_B;
+  w.rb = reinterpret_cast<unsigned char*>(w.cf + (size_t)g.area_B * (g.area_k / 2));
+  w.ext_x2 = reinterpret_cast<unsigned long long*>(w.rb + (size_t)g.area_B * term_bytes(g.area_d));
   w.ext_r2 = w.ext_x2 + kFusedMaxGrid;
   w.ext_r = w.ext_r2 + kFusedMaxGrid;
   return w;

@@ -189,11 +189,13 @@ __device__ __forceinline__ void add_low(const float (&low)[NB][4], float (&sum)[
 // `units` 16-byte units of NC operand columns from global to shared memory, all copies in flight.
 template <typename F>
 __device__ __forceinline__ void copy_columns(unsigned char* op, int stride, int units, int NC, F&& column) {
-  for (int c = 0; c < NC; ++c) {
-    const unsigned char* src = column(c);
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(op + c * stride);
-    for (int i = threadIdx.x; i < units; i += kT)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 16), "l"(src + i * 16) : "memory");
+  const int all = units * NC;
+  int f = (int)((long long)all * blockIdx.x / gridDim.x) + (int)threadIdx.x;   // (no two CTAs at the same place at a time)
+  for (int i = threadIdx.x; i < all; i += kT, f += kT) {
+    if (f >= all) f -= all;
+    const int c = f / units, u = f - c * units;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(op + c * stride + u * 16);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(column(c) + u * 16) : "memory");
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
@@ -277,11 +279,13 @@ __device__ __forceinline__ void stream_w(const GroupParams& g, const IoRef& io, 
   }
 }
 
-// NB: eight-token blocks at a time in the projection.  leave_from > 0: with that many gated tokens or
+// NB: eight-token blocks at a time in the projection.  kDirect: a build for calls of up to
+// kDirectTokens tokens (what the others need would cost it registers: 3 us at one token).  leave_from > 0: with that many gated tokens or
 // more W r is left to the tensor-core contraction that follows (r goes to g.r, the gated tokens to
 // g.fired).
-template <int NB, bool PF32>
-__global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io, int n_tokens, int n_slabs,
+template <int NB, bool PF32, bool kDirect>
+__global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__ GroupParams g, const __grid_constant__ IoRef io,
+                                                         int n_tokens, int n_slabs,
                                                          int leave_from) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ float2 s_unit[kSlots][GSI_MAX_TOKENS];    // ||r||^2, ||x||^2 of a 16-row unit of the basis
@@ -449,8 +453,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
     if (tid == 0 && cta == 0) *g.fused_call = tag;
     return true;
   };
-  const bool direct = n <= kDirectTokens;
-  if (!direct) {
+  if constexpr (!kDirect) {
     const int i0 = (int)((long long)n * (k / 2) * cta / G) * 2, i1 = (int)((long long)n * (k / 2) * (cta + 1) / G) * 2;
     for (int ib = i0; ib < i1; ib += kT / 8) {
       const int i = ib + tid / 8;
@@ -459,17 +462,8 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
       if (i < i1 && tid % 16 == 0) {   // (i0, i1 and ib are even)
         uint32_t t[3];
         split3_pair(s, nx, t);
-        const int c = i / k;
-        terms_store_pair(words.cb + (size_t)c * term_bytes(k), i - c * k, k, t);
-        __threadfence();
+        put128(words.cf + (i >> 1), t[0], t[1], t[2], tag);
       }
-    }
-    if (timed_out(ok)) return;
-    if (tid == 0) put(words.flag + cta, 0.f, tag);
-    if (warp == 0) {
-      double unused;
-      ok = warp_gather_sum(words.flag, 1, G, tag, unused);
-      __threadfence();
     }
   }
 
@@ -481,9 +475,9 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
     const int NC = min(per_block, n - tb), ncb = (NC + 7) / 8;
     if (tb > 0) __syncthreads();
     if (tid < NC) s_run[tid] = make_float2(0.f, 0.f);
-    if (direct) {
-      const int tail = ksteps * 16 - k / 2;   // pairs of the operand beyond k
-      for (int i = tid; i < tail * NC; i += kT) op_store_pair(op + (i / tail) * stride, k + 2 * (i % tail), 0u, 0u, 0u);
+    const int tail = ksteps * 16 - k / 2;   // pairs of the operand beyond k
+    for (int i = tid; i < tail * NC; i += kT) op_store_pair(op + (i / tail) * stride, k + 2 * (i % tail), 0u, 0u, 0u);
+    if constexpr (kDirect) {
       for (int ib = 0; ib < NC * k; ib += kT / 2) {
         const int i = ib + tid / 2;
         const float s = slab_sum(tb * k + i, i < NC * k, std::integral_constant<int, 2>());
@@ -495,12 +489,20 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
           op_store_pair(op + c * stride, i - c * k, t[0], t[1], t[2]);
         }
       }
-      if (timed_out(ok)) return;
     } else {
-      if (tb == 0 && timed_out(ok)) return;   // (every CTA's part of cb is there)
-      copy_columns(op, stride, ksteps * 12, NC, [&](int c) { return words.cb + (size_t)(tb + c) * term_bytes(k); });
-      __syncthreads();
+      const int half = k / 2, all = NC * half, mine = all > tid ? (all - tid + kT - 1) / kT : 0;
+      const int rot = (int)((long long)all * cta / G) + tid;   // (no two CTAs at the same place at a time)
+      auto place = [&](int u) {
+        const int f = rot + u * kT;
+        return f < all ? f : f - all;
+      };
+      ok = gather128([&](int u) { return words.cf + (size_t)tb * half + place(u); }, mine, tag,
+                     [&](int u, const Word128& w) {
+                       const int f = place(u), c = f / half;
+                       op_store_pair(op + c * stride, 2 * (f - c * half), w.a, w.b, w.c);
+                     }) && ok;
     }
+    if (timed_out(ok)) return;
     // basis rows: a unit x eight tokens per warp.  The units' norms wait in shared memory and are
     // added in order by the warp that hands in last; it sends them off while the image rows run.
     for (int uc = 0; uc == 0 || uc < pt; uc += kSlots) {
@@ -635,7 +637,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
     if (lane == 0) s_rho[t] = (float)(nr / nx);
     return nr < (double)g.eps * nx;   // false for NaN and for x = 0
   };
-  if (n <= kDecideTokens) {
+  if (kDirect || n <= kDecideTokens) {
     if (warp < n) {
       const bool fast = decide(warp);
       if (lane == 0) s_fast[warp] = fast;
@@ -693,25 +695,31 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(GroupParams g, IoRef io
   else stream_w<4>(g, io, words.rb, s_fired, smem, o0, o1);
 }
 
-template <int NB, bool PF32>
+template <int NB, bool PF32, bool kDirect>
 cudaError_t launch_fused_t(GroupParams g, IoRef io, int n_tokens, int n_slabs, int leave, int grid, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(k_forward_fused<NB, PF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kSmemFused);
-  if (e != cudaSuccess) return e;
+  auto kernel = k_forward_fused<NB, PF32, kDirect>;
+  static bool configured[64] = {};   // per device: the attribute belongs to the device's function
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+  if (dev >= 64 || !configured[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFused);
+    if (e != cudaSuccess) return e;
+    if (dev < 64) configured[dev] = true;
+  }
   void* args[] = {&g, &io, &n_tokens, &n_slabs, &leave};
-  return cudaLaunchCooperativeKernel((void*)k_forward_fused<NB, PF32>, dim3(grid), dim3(kT), args, kSmemFused, st);
+  return cudaLaunchCooperativeKernel((void*)kernel, dim3(grid), dim3(kT), args, kSmemFused, st);
 }
-template <int NB>
+template <int NB, bool kDirect>
 cudaError_t launch_fused_p(const GroupParams& g, const IoRef& io, int n, int slabs, int leave, int grid, cudaStream_t st) {
-  return g.p_f32 ? launch_fused_t<NB, true>(g, io, n, slabs, leave, grid, st)
-                 : launch_fused_t<NB, false>(g, io, n, slabs, leave, grid, st);
+  return g.p_f32 ? launch_fused_t<NB, true, kDirect>(g, io, n, slabs, leave, grid, st)
+                 : launch_fused_t<NB, false, kDirect>(g, io, n, slabs, leave, grid, st);
 }
 
 }  // namespace
 
 size_t fused_words_bytes(int d, int k, int max_tokens) {
-  return 8 * ((size_t)kFusedMaxGrid * (max_tokens * (kCols + 2) + 3) + 2 * (size_t)max_tokens + d) +
-         (size_t)max_tokens * (term_bytes(k) + term_bytes(d));
+  return 8 * ((size_t)kFusedMaxGrid * (max_tokens * (kCols + 2) + 2) + (size_t)max_tokens * (k + 2) + d) +
+         (size_t)max_tokens * term_bytes(d);
 }
 
 int fused_grid() {
@@ -737,9 +745,10 @@ cudaError_t launch_forward_fused(const GroupParams& g, const IoRef& io, int n_to
   const int grid = fused_grid();
   if (!grid) return cudaErrorInvalidDevice;
   const int slabs = fused_slabs(g.d, g.k, grid);
-  return n_tokens <= 8    ? launch_fused_p<1>(g, io, n_tokens, slabs, leave_from, grid, st)
-         : n_tokens <= 16 ? launch_fused_p<2>(g, io, n_tokens, slabs, leave_from, grid, st)
-                          : launch_fused_p<4>(g, io, n_tokens, slabs, leave_from, grid, st);
+  return n_tokens <= kDirectTokens ? launch_fused_p<1, true>(g, io, n_tokens, slabs, leave_from, grid, st)
+         : n_tokens <= 8           ? launch_fused_p<1, false>(g, io, n_tokens, slabs, leave_from, grid, st)
+         : n_tokens <= 16          ? launch_fused_p<2, false>(g, io, n_tokens, slabs, leave_from, grid, st)
+                                   : launch_fused_p<4, false>(g, io, n_tokens, slabs, leave_from, grid, st);
 }
 
 }  // namespace gsi
