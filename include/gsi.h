@@ -141,9 +141,10 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W_host_array,
  * max_tokens tokens (gsi_forward_n).  x [n][d] fp32; y [n][sum d_out] fp32;
  * gate_mask_out [n] bytes (1 = slow path, W r added); rho_out [n] fp32 or NULL.
  * Each token is processed independently of the others in the call (Algorithm 1
- * is per token); its rounding can depend on the size of the call: calls of 5 or
- * more tokens (bf16 basis; k, d and every d_out multiples of 128) sum in another
- * order and add W r from r rounded to bf16 (|dy| <= 3e-3 max|y|); with other
+ * is per token); its rounding can depend on the size of the call: calls of 2 or
+ * more tokens (bf16 basis; k, d and every d_out multiples of 128) beyond 32 tokens
+ * or n * d * sum d_out = 2^27 (in a stack always) sum in another order and add W r
+ * from r rounded to bf16 (|dy| <= 3e-3 max|y|); with other
  * shapes that rounding applies only from 33 gated tokens per call on, where
  * sum d_out * d is 2^25 or more, d a multiple of 64 and every d_out of 128.
  * Results of a given call are reproducible bit for bit.

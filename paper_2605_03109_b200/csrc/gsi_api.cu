@@ -28,6 +28,7 @@ struct Layout {
 
 constexpr int kTcMinFired = 5;  // fewer fired tokens: one pass of the CUDA-core GEMV
 constexpr double kOwnStreamBytes = 262144.0;   // W rows of a CTA up to which a gated residual stays on its group's share
+constexpr int kChains = 2;   // chains of a batched step side by side
 constexpr int kFrontMinTokens = 2;  // single-token calls: the CUDA-core front end
 
 bool tc_shapes_ok(const gsi_desc_t* d) {
@@ -158,11 +159,16 @@ struct gsi_stack {
   // the stack's own, forked from and joined to the caller's stream by events
   cudaStream_t aux = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  // batched steps: the chains of small kernels (projection, residual, gate, image) run on a
-  // stream of the stack's own with the highest priority, the gated-residual contractions stay
+  // batched steps: the chains of small kernels (projection, residual, gate, image) run on two
+  // streams of the stack's own with the highest priority; the gated-residual contractions stay
   // on the caller's stream: a contraction is ordered behind its group's gate by an event and
-  // runs beside the chains of the groups that follow (inputs are staged before the step)
-  cudaStream_t front_stream = nullptr;
+  // runs beside the chains of the groups that follow (inputs are staged before the step).
+  // alternate: small maps, where a step is the latency of its chains: those of consecutive groups
+  // on alternating streams (GPT-2 at 8 tokens, a quarter gated: 0.76 -> 0.55 ms).  With large
+  // maps the W stream sets the time, and a second chain only takes its SM slots (OPT at 64
+  // tokens 0.93 -> 1.02 ms for six layers): there it is for the second group of a declared pair.
+  cudaStream_t front[kChains] = {};
+  bool alternate = false;
   cudaEvent_t ev_resid = nullptr, ev_front_fork = nullptr, ev_front_join = nullptr;
   ~gsi_stack() {
     if (ev_fork) cudaEventDestroy(ev_fork);
@@ -171,7 +177,8 @@ struct gsi_stack {
     if (ev_resid) cudaEventDestroy(ev_resid);
     if (ev_front_fork) cudaEventDestroy(ev_front_fork);
     if (ev_front_join) cudaEventDestroy(ev_front_join);
-    if (front_stream) cudaStreamDestroy(front_stream);
+    for (cudaStream_t f : front)
+      if (f) cudaStreamDestroy(f);
   }
 };
 
@@ -651,18 +658,21 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
                 cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess))
       return GSI_ERR_CUDA;
   }
-  if (!s->persistent && !s->front_stream) {
+  if (!s->persistent && !s->ev_front_join) {
     bool any = false;   // some group takes the tensor-core front end at this batch
     for (const gsi_layer* h : s->groups)
       any = any || (h->has_tm && h->gp.front_min_tokens > 0 && s->B >= h->gp.front_min_tokens &&
                     !(h->desc.flags & (GSI_FLAG_DENSE | GSI_FLAG_STATIC_PROJECTION)));
     int least = 0, greatest = 0;
     if (any && (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess ||
-                cudaStreamCreateWithPriority(&s->front_stream, cudaStreamNonBlocking, greatest) != cudaSuccess ||
                 cudaEventCreateWithFlags(&s->ev_resid, cudaEventDisableTiming) != cudaSuccess ||
                 cudaEventCreateWithFlags(&s->ev_front_fork, cudaEventDisableTiming) != cudaSuccess ||
                 cudaEventCreateWithFlags(&s->ev_front_join, cudaEventDisableTiming) != cudaSuccess))
       return GSI_ERR_CUDA;
+    s->alternate = true;
+    for (const gsi_layer* h : s->groups) s->alternate = s->alternate && (double)h->lay.O * h->desc.d <= 8388608.0;
+    for (cudaStream_t& f : s->front)
+      if (any && cudaStreamCreateWithPriority(&f, cudaStreamNonBlocking, greatest) != cudaSuccess) return GSI_ERR_CUDA;
   }
   if (s->persistent) {
     // The cross-CTA exchange state of every group (accumulators, exchange words, arrival
@@ -798,14 +808,12 @@ static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t 
     }
     return GSI_OK;
   }
-  // fs: the stream the chains of small kernels run on
-  cudaStream_t fs = stream;
   ResidualLane lane{stream, s->ev_resid, false};
-  if (s->front_stream) {
-    if (cudaEventRecord(s->ev_front_fork, stream) != cudaSuccess ||
-        cudaStreamWaitEvent(s->front_stream, s->ev_front_fork, 0) != cudaSuccess)
-      return GSI_ERR_CUDA;
-    fs = s->front_stream;
+  const bool chains = s->front[0] != nullptr;
+  if (chains) {
+    if (cudaEventRecord(s->ev_front_fork, stream) != cudaSuccess) return GSI_ERR_CUDA;
+    for (cudaStream_t f : s->front)
+      if (cudaStreamWaitEvent(f, s->ev_front_fork, 0) != cudaSuccess) return GSI_ERR_CUDA;
   }
   auto enqueue_group = [&](int i, cudaStream_t st) -> bool {
     gsi_layer* h = s->groups[i];
@@ -820,28 +828,32 @@ static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t 
     io.log_step_stride = (long long)G * s->B;
     h->last_stream = stream;   // the joins below put all of the step's work in the caller's stream order
     return launch_generic_forward(h->gp, h->has_tm ? &h->tm : nullptr, io, s->B, st, nullptr,
-                                  s->front_stream ? &lane : nullptr, s->mode == 1) == cudaSuccess;
+                                  chains ? &lane : nullptr, s->mode == 1) == cudaSuccess;
   };
   for (int i = 0; i < G; ++i) {
-    if (s->aux && i + 1 < G && s->pair_first[i]) {
+    if (chains && s->alternate) {
+      if (!enqueue_group(i, s->front[i % kChains])) return GSI_ERR_CUDA;
+      continue;
+    }
+    const cudaStream_t main = chains ? s->front[0] : stream, side = chains ? s->front[1] : s->aux;
+    if (side && i + 1 < G && s->pair_first[i]) {
       // groups i and i+1 do not read each other's outputs: two chains of dependent launches
       // side by side (under stream capture this becomes a fork and a join in the graph)
-      if (cudaEventRecord(s->ev_fork, fs) != cudaSuccess ||
-          cudaStreamWaitEvent(s->aux, s->ev_fork, 0) != cudaSuccess)
+      if (cudaEventRecord(s->ev_fork, main) != cudaSuccess || cudaStreamWaitEvent(side, s->ev_fork, 0) != cudaSuccess)
         return GSI_ERR_CUDA;
-      if (!enqueue_group(i, fs) || !enqueue_group(i + 1, s->aux)) return GSI_ERR_CUDA;
-      if (cudaEventRecord(s->ev_join, s->aux) != cudaSuccess ||
-          cudaStreamWaitEvent(fs, s->ev_join, 0) != cudaSuccess)
+      if (!enqueue_group(i, main) || !enqueue_group(i + 1, side)) return GSI_ERR_CUDA;
+      if (cudaEventRecord(s->ev_join, side) != cudaSuccess || cudaStreamWaitEvent(main, s->ev_join, 0) != cudaSuccess)
         return GSI_ERR_CUDA;
       ++i;
       continue;
     }
-    if (!enqueue_group(i, fs)) return GSI_ERR_CUDA;
+    if (!enqueue_group(i, main)) return GSI_ERR_CUDA;
   }
-  if (s->front_stream &&   // the chains join the caller's stream, which holds the contractions
-      (cudaEventRecord(s->ev_front_join, fs) != cudaSuccess ||
-       cudaStreamWaitEvent(stream, s->ev_front_join, 0) != cudaSuccess))
-    return GSI_ERR_CUDA;
+  if (chains)   // the chains join the caller's stream, which holds the contractions
+    for (cudaStream_t f : s->front)
+      if (cudaEventRecord(s->ev_front_join, f) != cudaSuccess ||
+          cudaStreamWaitEvent(stream, s->ev_front_join, 0) != cudaSuccess)
+        return GSI_ERR_CUDA;
   if (use_counter && launch_advance_step(s->step, stream) != cudaSuccess) return GSI_ERR_CUDA;
   return GSI_OK;
 }

@@ -20,11 +20,11 @@ namespace {
 
 using namespace umma;
 
-constexpr int kStages3 = 4;
+constexpr int kStages3 = 2;   // (blocks of 82 KB find a slot beside the W stream sooner: four stages left a step 2-7 % slower)
 constexpr int kMaxN3 = 192;          // 3 terms x 64 tokens
 constexpr int kTmemCols3 = 256;      // power of two >= kMaxN3
 using Cfg3 = Cfg<kStages3, kMaxN3>;
-constexpr int kSmem3 = Cfg3::kSmem;  // 4 x (16 + 24) KB + slack
+constexpr int kSmem3 = Cfg3::kSmem;
 // residual / image: K = k is short (four 64-wide blocks at k = 256).  Up to 32 tokens the B
 // operand is small enough for four stages with two blocks per SM, so every weight box of a
 // tile is requested before the wait on the previous kernel; beyond, two stages.

@@ -255,6 +255,7 @@ cudaError_t launch_residual_gemm_tc(const GroupParams& g, const TmaMaps& tm, con
                                     int min_fired, bool mapped, int n_tokens,
                                     cudaStream_t stream, int* n_launches);
 int tc_splits(int O, int d);
+int tc_launches(int O, int d);   // kernels of a contraction
 bool tc_eligible(const GroupParams& g);
 // Batched front end on the tensor cores: c, r, gate and y = W_P c for n_tokens tokens.
 cudaError_t launch_front_tc(const GroupParams& g, const TmaMaps& tm, const IoRef& io,

@@ -374,9 +374,15 @@ cudaError_t dispatch_vpl(const GroupParams& g, const IoRef& io, int n_tokens, cu
 }
 
 // Which calls run as the one cooperative launch: those whose shape the tensor-core front end does
-// not take, and the small ones of the others.
-constexpr int kFusedFewTokens = 4;
-bool takes_fused(const GroupParams& g, bool front, int n_tokens) { return !front || n_tokens <= kFusedFewTokens; }
+// not take, and the small ones of the others unless they belong to a stack (whose chains of small
+// kernels run side by side: 48 GPT-2 groups of three tokens 0.72 ms, as cooperative launches 0.77
+// to 1.03 ms).  The line, measured over 768 x 2304 .. 4096 x 28672 (16 tokens, a tenth gated): the
+// one launch saves 5 us of launches, but adds W r of n tokens at 6 TFMA/s: 4096 x 4096 at 8 tokens
+// 25.5 against 30.5 us (all gated 30.7 against 30.4), at 48 tokens 37.2 against 31.6.
+bool takes_fused(const GroupParams& g, bool front, int n_tokens, bool in_stack) {
+  if (!front) return true;
+  return !in_stack && n_tokens <= 32 && (double)n_tokens * g.O * g.d <= 134217728.0;
+}
 
 // Gated tokens from which the fused launch leaves W r to the tensor-core contraction, 0 = never.
 // The fused launch reads W once for 32 tokens; the contraction reads it once for 64 but costs
@@ -391,6 +397,7 @@ int leave_to_contraction(const GroupParams& g, bool tc, int n_tokens) {
 cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, const IoRef& io,
                                    int n_tokens, cudaStream_t st, int* n_launches, ResidualLane* lane,
                                    bool per_stage) {
+  const bool in_stack = lane != nullptr;
   int dummy = 0;
   if (!n_launches) n_launches = &dummy;
   int grid = (g.O + kWarps - 1) / kWarps;
@@ -404,7 +411,7 @@ cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, cons
   }
   cudaError_t e;
   const bool front = tm && g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens;
-  if (!per_stage && takes_fused(g, front, n_tokens)) {
+  if (!per_stage && takes_fused(g, front, n_tokens, in_stack)) {
     const int leave = leave_to_contraction(g, tm != nullptr, n_tokens);
     if ((e = launch_forward_fused(g, io, n_tokens, leave, st)) != cudaSuccess) return e;
     *n_launches += 1;
@@ -442,15 +449,14 @@ cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, cons
 }
 
 int generic_launch_count(const GroupParams& g, int n_tokens, bool per_stage) {
-  // (a tensor-core contraction with one split over the depth writes y itself: no kernel that adds partial sums)
-  const int add = tc_splits(g.O, g.d) > 1 ? 1 : 0;
-  if (g.flags & GSI_FLAG_DENSE)
-    return (g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens) ? 2 + add : 1;
-  if (!per_stage && takes_fused(g, g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens, n_tokens))
-    return 1 + (leave_to_contraction(g, g.tc_min_fired > 0, n_tokens) ? 2 + add : 0);
+  const int tc = tc_launches(g.O, g.d);
+  const bool front = g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens;
+  if (g.flags & GSI_FLAG_DENSE) return front ? 2 + (tc_splits(g.O, g.d) > 1 ? 1 : 0) : 1;
+  if (!per_stage && takes_fused(g, front, n_tokens, true))
+    return 1 + (leave_to_contraction(g, g.tc_min_fired > 0, n_tokens) ? 1 + tc : 0);
   const bool stat = g.flags & GSI_FLAG_STATIC_PROJECTION;
-  if (g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens) return stat ? 4 : 5 + add;
-  return 4 + (stat ? 0 : 1 + (g.tc_min_fired > 0 ? 2 + add : 0));
+  if (front) return stat ? 4 : 4 + tc;
+  return 4 + (stat ? 0 : 1 + (g.tc_min_fired > 0 ? 1 + tc : 0));
 }
 
 cudaError_t launch_advance_step(int* step, cudaStream_t st) {

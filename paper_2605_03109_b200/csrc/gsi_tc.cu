@@ -48,6 +48,9 @@ __global__ void __launch_bounds__(256) k_pack_fired_bf16(GroupParams g, int min_
 // mapped == 0: B rows are the fired tokens compacted (N = fired count rounded up to 16).
 // mapped == 1: B rows are all n_tokens tokens of the call (row = token); only the columns
 //              of fired tokens are written out.
+// kCluster: the splits of a tile are a cluster; their sums meet in distributed shared memory, added
+// in split order by the ranks (a share of the columns each), and no partial sum goes to memory.
+template <bool kCluster>
 __global__ void __launch_bounds__(kThreadsTc, 2)
 k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, int min_fired, int splits,
                    int mapped, int n_tokens) {
@@ -94,7 +97,36 @@ k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, 
     }
     __syncthreads();
   }
-  if (skipped) {
+  if (kCluster && !skipped) {   // (the same for all blocks of the cluster)
+    float* part = reinterpret_cast<float*>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);   // [column][row]: the ring is consumed
+    if (!ok && threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
+    const unsigned long long mask = s_mask;
+    const int r = warp * 32 + lane;
+    for (int c0 = 0; c0 < N; c0 += 16) {
+      if (((mask >> c0) & 0xFFFFull) == 0ull) continue;
+      uint32_t v[16];
+      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
+      tmem_ld_wait();
+#pragma unroll
+      for (int c = 0; c < 16; ++c) part[(c0 + c) * kTM + r] = __uint_as_float(v[c]);
+    }
+    cluster_sync();
+#pragma unroll 2
+    for (int col = N * split / splits; col < N * (split + 1) / splits; ++col) {
+      if (!((mask >> col) & 1ull)) continue;
+      float v[8];   // (splits <= 8)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = q < splits ? ld_cluster(s32(part + col * kTM + r), q) : 0.f;
+      float sum = v[0];
+#pragma unroll
+      for (int q = 1; q < 8; ++q) sum += v[q];
+      const int tok = mapped ? col : g.fired[col];
+      asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(io.y + (size_t)tok * g.O + row0 + r), "f"(sum)
+                   : "memory");
+    }
+    cluster_sync();   // nobody leaves while its sums are being read
+  } else if (skipped) {
     // nothing to write
   } else if (!ok) {
     if (threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
@@ -243,6 +275,13 @@ cudaError_t launch_dense_gemm_tc(const GroupParams& g, const TmaMaps& tm, const 
   return cudaGetLastError();
 }
 
+// Deep narrow maps add their splits in distributed shared memory: 4096 x 16384 at 8 tokens 54 -> 50 us
+// a call, at 64 tokens 65.4 -> 64.5.  Wide maps have few splits, whose partial sums are cheap beside W
+// (12288 and 16384 rows, 64 tokens: a step 1.00 -> 1.27 ms as clusters); at small depths the two
+// cluster barriers cost what the second kernel does.
+static bool tc_cluster(int O, int d) { return d >= 4096 && tc_splits(O, d) >= 5; }
+int tc_launches(int O, int d) { return tc_splits(O, d) > 1 && !tc_cluster(O, d) ? 2 : 1; }
+
 int tc_splits(int O, int d) {
   const int tiles = O / kTM, nkb = d / kTK;
   if (tiles >= 148) return 1;   // a tile per CTA already fills the SMs: long pipelines, no partial sums to add
@@ -263,26 +302,32 @@ bool tc_eligible(const GroupParams& g) {
 cudaError_t launch_residual_gemm_tc(const GroupParams& g, const TmaMaps& tm, const IoRef& io,
                                     int min_fired, bool mapped, int n_tokens, cudaStream_t st,
                                     int* n_launches) {
-  cudaError_t e = cudaFuncSetAttribute(k_residual_gemm_tc,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-  if (e != cudaSuccess) return e;
   const int splits = tc_splits(g.O, g.d);
+  const bool cluster = tc_cluster(g.O, g.d);
+  auto kernel = cluster ? k_residual_gemm_tc<true> : k_residual_gemm_tc<false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+  if (e != cudaSuccess) return e;
   if (!mapped) k_pack_fired_bf16<<<dim3((g.d + 2047) / 2048, kMaxN), 256, 0, st>>>(g, min_fired);
-  if (mapped) {
-    // straight after the residual kernel: both may start while their predecessor drains
-    if ((e = launch_pdl(k_residual_gemm_tc, dim3((g.O / kTM) * splits), dim3(kThreadsTc), kTcSmem, st, g,
-                        tm, io, min_fired, splits, 1, n_tokens)) != cudaSuccess)
-      return e;
-    if (splits > 1 &&
-        (e = launch_pdl(k_add_partials, dim3((g.O + 1023) / 1024, g.B), dim3(256), 0, st, g, io,
-                        min_fired, splits, 1)) != cudaSuccess)
-      return e;
-  } else {
-    k_residual_gemm_tc<<<(g.O / kTM) * splits, kThreadsTc, kTcSmem, st>>>(g, tm, io, min_fired, splits, 0,
-                                                                          n_tokens);
-    if (splits > 1) k_add_partials<<<dim3((g.O + 1023) / 1024, g.B), 256, 0, st>>>(g, io, min_fired, splits, 0);
-  }
-  if (n_launches) *n_launches += (mapped ? 1 : 2) + (splits > 1 ? 1 : 0);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((g.O / kTM) * splits);
+  cfg.blockDim = dim3(kThreadsTc);
+  cfg.dynamicSmemBytes = kTcSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // straight after the residual (or pack) kernel
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = splits;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster ? 2 : 1;
+  if ((e = cudaLaunchKernelEx(&cfg, kernel, g, tm, io, min_fired, splits, mapped ? 1 : 0, n_tokens)) != cudaSuccess)
+    return e;
+  if (splits > 1 && !cluster &&
+      (e = launch_pdl(k_add_partials, dim3((g.O + 1023) / 1024, g.B), dim3(256), 0, st, g, io, min_fired, splits,
+                      mapped ? 1 : 0)) != cudaSuccess)
+    return e;
+  if (n_launches) *n_launches += (mapped ? 0 : 1) + tc_launches(g.O, g.d);
   return cudaGetLastError();
 }
 

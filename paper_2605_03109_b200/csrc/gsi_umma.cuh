@@ -2,7 +2,7 @@
 // kernels: D[128 x N] (fp32, tensor memory) = A[128 x K] * B[N x K]^T with bf16
 // operands that are both K-major in global memory.
 //
-//   producer thread   TMA (cp.async.bulk.tensor, 128-byte swizzle, no multicast) brings a
+//   producer warp     TMA (cp.async.bulk.tensor, 128-byte swizzle, no multicast) brings a
 //                     stage = A box 128 rows x 64 K-elements + N/16 B boxes of 16 rows into
 //                     shared memory and signals the stage's "full" mbarrier by byte count
 //   MMA thread        waits "full", issues tcgen05.mma (accumulator in tensor memory),
@@ -68,6 +68,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, unsigned
   for (unsigned it = 0; it < spin; ++it)
     if (mbar_try(b, parity)) return true;
   return false;
+}
+// All blocks of the cluster; a word of shared memory of its rank `rank`.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float ld_cluster(uint32_t local, int rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
 }
 // One box of a 2-D tensor map: x = first K element, y = first row.
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
@@ -192,24 +203,22 @@ __device__ __forceinline__ bool tile_mma(unsigned char* smem_raw, const CUtensor
   }
 
   if (warp == 0) {
-    if (lane == 0) {   // producer
-      for (int i = 0; i < nloc; ++i) {
-        const int stage = i % kStages;
-        const uint32_t sa = s32(smem + stage * C::kStageBytes), sb = sa + kABytes;
-        const int x = (kb0 + i) * kTK;
-        if (i >= kStages) {
-          if (!mbar_wait(&bar_empty[stage], ((i / kStages) - 1) & 1)) {
-            *s_fail = 1;
-            break;
-          }
-          mbar_expect_tx(&bar_full[stage], stage_bytes);
-          tma_load_2d(sa, map_a, x, a_row0, &bar_full[stage]);
-        } else {
-          mbar_expect_tx(&bar_full[stage], stage_bytes - (uint32_t)kABytes);   // A is on its way
-        }
-        for (int j = 0; j < N / kBBox; ++j)
-          tma_load_2d(sb + j * (kBBox * kTK * 2), map_b, x, b_row0 + j * kBBox, &bar_full[stage]);
+    // producer: one lane per B box (an issue takes about a hundred cycles, a stage has up to twelve)
+    for (int i = 0; i < nloc; ++i) {
+      const int stage = i % kStages;
+      const uint32_t sa = s32(smem + stage * C::kStageBytes), sb = sa + kABytes;
+      const int x = (kb0 + i) * kTK;
+      if (i >= kStages && !__all_sync(0xffffffffu, mbar_wait(&bar_empty[stage], ((i / kStages) - 1) & 1))) {
+        if (lane == 0) *s_fail = 1;
+        break;
       }
+      if (lane == 0)   // (the first kStages blocks of A are on their way)
+        mbar_expect_tx(&bar_full[stage], i >= kStages ? stage_bytes : stage_bytes - (uint32_t)kABytes);
+      __syncwarp();
+      if (lane < N / kBBox)
+        tma_load_2d(sb + lane * (kBBox * kTK * 2), map_b, x, b_row0 + lane * kBBox, &bar_full[stage]);
+      else if (lane == N / kBBox && i >= kStages)
+        tma_load_2d(sa, map_a, x, a_row0, &bar_full[stage]);
     }
     __syncwarp();
   } else if (warp == 1) {

@@ -967,6 +967,27 @@ def test_tensor_core_front_end_batched_projection_residual_image(k, n_tokens):
     assert np.array_equal(yb.cpu().numpy(), y) and np.array_equal(rhob.cpu().numpy(), rho)
 
 
+@pytest.mark.parametrize("n_tokens,d_out", [(3, (128,)), (17, (256, 128)), (64, (4096,)), (33, (8192,))])
+def test_tensor_core_residual_splits_meet_in_a_cluster(n_tokens, d_out):
+    """Deep narrow maps: the splits of a tile are a cluster (two, three and 32 tiles of eight
+    splits; the widest case has five and sums them through memory)."""
+    d, k = 4096, 128
+    x, P, Ws = make_small(d, k, d_out, n_tokens, seed=970 + n_tokens, noise=0.001, outlier_every=2)
+    g = G()
+    lay = g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n_tokens)
+    stack = g.Stack([lay])
+    stack.bind([x.cuda().unsqueeze(0).contiguous()], n_steps=1)
+    outs = []
+    for _ in range(2):
+        stack.step()
+        torch.cuda.synchronize()
+        outs.append(stack.ys[0].cpu().clone())
+    assert stack.status() == 0 and torch.equal(*outs)
+    gate = stack.gate_log[0, 0].cpu().numpy()
+    assert 0 < gate.sum() < n_tokens
+    compare_group(x, P, Ws, 0.05, outs[0].numpy(), gate, stack.rho_log[0, 0].cpu().numpy())
+
+
 def test_tensor_core_residual_gemm_gptj_shape_sampled_rows():
     """One GPT-J-shaped group at batch 64 (d=4096 -> 4096, k=256), 25 % outliers."""
     st = S.config5(0.25, batch=64, steps=1)
