@@ -29,6 +29,7 @@ struct Layout {
 constexpr int kTcMinFired = 5;  // fewer fired tokens: one pass of the CUDA-core GEMV
 constexpr double kOwnStreamBytes = 262144.0;   // W rows of a CTA up to which a gated residual stays on its group's share
 constexpr int kChains = 2;   // chains of a batched step side by side
+constexpr int kMaxSegments = 12;   // of a step with host buffers
 constexpr int kFrontMinTokens = 2;  // single-token calls: the CUDA-core front end
 
 bool tc_shapes_ok(const gsi_desc_t* d) {
@@ -169,6 +170,12 @@ struct gsi_stack {
   // tokens 0.93 -> 1.02 ms for six layers): there it is for the second group of a declared pair.
   cudaStream_t front[kChains] = {};
   bool alternate = false;
+  // steps with host buffers: the groups in up to kMaxSegments segments, whose inputs, work and
+  // outputs overlap (a copy stream per direction); segment i begins with group (persistent
+  // schedule: phase) segment[i]
+  std::vector<int> segment;
+  cudaStream_t copy_in = nullptr, copy_out = nullptr;
+  cudaEvent_t ev_begin = nullptr, ev_in[kMaxSegments] = {}, ev_run[kMaxSegments] = {};
   cudaEvent_t ev_resid = nullptr, ev_front_fork = nullptr, ev_front_join = nullptr;
   ~gsi_stack() {
     if (ev_fork) cudaEventDestroy(ev_fork);
@@ -179,6 +186,13 @@ struct gsi_stack {
     if (ev_front_join) cudaEventDestroy(ev_front_join);
     for (cudaStream_t f : front)
       if (f) cudaStreamDestroy(f);
+    if (copy_in) cudaStreamDestroy(copy_in);
+    if (copy_out) cudaStreamDestroy(copy_out);
+    if (ev_begin) cudaEventDestroy(ev_begin);
+    for (cudaEvent_t e : ev_in)
+      if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : ev_run)
+      if (e) cudaEventDestroy(e);
   }
 };
 
@@ -621,6 +635,8 @@ gsi_status_t gsi_stack_set_mode(gsi_stack_t s, int mode) {
   return GSI_OK;
 }
 
+static bool plan_segments(gsi_stack* s);
+
 gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps,
                             unsigned char* gate_log, float* rho_log, gsi_stream_t stream) {
   if (!s || !io || n_steps <= 0 || !gate_log) return GSI_ERR_INVALID_ARG;
@@ -763,6 +779,7 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
         launch_patch_pmax(s->dev_groups, dev_ptrs, G, stream) != cudaSuccess)
       return GSI_ERR_CUDA;
   }
+  if (!plan_segments(s)) return GSI_ERR_CUDA;
   // A set-up call: the descriptor table and the cleared exchange state must be in
   // device memory before a step may be enqueued on ANY stream.
   if (cudaStreamSynchronize(stream) != cudaSuccess) return GSI_ERR_CUDA;
@@ -780,14 +797,19 @@ gsi_status_t gsi_stack_seek(gsi_stack_t s, int step, gsi_stream_t stream) {
              : GSI_ERR_CUDA;
 }
 
-static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t stream) {
+// The groups [g0, g1) of a step (persistent schedule: the phases [g0, g1)) whose inputs are there
+// once `ready` (null: everything enqueued on `stream` so far) has happened.  `first` / `last`: the
+// range opens / closes the step.
+static gsi_status_t stack_enqueue_range(gsi_stack_t s, int g0, int g1, bool first, bool last, bool use_counter,
+                                        cudaEvent_t ready, gsi_stream_t stream) {
   const int G = (int)s->groups.size();
+  if (ready && cudaStreamWaitEvent(stream, ready, 0) != cudaSuccess) return GSI_ERR_CUDA;
   if (s->persistent) {
     PersistParams p{};
     p.groups = s->dev_groups;
     p.n_groups = G;
-    p.phase_first = s->dev_phase_first;
-    p.n_phases = s->n_phases;
+    p.phase_first = s->dev_phase_first + g0;
+    p.n_phases = g1 - g0;
     p.step = s->step;
     p.epoch = s->epoch;
     p.n_steps = s->n_steps;
@@ -799,6 +821,7 @@ static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t 
     p.trace = s->trace;
     p.spin_limit = s->spin_limit - 1;   // the kernels give up when a wait has polled more than this many times without success
     p.n_tokens = s->B;
+    p.last = last ? 1 : 0;
     // one launch per token of the step (up to kPersistMaxTokens; larger batches take the
     // batched kernels): each is a complete decode step of that token, the last one advances
     for (int t = 0; t < s->B; ++t) {
@@ -811,9 +834,11 @@ static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t 
   ResidualLane lane{stream, s->ev_resid, false};
   const bool chains = s->front[0] != nullptr;
   if (chains) {
-    if (cudaEventRecord(s->ev_front_fork, stream) != cudaSuccess) return GSI_ERR_CUDA;
+    if (first && cudaEventRecord(s->ev_front_fork, stream) != cudaSuccess) return GSI_ERR_CUDA;
     for (cudaStream_t f : s->front)
-      if (cudaStreamWaitEvent(f, s->ev_front_fork, 0) != cudaSuccess) return GSI_ERR_CUDA;
+      if ((first && cudaStreamWaitEvent(f, s->ev_front_fork, 0) != cudaSuccess) ||
+          (ready && cudaStreamWaitEvent(f, ready, 0) != cudaSuccess))
+        return GSI_ERR_CUDA;
   }
   auto enqueue_group = [&](int i, cudaStream_t st) -> bool {
     gsi_layer* h = s->groups[i];
@@ -830,13 +855,13 @@ static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t 
     return launch_generic_forward(h->gp, h->has_tm ? &h->tm : nullptr, io, s->B, st, nullptr,
                                   chains ? &lane : nullptr, s->mode == 1) == cudaSuccess;
   };
-  for (int i = 0; i < G; ++i) {
+  for (int i = g0; i < g1; ++i) {
     if (chains && s->alternate) {
       if (!enqueue_group(i, s->front[i % kChains])) return GSI_ERR_CUDA;
       continue;
     }
     const cudaStream_t main = chains ? s->front[0] : stream, side = chains ? s->front[1] : s->aux;
-    if (side && i + 1 < G && s->pair_first[i]) {
+    if (side && i + 1 < g1 && s->pair_first[i]) {
       // groups i and i+1 do not read each other's outputs: two chains of dependent launches
       // side by side (under stream capture this becomes a fork and a join in the graph)
       if (cudaEventRecord(s->ev_fork, main) != cudaSuccess || cudaStreamWaitEvent(side, s->ev_fork, 0) != cudaSuccess)
@@ -854,8 +879,55 @@ static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t 
       if (cudaEventRecord(s->ev_front_join, f) != cudaSuccess ||
           cudaStreamWaitEvent(stream, s->ev_front_join, 0) != cudaSuccess)
         return GSI_ERR_CUDA;
-  if (use_counter && launch_advance_step(s->step, stream) != cudaSuccess) return GSI_ERR_CUDA;
+  if (last && use_counter && launch_advance_step(s->step, stream) != cudaSuccess) return GSI_ERR_CUDA;
   return GSI_OK;
+}
+
+static gsi_status_t stack_enqueue(gsi_stack_t s, bool use_counter, gsi_stream_t stream) {
+  return stack_enqueue_range(s, 0, s->persistent ? s->n_phases : (int)s->groups.size(), true, true, use_counter,
+                             nullptr, stream);
+}
+
+// First group of unit u (a phase of the persistent schedule, else a group).
+static int unit_group(const gsi_stack* s, int u) {
+  if (!s->persistent) return u;
+  return u < s->n_phases ? s->host_phase_first[u] : (int)s->groups.size();
+}
+
+// Cuts a step with host buffers into segments of about equal bytes, and makes the streams and
+// events that overlap them.
+static bool plan_segments(gsi_stack* s) {
+  const int units = s->persistent ? s->n_phases : (int)s->groups.size();
+  auto bytes = [&](int u) {
+    double b = 0.0;
+    for (int i = unit_group(s, u); i < unit_group(s, u + 1); ++i)
+      b += 4.0 * s->B * ((double)s->groups[i]->desc.d + s->groups[i]->lay.O);
+    return b;
+  };
+  double total = 0.0;
+  for (int u = 0; u < units; ++u) total += bytes(u);
+  // A copy of 1 MB takes 20 us.  A further launch of the persistent kernel costs about that (its
+  // opening and closing ticks), so two halves from 3 MB on (28 GPT-J groups: 776 us in one piece,
+  // 729 in two); the chains of batched steps go on from segment to segment without a gap: 3 MB
+  // each (8 GPT-J layers: 821 us at 8 tokens and 1968 at 64, where the step alone takes 1200 and the
+  // copies as long; in one piece, before the alternating chains, 1076 and 3359).
+  int n = s->persistent ? (s->B == 1 && total >= 3.0e6 ? 2 : 1) : (int)(total / 3.0e6);
+  n = std::max(1, std::min(n, std::min(units, kMaxSegments)));
+  s->segment.assign(1, 0);
+  double at = 0.0;
+  for (int u = 0; u < units && (int)s->segment.size() < n; ++u) {
+    at += bytes(u);
+    const bool inside_pair = !s->persistent && s->pair_first[u];
+    if (at >= total * s->segment.size() / n && !inside_pair && u + 1 < units) s->segment.push_back(u + 1);
+  }
+  s->segment.push_back(units);
+  if (s->segment.size() == 2 || s->copy_in) return true;
+  bool ok = cudaStreamCreateWithFlags(&s->copy_in, cudaStreamNonBlocking) == cudaSuccess &&
+            cudaStreamCreateWithFlags(&s->copy_out, cudaStreamNonBlocking) == cudaSuccess &&
+            cudaEventCreateWithFlags(&s->ev_begin, cudaEventDisableTiming) == cudaSuccess;
+  for (cudaEvent_t& e : s->ev_in) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+  for (cudaEvent_t& e : s->ev_run) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+  return ok;
 }
 
 gsi_status_t gsi_stack_step(gsi_stack_t s, gsi_stream_t stream) {
@@ -886,15 +958,16 @@ gsi_status_t gsi_stack_step_host(gsi_stack_t s, const float* const* x_host, floa
     if (!x_host[i] || !y_host[i]) return GSI_ERR_INVALID_ARG;
   // Runs of groups whose buffers are adjacent both on the host and on the device
   // (a caller that carves them out of one arena) travel as ONE copy.
-  auto copy_runs = [&](bool to_device) -> bool {
-    for (int i = 0; i < G;) {
+  auto copy_runs = [&](bool to_device, int g0, int g1, cudaStream_t st) -> bool {
+    bool merge = true;
+    for (int i = g0; i < g1;) {
       const char* h0 = to_device ? reinterpret_cast<const char*>(x_host[i])
                                  : reinterpret_cast<const char*>(y_host[i]);
       const char* d0 = to_device ? reinterpret_cast<const char*>(s->io[i].x)
                                  : reinterpret_cast<const char*>(s->io[i].y);
       size_t bytes = 0;
       int j = i;
-      for (; j < G; ++j) {
+      for (; j < g1 && (merge || j == i); ++j) {
         const size_t b = to_device ? (size_t)s->B * s->groups[j]->desc.d * 4
                                    : (size_t)s->B * s->groups[j]->lay.O * 4;
         const char* hj = to_device ? reinterpret_cast<const char*>(x_host[j])
@@ -905,22 +978,50 @@ gsi_status_t gsi_stack_step_host(gsi_stack_t s, const float* const* x_host, floa
         bytes += b;
       }
       const cudaError_t e =
-          to_device ? cudaMemcpyAsync(const_cast<char*>(d0), h0, bytes, cudaMemcpyHostToDevice, stream)
-                    : cudaMemcpyAsync(const_cast<char*>(h0), d0, bytes, cudaMemcpyDeviceToHost, stream);
-      if (e != cudaSuccess) return false;
+          to_device ? cudaMemcpyAsync(const_cast<char*>(d0), h0, bytes, cudaMemcpyHostToDevice, st)
+                    : cudaMemcpyAsync(const_cast<char*>(h0), d0, bytes, cudaMemcpyDeviceToHost, st);
+      if (e != cudaSuccess) {
+        if (j == i + 1) return false;
+        (void)cudaGetLastError();   // neighbours by chance, in allocations of their own: one copy each
+        merge = false;
+        continue;
+      }
       i = j;
     }
     return true;
   };
-  if (!copy_runs(true)) return GSI_ERR_CUDA;
   s->last_stream = stream;
-  gsi_status_t st = stack_enqueue(s, false, stream);
-  if (st != GSI_OK) return st;
-  if (!copy_runs(false)) return GSI_ERR_CUDA;
-  if (cudaMemcpyAsync(gate_host, s->gate_log, (size_t)G * s->B, cudaMemcpyDeviceToHost, stream) !=
-      cudaSuccess)
+  const int n = (int)s->segment.size() - 1;
+  if (n == 1) {
+    if (!copy_runs(true, 0, G, stream)) return GSI_ERR_CUDA;
+    gsi_status_t st = stack_enqueue(s, false, stream);
+    if (st != GSI_OK) return st;
+    if (!copy_runs(false, 0, G, stream)) return GSI_ERR_CUDA;
+    if (cudaMemcpyAsync(gate_host, s->gate_log, (size_t)G * s->B, cudaMemcpyDeviceToHost, stream) != cudaSuccess)
+      return GSI_ERR_CUDA;
+    return cudaStreamSynchronize(stream) == cudaSuccess ? GSI_OK : GSI_ERR_CUDA;
+  }
+  // Segment i + 1 is copied in and segment i - 1 copied out while segment i runs.
+  auto ok = [](cudaError_t e) { return e == cudaSuccess; };
+  if (!ok(cudaEventRecord(s->ev_begin, stream)) || !ok(cudaStreamWaitEvent(s->copy_in, s->ev_begin, 0)))
     return GSI_ERR_CUDA;
-  return cudaStreamSynchronize(stream) == cudaSuccess ? GSI_OK : GSI_ERR_CUDA;
+  for (int i = 0; i < n; ++i)
+    if (!copy_runs(true, unit_group(s, s->segment[i]), unit_group(s, s->segment[i + 1]), s->copy_in) ||
+        !ok(cudaEventRecord(s->ev_in[i], s->copy_in)))
+      return GSI_ERR_CUDA;
+  for (int i = 0; i < n; ++i) {
+    gsi_status_t st = stack_enqueue_range(s, s->segment[i], s->segment[i + 1], i == 0, i + 1 == n, false, s->ev_in[i], stream);
+    if (st != GSI_OK) return st;
+    if (!ok(cudaEventRecord(s->ev_run[i], stream))) return GSI_ERR_CUDA;
+  }
+  for (int i = 0; i < n; ++i)   // (after all work is enqueued: a copy to pageable memory holds the host)
+    if (!ok(cudaStreamWaitEvent(s->copy_out, s->ev_run[i], 0)) ||
+        !copy_runs(false, unit_group(s, s->segment[i]), unit_group(s, s->segment[i + 1]), s->copy_out))
+      return GSI_ERR_CUDA;
+  if (!ok(cudaMemcpyAsync(gate_host, s->gate_log, (size_t)G * s->B, cudaMemcpyDeviceToHost, stream)) ||
+      !ok(cudaEventRecord(s->ev_begin, s->copy_out)) || !ok(cudaStreamWaitEvent(stream, s->ev_begin, 0)))
+    return GSI_ERR_CUDA;
+  return ok(cudaStreamSynchronize(stream)) ? GSI_OK : GSI_ERR_CUDA;
 }
 
 gsi_status_t gsi_stack_set_trace(gsi_stack_t s, unsigned long long* cycles) {

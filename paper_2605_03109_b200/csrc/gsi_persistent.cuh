@@ -74,6 +74,7 @@ struct PersistParams {
   int use_counter;             // 0: I/O slot 0, counter not advanced
   int n_tokens, token;         // tokens per step, and the one this launch processes (one launch per token)
   int advance;                 // this launch advances the step counter (the last token's launch)
+  int last;                    // this launch ends the pass over the groups (a pass may be cut into launches: each group in one of them)
   unsigned char* gate_log;     // [n_steps][n_groups]
   float* rho_log;              // same shape or nullptr
   int log_step_stride;

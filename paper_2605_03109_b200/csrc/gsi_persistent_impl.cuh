@@ -1568,7 +1568,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
   // Every CTA read the counters at its start and has since taken part in the
   // last group's exchange, so they may advance now.
   if (cta == 0 && tid == 0 && ok && !*abort) {
-    *p.epoch = epoch + 1;
+    if (p.last) *p.epoch = epoch + 1;
     if (p.use_counter && p.advance) *p.step = step + 1;
   }
 }

@@ -329,6 +329,35 @@ def test_stack_step_host_matches_device_step(mode):
     assert torch.equal(gate_ref, gate_host)
 
 
+@pytest.mark.parametrize("n_tokens,pinned", [(1, True), (1, False), (16, True)])
+def test_step_host_in_segments_matches_the_device_step(n_tokens, pinned):
+    """Steps with enough host data run in segments whose copies overlap the work (single tokens: two
+    launches of one pass; batches: up to twelve): same bits as the device step, host and device steps
+    mixed on the same stack."""
+    g = G()
+    n_groups, d, k, d_out = (28, 256, 64, (30008,)) if n_tokens == 1 else (12, 512, 128, (16384,))
+    groups = [make_small(d, k, d_out, 2 * n_tokens, seed=8100 + i, noise=0.001, outlier_every=3 * (i % 2))
+              for i in range(n_groups)]
+    layers = [g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n_tokens) for _, P, Ws in groups]
+    stack = g.Stack(layers)
+    stack.bind([x[:n_tokens].cuda().contiguous() for x, _, _ in groups], n_steps=1)
+    assert stack.is_persistent() == (n_tokens == 1)
+    hold = (lambda t: t.pin_memory()) if pinned else (lambda t: t)
+    ys = [hold(torch.empty(n_tokens * sum(d_out))) for _ in groups]
+    gate = hold(torch.empty((n_groups, n_tokens), dtype=torch.uint8))
+    for part in (0, 1, 0):
+        xs = [hold(x[part * n_tokens:(part + 1) * n_tokens].contiguous()) for x, _, _ in groups]
+        stack.step_host(xs, ys, gate)
+        host = [y.clone() for y in ys], gate.clone()
+        stack.step()          # the inputs of the host step are in the device buffers now
+        torch.cuda.synchronize()
+        assert stack.status() == 0
+        assert torch.equal(stack.gate_log[0].cpu(), host[1])
+        assert part == 1 or 0 < int(host[1].sum()) < n_groups * n_tokens
+        for y, yh in zip(stack.ys, host[0]):
+            assert torch.equal(y.cpu().reshape(-1), yh)
+
+
 def test_gptj_layer_full_size_sampled_rows():
     """One GPT-J-shaped layer at full size (k=256, eps=0.05), batch 1, in the
     launch configuration the benchmark uses; the oracle evaluates a sample of
