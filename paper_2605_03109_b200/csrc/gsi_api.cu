@@ -516,16 +516,15 @@ gsi_status_t gsi_stack_create(int n_groups, const gsi_handle_t* groups, void* wo
   return GSI_OK;
 }
 
-// The basis rows and the image rows are dealt to the CTAs of a group's share in units of 16
-// rows: the least share whose rows fit a CTA's buffers.
-static int least_share(const gsi_layer* h) {
-  const int pt = (h->desc.d + 15) / 16, ot = (h->lay.O + 15) / 16;
-  return std::max((pt + kPersistMaxPRows / 16 - 1) / (kPersistMaxPRows / 16),
-                  (ot + kPersistMaxORows / 16 - 1) / (kPersistMaxORows / 16));
-}
+// Basis rows and image rows are dealt to the CTAs of a group's shares in units of 16 rows: the
+// least shares whose rows fit a CTA's buffers.
+static int p_tiles(const gsi_layer* h) { return (h->desc.d + 15) / 16; }
+static int o_tiles(const gsi_layer* h) { return (h->lay.O + 15) / 16; }
+static int least_p_share(const gsi_layer* h) { return (p_tiles(h) + kPersistMaxPRows / 16 - 1) / (kPersistMaxPRows / 16); }
+static int least_o_share(const gsi_layer* h) { return (o_tiles(h) + kPersistMaxORows / 16 - 1) / (kPersistMaxORows / 16); }
 static bool rows_fit(const gsi_layer* h, int ctas) {
   if ((h->desc.flags & GSI_FLAG_DENSE) || h->desc.k <= 0) return true;
-  return least_share(h) <= ctas;
+  return std::max(least_p_share(h), least_o_share(h)) <= ctas;
 }
 
 // W stream geometry of a group: whole rows per contiguous piece of at most 32 KB.
@@ -556,53 +555,76 @@ static bool persistent_eligible(const gsi_stack* s, int grid) {
   return true;
 }
 
-// Time of a phase of groups [i, i + len) in microseconds as the shares in `ncta` (filled in) leave
-// it, or a negative number when the rows do not fit.  A tick costs about 4 us whatever it carries
-// (the barriers, the scalar code and the latency of its sections); on top of that either the memory
-// system (6 bytes per picosecond) or the CTA with the longest row passes: rounds of fifteen 16-row
-// units, 0.85 us each at k = 256, and pass 1, 0.1 us per unit (per-warp timeline at the GPT-J
-// shapes).  The CTAs go one by one to the group whose rows take longest, basis rows counting
-// twice (pass 1 and residual).
-static double phase_cost(const gsi_stack* s, int i, int len, int* ncta) {
-  double bytes = 0.0, load[kPersistMaxLen];
-  int left = s->grid;
-  for (int j = 0; j < len; ++j) {
-    const gsi_layer* h = s->groups[i + j];
-    ncta[j] = least_share(h);
-    left -= ncta[j];
-    load[j] = (2.0 * h->desc.d + h->lay.O) * h->desc.k;
-    bytes += 2.0 * ((double)h->desc.d + h->lay.O) * h->desc.k;
-  }
-  if (left < 0) return -1.0;
+// Deals `grid` CTAs to `len` groups, at least least[j] to each, the next one always to the group
+// with the most load per CTA.  False when they do not suffice.
+static bool deal_ctas(int grid, int len, const double* load, const int* least, int* ncta) {
+  int left = grid;
+  for (int j = 0; j < len; ++j) left -= ncta[j] = least[j];
+  if (left < 0) return false;
   for (; left > 0; --left) {
     int at = 0;
     for (int j = 1; j < len; ++j)
       if (load[j] / ncta[j] > load[at] / ncta[at]) at = j;
     ++ncta[at];
   }
-  double rows = 0.0;
+  return true;
+}
+
+struct Shares {
+  int p = 0, o = 0, w = 0;   // CTAs for the basis rows, for the image rows, for W r beside the others of the phase
+};
+
+// Time of a phase of groups [i, i + len) in microseconds as the shares (filled in) leave it, or a
+// negative number when the rows do not fit.  Basis and image rows are dealt on their own, so that
+// every CTA carries about the same bytes of either: with one share per group, the CTAs of a wide
+// basis turn its slab over twice (pass 1, residual) in their ring, 147 KB each time at GPT-J's
+// 16384 -> 4096, while those beside them wait (28 GPT-J layers, nothing gated: 254 -> 219 us; 26
+// OPT layers at k = 512: 532 -> 518).  A tick costs about 4 us whatever it carries (the
+// barriers, the scalar code and the latency of its sections); on top of that either the memory
+// system (6 bytes per picosecond), or the CTA with the most rows: rounds of fifteen 16-row units,
+// 0.85 us each at k = 256, and pass 1, 0.1 us per unit.
+static double phase_cost(const gsi_stack* s, int i, int len, Shares* share) {
+  double bytes = 0.0, load[3][kPersistMaxLen];
+  int least[2][kPersistMaxLen], one[kPersistMaxLen], n[3][kPersistMaxLen];
   for (int j = 0; j < len; ++j) {
     const gsi_layer* h = s->groups[i + j];
-    const int pt = ((h->desc.d + 15) / 16 + ncta[j] - 1) / ncta[j], ot = ((h->lay.O + 15) / 16 + ncta[j] - 1) / ncta[j];
-    const int rounds = (pt + ot + kPersistConsumerWarps - 1) / kPersistConsumerWarps;
-    rows = std::max(rows, (0.85 * rounds + 0.1 * pt) * h->desc.k / 256.0);
+    load[0][j] = (double)h->desc.d * h->desc.k;
+    load[1][j] = (double)h->lay.O * h->desc.k;
+    load[2][j] = (double)h->lay.O * h->desc.d;
+    least[0][j] = least_p_share(h);
+    least[1][j] = least_o_share(h);
+    one[j] = 1;
+    bytes += 2.0 * ((double)h->desc.d + h->lay.O) * h->desc.k;
   }
+  if (!deal_ctas(s->grid, len, load[0], least[0], n[0]) || !deal_ctas(s->grid, len, load[1], least[1], n[1]) ||
+      !deal_ctas(s->grid, len, load[2], one, n[2]))
+    return -1.0;
+  double pt = 0.0, ot = 0.0;   // most units of one CTA, in units of k = 256
+  for (int j = 0; j < len; ++j) {
+    const gsi_layer* h = s->groups[i + j];
+    pt = std::max(pt, (p_tiles(h) + n[0][j] - 1) / n[0][j] * h->desc.k / 256.0);
+    ot = std::max(ot, (o_tiles(h) + n[1][j] - 1) / n[1][j] * h->desc.k / 256.0);
+    share[j].p = n[0][j];
+    share[j].o = n[1][j];
+    share[j].w = n[2][j];
+  }
+  const double rows = 0.85 * std::ceil((pt + ot) / kPersistConsumerWarps) + 0.1 * pt;
   return 4.0 + std::max(bytes / 6.0e6, rows);
 }
 
 // The phases of the persistent schedule: consecutive groups in one phase as far as that shortens
 // the step (inputs are staged before it), chosen over all partitions of the order.
-static void plan_phases(gsi_stack* s, std::vector<int>* first, std::vector<int>* share) {
+static void plan_phases(gsi_stack* s, std::vector<int>* first, std::vector<Shares>* share) {
   const int G = (int)s->groups.size();
   std::vector<double> best(G + 1, 0.0);   // cost of groups [i, G)
   std::vector<int> len(G, 1);
-  int ncta[kPersistMaxLen];
+  Shares parts[kPersistMaxLen];
   auto dense = [&](int i) { return (s->groups[i]->desc.flags & GSI_FLAG_DENSE) != 0; };
   for (int i = G - 1; i >= 0; --i) {
     best[i] = -1.0;
     for (int l = 1; l <= kPersistMaxLen && i + l <= G; ++l) {
       if (l > 1 && (dense(i) || dense(i + l - 1))) break;   // a dense group is a phase of its own
-      const double c = dense(i) ? 4.0 : phase_cost(s, i, l, ncta);
+      const double c = dense(i) ? 4.0 : phase_cost(s, i, l, parts);
       if (c < 0.0) break;
       if (best[i] < 0.0 || c + best[i + l] < best[i]) {
         best[i] = c + best[i + l];
@@ -611,7 +633,7 @@ static void plan_phases(gsi_stack* s, std::vector<int>* first, std::vector<int>*
     }
   }
   first->clear();
-  share->assign(G, s->grid);
+  share->assign(G, Shares{s->grid, s->grid, s->grid});
   for (int i = 0; i < G; i += len[i]) {
     first->push_back(i);
     if (!dense(i)) (void)phase_cost(s, i, len[i], share->data() + i);
@@ -733,7 +755,7 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
       pg.bar = h->bar;
       pg.x_step_stride = (long long)s->B * gp.d;
     }
-    std::vector<int> share;
+    std::vector<Shares> share;
     plan_phases(s, &s->host_phase_first, &share);
     s->has_pairs = false;
     s->common_k = -1;
@@ -741,26 +763,28 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
       const int i0 = s->host_phase_first[ph];
       const int i1 = ph + 1 < s->host_phase_first.size() ? s->host_phase_first[ph + 1] : G;
       if (i1 - i0 > 1) s->has_pairs = true;
-      int at = 0;
+      Shares at;
       for (int i = i0; i < i1; ++i) {
         PersistGroup& pg = s->host_groups[i];
         const gsi_layer* h = s->groups[i];
-        pg.cta0 = at;
-        pg.ncta = share[i];
+        pg.cta0 = at.p;
+        pg.ncta = share[i].p;
+        pg.o_cta0 = at.o;
+        pg.o_ncta = share[i].o;
         pg.phase_len = i1 - i0;
-        at += share[i];
         // rows are dealt in groups of 16: CTA c of the share owns groups [c n / ncta, (c + 1) n / ncta)
         // (the first n CTAs one group each when there are fewer groups than CTAs)
-        const int pgroups = (pg.d + 15) / 16, ogroups = (pg.O + 15) / 16;
-        pg.p_rows = 16 * ((pgroups + pg.ncta - 1) / pg.ncta);
-        pg.o_rows = 16 * ((ogroups + pg.ncta - 1) / pg.ncta);
-        pg.n_contrib = std::min(pg.ncta, pgroups);
-        // W r on the group's own share where a CTA's rows are few pieces: such a stream is a chain
+        pg.p_rows = 16 * ((p_tiles(h) + pg.ncta - 1) / pg.ncta);
+        pg.n_contrib = std::min(pg.ncta, p_tiles(h));
+        // W r on a share of the group's own where a CTA's rows are few pieces: such a stream is a chain
         // of latencies (2.5 us whatever its size), and those of a phase then run side by side
-        const bool own = !(pg.flags & GSI_FLAG_DENSE) && w_rows_fit(h, pg.ncta) &&
-                         (double)((pg.O + pg.ncta - 1) / pg.ncta) * pg.d * 2 <= kOwnStreamBytes;
-        pg.w_cta0 = (short)(own ? pg.cta0 : 0);
-        pg.w_ncta = (short)(own ? pg.ncta : s->grid);
+        const bool own = !(pg.flags & GSI_FLAG_DENSE) && w_rows_fit(h, share[i].w) &&
+                         (double)((pg.O + share[i].w - 1) / share[i].w) * pg.d * 2 <= kOwnStreamBytes;
+        pg.w_cta0 = (short)(own ? at.w : 0);
+        pg.w_ncta = (short)(own ? share[i].w : s->grid);
+        at.p += share[i].p;
+        at.o += share[i].o;
+        at.w += share[i].w;
         for (int j = 0; j < h->gp.n_maps; ++j)
           pg.w_rows[j] = (short)((h->gp.d_out[j] + pg.w_ncta - 1) / pg.w_ncta);
         if (!(pg.flags & GSI_FLAG_DENSE)) s->common_k = s->common_k < 0 || s->common_k == pg.k ? pg.k : 0;

@@ -48,11 +48,13 @@ struct PersistGroup {
   float eps;
   unsigned flags;
   float pmax;                        // max |P| (patched in on the device at bind time)
-  int p_rows, o_rows;                // most rows one CTA owns of P and of the images (multiples of 16)
+  int p_rows;                        // most rows of P one CTA owns (a multiple of 16)
   int n_contrib;                     // CTAs that own basis rows: the first min(ncta, ceil(d / 16)) of the share
   // Consecutive groups form a phase (their inputs are staged before the step): CTAs
-  // [cta0, cta0 + ncta) run this group's projection, residual and image.
-  int cta0, ncta;                    // this group's share of the grid (0, grid when alone)
+  // [cta0, cta0 + ncta) run this group's projection and residual, CTAs [o_cta0, o_cta0 + o_ncta)
+  // its image.
+  int cta0, ncta;                    // this group's shares of the grid (0, grid when alone)
+  int o_cta0, o_ncta;
   int phase_len;                     // groups in this group's phase
   // W stream (gated residual, dense baseline): CTA w_cta0 + i, i < w_ncta, owns rows
   // [i w_rows[j], (i + 1) w_rows[j]) of every map j (one contiguous run of memory), copied as

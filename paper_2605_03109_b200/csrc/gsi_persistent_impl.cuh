@@ -3,11 +3,10 @@
 // One CTA per SM.  Each CTA owns a fixed slab of rows of every basis P and of every
 // (concatenated) image W_P, and a fixed set of rows of every weight matrix W.  A producer
 // warp streams ALL weights from HBM into a ring of shared-memory slots: the slabs of P and
-// W_P with bulk async copies, the rows of W (gated residual, dense baseline) as TMA boxes of
-// up to 30 rows x 256 columns.  Weight addresses never depend on x, so the next group's slabs
+// W_P and whole rows of W (gated residual, dense baseline), all by bulk async copies.  Weight addresses never depend on x, so the next group's slabs
 // arrive while the current group waits on its exchange.  Fifteen consumer warps run
-// Algorithm 1 per group (two consecutive groups declared independent share a phase on two
-// parts of the grid).  A phase has ONE grid-wide exchange:
+// Algorithm 1 per group (consecutive groups share a phase; their basis rows and their image
+// rows are dealt to parts of the grid of their own).  A phase has ONE grid-wide exchange:
 //
 //   statistics  one warp: max |x| and sum x^2 over this CTA's rows of x (requested and
 //               published one row pass ahead: the inputs of a stack are pre-staged); the
@@ -69,17 +68,20 @@ constexpr unsigned long long kOne = 1ull << kCountShift;
 
 // What one CTA does in one tick of a launch, worked out once at the start of the launch.
 // Rows are dealt in groups of 16 (one tile row).
-struct Plan {
-  short gi;        // the group whose fast path (or dense stream) this CTA runs in this tick
+struct alignas(16) Plan {
+  short gi;        // the group whose basis rows (or dense stream) this CTA runs in this tick
+  short go;        // the group whose image rows it runs
   short gi0;       // first group of the tick's phase
+  short pg, og;                  // 16-row groups of the basis slab (of gi) and of the image slab (of go)
+  short pchunks, ochunks;        // ... their ring chunks
+  short pt0, ot0;                // ... and the first ones
+  short lc, n_contrib;           // index within gi's share of the grid; CTAs that own basis rows of gi
+  short o_contrib;               // CTAs that own basis rows of go
   unsigned char len;             // groups in this phase
   unsigned char kind;            // 0 nothing (closing ticks), 1 gated subspace group, 2 dense group
-  unsigned char zeroer;          // this CTA clears the group's counters for the next launch
-  short pg, og;                  // 16-row groups of the basis slab and of the image slab
-  short pchunks, ochunks;        // ... and their ring chunks
-  int p0, o0;                    // first rows
-  short lc, n_contrib;           // index within the group's share of the grid; CTAs that own basis rows
-  short gc_log2;                 // log2 of the 16-row groups per 16 KB chunk
+  unsigned char zeroer;          // this CTA clears the counters of gi for the next launch
+  unsigned char gc_log2, oc_log2;   // log2 of the 16-row groups per 16 KB chunk, of gi and of go (k = 512 >> log2)
+  unsigned char o_fp8;           // the image of go holds FP8 codes
 };
 static_assert(sizeof(Plan) == 32, "one plan record");
 
@@ -111,16 +113,15 @@ constexpr int kOffLin = 1024;       // producer: ring position (bytes placed bef
 constexpr int kOffOff = 1280;       // offset of every chunk in flight within the ring (kNB words), for the consumers
 constexpr int kOffMisc = 1536;      // scalars
 constexpr int kOffTrace = 1792;     // cycle counters of the trace (16 words)
-constexpr int kOffProd = 1920;      // state of the producer thread (16 bytes)
 constexpr int kOffX = 2048;         // x of this CTA's basis rows, three buffers (kPersistMaxPRows floats each)
 constexpr int kOffXt = kOffX + 3 * kPersistMaxPRows * 4;  // ... as three bf16 terms in A-operand order, two buffers
 constexpr int kXtBytes = kPersistMaxPRows / 16 * 256;     // (256 B per tile row)
-constexpr int kOffCb = kOffXt + 2 * kXtBytes;                 // c as three bf16 terms in B-operand order (32 tile columns x 256 B)
-constexpr int kOffFx = kOffCb + 8192;                     // fixed-point partial c and ||x||^2, source of the bulk reduction (514 words)
+constexpr int kOffCb = kOffXt + 2 * kXtBytes;                 // c of gi and of go as three bf16 terms in B-operand order (32 tile columns x 256 B each)
+constexpr int kOffFx = kOffCb + 2 * 8192;                     // fixed-point partial c and ||x||^2, source of the bulk reduction (514 words)
 constexpr int kOffPlan = kOffFx + 4224;                   // the launch's plan (kPersistMaxTicks records)
 constexpr int kOffSettle = kOffPlan + kPersistMaxTicks * 32;   // one record per group
 constexpr int kOffDesc = kOffSettle + kPersistMaxTicks * 32;   // descriptors of this CTA's groups, by phase
-constexpr int kDescSlots = 8;
+constexpr int kDescSlots = 8;   // two per phase, four phases
 constexpr int kOffYacc = kOffDesc + kDescSlots * 512;     // W stream: per-warp partial results (kNW x kPersistMaxWRows floats)
 constexpr int kOffRing = ((kOffYacc + kNW * kPersistMaxWRows * 4 + 1023) / 1024) * 1024;
 constexpr int kRingBytes = (232448 - kOffRing) / 1024 * 1024;
@@ -129,10 +130,16 @@ static_assert(kSmemBytes <= 232448, "shared memory budget of one sm_100 CTA");
 static_assert(kOffXt % 16 == 0 && kOffCb % 16 == 0 && kOffFx % 16 == 0 && kOffSettle % 16 == 0 && kOffPlan % 16 == 0 && kOffDesc % 16 == 0, "alignment");
 static_assert(sizeof(PersistGroup) <= 512 && sizeof(PersistGroup) % 4 == 0, "descriptor slot");
 constexpr int kDescWords = (int)(sizeof(PersistGroup) / 4);
+static_assert(2 * kDescWords <= kNC, "one thread per descriptor word");
+
+// Descriptor of the group whose basis rows (image = 0) or image rows (1) this CTA runs in phase ph.
+__device__ __forceinline__ unsigned char* desc_slot(unsigned char* smem, int ph, int image) {
+  return smem + kOffDesc + ((ph & 3) * 2 + image) * 512;
+}
 
 struct Misc {
   int abort;
-  unsigned amax_bits[2];    // by tick parity: max |x| of the phase's group (>= 0x7f800000: a non-finite token)
+  unsigned amax_bits[2][2]; // by role (basis rows, image rows) and tick parity: max |x| of the CTA's group (>= 0x7f800000: a non-finite token)
   float x2_part[2];         // this CTA's sum of x^2 over its rows, by tick parity
   unsigned fire[2];         // decisions on the previous phase's groups, by tick parity: bit u = stream W of group u
   double x2;                // ||x||^2 of this phase's group
@@ -276,189 +283,159 @@ struct Trace {
 // pair n % kNB.  The producer publishes the offset of chunk n in s_off[n % kNB] before it arms
 // the chunk's "full" barrier; producer and consumers walk the same sequence of chunks, so a
 // consumer needs only the sequence number.
-struct Producer {      // state of the producer thread, kept in shared memory
-  unsigned n;          // sequence number of the next chunk
-  unsigned lin;        // bytes placed so far
-  unsigned tail_n;     // oldest chunk not yet given back by the consumers
-  unsigned tail_lin;   // where it starts
-};
-
-// Reserve `bytes` for chunk n: waits (bounded) until the consumers have given back every
-// older chunk that still overlaps the place, and a barrier pair is free.  Returns the
-// offset, or 0xffffffff when a wait gave up.  Out of line: one copy for every kind of chunk.
-__device__ __noinline__ unsigned producer_acquire(unsigned char* smem, unsigned bytes) {
-  Producer& pr = *reinterpret_cast<Producer*>(smem + kOffProd);
-  uint64_t* empty = reinterpret_cast<uint64_t*>(smem + kOffBar) + kNB;
-  unsigned* s_lin = reinterpret_cast<unsigned*>(smem + kOffLin);
-  unsigned* s_off = reinterpret_cast<unsigned*>(smem + kOffOff);
-  volatile int* abort = &reinterpret_cast<Misc*>(smem + kOffMisc)->abort;
-  unsigned n = pr.n, lin = pr.lin, tail_n = pr.tail_n, tail_lin = pr.tail_lin;
-  unsigned off = lin % (unsigned)kRingBytes;
-  if (off + bytes > (unsigned)kRingBytes) {
-    lin += (unsigned)kRingBytes - off;
-    off = 0;
-  }
-  const unsigned start = lin;
-  lin += bytes;
-  while (n - tail_n >= (unsigned)kNB || (tail_n < n && lin - tail_lin > (unsigned)kRingBytes)) {
-    if (!mbar_wait(&empty[tail_n % kNB], (tail_n / kNB) & 1u, abort)) return 0xffffffffu;
-    ++tail_n;
-    tail_lin = tail_n < n ? s_lin[tail_n % kNB] : start;
-  }
-  if (tail_n == n) tail_lin = start;
-  s_lin[n % kNB] = start;
-  s_off[n % kNB] = off;
-  pr.lin = lin;
-  pr.tail_n = tail_n;
-  pr.tail_lin = tail_lin;
-  return off;
-}
-
-// The W stream of one group for this CTA: its w_rows[j] consecutive rows of every map j are
-// one contiguous run of memory, copied as contiguous pieces of w_pr whole rows (at most 32 KB:
-// large contiguous copies are what reaches the memory system's bandwidth).
-__device__ __forceinline__ bool produce_w(const PersistGroup& g, unsigned char* smem) {
-  Producer& prs = *reinterpret_cast<Producer*>(smem + kOffProd);
+//
+// The producer is one thread and ONE loop over chunks, its state in registers: every run of weights
+// (basis slab, image slab, a CTA's rows of one map) is contiguous memory, cut into chunks by the
+// same few instructions, and the next runs' addresses are fetched a tick ahead.  With the chunk
+// placed by an out-of-line function, its state in shared memory and a copy of the loop per kind of
+// run, a 16 KB chunk took 0.43 us to issue, and the ring could not turn over faster than 37 KB/us
+// per SM whatever the memory gave (28 GPT-J layers, nothing gated: 351 -> 254 us).
+__device__ void producer(const PersistParams& p, unsigned char* smem, Misc* misc) {
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kOffBar);
   uint64_t* empty = full + kNB;
   unsigned* s_lin = reinterpret_cast<unsigned*>(smem + kOffLin);
   unsigned* s_off = reinterpret_cast<unsigned*>(smem + kOffOff);
-  unsigned char* base = smem + kOffRing;
-  volatile int* abort = &reinterpret_cast<Misc*>(smem + kOffMisc)->abort;
-  // the ring state in registers for the length of the stream (thousands of pieces, one every
-  // few hundred cycles: the out-of-line acquire with its state in shared memory is too slow)
-  unsigned n = prs.n, lin = prs.lin, tail_n = prs.tail_n, tail_lin = prs.tail_lin;
-  bool ok = true;
-  const int cta = (int)blockIdx.x - g.w_cta0;
-  const int d = g.d, pr = g.w_pr;
-  if (cta < 0 || cta >= g.w_ncta) return true;
-  for (int j = 0; j < g.n_maps && ok; ++j) {
-    const int dout = g.off[j + 1] - g.off[j], rows = g.w_rows[j];
-    const int row0 = cta * rows;
-    const int live = min(rows, dout - row0);
-    for (int r0 = 0; r0 < live; r0 += pr) {
-      const uint32_t bytes = (uint32_t)min(pr, live - r0) * d * 2;
-      unsigned off = lin % (unsigned)kRingBytes;
-      if (off + bytes > (unsigned)kRingBytes) {
-        lin += (unsigned)kRingBytes - off;
-        off = 0;
-      }
-      const unsigned start = lin;
-      lin += bytes;
-      while (n - tail_n >= (unsigned)kNB || (tail_n < n && lin - tail_lin > (unsigned)kRingBytes)) {
-        if (!mbar_wait(&empty[tail_n % kNB], (tail_n / kNB) & 1u, abort)) {
-          ok = false;
-          break;
-        }
-        ++tail_n;
-        tail_lin = tail_n < n ? s_lin[tail_n % kNB] : start;
-      }
-      if (!ok) break;
-      if (tail_n == n) tail_lin = start;
-      s_lin[n % kNB] = start;
-      s_off[n % kNB] = off;
-      uint64_t* fb = &full[n % kNB];
-      mbar_expect_tx(fb, bytes);
-      bulk_g2s(base + off, g.W[j] + (size_t)(row0 + r0) * d, bytes, fb);
-      ++n;
-    }
-  }
-  prs.n = n;
-  prs.lin = lin;
-  prs.tail_n = tail_n;
-  prs.tail_lin = tail_lin;
-  return ok;
-}
-
-// Tile rows [a, b) (16 matrix rows each, row_bytes bytes) of a tiled matrix of rank k as chunks
-// of whole tile rows (as many per chunk as 16 KB hold of the bf16 form).
-__device__ __forceinline__ bool produce_rows(const void* base, int k, int row_bytes, int a, int b,
-                                             unsigned char* smem) {
-  Producer& pr = *reinterpret_cast<Producer*>(smem + kOffProd);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kOffBar);
-  const int gc = kChunk / (k * 32);
-  for (int r = a; r < b; r += gc) {
-    const int groups = min(gc, b - r);
-    const uint32_t bytes = (uint32_t)(groups * row_bytes);
-    const unsigned off = producer_acquire(smem, bytes);
-    if (off == 0xffffffffu) return false;
-    uint64_t* fb = &full[pr.n % kNB];
-    mbar_expect_tx(fb, bytes);
-    bulk_g2s(smem + kOffRing + off, static_cast<const char*>(base) + (size_t)r * row_bytes, bytes, fb);
-    ++pr.n;
-  }
-  return true;
-}
-
-__device__ void producer(const PersistParams& p, unsigned char* smem, Misc* misc) {
-  Producer& pr = *reinterpret_cast<Producer*>(smem + kOffProd);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kOffBar);
-  pr.n = 0;
-  pr.lin = 0;
-  pr.tail_n = 0;
-  pr.tail_lin = 0;
   volatile int* abort = &misc->abort;
+  unsigned n = 0;          // sequence number of the next chunk
+  unsigned lin = 0;        // bytes placed so far
+  unsigned off = 0;        // lin % kRingBytes
+  unsigned tail_n = 0;     // oldest chunk not yet given back by the consumers
+  unsigned tail_lin = 0;   // where it starts
   bool ok = true;
   // ticks: tick t runs the rows of phase t, pass 1 of phase t + 1 and the gated residuals of
   // phase t - 2; the work of a tick, in ring order (the order in which the consumers give the
-  // chunks back): the basis slab of phase t + 1 for pass 1 (that of the first phase comes before
-  // the first tick), the basis slab of phase t again for its residual rows, the image slab of
-  // phase t, the W pieces of the gated groups (or of a dense group)
+  // chunks back): run 0 the basis slab of phase t + 1 for pass 1 (that of the first phase in tick
+  // -1), run 1 the basis slab of phase t again for its residual rows (from the L2), run 2 the image
+  // slab of phase t, then the W rows of the gated groups and of a dense group, map by map (large
+  // contiguous pieces of whole rows are what reaches the memory system's bandwidth)
   const Plan* plan = reinterpret_cast<const Plan*>(smem + kOffPlan);
   const int n_ticks = p.n_phases + 2;
-  if (plan[0].kind == 1) {
-    const PersistGroup* g0 = p.groups + plan[0].gi;
-    ok = produce_rows(g0->P, g0->k, g0->k * 32, plan[0].p0 >> 4, (plan[0].p0 >> 4) + plan[0].pg, smem);
-  }
+  const int cta = (int)blockIdx.x;
+  auto basis_of = [&](int ph) -> const unsigned char* {
+    if (ph >= p.n_phases || plan[ph].kind != 1) return nullptr;
+    const Plan& pl = plan[ph];
+    return reinterpret_cast<const unsigned char*>(p.groups[pl.gi].P) + (size_t)pl.pt0 * (kChunk >> pl.gc_log2);
+  };
+  auto image_row_bytes = [&](const Plan& pl) {   // of 16 rows: one byte per element and 16 scales, or two bytes
+    const int b = kChunk >> pl.oc_log2;
+    return pl.o_fp8 ? b / 2 + 64 : b;
+  };
+  auto image_of = [&](int ph) -> const unsigned char* {
+    if (ph >= p.n_phases || plan[ph].kind != 1) return nullptr;
+    const Plan& pl = plan[ph];
+    return reinterpret_cast<const unsigned char*>(p.groups[pl.go].WP) + (size_t)pl.ot0 * image_row_bytes(pl);
+  };
+  const unsigned char *src_p = nullptr, *src_pn = basis_of(0), *src_i = nullptr, *src_in = image_of(0);
 #pragma unroll 1
-  for (int t = 0; t < n_ticks && ok; ++t) {
-    const Plan& pl = plan[t];
-    const PersistGroup* g = p.groups + pl.gi;   // read only when the tick has a group
-    if (t + 1 < p.n_phases && plan[t + 1].kind == 1) {
-      const Plan& pn = plan[t + 1];
-      const PersistGroup* gn = p.groups + pn.gi;
-      ok = produce_rows(gn->P, gn->k, gn->k * 32, pn.p0 >> 4, (pn.p0 >> 4) + pn.pg, smem);
-    }
-    if (ok && pl.kind == 1) {
-      ok = produce_rows(g->P, g->k, g->k * 32, pl.p0 >> 4, (pl.p0 >> 4) + pl.pg, smem);   // once more, for the residual rows
-      if (ok)
-        ok = produce_rows(g->WP, g->k, persist_image_row_bytes(g->k, g->flags & GSI_FLAG_FP8_IMAGE), pl.o0 >> 4,
-                          (pl.o0 >> 4) + pl.og, smem);
-    }
+  for (int t = -1; t < n_ticks && ok; ++t) {
+    const unsigned char* src_pf = basis_of(t + 2);   // (used in the next tick: their latency is hidden)
+    const unsigned char* src_if = image_of(t + 2);
     unsigned wmask = 0;
-    const int len_pp = t >= 2 ? plan[t - 2].len : 0, g_pp = t >= 2 ? plan[t - 2].gi0 : 0;
-    if (ok && len_pp > 0) {
-      // the decision on phase t - 2 (taken by the consumers during tick t - 1)
-      const unsigned want = (unsigned)(t - 1);   // (phase + 1)
-      unsigned v = 0, it = 0;
-      for (;;) {
-        v = misc->decision[(t - 2) & 3];
-        if ((v >> 8) == want) break;
-        if (++it > kLocalSpinLimit || *abort) {
-          ok = false;
-          break;
-        }
-      }
-      wmask = v & 0xffu;
-    }
-    // one call site for every W stream of the tick: the gated groups, then a dense group
-    if (wmask || pl.kind == 2) {
+    const PersistGroup* gw = nullptr;   // the group whose W rows stream, and its next map
+    int map = 0;
+    bool dense = t >= 0 && plan[t].kind == 2;
 #pragma unroll 1
-      for (; ok && (wmask || pl.kind == 2);) {
-        const PersistGroup* gw = g;
-        if (wmask) gw = &p.groups[g_pp + __ffs(wmask) - 1];
-        ok = produce_w(*gw, smem);
-        if (!wmask) break;
-        wmask &= wmask - 1;
+    for (int run = 0; ok; ++run) {
+      const unsigned char* src = nullptr;
+      uint32_t left = 0, piece = kChunk;
+      if (run == 0) {
+        src = src_pn;
+        if (src) left = (uint32_t)plan[t + 1].pg * (kChunk >> plan[t + 1].gc_log2);
+      } else if (run == 1) {
+        src = src_p;
+        if (src) left = (uint32_t)plan[t].pg * (kChunk >> plan[t].gc_log2);
+      } else if (run == 2) {
+        src = src_i;
+        if (src) {
+          const int rb = image_row_bytes(plan[t]);
+          left = (uint32_t)plan[t].og * rb;
+          piece = (uint32_t)rb << plan[t].oc_log2;
+        }
+      } else {
+        if (run == 3 && t >= 2 && plan[t - 2].len > 0) {
+          // the decision on phase t - 2 (taken by the consumers during tick t - 1)
+          const unsigned want = (unsigned)(t - 1);   // (phase + 1)
+          unsigned v = 0, it = 0;
+          for (;;) {
+            v = misc->decision[(t - 2) & 3];
+            if ((v >> 8) == want) break;
+            if (++it > kLocalSpinLimit || *abort) {
+              ok = false;
+              break;
+            }
+          }
+          if (!ok) break;
+          wmask = v & 0xffu;
+        }
+        if (!gw || map == gw->n_maps) {   // the next group: the gated ones, then a dense one
+          if (wmask) {
+            gw = p.groups + plan[t - 2].gi0 + __ffs(wmask) - 1;
+            wmask &= wmask - 1;
+          } else if (dense) {
+            gw = p.groups + plan[t].gi;
+            dense = false;
+          } else {
+            break;
+          }
+          map = 0;
+        }
+        const int wc = cta - gw->w_cta0;
+        if (wc < 0 || wc >= gw->w_ncta) {
+          map = gw->n_maps;
+          continue;
+        }
+        const int rows = gw->w_rows[map], row0 = wc * rows;
+        const int live = min(rows, gw->off[map + 1] - gw->off[map] - row0);
+        if (live > 0) {
+          const uint32_t rb = (uint32_t)gw->d * 2;
+          src = reinterpret_cast<const unsigned char*>(gw->W[map]) + (size_t)row0 * rb;
+          left = (uint32_t)live * rb;
+          piece = (uint32_t)gw->w_pr * rb;
+        }
+        ++map;
+      }
+#pragma unroll 1
+      while (left) {
+        const uint32_t bytes = min(piece, left);
+        if (off + bytes > (unsigned)kRingBytes) {   // a chunk never wraps
+          lin += (unsigned)kRingBytes - off;
+          off = 0;
+        }
+        const unsigned start = lin, slot = n % kNB;
+        lin += bytes;
+        // wait (bounded) until the consumers have given back every older chunk that still overlaps
+        // the place, and a barrier pair is free
+        while (n - tail_n >= (unsigned)kNB || (tail_n < n && lin - tail_lin > (unsigned)kRingBytes)) {
+          if (!mbar_wait(&empty[tail_n % kNB], (tail_n / kNB) & 1u, abort)) {
+            ok = false;
+            break;
+          }
+          ++tail_n;
+          tail_lin = tail_n < n ? s_lin[tail_n % kNB] : start;
+        }
+        if (!ok) break;
+        if (tail_n == n) tail_lin = start;
+        s_lin[slot] = start;
+        s_off[slot] = off;
+        mbar_expect_tx(&full[slot], bytes);
+        bulk_g2s(smem + kOffRing + off, src, bytes, &full[slot]);
+        ++n;
+        off += bytes;
+        src += bytes;
+        left -= bytes;
       }
     }
+    src_p = src_pn;
+    src_pn = src_pf;
+    src_i = src_in;
+    src_in = src_if;
   }
   if (!ok && !*abort) fail(p, misc, 1);
   // Every copy issued must have landed before the CTA may give up its shared
   // memory: wait (bounded) for the last kNB chunks.
   {
-    const unsigned first = pr.n > (unsigned)kNB ? pr.n - kNB : 0;
-    for (unsigned c = first; c < pr.n; ++c) {
+    const unsigned first = n > (unsigned)kNB ? n - kNB : 0;
+    for (unsigned c = first; c < n; ++c) {
       const unsigned slot = c % kNB, ph = (c / kNB) & 1u;
       for (unsigned it = 0; it < kLocalSpinLimit; ++it)
         if (mbar_try(&full[slot], ph)) break;
@@ -792,8 +769,8 @@ __device__ __forceinline__ unsigned w_stream(const PersistGroup* gp, const float
   return w_run(gp, q, in, y, dense, smem, n, status, traced);
 }
 
-// The statistics warp: the group's max |x| for tick `tt` from the tagged words of all
-// contributing CTAs (lane l owns words l, l+32, ...).  `first` holds a first round of loads
+// The statistics warp (the warp before it for the group of the CTA's image rows): the group's
+// max |x| for tick `tt` from the tagged words of all contributing CTAs (lane l owns words l, l+32, ...).  `first` holds a first round of loads
 // issued earlier (split phase: they flew while the warp did other work); further rounds are
 // polled here.  Out of line.
 constexpr int kXmaxWords = (kPersistMaxGrid + 31) / 32;
@@ -805,14 +782,14 @@ __device__ __forceinline__ void xmax_issue(const unsigned* xmax, int n_contrib, 
     w[i] = w_i < n_contrib ? ld_relaxed_u32(xmax + w_i) : 0xffffffffu;   // all loads in flight together
   }
 }
-__device__ __noinline__ void xmax_collect(unsigned char* smem, int tt, unsigned tag, unsigned spin_limit,
+__device__ __noinline__ void xmax_collect(unsigned char* smem, int tt, int image, unsigned tag, unsigned spin_limit,
                                           int* status, unsigned w0, unsigned w1, unsigned w2,
                                           unsigned w3, unsigned w4) {
   static_assert(kXmaxWords == 5, "argument list");
   const Plan& pn = reinterpret_cast<const Plan*>(smem + kOffPlan)[tt];
+  const int n_contrib = image ? pn.o_contrib : pn.n_contrib;
   Misc* misc = reinterpret_cast<Misc*>(smem + kOffMisc);
-  const PersistGroup& gn =
-      *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (tt & (kDescSlots - 1)) * 512);
+  const PersistGroup& gn = *reinterpret_cast<const PersistGroup*>(desc_slot(smem, tt, image));
   const int lane = threadIdx.x & 31;
   unsigned w[kXmaxWords] = {w0, w1, w2, w3, w4};
   unsigned m = 0, it = 0;
@@ -821,7 +798,7 @@ __device__ __noinline__ void xmax_collect(unsigned char* smem, int tt, unsigned 
     m = 0;
 #pragma unroll
     for (int i = 0; i < kXmaxWords; ++i) {
-      if (lane + 32 * i < pn.n_contrib) {
+      if (lane + 32 * i < n_contrib) {
         all = all && ((w[i] >> 31) == tag);
         m = max(m, w[i] & 0x7fffffffu);
       }
@@ -831,11 +808,11 @@ __device__ __noinline__ void xmax_collect(unsigned char* smem, int tt, unsigned 
       if (!misc->abort && lane == 0) fail_at(status, misc, 4);
       break;
     }
-    xmax_issue(gn.xmax, pn.n_contrib, w);
+    xmax_issue(gn.xmax, n_contrib, w);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) misc->amax_bits[tt & 1] = m;
+  if (lane == 0) misc->amax_bits[image][tt & 1] = m;
 }
 
 // The statistics warp, for tick `tt`: (request = true) ask for this CTA's rows of x into buffer
@@ -847,13 +824,12 @@ __device__ __noinline__ void stat_warp_step(unsigned char* smem, int tt, bool re
   const Plan& pn = reinterpret_cast<const Plan*>(smem + kOffPlan)[tt];
   if (pn.kind != 1) return;
   const int lane = threadIdx.x & 31;
-  const PersistGroup& gn =
-      *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (tt & (kDescSlots - 1)) * 512);
+  const PersistGroup& gn = *reinterpret_cast<const PersistGroup*>(desc_slot(smem, tt, 0));
   float* sx = reinterpret_cast<float*>(smem + kOffX) + (tt % 3) * kPersistMaxPRows;
   const int rows = pn.pg * 16;
   if (request) {
-    const float* src = gn.x + (long long)slot_io * gn.x_step_stride + (size_t)token * gn.d + pn.p0;
-    const int live = min(rows, gn.d - pn.p0);   // rows past d belong to the zero padding of P
+    const float* src = gn.x + (long long)slot_io * gn.x_step_stride + (size_t)token * gn.d + pn.pt0 * 16;
+    const int live = min(rows, gn.d - pn.pt0 * 16);   // rows past d belong to the zero padding of P
 #pragma unroll 1
     for (int i = lane; i < rows; i += 32) {
       if (i < live)
@@ -919,17 +895,20 @@ __device__ __forceinline__ void make_plan(const PersistParams& p, unsigned char*
 #pragma unroll 1
   for (int t = threadIdx.x; t < n_ticks; t += kThreadsP) {
     Plan pl{};
-    pl.gi = pl.gi0 = -1;
+    pl.gi = pl.go = pl.gi0 = -1;
     if (t < p.n_phases) {
       const int gi0 = __ldg(p.phase_first + t);
       const PersistGroup* ga = p.groups + gi0;
       const int len = kPairs ? __ldg(&ga->phase_len) : 1;
-      int gi = gi0;
-      if (kPairs)
+      int gi = gi0, go = gi0;
+      if (kPairs) {
         while (gi + 1 < gi0 + len && cta >= __ldg(&p.groups[gi + 1].cta0)) ++gi;
-      const PersistGroup* g = p.groups + gi;
+        while (go + 1 < gi0 + len && cta >= __ldg(&p.groups[go + 1].o_cta0)) ++go;
+      }
+      const PersistGroup *g = p.groups + gi, *gq = p.groups + go;
       const bool dense = __ldg(&g->flags) & GSI_FLAG_DENSE;
       pl.gi = (short)gi;
+      pl.go = (short)go;
       pl.gi0 = (short)gi0;
       pl.len = (unsigned char)len;
       pl.kind = dense ? 2 : 1;
@@ -942,15 +921,19 @@ __device__ __forceinline__ void make_plan(const PersistParams& p, unsigned char*
         const int gc = 1 << gcl;
         int a, b;
         deal((__ldg(&g->d) + 15) >> 4, ncta, lc, a, b);
-        pl.p0 = a * 16;
+        pl.pt0 = (short)a;
         pl.pg = (short)(b - a);
         pl.pchunks = (short)((b - a + gc - 1) >> gcl);
-        deal((__ldg(&g->O) + 15) >> 4, ncta, lc, a, b);
-        pl.o0 = a * 16;
+        const int ocl = kK ? gcl : 31 - __clz(kChunk / (__ldg(&gq->k) * 32));
+        deal((__ldg(&gq->O) + 15) >> 4, __ldg(&gq->o_ncta), cta - __ldg(&gq->o_cta0), a, b);
+        pl.ot0 = (short)a;
         pl.og = (short)(b - a);
-        pl.ochunks = (short)((b - a + gc - 1) >> gcl);
+        pl.ochunks = (short)((b - a + (1 << ocl) - 1) >> ocl);
         pl.n_contrib = (short)__ldg(&g->n_contrib);
-        pl.gc_log2 = (short)gcl;
+        pl.o_contrib = (short)__ldg(&gq->n_contrib);
+        pl.gc_log2 = (unsigned char)gcl;
+        pl.oc_log2 = (unsigned char)ocl;
+        pl.o_fp8 = (__ldg(&gq->flags) & GSI_FLAG_FP8_IMAGE) != 0;
       }
     }
     plan[t] = pl;
@@ -991,21 +974,26 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
   tr.start(p, smem);
 
   const Settle* settle = reinterpret_cast<const Settle*>(smem + kOffSettle);
-  // the descriptor of the group this CTA runs in phase ph (read only when there is one)
+  // the descriptors of the groups whose basis rows and whose image rows this CTA runs in phase
+  // ph (read only when there are such)
   auto desc = [&](int ph) -> const PersistGroup& {
-    return *reinterpret_cast<const PersistGroup*>(smem + kOffDesc + (ph & (kDescSlots - 1)) * 512);
+    return *reinterpret_cast<const PersistGroup*>(desc_slot(smem, ph, 0));
   };
-  // ... from the device table into its slot (threads 0 .. kDescWords - 1)
+  auto desc_o = [&](int ph) -> const PersistGroup& {
+    return *reinterpret_cast<const PersistGroup*>(desc_slot(smem, ph, kPairs ? 1 : 0));
+  };
+  // ... from the device table into their slots (one thread per word)
+  const int d_role = kPairs && tid >= kDescWords ? 1 : 0, d_word = tid - d_role * kDescWords;
   auto desc_load = [&](int ph) -> uint32_t {
-    return ph < p.n_phases && tid < kDescWords ? __ldg(reinterpret_cast<const uint32_t*>(p.groups + plan[ph].gi) + tid)
-                                               : 0u;
+    return ph < p.n_phases && d_word < kDescWords
+               ? __ldg(reinterpret_cast<const uint32_t*>(p.groups + (d_role ? plan[ph].go : plan[ph].gi)) + d_word)
+               : 0u;
   };
   auto desc_store = [&](int ph, uint32_t w) {
-    if (ph < p.n_phases && tid < kDescWords)
-      reinterpret_cast<uint32_t*>(smem + kOffDesc + (ph & (kDescSlots - 1)) * 512)[tid] = w;
+    if (ph < p.n_phases && d_word < kDescWords) reinterpret_cast<uint32_t*>(desc_slot(smem, ph, d_role))[d_word] = w;
   };
   // the operand rows / columns beyond the three terms stay zero for the whole launch
-  for (int i = tid; i < (2 * kXtBytes + 8192) / 4; i += kNC) reinterpret_cast<uint32_t*>(smem + kOffXt)[i] = 0u;
+  for (int i = tid; i < (2 * kXtBytes + 2 * 8192) / 4; i += kNC) reinterpret_cast<uint32_t*>(smem + kOffXt)[i] = 0u;
   // the descriptors of the first two phases (descriptors are staged three phases ahead; the
   // tick before the first phase stages the third)
   {
@@ -1017,11 +1005,15 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
   if (warp == kStatWarp) {   // the first phase's rows of x: nothing ran ahead of them
     stat_warp_step(smem, 0, true, slot_io, p.token, tag);
     stat_warp_step(smem, 0, false, slot_io, p.token, tag);
-    if (plan[0].kind == 1) {
-      unsigned xw[kXmaxWords];
-      xmax_issue(desc(0).xmax, plan[0].n_contrib, xw);
-      xmax_collect(smem, 0, tag, p.spin_limit, p.status, xw[0], xw[1], xw[2], xw[3], xw[4]);
-    }
+  }
+  // the statistics warp collects max |x| of the group of the CTA's basis rows, the warp before it
+  // that of the group of its image rows
+  const bool xmax_warp = warp == kStatWarp || (kPairs && warp == kStatWarp - 1);
+  const int xmax_role = kPairs && warp != kStatWarp ? 1 : 0;
+  if (xmax_warp && plan[0].kind == 1) {
+    unsigned xw[kXmaxWords];
+    xmax_issue(xmax_role ? desc_o(0).xmax : desc(0).xmax, xmax_role ? plan[0].o_contrib : plan[0].n_contrib, xw);
+    xmax_collect(smem, 0, xmax_role, tag, p.spin_limit, p.status, xw[0], xw[1], xw[2], xw[3], xw[4]);
   }
 
   unsigned mask_pp = 0;          // gates that fired in the phase before the previous one
@@ -1035,9 +1027,9 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     const Plan pf = t + 1 < p.n_phases ? plan[t + 1] : Plan{};   // the phase whose pass 1 runs in this tick
     const bool gsi = pl.kind == 1, dense = pl.kind == 2, gsi_f = pf.kind == 1;
     const PersistGroup& g = desc(t);            // read only when the tick has a group
-    const int k = gsi ? (kK ? kK : g.k) : 0;
-    const int KT = k >> 4;                      // tile columns
-    const int pg = pl.pg, og = pl.og, pchunks = pl.pchunks, ochunks = pl.ochunks, gcl = pl.gc_log2;
+    const PersistGroup& g_o = desc_o(t);        // ... and image rows of this one
+    const int k = gsi ? (kK ? kK : g.k) : 0, k_o = gsi ? (kK ? kK : g_o.k) : 0;
+    const int pg = pl.pg, og = pl.og, pchunks = pl.pchunks, ochunks = pl.ochunks;
     const int n_contrib = pl.n_contrib, lc = pl.lc;
     const int len_p = t >= 1 ? plan[t - 1].len : 0, g_p = t >= 1 ? plan[t - 1].gi0 : 0;
     const float* s_x = s_xb + ((t + 3) % 3) * kPersistMaxPRows;
@@ -1203,7 +1195,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
           }
       if (!okf && !*abort) fail(p, misc, 5);
       // fixed-point scale: |partial c_j| <= amax * rows * max|P| < 2^e
-      const unsigned amax_f = misc->amax_bits[(t + 1) & 1];
+      const unsigned amax_f = misc->amax_bits[0][(t + 1) & 1];
       const float bound = __uint_as_float(amax_f) * (float)gf.p_rows * gf.pmax;
       double scale = 0.0;
       if (amax_f < 0x7f800000u && bound > 0.f && bound < 3.0e38f)
@@ -1235,7 +1227,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     if (gsi_f && tid == kNC - 1 && pf.pg > 0) {   // ||x||^2 of phase t + 1 over this CTA's rows
       const PersistGroup& gf = desc(t + 1);
       const int kf = kK ? kK : gf.k;
-      const unsigned amax_f = misc->amax_bits[(t + 1) & 1];
+      const unsigned amax_f = misc->amax_bits[0][(t + 1) & 1];
       const double amax = (double)__uint_as_float(amax_f);
       const float bound = __uint_as_float(amax_f) * (float)gf.p_rows * gf.pmax;
       const bool fin = amax_f < 0x7f800000u && bound > 0.f && bound < 3.0e38f;
@@ -1248,16 +1240,10 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     if (warp == kStatWarp && t + 2 < n_ticks) stat_warp_step(smem, t + 2, false, slot_io, p.token, tag);
     tr.mark(3);
 
-    // the scale of the sums of phase t (sent a tick ago), and whether its token is finite
-    bool nonfinite = false;
-    double inv_scale = 0.0;
-    if (gsi) {
-      const unsigned amax_bits = misc->amax_bits[t & 1];
-      nonfinite = amax_bits >= 0x7f800000u;
-      const float bound = __uint_as_float(amax_bits) * (float)g.p_rows * g.pmax;
-      if (!nonfinite && bound > 0.f && bound < 3.0e38f)
-        inv_scale = pow2d(max((int)((__float_as_uint(bound) >> 23) & 0xFFu), 1) - 126 - 43);
-    }
+    // whether the tokens of phase t are finite
+    const bool nonfinite = gsi && misc->amax_bits[0][t & 1] >= 0x7f800000u;
+    const bool nonfinite_o = kPairs ? gsi && misc->amax_bits[1][t & 1] >= 0x7f800000u : nonfinite;
+    const bool two = kPairs && pl.go != pl.gi;   // basis rows of one group, image rows of another
 
     // ---- E. wait until every contributing CTA has been added: four warps poll a quarter of
     //      the accumulators of c each (contiguous words, all loads of a lane in flight together,
@@ -1266,20 +1252,35 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     //      threshold on lane 8 + u, and on lane 7 this phase's ||x||^2.
     if (gsi && (warp == 0 || (warp >= 2 && warp <= 4))) {
       constexpr int kWpl = kK ? (kK + 127) / 128 : 4;   // words per lane
+      constexpr int kRoles = kPairs ? 2 : 1;
       const int q4 = warp == 0 ? 0 : warp - 1;          // this warp's quarter of the words
-      unsigned long long w[kWpl];
+      const unsigned long long* src[kRoles];
+      int want[kRoles], kr[kRoles];
+      src[0] = acc;
+      want[0] = n_contrib;
+      kr[0] = k;
+      if constexpr (kPairs) {
+        src[1] = g_o.acc + (size_t)parity * (k_o + 4);
+        want[1] = pl.o_contrib;
+        kr[1] = two ? k_o : 0;
+      }
+      unsigned long long w[kRoles][kWpl];
       unsigned it = 0;
       bool done = false;
       while (!done) {
         bool all = true;
 #pragma unroll
-        for (int i = 0; i < kWpl; ++i) {
-          const int j = (q4 + 4 * i) * 32 + lane;
-          w[i] = j < k ? ld_relaxed_u64(acc + j) : ((unsigned long long)n_contrib << kCountShift);
-        }
+        for (int r = 0; r < kRoles; ++r)
 #pragma unroll
-        for (int i = 0; i < kWpl; ++i)
-          all = all && ((unsigned)((w[i] + (kOne >> 1)) >> kCountShift) == (unsigned)n_contrib);
+          for (int i = 0; i < kWpl; ++i) {
+            const int j = (q4 + 4 * i) * 32 + lane;
+            w[r][i] = j < kr[r] ? ld_relaxed_u64(src[r] + j) : ((unsigned long long)want[r] << kCountShift);
+          }
+#pragma unroll
+        for (int r = 0; r < kRoles; ++r)
+#pragma unroll
+          for (int i = 0; i < kWpl; ++i)
+            all = all && ((unsigned)((w[r][i] + (kOne >> 1)) >> kCountShift) == (unsigned)want[r]);
         done = __all_sync(0xffffffffu, all);
         if (!done && (++it > p.spin_limit || ((it & 1023u) == 0 && *abort))) {
           if (!*abort && lane == 0) fail(p, misc, 6);
@@ -1287,16 +1288,26 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
         }
       }
 #pragma unroll
-      for (int i = 0; i < kWpl; ++i) {
-        const int j = (q4 + 4 * i) * 32 + lane;
-        if (j < k) {
-          const long long val = (long long)(w[i] - ((unsigned long long)n_contrib << kCountShift));
-          unsigned short tm[3];
-          split3((float)((double)val * inv_scale), tm);
-          const int slot = term_slot(j >> 4, j & 15, 0);
-          s_cb[slot] = tm[0];
-          s_cb[slot + 16] = tm[1];   // the next term is the next column of the operand: four lanes on
-          s_cb[slot + 32] = tm[2];
+      for (int r = 0; r < kRoles; ++r) {
+        // the scale of the sums (sent a tick ago)
+        const PersistGroup& gr = r ? g_o : g;
+        const unsigned amax_bits = misc->amax_bits[r][t & 1];
+        const float bound = __uint_as_float(amax_bits) * (float)gr.p_rows * gr.pmax;
+        double inv_scale = 0.0;
+        if (amax_bits < 0x7f800000u && bound > 0.f && bound < 3.0e38f)
+          inv_scale = pow2d(max((int)((__float_as_uint(bound) >> 23) & 0xFFu), 1) - 126 - 43);
+#pragma unroll
+        for (int i = 0; i < kWpl; ++i) {
+          const int j = (q4 + 4 * i) * 32 + lane;
+          if (j < kr[r]) {
+            const long long val = (long long)(w[r][i] - ((unsigned long long)want[r] << kCountShift));
+            unsigned short tm[3];
+            split3((float)((double)val * inv_scale), tm);
+            unsigned short* cb = s_cb + r * (8192 / 2) + term_slot(j >> 4, j & 15, 0);
+            cb[0] = tm[0];
+            cb[16] = tm[1];   // the next term is the next column of the operand: four lanes on
+            cb[32] = tm[2];
+          }
         }
       }
     }
@@ -1337,7 +1348,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
       if (w_bar) __threadfence();   // acquire: the barrier below hands the visibility on to the CTA
       if (w_x2) {
         const long long val = (long long)(w - ((unsigned long long)n_contrib << kCountShift));
-        const double amax = (double)__uint_as_float(misc->amax_bits[t & 1]);
+        const double amax = (double)__uint_as_float(misc->amax_bits[0][t & 1]);
         const double x2 = nonfinite ? __longlong_as_double(0x7ff8000000000000ll)
                           : val > 0 ? (double)val * pow2d(exp_above(amax * amax * (double)g.p_rows) - 43)
                                     : 0.0;
@@ -1404,8 +1415,10 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     // (this warp then fetches the words of the other CTAs for the next phase: the loads fly
     // during its row units, the check comes after them)
     unsigned xw[kXmaxWords];
-    const bool xmax_next = warp == kStatWarp && t + 2 < n_ticks && plan[t + 2].kind == 1;
-    if (xmax_next) xmax_issue(desc(t + 2).xmax, plan[t + 2].n_contrib, xw);
+    const bool xmax_next = xmax_warp && t + 2 < n_ticks && plan[t + 2].kind == 1;
+    if (xmax_next)
+      xmax_issue(xmax_role ? desc_o(t + 2).xmax : desc(t + 2).xmax,
+                 xmax_role ? plan[t + 2].o_contrib : plan[t + 2].n_contrib, xw);
 
     // ---- G / I. the row passes on the tensor cores, one copy of the code for both: part 0 the
     //      residual rows of the basis slab (still in the ring), part 1 the image rows.  A unit
@@ -1420,9 +1433,12 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
       const int ngroups = image ? og : pg;
       const int id0 = image ? pg : 0;
       const unsigned n0 = image ? n : n_pr;
-      const int row_base = image ? pl.o0 : pl.p0, row_end = image ? g.O : g.d;
-      float* out = image ? g.y + (size_t)p.token * g.O : g.r;
-      const bool f8 = image && (g.flags & GSI_FLAG_FP8_IMAGE);
+      const int row_base = (image ? pl.ot0 : pl.pt0) * 16, row_end = image ? g_o.O : g.d;
+      float* out = image ? g_o.y + (size_t)p.token * g_o.O : g.r;
+      const bool f8 = image && pl.o_fp8;
+      const int KT = kK ? kK >> 4 : (image ? k_o : k) >> 4;   // tile columns
+      const int gcl = image ? pl.oc_log2 : pl.gc_log2;
+      const unsigned char* cb = reinterpret_cast<const unsigned char*>(s_cb) + (image && two ? 8192 : 0) + lane * 8;
       if (image) n += ochunks;
       float sr = 0.f;
       // A warp touches only the chunks its units lie in: it waits for the chunk, runs the unit
@@ -1440,7 +1456,6 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
           // (the outcome is taken for the warp as a whole: lanes must not part ways here)
           if (!__all_sync(0xffffffffu, mbar_wait(&full_b[seq % kNB], (seq / kNB) & 1u, abort))) ok = false;
           if (!ok) break;
-          const unsigned char* cb = reinterpret_cast<const unsigned char*>(s_cb) + lane * 8;
           float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
           float sc_lo = 1.f, sc_hi = 1.f;   // FP8 image: the scales of rows lg and lg + 8
           if (f8) {
@@ -1486,7 +1501,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
               const int row = R * 16 + lg + 8 * h;
               if (row_base + row < row_end) {
                 if (image) {
-                  out[row_base + row] = nonfinite ? __int_as_float(0x7fc00000) : dot;
+                  out[row_base + row] = nonfinite_o ? __int_as_float(0x7fc00000) : dot;
                 } else {
                   const float rv = s_x[row] - dot;
                   out[row_base + row] = rv;
@@ -1524,7 +1539,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
       tr.mark(image ? 8 : 5);
     }
     if (!ok && !*abort) fail(p, misc, 8);   // (the CTA leaves together, behind the next barrier)
-    if (xmax_next) xmax_collect(smem, t + 2, tag, p.spin_limit, p.status, xw[0], xw[1], xw[2], xw[3], xw[4]);
+    if (xmax_next) xmax_collect(smem, t + 2, xmax_role, tag, p.spin_limit, p.status, xw[0], xw[1], xw[2], xw[3], xw[4]);
 
     mask_pp = mask_p;
     }

@@ -844,6 +844,8 @@ def test_persistent_trace_counters_do_not_change_results():
     [(256, 64, (264,)), (16384, 512, (64,)), (1024, 128, (8, 2056)), (2048, 512, (4096,))],
     # a dense group between phases of several
     [(512, 128, (512,)), (768, 128, (256,)), "dense", (512, 128, (128,)), (512, 128, (640,))],
+    # wide bases beside wide images: most CTAs run basis rows of one group and image rows of another
+    [(4096, 256, (72,)), (320, 256, (16392,)), (512, 256, (24, 40)), (1040, 256, (272,))],
 ])
 def test_persistent_phases_of_several_groups(shapes):
     """Consecutive groups share a phase (its CTAs split between them): every group's gates and
