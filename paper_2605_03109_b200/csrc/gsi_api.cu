@@ -527,8 +527,16 @@ static bool rows_fit(const gsi_layer* h, int ctas) {
   return std::max(least_p_share(h), least_o_share(h)) <= ctas;
 }
 
-// W stream geometry of a group: whole rows per contiguous piece of at most 32 KB.
-static int w_piece_rows(int d) { return std::max(1, kPersistPieceBytes / (d * 2)); }
+// W stream geometry of a CTA's `rows` rows: whole rows per contiguous piece of at most 32 KB, fewer
+// where that leaves teams of consumer warps idle (see w_geometry in the kernel; two rows at least, the
+// step of a team).  d = 768, 62 rows: five rows on 15 teams, against 21 on three (12 GPT-2 layers with
+// 67 % gated 127 -> 117 us); cutting smaller where all teams have work costs (28 GPT-J
+// layers, all gated, 16 KB pieces: 2.23 -> 2.57 ms).
+static int w_piece_rows(int d, int rows) {
+  const int most = std::max(1, kPersistPieceBytes / (d * 2));
+  const int teams = std::max(1, kPersistConsumerWarps / ((d / 8 + 127) / 128));
+  return std::min(most, std::max(2, (rows + teams - 1) / teams));
+}
 
 // A row of W fits a piece, and the per-warp partial results of the W stream hold every row a
 // CTA owns of every map of a group.
@@ -735,7 +743,6 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
       pg.P = reinterpret_cast<const uint16_t*>(h->ws + h->lay.pk_pp);
       pg.WP = reinterpret_cast<const uint16_t*>(h->ws + h->lay.pk_wpp);
       for (int j = 0; j < gp.n_maps; ++j) pg.W[j] = gp.W[j];
-      pg.w_pr = w_piece_rows(gp.d);
       for (int j = 0; j <= gp.n_maps; ++j) pg.off[j] = gp.off[j];
       pg.n_maps = gp.n_maps;
       pg.d = gp.d;
@@ -785,8 +792,10 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
         at.p += share[i].p;
         at.o += share[i].o;
         at.w += share[i].w;
+        int w_rows = 0;
         for (int j = 0; j < h->gp.n_maps; ++j)
-          pg.w_rows[j] = (short)((h->gp.d_out[j] + pg.w_ncta - 1) / pg.w_ncta);
+          w_rows += pg.w_rows[j] = (short)((h->gp.d_out[j] + pg.w_ncta - 1) / pg.w_ncta);
+        pg.w_pr = w_piece_rows(pg.d, w_rows);
         if (!(pg.flags & GSI_FLAG_DENSE)) s->common_k = s->common_k < 0 || s->common_k == pg.k ? pg.k : 0;
       }
     }

@@ -62,7 +62,6 @@ constexpr int kChunk = 16384;               // largest chunk
 static_assert(kPersistMaxWRows <= kPersistConsumerWarps * 32, "one thread per row of a W stream");
 constexpr int kWVecMax = 5;                 // 16-byte vectors of a row one lane may own in the W stream (d <= 16384)
 constexpr unsigned kLocalSpinLimit = 1u << 20;   // waits inside the CTA (ring, producer hand-off)
-constexpr int kP1Chunks = 7;                // chunks of a basis slab that pass 1 waits for at a time
 constexpr int kCountShift = 54;
 constexpr unsigned long long kOne = 1ull << kCountShift;
 
@@ -112,7 +111,7 @@ constexpr int kOffBar = 0;          // full[kNB], empty[kNB]
 constexpr int kOffLin = 1024;       // producer: ring position (bytes placed before it) of every chunk in flight (kNB words)
 constexpr int kOffOff = 1280;       // offset of every chunk in flight within the ring (kNB words), for the consumers
 constexpr int kOffMisc = 1536;      // scalars
-constexpr int kOffTrace = 1792;     // cycle counters of the trace (16 words)
+constexpr int kOffTrace = 1792;     // cycle counters of the trace (16 words), time of the last mark
 constexpr int kOffX = 2048;         // x of this CTA's basis rows, three buffers (kPersistMaxPRows floats each)
 constexpr int kOffXt = kOffX + 3 * kPersistMaxPRows * 4;  // ... as three bf16 terms in A-operand order, two buffers
 constexpr int kXtBytes = kPersistMaxPRows / 16 * 256;     // (256 B per tile row)
@@ -253,26 +252,29 @@ __device__ __forceinline__ void fail(const PersistParams& p, Misc* misc, int sit
 // Optional cycle trace (thread 0 of every CTA; sections of the per-phase pipeline, summed
 // over phases in shared memory and added to p.trace when the CTA ends); p.trace == nullptr
 // disables it.
-struct Trace {
-  unsigned long long* acc;   // shared
-  long long t;
-  __device__ __forceinline__ void start(const PersistParams& p, unsigned char* smem) {
-    acc = (threadIdx.x == 0 && p.trace) ? reinterpret_cast<unsigned long long*>(smem + kOffTrace) : nullptr;
-    if (acc) {
-      for (int i = 0; i < 16; ++i) acc[i] = 0ull;
-      t = clock64();
+struct Trace {   // (no state in registers: the time of the last mark lies in shared memory too)
+  const PersistParams& p;
+  unsigned char* smem;
+  __device__ __forceinline__ bool on() const { return threadIdx.x == 0 && p.trace; }
+  __device__ __forceinline__ unsigned long long* acc() const {
+    return reinterpret_cast<unsigned long long*>(smem + kOffTrace);
+  }
+  __device__ __forceinline__ void start() const {
+    if (on()) {
+      for (int i = 0; i < 16; ++i) acc()[i] = 0ull;
+      acc()[16] = clock64();
     }
   }
-  __device__ __forceinline__ void mark(int section) {
-    if (acc) {
-      const long long now = clock64();
-      acc[section] += (unsigned long long)(now - t);
-      t = now;
+  __device__ __forceinline__ void mark(int section) const {
+    if (on()) {
+      const unsigned long long now = clock64();
+      acc()[section] += now - acc()[16];
+      acc()[16] = now;
     }
   }
-  __device__ __forceinline__ void flush(const PersistParams& p) {
-    if (acc)
-      for (int i = 0; i < 16; ++i) p.trace[(size_t)blockIdx.x * 16 + i] += acc[i];
+  __device__ __forceinline__ void flush() const {
+    if (on())
+      for (int i = 0; i < 16; ++i) p.trace[(size_t)blockIdx.x * 16 + i] += acc()[i];
   }
 };
 
@@ -551,87 +553,6 @@ __device__ __forceinline__ bool grid_wait(const unsigned* ctr, unsigned target, 
   return true;
 }
 
-// Chunks [n0, n0 + count) have landed (lane c waits for chunk c, all waits in flight together).
-__device__ __forceinline__ bool chunks_landed(unsigned char* smem, unsigned n0, int count,
-                                              volatile int* abort) {
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kOffBar);
-  const int lane = threadIdx.x & 31;
-  bool mine_ok = true;
-  if (lane < count) {
-    const unsigned seq = n0 + lane;
-    mine_ok = mbar_wait(&full[seq % kNB], (seq / kNB) & 1u, abort);
-  }
-  return __all_sync(0xffffffffu, mine_ok);
-}
-
-// One piece of the W stream for one warp: rows_p rows of rvec vectors; this lane owns vectors
-// lane + 32 i (i < VPL) of the warp's range (first = pointer to its first vector of row 0,
-// nvalid = how many of its VPL vectors exist); `in` holds its share of the input.  RPI rows at
-// a time (2 or 1: more rows in flight cost registers that the tick loop around the stream
-// needs); two rows share five shuffles (the first level sends half of the values to the
-// partner).  Results to part[row].
-// The piece goes back to the producer (release_n arrivals on `eb`) as soon as its last rows
-// are in registers, before the sums over the lanes: the arrival is predicated on a value that
-// every load of the warp feeds (a comparison that never fails), so it cannot be issued before
-// those loads have returned.
-template <int VPL, int RPI>
-__device__ __forceinline__ void w_piece(const uint4* first, int rvec, int rows_p, int nvalid,
-                                        const unsigned long long (&in)[kWVecMax][4], float* part,
-                                        uint64_t* eb, uint32_t release_n) {
-  const int lane = threadIdx.x & 31;
-  constexpr unsigned kNever = 0x7fc5a5a5u;   // a NaN pattern no arithmetic instruction produces
-#pragma unroll 1
-  for (int ra = 0; ra < rows_p; ra += RPI) {
-    unsigned long long a[RPI], b[RPI];   // two chains of dependent additions per row
-#pragma unroll
-    for (int q = 0; q < RPI; ++q) a[q] = b[q] = 0ull;
-    uint4 w[VPL][RPI];
-#pragma unroll
-    for (int i = 0; i < VPL; ++i)
-#pragma unroll
-      for (int q = 0; q < RPI; ++q) {
-        // rows past the piece read the last row again (dropped below); vectors past the row's
-        // end are not read at all
-        w[i][q] = make_uint4(0u, 0u, 0u, 0u);
-        if (i < nvalid) w[i][q] = first[(size_t)min(ra + q, rows_p - 1) * rvec + 32 * i];
-      }
-#pragma unroll
-    for (int i = 0; i < VPL; ++i)
-#pragma unroll
-      for (int q = 0; q < RPI; ++q) {
-        fma2(a[q], bf16x2_to_f32x2(w[i][q].x), in[i][0]);
-        fma2(b[q], bf16x2_to_f32x2(w[i][q].y), in[i][1]);
-        fma2(a[q], bf16x2_to_f32x2(w[i][q].z), in[i][2]);
-        fma2(b[q], bf16x2_to_f32x2(w[i][q].w), in[i][3]);
-      }
-    float v[RPI];
-#pragma unroll
-    for (int q = 0; q < RPI; ++q) v[q] = sum2(a[q]) + sum2(b[q]);
-    const bool last = ra + RPI >= rows_p;
-    float v0 = v[0];
-    int q_mine = 0, keep = 31;   // the row this lane ends up with, and which lanes write (lane & keep == 0)
-    if constexpr (RPI == 2) {
-      const bool up = lane & 16;
-      const float s0 = up ? v[0] : v[1];
-      const float r0v = __shfl_xor_sync(0xffffffffu, s0, 16);
-      v0 = (up ? v[1] : v[0]) + r0v;
-      q_mine = lane >> 4;
-      keep = 15;
-    }
-    // v0 now depends on every row loaded above
-    if (last) {
-      __syncwarp();
-      if (lane == 0 && __float_as_uint(v0) != kNever) mbar_arrive_n(eb, release_n);
-    }
-    if constexpr (RPI == 1) v0 += __shfl_xor_sync(0xffffffffu, v0, 16);
-    v0 += __shfl_xor_sync(0xffffffffu, v0, 8);
-    v0 += __shfl_xor_sync(0xffffffffu, v0, 4);
-    v0 += __shfl_xor_sync(0xffffffffu, v0, 2);
-    v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
-    if ((lane & keep) == 0 && ra + q_mine < rows_p) part[ra + q_mine] = v0;
-  }
-}
-
 // ---- W stream: y_rows (+)= W_rows . src (src = r of a gated group, or x for the dense
 // baseline), pieces of whole rows taken from the ring in the producer's order.  The consumer
 // warps form teams of nw warps; a team takes every T-th piece, so T pieces are worked on at
@@ -639,13 +560,14 @@ __device__ __forceinline__ void w_piece(const uint4* first, int rvec, int rows_p
 // others.  Within a team every warp owns a range of columns and keeps its share of src in
 // registers for the whole stream (four or five 16-byte vectors of W per lane and row; no
 // staging in shared memory).  The partial sums of a row meet in shared memory and are added
-// in warp order at the end (reproducible).  `n` is the consumers' chunk sequence number on
-// entry, the return value the one after the stream; a wait that gave up sets the abort flag.
-// Inlined at its two call sites (an out-of-line call makes the tick loop keep its state in
-// local memory); both sit where little of the tick's state is alive.
+// in warp order at the end (reproducible).  Inlined at its two call sites (an out-of-line call
+// makes the tick loop keep its state in local memory); both sit where little of the tick's state
+// is alive.
 // How the consumer warps share a W stream of input width d.
 struct WGeo {
   int d, pr, n_maps, rvec, vpl, nw, T, team, wi, v_lo, v_hi, nvalid;
+  int rows;   // this CTA's rows of all maps
+  bool half;  // their partial sums fit one half of the buffer: such streams alternate between the halves
   bool active;
   uint32_t release_n;
 };
@@ -656,8 +578,12 @@ __device__ __forceinline__ WGeo w_geometry(const PersistGroup* gp) {
   q.pr = gp->w_pr;
   q.n_maps = gp->n_maps;
   q.rvec = q.d >> 3;                                         // 16-byte vectors per row
-  q.vpl = q.rvec > 4 * kNC ? 5 : 4;
-  q.nw = (q.rvec + 32 * q.vpl - 1) / (32 * q.vpl);           // warps of a team
+  // warps of a team, at four vectors per lane and two rows at a time, or at five and one where pieces
+  // are single rows or that gives more teams (d = 8192: two of seven warps against one of eight; 27.7 -> 21.8 us per
+  // stream of 134 MB)
+  const int nw4 = (q.rvec + 127) / 128, nw5 = (q.rvec + 159) / 160;
+  q.vpl = q.pr == 1 || kNW / nw5 > kNW / nw4 ? 5 : 4;
+  q.nw = q.vpl == 5 ? nw5 : nw4;
   q.T = kNW / q.nw;                                          // teams
   q.team = warp / q.nw;
   q.wi = warp - q.team * q.nw;
@@ -665,6 +591,14 @@ __device__ __forceinline__ WGeo w_geometry(const PersistGroup* gp) {
   q.v_lo = min(q.rvec, q.wi * 32 * q.vpl);                   // this warp's vectors of every row
   q.v_hi = min(q.rvec, q.v_lo + 32 * q.vpl);
   q.nvalid = (q.v_hi - q.v_lo - lane + 31) >> 5;             // how many of this lane's vectors exist
+  const int cta = (int)blockIdx.x - gp->w_cta0;              // (within the group's share of the stream)
+  q.rows = 0;
+#pragma unroll 1
+  for (int j = 0; j < q.n_maps; ++j) {
+    const int rows = gp->w_rows[j];
+    q.rows += max(min(rows, gp->off[j + 1] - gp->off[j] - cta * rows), 0);
+  }
+  q.half = q.nw * q.rows <= kNW * kPersistMaxWRows / 2;
   q.release_n = q.wi == 0 ? (uint32_t)(kNW - q.nw + 1) : 1u; // a team's first warp also arrives for all other warps
   return q;
 }
@@ -686,87 +620,167 @@ __device__ __forceinline__ void w_load_in(const WGeo& q, const float* src, unsig
   }
 }
 
-__device__ __forceinline__ unsigned w_run(const PersistGroup* gp, const WGeo& q,
-                                          const unsigned long long (&in)[kWVecMax][4], float* y, bool dense,
-                                          unsigned char* smem, unsigned n, int* status, bool traced) {
+// What remains of a stream after its pieces: thread i adds row i's partial sums to y.
+struct WSum {
+  float* yp;        // y of this thread's row, or nullptr
+  float yold;       // ... so far (the image row, written by another CTA and visible by now)
+  int base, rows, nw;   // the partial sums: s_part[base + wi * rows + row]
+  bool half;
+};
+
+// The pieces of one stream for this warp's team.  RPI rows of VPL vectors per lane at a time (more
+// rows in flight cost registers that the tick loop around the stream needs).  A piece goes back to the
+// producer as soon as its last rows are in registers: the arrival is predicated on a value that the
+// warp's loads feed (a comparison that never fails), so it cannot be issued before those have
+// returned.  Single rows (the widest inputs, few teams): the sums over the lanes are taken one step
+// later, while the next row is on its way from shared memory (16384 -> 4096: 30.5 -> 22.3 us per
+// stream with that and the input share of the next stream fetched early).  Two rows share five
+// shuffles (the first level sends half of the values to the partner), and the other teams hide them.
+template <int VPL, int RPI>
+__device__ __forceinline__ unsigned w_pieces_t(const PersistGroup* gp, const WGeo& q,
+                                               const unsigned long long (&in)[kWVecMax][4], float* part,
+                                               unsigned char* smem, unsigned n, int cta, bool& ok, const Trace& tr) {
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kOffBar);
   uint64_t* empty = full + kNB;
   const unsigned* s_off = reinterpret_cast<const unsigned*>(smem + kOffOff);
   unsigned char* ring = smem + kOffRing;
-  float* s_part = reinterpret_cast<float*>(smem + kOffYacc);
-  Misc* misc = reinterpret_cast<Misc*>(smem + kOffMisc);
-  volatile int* abort = &misc->abort;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int cta = (int)blockIdx.x - gp->w_cta0;   // (within the group's share of the stream)
-  Trace tr;
-  tr.acc = (traced && tid == 0) ? reinterpret_cast<unsigned long long*>(smem + kOffTrace) : nullptr;
-  tr.t = clock64();
-  const int pr = q.pr, n_maps = q.n_maps, rvec = q.rvec, nw = q.nw, T = q.T, team = q.team, wi = q.wi;
-  const bool active = q.active;
-  bool ok = true;
-  // thread i owns row i of this CTA's rows (all maps, in order): its y so far (the image row,
-  // written by another CTA and visible by now) is fetched while the stream runs
-  float* yp = nullptr;
-  float yold = 0.f;
-  {
-    int yb = 0;
-#pragma unroll 1
-    for (int j = 0; j < n_maps; ++j) {
-      const int dout = gp->off[j + 1] - gp->off[j], rows = gp->w_rows[j];
-      const int live = max(min(rows, dout - cta * rows), 0);
-      if (tid >= yb && tid < yb + live) yp = y + gp->off[j] + cta * rows + (tid - yb);
-      yb += live;
+  volatile int* abort = &reinterpret_cast<Misc*>(smem + kOffMisc)->abort;
+  const int lane = threadIdx.x & 31;
+  constexpr unsigned kNever = 0x7fc5a5a5u;   // a NaN pattern no arithmetic instruction produces
+  float held[RPI];     // this lane's sums of the rows before, not yet summed over the lanes
+  int held_at = -1, held_rows = 0;
+  auto settle = [&]() {
+    if (held_at < 0) return;
+    float v0 = held[0];
+    int mine = 0, keep = 31;   // the row this lane ends up with, and which lanes write (lane & keep == 0)
+    if constexpr (RPI == 2) {
+      const bool up = lane & 16;
+      const float s0 = up ? held[0] : held[1];
+      v0 = (up ? held[1] : held[0]) + __shfl_xor_sync(0xffffffffu, s0, 16);
+      mine = lane >> 4;
+      keep = 15;
+    } else {
+      v0 += __shfl_xor_sync(0xffffffffu, v0, 16);
     }
-    if (yp && !dense) yold = __ldcg(yp);
-  }
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 8);
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 4);
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 2);
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
+    if ((lane & keep) == 0 && mine < held_rows) part[held_at + mine] = v0;
+  };
   int ybase = 0, pi = 0;   // rows of the maps before this one; pieces of this stream so far
-  tr.mark(10);
 #pragma unroll 1
-  for (int j = 0; j < n_maps; ++j) {
-    const int dout = gp->off[j + 1] - gp->off[j], rows = gp->w_rows[j];
-    const int live = min(rows, dout - cta * rows);
+  for (int j = 0; j < q.n_maps; ++j) {
+    const int rows = gp->w_rows[j];
+    const int live = min(rows, gp->off[j + 1] - gp->off[j] - cta * rows);
 #pragma unroll 1
-    for (int r0 = 0; r0 < live; r0 += pr, ++pi) {
-      const int rows_p = min(pr, live - r0);
+    for (int r0 = 0; r0 < live; r0 += q.pr, ++pi) {
+      const int rows_p = min(q.pr, live - r0);
       const unsigned slot = n % kNB, ph = (n / kNB) & 1u;
       ++n;
-      if (!active || pi % T != team) continue;
+      if (!q.active || pi % q.T != q.team) continue;
       if (ok && !__all_sync(0xffffffffu, mbar_wait(&full[slot], ph, abort))) ok = false;   // (for the warp as a whole)
       tr.mark(11);
-      if (ok) {
-        const uint4* piece = reinterpret_cast<const uint4*>(ring + s_off[slot]) + q.v_lo + lane;
-        float* part = s_part + wi * kPersistMaxWRows + ybase + r0;
-        uint64_t* eb = &empty[slot];
-        if (q.vpl == 5) w_piece<5, 1>(piece, rvec, rows_p, q.nvalid, in, part, eb, q.release_n);
-        else if (pr >= 2) w_piece<4, 2>(piece, rvec, rows_p, q.nvalid, in, part, eb, q.release_n);
-        else w_piece<4, 1>(piece, rvec, rows_p, q.nvalid, in, part, eb, q.release_n);
+      if (!ok) continue;
+      const uint4* first = reinterpret_cast<const uint4*>(ring + s_off[slot]) + q.v_lo + lane;
+#pragma unroll 1
+      for (int ra = 0; ra < rows_p; ra += RPI) {
+        unsigned long long a[RPI], b[RPI];   // two chains of dependent additions per row
+#pragma unroll
+        for (int r = 0; r < RPI; ++r) a[r] = b[r] = 0ull;
+        uint4 w[VPL][RPI];
+#pragma unroll
+        for (int i = 0; i < VPL; ++i)
+#pragma unroll
+          for (int r = 0; r < RPI; ++r) {
+            // rows past the piece read the last row again (dropped below); vectors past the row's
+            // end are not read at all
+            w[i][r] = make_uint4(0u, 0u, 0u, 0u);
+            if (i < q.nvalid) w[i][r] = first[(size_t)min(ra + r, rows_p - 1) * q.rvec + 32 * i];
+          }
+        if (RPI == 1) settle();
+#pragma unroll
+        for (int i = 0; i < VPL; ++i)
+#pragma unroll
+          for (int r = 0; r < RPI; ++r) {
+            fma2(a[r], bf16x2_to_f32x2(w[i][r].x), in[i][0]);
+            fma2(b[r], bf16x2_to_f32x2(w[i][r].y), in[i][1]);
+            fma2(a[r], bf16x2_to_f32x2(w[i][r].z), in[i][2]);
+            fma2(b[r], bf16x2_to_f32x2(w[i][r].w), in[i][3]);
+          }
+        float all = 0.f;
+#pragma unroll
+        for (int r = 0; r < RPI; ++r) {
+          held[r] = sum2(a[r]) + sum2(b[r]);
+          all += held[r];
+        }
+        held_at = ybase + r0 + ra;
+        held_rows = rows_p - ra;
+        if (ra + RPI >= rows_p) {   // `all` depends on every row loaded above
+          __syncwarp();
+          if (lane == 0 && __float_as_uint(all) != kNever) mbar_arrive_n(&empty[slot], q.release_n);
+        }
+        if (RPI > 1) settle();
       }
       tr.mark(12);
     }
     ybase += max(live, 0);
   }
-  if (!ok && !*abort) fail_at(status, misc, 3);
-  csync();
-  // rows back to y: the warps' partial sums in warp order, onto the value fetched at the start
-  if (ok && yp) {
-    float acc = 0.f;
-#pragma unroll 1
-    for (int q = 0; q < nw; ++q) acc += s_part[q * kPersistMaxWRows + tid];
-    *yp = yold + acc;
-  }
-  csync();   // the partial sums may be overwritten by the next stream
-  tr.mark(13);
+  if (RPI == 1) settle();
   return n;
 }
 
+// Runs the pieces of one stream: `n` is the consumers' chunk sequence number on entry, the return
+// value the one after the stream; a wait that gave up sets the abort flag.  `flip` alternates the
+// halves of the buffer of partial sums from stream to stream.
+__device__ __forceinline__ unsigned w_pieces(const PersistGroup* gp, const WGeo& q,
+                                             const unsigned long long (&in)[kWVecMax][4], float* y, bool dense,
+                                             unsigned char* smem, unsigned n, const Trace& tr, unsigned& flip,
+                                             WSum& ws) {
+  const int tid = threadIdx.x;
+  const int cta = (int)blockIdx.x - gp->w_cta0;   // (within the group's share of the stream)
+  // thread i owns row i of this CTA's rows (all maps, in order): its y so far is fetched while the
+  // stream runs
+  ws.yp = nullptr;
+  ws.yold = 0.f;
+  ws.nw = q.nw;
+  int yb = 0;
+#pragma unroll 1
+  for (int j = 0; j < q.n_maps; ++j) {
+    const int dout = gp->off[j + 1] - gp->off[j], rows = gp->w_rows[j];
+    const int live = max(min(rows, dout - cta * rows), 0);
+    if (tid >= yb && tid < yb + live) ws.yp = y + gp->off[j] + cta * rows + (tid - yb);
+    yb += live;
+  }
+  if (ws.yp && !dense) ws.yold = __ldcg(ws.yp);
+  ws.rows = q.rows;
+  ws.half = q.half;
+  ws.base = q.half ? (int)(flip & 1u) * (kNW * kPersistMaxWRows / 2) : 0;
+  ++flip;
+  tr.mark(10);
+  float* part = reinterpret_cast<float*>(smem + kOffYacc) + ws.base + q.wi * q.rows;
+  bool ok = true;
+  if (q.vpl == 5) n = w_pieces_t<5, 1>(gp, q, in, part, smem, n, cta, ok, tr);
+  else n = w_pieces_t<4, 2>(gp, q, in, part, smem, n, cta, ok, tr);
+  Misc* misc = reinterpret_cast<Misc*>(smem + kOffMisc);
+  if (!ok && !*(volatile int*)&misc->abort) fail(tr.p, misc, 3);
+  return n;
+}
 
-// Geometry, input share and stream in one go.
-__device__ __forceinline__ unsigned w_stream(const PersistGroup* gp, const float* src, float* y, bool dense,
-                                             unsigned char* smem, unsigned n, int* status, bool traced) {
-  const WGeo q = w_geometry(gp);
-  unsigned long long in[kWVecMax][4];
-  w_load_in(q, src, in);
-  return w_run(gp, q, in, y, dense, smem, n, status, traced);
+// Rows back to y: the warps' partial sums in warp order, onto the value fetched at the start.  The
+// next stream writes its partial sums to the other half of the buffer, and the one after it lies
+// behind that stream's barrier; where one of the two does not fit a half (`apart` = false), a second barrier
+// keeps them apart.
+__device__ __forceinline__ void w_finish(const WSum& ws, unsigned char* smem, bool apart) {
+  const float* s_part = reinterpret_cast<const float*>(smem + kOffYacc) + ws.base + threadIdx.x;
+  csync();
+  if (ws.yp) {
+    float acc = 0.f;
+#pragma unroll 1
+    for (int q = 0; q < ws.nw; ++q) acc += s_part[q * ws.rows];
+    *ws.yp = ws.yold + acc;
+  }
+  if (!apart) csync();
 }
 
 // The statistics warp (the warp before it for the group of the CTA's image rows): the group's
@@ -965,13 +979,11 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
   constexpr int kP1 = kStatWarp - kP1First;   // ... while warps 5..13 run pass 1 of the phase after it
 
   unsigned n = 0;   // chunk sequence number: advances exactly as in producer()
-  const int step = p.use_counter ? *p.step : 0;
-  const int slot_io = step % p.n_steps;
-  const int epoch = *p.epoch;
-  const unsigned parity = (unsigned)epoch & 1u, tag = ((unsigned)epoch + 1u) & 1u;
+  const int slot_io = (p.use_counter ? *p.step : 0) % p.n_steps;
+  const unsigned parity = (unsigned)*p.epoch & 1u, tag = parity ^ 1u;
   const int n_ticks = p.n_phases + 2;
-  Trace tr;
-  tr.start(p, smem);
+  const Trace tr{p, smem};
+  tr.start();
 
   const Settle* settle = reinterpret_cast<const Settle*>(smem + kOffSettle);
   // the descriptors of the groups whose basis rows and whose image rows this CTA runs in phase
@@ -1038,67 +1050,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     // the descriptor of the phase three ahead: requested now, stored before the barrier that ends the exchange
     const uint32_t desc_word = desc_load(t + 3);
 
-    // ---- a run of dense groups (the dense baseline): nothing of the exchange machinery has
-    //      work in these ticks.  Per tick: post the (empty) decision on the previous phase for
-    //      the producer, stream, close with the grid barrier that keeps a dense stack in model
-    //      order.  The inputs of a stack are staged before the step, so the next group's input
-    //      is asked into the L2 while this group streams, and this CTA's share of it into
-    //      registers while the barrier is waited for.
-    auto not_gated = [&](int ph) { return ph >= p.n_phases || plan[ph].kind != 1; };
-    const bool plain = dense && !mask_pp && (t == 0 || plan[t - 1].kind == 2) && not_gated(t + 1) && not_gated(t + 2);
     const unsigned mask_stream = mask_pp;   // the gated residuals this tick streams: phase t - 2
-    if (plain) {
-      auto x_of = [&](const PersistGroup& gg) {
-        return gg.x + (long long)slot_io * gg.x_step_stride + (size_t)p.token * gg.d;
-      };
-      unsigned long long in[kWVecMax][4];
-      WGeo q = w_geometry(&g);
-      w_load_in(q, x_of(g), in);
-      uint32_t dword = desc_word;   // descriptors of the phase after the next, requested at the top of the tick
-      int tt = t;
-      for (;;) {
-        const Plan plc = plan[tt];
-        const PersistGroup& gc = desc(tt);
-        if (tt != t) dword = desc_load(tt + 3);
-        if (plc.zeroer && tid < 2) gc.bar[2 * tid + (parity ^ 1u)] = 0u;
-        if (tid == 0 && tt >= 1) misc->decision[(tt - 1) & 3] = (unsigned)tt << 8;
-        const bool more = tt + 1 < n_ticks && plan[tt + 1].kind == 2 && not_gated(tt + 2) && not_gated(tt + 3);
-        if (warp == kStatWarp && tt + 1 < n_ticks) {
-          const Plan& pn = plan[tt + 1];
-          if (pn.kind == 2) {
-            const char* xn = reinterpret_cast<const char*>(x_of(desc(tt + 1)));
-            for (int i = lane * 128; i < desc(tt + 1).d * 4; i += 32 * 128)
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(xn + i));
-          }
-        }
-        tr.mark(0);
-        n = w_run(&gc, q, in, gc.y + (size_t)p.token * gc.O, true, smem, n, p.status, p.trace != nullptr);
-        if (tr.acc) tr.t = clock64();
-        desc_store(tt + 3, dword);   // (its latency ran under the stream)
-        if (tid == 0) red_relaxed_u32(gc.bar + parity, 1u);
-        if (more) {   // in flight while the barrier is waited for
-          const PersistGroup& gn = desc(tt + 1);
-          q = w_geometry(&gn);
-          w_load_in(q, x_of(gn), in);
-        }
-        if (tid == 0) {
-          grid_wait(gc.bar + parity, (unsigned)G, p, misc);
-          if (cta == 0) p.gate_log[((size_t)slot_io * p.log_step_stride + plc.gi) * p.n_tokens + p.token] = 1;
-          misc->stop[1] = *abort;
-        }
-        csync();
-        tr.mark(6);
-        if (misc->stop[1]) {   // decided before the barrier: the same for every warp
-      async_drain();
-      return;
-    }
-        if (!more) break;
-        ++tt;
-      }
-      t = tt;   // the loop's increment moves on to the tick after the run
-      mask_pp = 0;
-      continue;
-    } else {
     // ---- A. the bulk reduction of the previous tick has read its source
     if (lane == 0 || tid == kNC - 1) bulk_reduce_wait_read();   // the lanes that issue bulk reductions
     if (t >= 0 && pl.zeroer) {  // this CTA clears the group's counters for the next launch
@@ -1153,34 +1105,34 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
 #pragma unroll
           for (int v = 0; v < 4; ++v) cacc[s3][m][v] = 0.f;
       const unsigned short* xt = s_xt + ((t + 1) & 1) * (kXtBytes / 2);
-      // (a slab of few chunks is waited for as a whole; a larger one streams through the ring)
+      // chunk by chunk as they land; a chunk goes back as soon as its tiles are in registers (the last
+      // mma has issued).  (Seven chunks at a time, rows one by one: 1.5 us for 13 units of k = 256, and
+      // a slab larger than the ring waited for itself; 26 OPT layers at k = 512, nothing gated, 518 -> 494 us.)
+      const uint32_t share = unit_share(wp1, nf);
 #pragma unroll 1
-      for (int cb = 0; p1_active && okf && cb < pf.pchunks; cb += kP1Chunks) {
-        const int cn = min(kP1Chunks, pf.pchunks - cb);
-        okf = chunks_landed(smem, n_pf + cb, cn, abort);
-        if (!okf) break;
-        const int R1 = min((int)pf.pg, (cb + cn) << gclf);
-#pragma unroll 1
-        for (int R = cb << gclf; R < R1; ++R) {
-          const uint2 ax = *reinterpret_cast<const uint2*>(xt + (R * 32 + lane) * 4);
+      for (int c = 0; p1_active && c < pf.pchunks; ++c) {
+        const unsigned seq = n_pf + c, slot = seq % kNB;
+        if (!__all_sync(0xffffffffu, mbar_wait(&full_b[slot], (seq / kNB) & 1u, abort))) {   // (for the warp as a whole)
+          okf = false;
+          break;
+        }
+        const int R0 = c << gclf, R1 = min((int)pf.pg, R0 + (1 << gclf));
+        const unsigned char* trow = ring + s_off[slot] + wp1 * tpw * 512 + lane * 16;
+        const unsigned short* xr = xt + (R0 * 32 + lane) * 4;
+#pragma unroll (kK && kK < 512 ? 2 : 1)
+        for (int R = R0; R < R1; ++R, trow += KTf * 512, xr += 128) {
+          const uint2 ax = *reinterpret_cast<const uint2*>(xr);
           const uint4 a = make_uint4(ax.x, 0u, ax.y, 0u);
-          const int ci = R >> gclf, rr = R - (ci << gclf);
-          const unsigned char* trow = ring + s_off[(n_pf + ci) % kNB] + (size_t)rr * KTf * 512 + lane * 16;
 #pragma unroll
           for (int s3 = 0; s3 < kTpwMax; ++s3) {
-            const int kt = wp1 * tpw + s3;
-            if (s3 < tpw && kt < KTf) {
-              const uint4 w = ldsm_tile_trans(trow + kt * 512);
+            if (s3 < tpw && wp1 * tpw + s3 < KTf) {
+              const uint4 w = ldsm_tile_trans(trow + s3 * 512);
               mma_bf16(cacc[s3][0], a, w.x, w.y);
               mma_bf16(cacc[s3][1], a, w.z, w.w);
             }
           }
         }
-        if (lane == 0) {   // (every tile of the chunks is in registers: the last mma has issued)
-          const uint32_t share = unit_share(wp1, nf);
-#pragma unroll 1
-          for (int c = cb; c < cb + cn; ++c) mbar_arrive_n(&empty[(n_pf + c) % kNB], share);
-        }
+        if (lane == 0) mbar_arrive_n(&empty[slot], share);
       }
       // the three terms of x sit in rows 0..2 = lanes 0-3, 4-7, 8-11: fold them onto lanes 0-3
 #pragma unroll
@@ -1542,49 +1494,87 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     if (xmax_next) xmax_collect(smem, t + 2, xmax_role, tag, p.spin_limit, p.status, xw[0], xw[1], xw[2], xw[3], xw[4]);
 
     mask_pp = mask_p;
-    }
 
     // ---- H. the W streams of the tick, one call site, after the row passes (little of the
     //      tick's state is alive here): the gated residuals of the phase before the previous
-    //      one, then this phase's own stream if it is a dense group (followed by a grid barrier
-    //      that keeps a dense stack in model order).
+    //      one, then this phase's own stream if it is a dense group, followed by a grid barrier
+    //      that keeps a dense stack in model order.  In a run of dense groups (the dense baseline)
+    //      nothing of the exchange machinery has work: the loop goes on to the next tick's stream by
+    //      itself.  While the sums of one stream meet, the next one's input share is on its way (the
+    //      inputs of a stack are staged before the step; r of a gated group is visible: warp 1 waited
+    //      for every CTA's arrival during this tick's exchange).
     if (mask_stream || dense) {
       const int g_pp = plan[t - 2 >= 0 ? t - 2 : 0].gi0;
-      unsigned left = mask_stream;
+      unsigned left = mask_stream, flip = 0;
+      bool own = false;   // the stream is the dense group of this tick
+      // the next stream that this CTA has rows of
+      auto next_stream = [&]() -> const PersistGroup* {
+        while (left) {
+          const PersistGroup* g_w = p.groups + g_pp + __ffs(left) - 1;
+          left &= left - 1;
+          if (cta >= g_w->w_cta0 && cta < g_w->w_cta0 + g_w->w_ncta) return g_w;
+        }
+        if (!dense) return nullptr;
+        own = true;
+        return p.groups + plan[t].gi;
+      };
+      auto src_of = [&](const PersistGroup* g_w) -> const float* {
+        return own ? g_w->x + (long long)slot_io * g_w->x_step_stride + (size_t)p.token * g_w->d : g_w->r;
+      };
+      auto not_gated = [&](int ph) { return ph >= p.n_phases || plan[ph].kind != 1; };
+      const PersistGroup* gw = next_stream();
+      WGeo q{};
+      unsigned long long in[kWVecMax][4];
+      if (gw) {
+        q = w_geometry(gw);
+        w_load_in(q, src_of(gw), in);
+      }
+      tr.mark(9);
 #pragma unroll 1
-      while (left || dense) {
-        const bool own = !left;   // the dense group of this tick
-        const PersistGroup* gw = own ? &desc(t) : p.groups + g_pp + __ffs(left) - 1;
-        left &= left - 1;
-        if (!own && (cta < gw->w_cta0 || cta >= gw->w_cta0 + gw->w_ncta)) continue;
-        // (a gated group's r and image rows are visible: warp 1 waited for every CTA's arrival
-        // during this tick's exchange)
-        const float* src = !own ? gw->r
-                                : gw->x + (long long)slot_io * gw->x_step_stride + (size_t)p.token * gw->d;
-        tr.mark(9);
-        n = w_stream(gw, src, gw->y + (size_t)p.token * gw->O, own, smem, n, p.status, p.trace != nullptr);
-        if (tr.acc) tr.t = clock64();
-        if (own) {
-          if (tid == 0) {
-            red_relaxed_u32(gw->bar + parity, 1u);
-            grid_wait(gw->bar + parity, (unsigned)G, p, misc);
-            if (cta == 0)
-              p.gate_log[((size_t)slot_io * p.log_step_stride + plan[t].gi) * p.n_tokens + p.token] = 1;
-          }
-          csync();
-          break;
+      while (gw) {
+        WSum ws;
+        n = w_pieces(gw, q, in, gw->y + (size_t)p.token * gw->O, own, smem, n, tr, flip, ws);
+        unsigned* bar = gw->bar + parity;
+        const bool close = own;   // a grid barrier ends this stream
+        if (!own) gw = next_stream();
+        else gw = !mask_pp && plan[t + 1].kind == 2 && not_gated(t + 2) && not_gated(t + 3) ? p.groups + plan[t + 1].gi : nullptr;
+        if (gw) {
+          q = w_geometry(gw);
+          w_load_in(q, src_of(gw), in);
+        }
+        w_finish(ws, smem, close || !gw || (ws.half && q.half));
+        tr.mark(13);
+        if (!close) continue;
+        if (tid == 0) {
+          red_relaxed_u32(bar, 1u);
+          grid_wait(bar, (unsigned)G, p, misc);
+          if (cta == 0)
+            p.gate_log[((size_t)slot_io * p.log_step_stride + plan[t].gi) * p.n_tokens + p.token] = 1;
+          misc->stop[1] = *abort;
+        }
+        csync();
+        tr.mark(6);
+        if (misc->stop[1]) {   // decided before the barrier: the same for every warp
+          async_drain();
+          return;
+        }
+        if (gw) {   // on to the next tick: its (empty) decision for the producer, its counters
+          ++t;
+          desc_store(t + 3, desc_load(t + 3));
+          if (tid == 0) misc->decision[(t - 1) & 3] = (unsigned)t << 8;
+          if (plan[t].zeroer && tid < 2) gw->bar[2 * tid + (parity ^ 1u)] = 0u;
         }
       }
       tr.mark(6);
     }
   }
   async_drain();
-  tr.flush(p);
+  tr.flush();
   // Every CTA read the counters at its start and has since taken part in the
   // last group's exchange, so they may advance now.
   if (cta == 0 && tid == 0 && ok && !*abort) {
-    if (p.last) *p.epoch = epoch + 1;
-    if (p.use_counter && p.advance) *p.step = step + 1;
+    if (p.last) *p.epoch += 1;
+    if (p.use_counter && p.advance) *p.step += 1;
   }
 }
 

@@ -846,6 +846,8 @@ def test_persistent_trace_counters_do_not_change_results():
     [(512, 128, (512,)), (768, 128, (256,)), "dense", (512, 128, (128,)), (512, 128, (640,))],
     # wide bases beside wide images: most CTAs run basis rows of one group and image rows of another
     [(4096, 256, (72,)), (320, 256, (16392,)), (512, 256, (24, 40)), (1040, 256, (272,))],
+    # W streams by teams of every width: single rows of five vectors a lane, pairs of rows of four, few rows
+    [(8192, 128, (304, 40)), (6144, 64, (520,)), (9216, 64, (152,)), (320, 64, (3000, 8)), (4096, 128, (1480,))],
 ])
 def test_persistent_phases_of_several_groups(shapes):
     """Consecutive groups share a phase (its CTAs split between them): every group's gates and
