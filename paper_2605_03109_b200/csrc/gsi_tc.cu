@@ -275,19 +275,28 @@ cudaError_t launch_dense_gemm_tc(const GroupParams& g, const TmaMaps& tm, const 
   return cudaGetLastError();
 }
 
-// Deep narrow maps add their splits in distributed shared memory: 4096 x 16384 at 8 tokens 54 -> 50 us
-// a call, at 64 tokens 65.4 -> 64.5.  Wide maps have few splits, whose partial sums are cheap beside W
-// (12288 and 16384 rows, 64 tokens: a step 1.00 -> 1.27 ms as clusters); at small depths the two
-// cluster barriers cost what the second kernel does.
-static bool tc_cluster(int O, int d) { return d >= 4096 && tc_splits(O, d) >= 5; }
+// The splits of a tile are a cluster that adds them in distributed shared memory (64 tokens, all gated:
+// 8192 x 4096 37.9 -> 34.8 us a call, 8192 x 16384 88.0 -> 83.5; 12 GPT-2 layers at 8 tokens, a quarter
+// gated 552 -> 422, at 64 tokens 710 -> 563).  Up to 2^20 entries of W the second kernel costs no more
+// than the two cluster barriers (768 x 768, 64 tokens: 27.1 / 27.5 us).
+static bool tc_cluster(int O, int d) { return (double)O * d > 1048576.0 && tc_splits(O, d) > 1; }
 int tc_launches(int O, int d) { return tc_splits(O, d) > 1 && !tc_cluster(O, d) ? 2 : 1; }
 
 int tc_splits(int O, int d) {
   const int tiles = O / kTM, nkb = d / kTK;
-  if (tiles >= 148) return 1;   // a tile per CTA already fills the SMs: long pipelines, no partial sums to add
-  int s = (2 * 148 + tiles - 1) / tiles;
-  if (s > 8) s = 8;
+  // A tile per CTA (nearly) fills the SMs: long pipelines, no partial sums to add.  (4096 deep, 64
+  // tokens, all gated: 140 tiles 55.0 us a call without a split, 56.8 with two; 112 tiles 51.0 against
+  // 49.2 with few gated.  16384 deep, where the idle SMs cost more than the sums: 128 tiles 136.5 / 126.8.)
+  if (tiles >= 148 || (tiles >= 128 && d <= 4096)) return 1;
+  // No more clusters than are resident at a time (a second wave of a few costs more than it balances;
+  // as the occupancy calculator gives them for clusters of 1, 2, ... blocks at two blocks per SM: they
+  // do not straddle groups of SMs).  64 tokens, all gated: 12288 x 4096 (96 tiles) 60.8 us as three
+  // splits, 48.2 as two; 6144 x 4096 (48 tiles) 42.7 as six, 33.7 as four; 10240 x 4096 (80 tiles)
+  // 41.3 as three, 44.7 as two.
+  constexpr int kResident[9] = {0, 296, 148, 93, 71, 56, 45, 37, 33};
+  int s = 8;
   if (s > nkb / 4) s = nkb / 4;
+  while (s > 1 && tiles > kResident[s]) --s;
   if (s < 1) s = 1;
   return s;
 }

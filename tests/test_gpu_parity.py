@@ -881,6 +881,32 @@ def test_persistent_phases_of_several_groups(shapes):
         assert eps == 0.0 or gate[:, i].tolist() == [int(v) for v in live]
 
 
+@pytest.mark.parametrize("d,k,d_out,n", [
+    (512, 128, (16384,), 64),          # a block per tile
+    (768, 128, (10240,), 33),          # three splits, clusters of three
+    (1024, 128, (2048, 128), 17),      # four, two maps
+    (2048, 256, (5120,), 64),          # six
+    (4096, 128, (1024, 384), 2),       # eight; W requested once the gate is known
+    (4096, 128, (128,), 16),           # splits of a small map: partial sums in memory
+])
+def test_batched_residual_in_splits_and_clusters(d, k, d_out, n):
+    """Every form of the batched contraction, in steps in which none, some and all tokens are gated."""
+    g = G()
+    x, P, Ws = make_small(d, k, d_out, n, seed=9100 + d + k, noise=0.001)
+    out, _, _ = make_small(d, k, d_out, n, seed=9100 + d + k, noise=0.001, outlier_every=1)
+    live = [torch.zeros(n, dtype=torch.bool), torch.arange(n) % 3 == 1, torch.ones(n, dtype=torch.bool)]
+    xs = torch.stack([torch.where(m[:, None], out, x) for m in live]).contiguous()
+    stack = g.Stack([g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n)], mode=1)
+    stack.bind([xs.cuda()], n_steps=len(live))
+    for s, m in enumerate(live):
+        stack.step()
+        torch.cuda.synchronize()
+        assert stack.status() == 0
+        gate = stack.gate_log[s, 0].cpu().numpy()
+        assert gate.tolist() == m.int().tolist()
+        compare_group(xs[s], P, Ws, 0.05, stack.ys[0].cpu().reshape(n, -1).numpy(), gate)
+
+
 def test_persistent_nonfinite_token():
     g = G()
     x, P, Ws = make_small(256, 64, (64,), 3, seed=41)
