@@ -1500,9 +1500,9 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
     //      one, then this phase's own stream if it is a dense group, followed by a grid barrier
     //      that keeps a dense stack in model order.  In a run of dense groups (the dense baseline)
     //      nothing of the exchange machinery has work: the loop goes on to the next tick's stream by
-    //      itself.  While the sums of one stream meet, the next one's input share is on its way (the
-    //      inputs of a stack are staged before the step; r of a gated group is visible: warp 1 waited
-    //      for every CTA's arrival during this tick's exchange).
+    //      itself, the next group's input share on its way while the barrier is waited for (the inputs of a
+    //      stack are staged before the step; r of a gated group is visible: warp 1 waited for every
+    //      CTA's arrival during this tick's exchange).
     if (mask_stream || dense) {
       const int g_pp = plan[t - 2 >= 0 ? t - 2 : 0].gi0;
       unsigned left = mask_stream, flip = 0;
@@ -1516,7 +1516,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
         }
         if (!dense) return nullptr;
         own = true;
-        return p.groups + plan[t].gi;
+        return &desc(t);
       };
       auto src_of = [&](const PersistGroup* g_w) -> const float* {
         return own ? g_w->x + (long long)slot_io * g_w->x_step_stride + (size_t)p.token * g_w->d : g_w->r;
@@ -1533,20 +1533,25 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
 #pragma unroll 1
       while (gw) {
         WSum ws;
+        if (own && warp == kStatWarp && plan[t + 1].kind == 2) {   // the next dense group's input, into the L2
+          const PersistGroup& g_n = desc(t + 1);
+          const char* x_n = reinterpret_cast<const char*>(src_of(&g_n));
+          for (int i = lane * 128; i < g_n.d * 4; i += 32 * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(x_n + i));
+        }
         n = w_pieces(gw, q, in, gw->y + (size_t)p.token * gw->O, own, smem, n, tr, flip, ws);
         unsigned* bar = gw->bar + parity;
         const bool close = own;   // a grid barrier ends this stream
         if (!own) gw = next_stream();
-        else gw = !mask_pp && plan[t + 1].kind == 2 && not_gated(t + 2) && not_gated(t + 3) ? p.groups + plan[t + 1].gi : nullptr;
-        if (gw) {
-          q = w_geometry(gw);
-          w_load_in(q, src_of(gw), in);
-        }
+        else gw = !mask_pp && plan[t + 1].kind == 2 && not_gated(t + 2) && not_gated(t + 3) ? &desc(t + 1) : nullptr;
+        if (gw) q = w_geometry(gw);
         w_finish(ws, smem, close || !gw || (ws.half && q.half));
         tr.mark(13);
+        if (close && tid == 0) red_relaxed_u32(bar, 1u);
+        if (gw) w_load_in(q, src_of(gw), in);
         if (!close) continue;
+        const uint32_t dword = gw ? desc_load(t + 4) : 0u;
         if (tid == 0) {
-          red_relaxed_u32(bar, 1u);
           grid_wait(bar, (unsigned)G, p, misc);
           if (cta == 0)
             p.gate_log[((size_t)slot_io * p.log_step_stride + plan[t].gi) * p.n_tokens + p.token] = 1;
@@ -1560,7 +1565,7 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
         }
         if (gw) {   // on to the next tick: its (empty) decision for the producer, its counters
           ++t;
-          desc_store(t + 3, desc_load(t + 3));
+          desc_store(t + 3, dword);
           if (tid == 0) misc->decision[(t - 1) & 3] = (unsigned)t << 8;
           if (plan[t].zeroer && tid < 2) gw->bar[2 * tid + (parity ^ 1u)] = 0u;
         }
