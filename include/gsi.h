@@ -301,16 +301,13 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io_host_array,
 /*
  * Declares that groups first_group and first_group + 1 do not read each other's
  * outputs (two branches of one block: in GPT-J the attention output projection
- * and the MLP down projection), so the persistent kernel may run their
- * projections, gates and images at the same time on two parts of the grid
- * (Algorithm 1 itself is unchanged; a gated residual still streams W with the
- * whole grid).  Outside persistent mode (per-stage and batched kernels) the
- * second group of a pair is enqueued on a stream of the stack's own, forked
+ * and the MLP down projection).  In the per-stage and batched kernels the
+ * second group of a pair is then enqueued on a stream of the stack's own, forked
  * from and joined to the caller's stream by events, so the two chains of
  * launches run side by side (and a stream capture records a fork and a join).
- * Off by default; a group belongs to at most one pair; in persistent mode a
- * pair whose rows do not fit its share of the grid runs one group after the
- * other.  Takes effect at the next gsi_stack_bind.
+ * Off by default; a group belongs to at most one pair.  The persistent kernel
+ * needs no declaration: a step's inputs are given, so it puts consecutive groups
+ * into one phase itself.  Takes effect at the next gsi_stack_bind.
  */
 gsi_status_t gsi_stack_set_concurrent(gsi_stack_t s, int first_group, int enable);
 
