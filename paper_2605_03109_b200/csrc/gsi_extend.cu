@@ -31,6 +31,7 @@ namespace {
 using namespace exchange;
 
 constexpr int kT = 512, kW = kT / 32;
+constexpr int kHoldOff = 400;  // cycles between a CTA's norm word and its first look at the others'
 constexpr int kStage = 4096;   // floats of x, r1 or v in shared memory at a time
 
 __device__ __forceinline__ uint16_t to_bf16_bits(float v) {
@@ -86,6 +87,8 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
 #pragma unroll 1
   for (int pass = 1; pass <= 2; ++pass) {
     const unsigned tag = call + (unsigned)pass;
+    // (the first CTAs are done with pass 1, and at the words of pass 2, while a late one may still read)
+    unsigned long long* const r2_words = words.ext_r2 + (pass - 1) * kFusedMaxGrid;
     bool ok = true;
     // partial c of a slab of rows x 32 columns
     if (cta < n_slabs * n_cb) {
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
 #pragma unroll
         for (int w = 0; w < kW; ++w) s += s_part[w * kCols + tid];
         if (cb * kCols + tid < k) put(words.c + (size_t)slab * k + cb * kCols + tid, s, tag);
-      } else if (tid == kCols && cb == 0) {
+      } else if (pass == 1 && tid == kCols && cb == 0) {   // (pass 2 needs no ||x||^2)
         float s = 0.f;
 #pragma unroll
         for (int w = 0; w < kW; ++w) s += s_c[w];
@@ -184,11 +187,14 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       float s = 0.f;
 #pragma unroll
       for (int w = 0; w < kW; ++w) s += s_part[w];
-      put(words.ext_r2 + cta, s, tag);
+      put(r2_words + cta, s, tag);
     }
-    if (warp < 2) {
+    if (warp < 3 - pass) {
+      // (First polls that arrive ahead of the words hold them up: all CTAs read the same few lines.  Asking
+      // at once, this exchange took 1.7 or 2.7 to 4 us, by where the words lie in memory.)
+      for (const long long t0 = clock64(); clock64() - t0 < kHoldOff;) {}
       double s = 0.0;
-      ok = warp ? warp_gather_sum(words.ext_x2, 1, n_slabs, tag, s) : warp_gather_sum(words.ext_r2, 1, G, tag, s);
+      ok = warp ? warp_gather_sum(words.ext_x2, 1, n_slabs, tag, s) : warp_gather_sum(r2_words, 1, G, tag, s);
       if (lane == 0) s_norm[warp] = s;
     }
     if (give_up(ok)) return;

@@ -1279,6 +1279,28 @@ def test_extend_basis_edges_and_copies(d, k_act, k_cap, d_out, fp8):
         assert np.all((cg == want8["codes"]) | ((cg | want8["codes"]) == 0x80))
 
 
+def test_extend_basis_passes_have_norm_words_of_their_own():
+    """A CTA may be at pass 2 while a late one still reads the norm words of pass 1, so pass 2 writes
+    none of those.  Once a column is appended the words show it (their upper half is the pass's
+    tag): of pass 1 the ||x||^2 of every slab and the ||r||^2 of every CTA are still there."""
+    g = G()
+    d, k_act, k_cap = 4096, 30, 200
+    q, P, Ws = _extend_case(d, k_act, k_cap, (264,), 765, "f32")
+    lay = g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=1)
+    x = torch.randn(d, generator=torch.Generator().manual_seed(766))
+
+    def words(tag):
+        return int((lay.workspace.view(torch.int64) >> 32 == tag).sum())
+    before = words(1), words(2)
+    appended, _ = lay.extend_basis(x.cuda(), 0.05, torch.tensor([k_act], dtype=torch.int32, device="cuda"))
+    torch.cuda.synchronize()
+    assert lay.status() == 0 and appended.item() == 1
+    ctas = min(torch.cuda.get_device_properties(0).multi_processor_count, 160)
+    slabs = ctas // ((k_cap + 31) // 32)
+    assert words(1) - before[0] == slabs + ctas
+    assert words(2) - before[1] == slabs * k_cap + ctas
+
+
 def test_extend_basis_sequence_then_forward_sees_the_new_columns():
     """A stream of tokens, some in the span, some not: the GPU basis and the oracle's evolve
     independently from the same start and stay together (same decisions, same columns to
