@@ -22,6 +22,9 @@ __device__ __forceinline__ unsigned long long get(const unsigned long long* p) {
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
+// Orders this thread's accesses, and what it has learned of others', for the whole GPU (__threadfence()
+// is sequentially consistent on top of that, which nothing here needs).
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ bool is(unsigned long long w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
 __device__ __forceinline__ float val(unsigned long long w) { return __uint_as_float((unsigned)w); }
 
@@ -109,8 +112,9 @@ __device__ __forceinline__ bool warp_gather_sum(const unsigned long long* p, siz
 
 // The exchange area of a handle (or of the allocation-free entry point).  A location holds words
 // of one kind only, so a stale payload is never taken for a call's number.  What every CTA reads in
-// bulk only when some token is gated (rb) is plain memory, ordered by a fence before the norm words
-// and one after them; a barrier of its own for c, with its fences, took 6 us where the words take 2.
+// bulk only when some token is gated (rb) is plain memory: the warp that sends a CTA's norm words
+// fences between learning that the CTA's rows are written and the words, a reader fences between the
+// words and rb, and a warp that passes a decision on does both; a barrier of its own for c, with its fences, took 6 us where the words take 2.
 // Every CTA starts a bulk read at another place: 148 readers in step at one place get 13 KB per
 // microsecond and SM, spread out 50.
 struct Area {

@@ -558,7 +558,6 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
         }
         return v;
       };
-      if (warp < nu * ncb) __threadfence();   // r before the word that announces it
       if (uc + nu >= pt) {
         __syncwarp();
         int before = 0;
@@ -570,6 +569,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
         before = __shfl_sync(0xffffffffu, before, 0);
         __syncwarp();
         if (before == kW - 1) {
+          fence_gpu();   // the CTA's r, which this warp now knows to be written, before the word that announces it
           for (int t = lane; t < NC; t += 32) {
             const float2 v = add_units(t);
             put128(words.norm + (size_t)cta * n + tb + t, __float_as_uint(v.x), __float_as_uint(v.y), 0u, tag);
@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
       all = __all_sync(0xffffffffu, all);
     }
     ok = ok && all;
-    __threadfence();
+    fence_gpu();
     double sr = 0.0, sx = 0.0;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
@@ -645,6 +645,8 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
   } else {
     for (int t = cta + warp * G; t < n; t += kW * G) {
       const bool fast = decide(t);
+      __syncwarp();   // what the lanes have seen (every CTA's r), before the word that announces it
+      if (lane == 0) fence_gpu();
       if (lane == 0 && ok) put128(words.gate + t, __float_as_uint(s_rho[t]), fast ? 1u : 0u, 0u, tag);
     }
     __syncwarp();
@@ -654,7 +656,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
       ok = ok && w.tag == tag;
       s_fast[warp * 32 + lane] = w.b != 0u;
       s_rho[warp * 32 + lane] = __uint_as_float(w.a);
-      __threadfence();
+      fence_gpu();
     }
   }
   if (timed_out(ok)) return;

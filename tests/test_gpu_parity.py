@@ -109,6 +109,27 @@ def test_one_launch_forward_on_two_streams_at_once():
     assert all(torch.equal(y, refs[i]) for i, y in outs)
 
 
+@pytest.mark.parametrize("n", [1, 3, 8, 33])
+def test_one_launch_calls_back_to_back_stream_their_own_residual(n):
+    """Calls with every token gated, enqueued without a pause and alternating between two inputs: W r
+    of a call is that of its own r (which the CTAs hand to one another through plain memory)."""
+    g = G()
+    x, P, Ws = make_small(1512, 72, (1000, 64), 2 * n, seed=77 + n, outlier_every=1)
+    lay = g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n)
+    xs = [x[:n].cuda().contiguous(), x[n:].cuda().contiguous()]
+    refs = []
+    for xi in xs:
+        y, gate, _ = lay.forward(xi)
+        torch.cuda.synchronize()
+        assert int(gate.sum()) == n
+        refs.append(y.clone())
+    compare_group(x[:n], P, Ws, 0.05, refs[0].cpu().numpy(), np.ones(n, np.uint8))
+    outs = [lay.forward(xs[i % 2])[0] for i in range(200)]
+    torch.cuda.synchronize()
+    assert lay.status() == 0
+    assert all(torch.equal(y, refs[i % 2]) for i, y in enumerate(outs))
+
+
 def test_config1_literal_batch1_all_tokens():
     st = S.config1()
     m = S.materialize_group(st, 0, 0, st.steps)
