@@ -190,7 +190,7 @@ gsi_status_t gsi_forward_host(gsi_handle_t h, const float* x_host, int n_tokens,
  * The first call on each device resolves the array's device address (with that
  * device current); make that first call before any stream capture begins.  The
  * call allocates nothing and frees nothing.  All calls on a device share the one
- * array, which keeps the previous call's contents; every word carries the number of
+ * array, which keeps the previous call's contents; every word carries a tag of
  * the call that wrote it, so nothing is cleared between calls.  Two calls whose
  * kernels overlap on the GPU (different streams, or one stream per thread) race
  * on the array - serialise them.
@@ -245,6 +245,16 @@ gsi_status_t gsi_get_image_fp8(gsi_handle_t h, const void** tiled_out, size_t* b
  * 0, or a GSI_ERR_* code recorded by a kernel (e.g. a bounded wait that gave
  * up).  Kernels never trap. */
 gsi_status_t gsi_get_status(gsi_handle_t h, int* device_status);
+
+/*
+ * Polls a wait between the CTAs of one launch (gsi_forward*, gsi_extend_basis) may take before the
+ * CTA gives up, records GSI_ERR_TIMEOUT in the status word and returns; 0 restores the default
+ * (2^20, about a second).  After a time-out the outputs of that call are undefined and the status
+ * word stays set; the calls that follow are not affected.  Applies from the next call (a captured
+ * call keeps the limit it was captured with).  A very small value makes the time-out path testable
+ * without hanging anything.
+ */
+gsi_status_t gsi_set_spin_limit(gsi_handle_t h, unsigned polls);
 
 gsi_status_t gsi_destroy(gsi_handle_t h);
 

@@ -20,7 +20,7 @@ GSI_MAX_MAPS, GSI_MAX_TOKENS = 8, 64
 EXPORTED = [
     "gsi_status_string", "gsi_build_image", "gsi_workspace_bytes", "gsi_create",
     "gsi_forward", "gsi_forward_n", "gsi_forward_host", "gsi_forward_static", "gsi_extend_basis", "gsi_get_image", "gsi_get_image_fp8", "gsi_get_status",
-    "gsi_destroy", "gsi_stack_workspace_bytes", "gsi_stack_create", "gsi_stack_bind",
+    "gsi_set_spin_limit", "gsi_destroy", "gsi_stack_workspace_bytes", "gsi_stack_create", "gsi_stack_bind",
     "gsi_stack_set_mode", "gsi_stack_set_concurrent", "gsi_stack_is_persistent", "gsi_stack_set_trace", "gsi_stack_set_spin_limit", "gsi_stack_seek", "gsi_stack_step", "gsi_stack_launches_per_step",
     "gsi_stack_step_host", "gsi_stack_get_status", "gsi_stack_destroy",
 ]
@@ -65,6 +65,7 @@ def _load():
     l.gsi_get_image_fp8.argtypes = [vp, C.POINTER(vp), C.POINTER(C.c_size_t)]
     l.gsi_extend_basis.argtypes = [vp, vp, C.c_float, vp, vp, vp, vp]
     l.gsi_get_status.argtypes = [vp, C.POINTER(i)]
+    l.gsi_set_spin_limit.argtypes = [vp, C.c_uint]
     l.gsi_destroy.argtypes = [vp]
     l.gsi_stack_workspace_bytes.restype = sz
     l.gsi_stack_workspace_bytes.argtypes = [i]
@@ -259,6 +260,10 @@ class Layer:
         codes = tiles.permute(0, 5, 2, 1, 4, 3, 6).reshape(R * 16, k)[:O].clone()
         scales = raw[:, KT * 256:].contiguous().view(torch.float32).reshape(R * 16)[:O].clone()
         return codes, scales
+
+    def set_spin_limit(self, polls: int):
+        """Polls a wait between the CTAs of one launch may take (0 = the default)."""
+        _check(lib.gsi_set_spin_limit(self.handle, int(polls)), "gsi_set_spin_limit")
 
     def status(self) -> int:
         v = C.c_int()

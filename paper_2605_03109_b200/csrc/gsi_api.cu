@@ -305,7 +305,8 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W, const void
   g.cpart3 = reinterpret_cast<float*>(h->ws + L.f_cpart);
   g.normpart3 = reinterpret_cast<float*>(h->ws + L.f_normpart);
   g.fused_words = reinterpret_cast<unsigned long long*>(h->ws + L.fused);
-  g.fused_call = reinterpret_cast<unsigned*>(ctrl + 32);
+  g.tickets = reinterpret_cast<unsigned long long*>(ctrl + 32);
+  g.spin_limit = kFusedSpinLimit;
   g.area_B = g.B;
   g.area_k = g.k;
   g.area_d = g.d;
@@ -454,6 +455,12 @@ gsi_status_t gsi_get_status(gsi_handle_t h, int* device_status) {
   if (cudaStreamSynchronize(h->last_stream) != cudaSuccess) return GSI_ERR_CUDA;
   if (cudaMemcpy(device_status, h->gp.status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
     return GSI_ERR_CUDA;
+  return GSI_OK;
+}
+
+gsi_status_t gsi_set_spin_limit(gsi_handle_t h, unsigned polls) {
+  if (!h) return GSI_ERR_INVALID_ARG;
+  h->gp.spin_limit = polls ? polls : kFusedSpinLimit;
   return GSI_OK;
 }
 

@@ -121,9 +121,11 @@ struct GroupParams {
   // calls in one launch (gsi_fused.cu)
   unsigned long long* fused_words;   // exchange area, laid out for ...
   int area_B, area_k, area_d;        // ... the largest call that uses it
-  unsigned* fused_call;              // calls so far
+  unsigned long long* tickets;       // counts their launches (exchange::first_tag)
+  unsigned spin_limit;               // polls their waits may take
 };
 constexpr int kFusedMaxGrid = 160;
+constexpr unsigned kFusedSpinLimit = 1u << 20;   // default: about a second
 
 // The block that arrives last (of n_blocks) sums the per-part norm partials in part
 // order in double precision, writes gate / rho (Eq. (3.3)) and the ascending list of

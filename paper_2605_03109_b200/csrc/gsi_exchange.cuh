@@ -1,6 +1,6 @@
 // Words that carry their own validity between the CTAs of one cooperative launch: 64 bits, an
-// fp32 value in the lower half and the number of the call that wrote it in the upper half,
-// written and read whole.  A reader that sees this call's number has the value: one L2 round
+// fp32 value in the lower half and the tag of the call that wrote it in the upper half,
+// written and read whole.  A reader that sees this call's tag has the value: one L2 round
 // trip, no fence, no counter, nothing to clear between calls.  Every wait is bounded.
 #pragma once
 
@@ -10,7 +10,6 @@ namespace gsi {
 namespace exchange {
 
 constexpr int kCols = 32;              // columns of c per CTA in the projection: 64-byte pieces of a basis row
-constexpr unsigned kSpinF = 1u << 20;
 
 __device__ __forceinline__ void put(unsigned long long* p, float v, unsigned tag) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p),
@@ -28,7 +27,7 @@ __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" 
 __device__ __forceinline__ bool is(unsigned long long w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
 __device__ __forceinline__ float val(unsigned long long w) { return __uint_as_float((unsigned)w); }
 
-// Wider words: 96 bits of payload and the call's number, written and read as one 128-bit access.
+// Wider words: 96 bits of payload and the call's tag, written and read as one 128-bit access.
 struct Word128 {
   uint32_t a, b, c, tag;
 };
@@ -51,12 +50,12 @@ __device__ __forceinline__ Word128 get128(const Word128* p) {
   return w;
 }
 
-// Words at(0) .. at(count - 1), four in flight; false when a wait ran out.
+// Words at(0) .. at(count - 1), four in flight; false when a wait ran out (`limit` polls).
 template <typename P, typename F>
-__device__ __forceinline__ bool gather128(P&& at, int count, unsigned tag, F&& take) {
+__device__ __forceinline__ bool gather128(P&& at, int count, unsigned tag, unsigned limit, F&& take) {
   for (int i0 = 0; i0 < count; i0 += 4) {
     Word128 w[4];
-    for (unsigned it = 0;; ++it) {
+    for (unsigned it = 1;; ++it) {
       bool all = true;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -65,7 +64,7 @@ __device__ __forceinline__ bool gather128(P&& at, int count, unsigned tag, F&& t
       for (int u = 0; u < 4; ++u)
         if (i0 + u < count) all = all && w[u].tag == tag;
       if (all) break;
-      if (it > kSpinF) return false;
+      if (it >= limit) return false;
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -76,10 +75,11 @@ __device__ __forceinline__ bool gather128(P&& at, int count, unsigned tag, F&& t
 
 // `count` words p[i * stride] in order, kIn in flight; false when a wait ran out.
 template <int kIn = 8, typename F>
-__device__ __forceinline__ bool gather(const unsigned long long* p, size_t stride, int count, unsigned tag, F&& take) {
+__device__ __forceinline__ bool gather(const unsigned long long* p, size_t stride, int count, unsigned tag,
+                                       unsigned limit, F&& take) {
   for (int i0 = 0; i0 < count; i0 += kIn) {
     unsigned long long w[kIn];
-    for (unsigned it = 0;; ++it) {
+    for (unsigned it = 1;; ++it) {
       bool all = true;
 #pragma unroll
       for (int u = 0; u < kIn; ++u)
@@ -88,7 +88,7 @@ __device__ __forceinline__ bool gather(const unsigned long long* p, size_t strid
       for (int u = 0; u < kIn; ++u)
         if (i0 + u < count) all = all && is(w[u], tag);
       if (all) break;
-      if (it > kSpinF) return false;
+      if (it >= limit) return false;
     }
 #pragma unroll
     for (int u = 0; u < kIn; ++u)
@@ -99,19 +99,35 @@ __device__ __forceinline__ bool gather(const unsigned long long* p, size_t strid
 
 // Sum of `count` words by one warp in double (lane l: words l, l + 32, ...; fixed order).
 __device__ __forceinline__ bool warp_gather_sum(const unsigned long long* p, size_t stride, int count, unsigned tag,
-                                                double& sum) {
+                                                unsigned limit, double& sum) {
   const int lane = threadIdx.x & 31;
   double s = 0.0;
   const int mine = count > lane ? (count - lane + 31) / 32 : 0;
-  const bool ok = gather(p + (size_t)lane * stride, 32 * stride, mine, tag, [&](int, float v) { s += (double)v; });
+  const bool ok = gather(p + (size_t)lane * stride, 32 * stride, mine, tag, limit, [&](int, float v) { s += (double)v; });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   sum = s;
   return __all_sync(0xffffffffu, ok);
 }
 
+// The first of a launch's four tags, and a CTA's leave.  The CTAs of a launch add kTickets to the
+// counter between them (block 0 what the others leave of it), each when it has done with its waits, so
+// its multiple of kTickets changes when the last one leaves: they all read the same launch number
+// whenever they begin, whatever the size of the grid, and a launch whose waits ran out, in part
+// before its last CTA had begun, shares no tag with the next.
+constexpr unsigned kTickets = 256;
+static_assert(kFusedMaxGrid <= (int)kTickets, "one at least for block 0");
+__device__ __forceinline__ unsigned first_tag(const unsigned long long* counter) {
+  return (unsigned)(*counter / kTickets) * 4u + 1u;
+}
+__device__ __forceinline__ void leave_launch(unsigned long long* counter) {   // one thread, behind a barrier
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(counter),
+               "l"(blockIdx.x == 0 ? (unsigned long long)(kTickets - (gridDim.x - 1)) : 1ull)
+               : "memory");
+}
+
 // The exchange area of a handle (or of the allocation-free entry point).  A location holds words
-// of one kind only, so a stale payload is never taken for a call's number.  What every CTA reads in
+// of one kind only, so a stale payload is never taken for a tag.  What every CTA reads in
 // bulk only when some token is gated (rb) is plain memory: the warp that sends a CTA's norm words
 // fences between learning that the CTA's rows are written and the words, a reader fences between the
 // words and rb, and a warp that passes a decision on does both; a barrier of its own for c, with its fences, took 6 us where the words take 2.

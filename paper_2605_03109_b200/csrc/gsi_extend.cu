@@ -40,8 +40,8 @@ __device__ __forceinline__ uint16_t to_bf16_bits(float v) {
 }
 
 // Elements [i0, i0 + n) of a vector into shared memory, from plain floats or from tagged words.
-__device__ __forceinline__ bool stage(float* s, const float* x, const unsigned long long* words, unsigned tag, int i0,
-                                      int n) {
+__device__ __forceinline__ bool stage(float* s, const float* x, const unsigned long long* words, unsigned tag,
+                                      unsigned limit, int i0, int n) {
   bool ok = true;
   for (int ib = 0; ib < n; ib += 8 * kT) {
     if (x) {
@@ -53,7 +53,7 @@ __device__ __forceinline__ bool stage(float* s, const float* x, const unsigned l
     } else {
       const int first = ib + (int)threadIdx.x;
       const int cnt = n > first ? min(8, (n - first + kT - 1) / kT) : 0;
-      ok = gather(words + i0 + first, kT, cnt, tag, [&](int u, float v) { s[first + u * kT] = v; }) && ok;
+      ok = gather(words + i0 + first, kT, cnt, tag, limit, [&](int u, float v) { s[first + u * kT] = v; }) && ok;
     }
   }
   return ok;
@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
   __shared__ double s_norm[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = gridDim.x, cta = blockIdx.x, d = g.d, k = g.k, KV = k / 8;
-  const unsigned call = *g.fused_call;
+  const unsigned tag1 = first_tag(g.tickets);
   const int col = *a.k_active;
   const Area words = area_of(g);
   const int p0 = (int)((long long)d * cta / G), p1 = (int)((long long)d * (cta + 1) / G);
@@ -79,16 +79,16 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
   auto give_up = [&](bool ok) -> bool {   // the same answer for every thread
     if (!__syncthreads_or(!ok)) return false;
     if (tid == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
-    if (tid == 0 && cta == 0) *g.fused_call = call + 3u;
+    if (tid == 0) leave_launch(g.tickets);
     return true;
   };
 
   float inv = 0.f;
 #pragma unroll 1
   for (int pass = 1; pass <= 2; ++pass) {
-    const unsigned tag = call + (unsigned)pass;
     // (the first CTAs are done with pass 1, and at the words of pass 2, while a late one may still read)
     unsigned long long* const r2_words = words.ext_r2 + (pass - 1) * kFusedMaxGrid;
+    const unsigned tag = tag1 + (unsigned)(pass - 1);
     bool ok = true;
     // partial c of a slab of rows x 32 columns
     if (cta < n_slabs * n_cb) {
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       for (int rb = r0; rb < r1; rb += kStage) {
         const int n = min(kStage, r1 - rb);
         __syncthreads();
-        ok = stage(s_v, pass == 1 ? a.x : nullptr, words.ext_r, tag - 1u, rb, n) && ok;
+        ok = stage(s_v, pass == 1 ? a.x : nullptr, words.ext_r, tag1, g.spin_limit, rb, n) && ok;
         __syncthreads();
         for (int base = warp * 8 + sub; base < n; base += kW * 8 * 4) {
           float p[4][8];
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
     // c: every CTA adds all partials in slab order
     for (int j = tid; j < k; j += kT) {
       float s = 0.f;
-      ok = gather(words.c + j, k, n_slabs, tag, [&](int, float v) { s += v; }) && ok;
+      ok = gather(words.c + j, k, n_slabs, tag, g.spin_limit, [&](int, float v) { s += v; }) && ok;
       s_c[j] = s;
     }
     if (give_up(ok)) return;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       // at once, this exchange took 1.7 or 2.7 to 4 us, by where the words lie in memory.)
       for (const long long t0 = clock64(); clock64() - t0 < kHoldOff;) {}
       double s = 0.0;
-      ok = warp ? warp_gather_sum(words.ext_x2, 1, n_slabs, tag, s) : warp_gather_sum(r2_words, 1, G, tag, s);
+      ok = warp ? warp_gather_sum(words.ext_x2, 1, n_slabs, tag, g.spin_limit, s) : warp_gather_sum(r2_words, 1, G, tag, g.spin_limit, s);
       if (lane == 0) s_norm[warp] = s;
     }
     if (give_up(ok)) return;
@@ -213,15 +213,17 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       if (cta == 0 && tid == 0) {
         if (a.appended_out) *a.appended_out = go ? 1 : 0;
         if (go) *a.k_active = col + 1;   // (every CTA has read it: its norms are here)
-        *g.fused_call = call + 3u;
       }
-      if (!go) return;
+      if (!go) {
+        if (tid == 0) leave_launch(g.tickets);
+        return;
+      }
     }
     __syncthreads();
   }
 
   // ---- store: the image column is W times what the basis really holds
-  const unsigned tag = call + 3u;
+  const unsigned tag = tag1 + 2u;
   float m = 0.f;
   for (int i = p0 + tid; i < p1; i += kT) {
     const float v = g.r[i] * inv;
@@ -253,7 +255,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
     const int n = min(kStage, d - c0);
     const bool last = c0 + n == d;
     __syncthreads();
-    if (give_up(stage(s_v, nullptr, words.ext_r, tag, c0, n))) return;
+    if (give_up(stage(s_v, nullptr, words.ext_r, tag, g.spin_limit, c0, n))) return;
     for (int row = o0 + warp; row < o1; row += kW) {
       int j = 0;
       while (j + 1 < g.n_maps && row >= g.off[j + 1]) ++j;
@@ -288,6 +290,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
       }
     }
   }
+  if (tid == 0) leave_launch(g.tickets);
   if (a.WP8) {
     __syncthreads();   // the column is in this CTA's rows
     for (int R = o0 / 16; R * 16 < o1; ++R) {

@@ -20,7 +20,7 @@
 // at 4096 x 256 -> 28672 41.7 -> 16.0 us; 21 tokens at 3000 x 200 -> 1576 84 -> 46 us (on CUDA-core
 // FMAs this kernel took 112 us there); 16 tokens, fp32 basis, 768 x 128 -> 2304 48.5 -> 23.7 us.
 //
-// The exchanges are words that carry the call's number (gsi_exchange.cuh): a release / acquire
+// The exchanges are words that carry the call's tag (gsi_exchange.cuh): a release / acquire
 // barrier would cost two L2 round trips and a fence where these cost one.  Every token's sums run
 // in an order that depends on the shape alone: results are reproducible, and a token's are the
 // same in a call of any size.
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lg = lane >> 2, lt = lane & 3;
   const int G = gridDim.x, cta = blockIdx.x;
   const int d = g.d, k = g.k, n = n_tokens;
-  const unsigned tag = *g.fused_call + 1u;
+  const unsigned tag = first_tag(g.tickets);
   const Area words = area_of(g);
   unsigned long long* cw = words.c;
   const int slot = io_slot(io);
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
       end[r] = n_slabs * (q * R + r + 1) / kSegs - a;
     }
     if (live)
-      ok = gather<Q == 2 ? 12 : 4>(cw + (size_t)a * n * k + i, (size_t)n * k, end[R - 1], tag, [&](int u, float v) {
+      ok = gather<Q == 2 ? 12 : 4>(cw + (size_t)a * n * k + i, (size_t)n * k, end[R - 1], tag, g.spin_limit, [&](int u, float v) {
 #pragma unroll
              for (int r = 0; r < R; ++r)
                if (u < end[r] && (r == 0 || u >= end[r - 1])) run[r] += v;
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
   auto timed_out = [&](bool good) -> bool {   // the same answer for every thread
     if (!__syncthreads_or(!good)) return false;
     if (tid == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
-    if (tid == 0 && cta == 0) *g.fused_call = tag;
+    if (tid == 0) leave_launch(g.tickets);
     return true;
   };
   if constexpr (!kDirect) {
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
         const int f = rot + u * kT;
         return f < all ? f : f - all;
       };
-      ok = gather128([&](int u) { return words.cf + (size_t)tb * half + place(u); }, mine, tag,
+      ok = gather128([&](int u) { return words.cf + (size_t)tb * half + place(u); }, mine, tag, g.spin_limit,
                      [&](int u, const Word128& w) {
                        const int f = place(u), c = f / half;
                        op_store_pair(op + c * stride, 2 * (f - c * half), w.a, w.b, w.c);
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
     constexpr int kPer = kFusedMaxGrid / 32;
     Word128 w[kPer];
     bool all = false;
-    for (unsigned it = 0; !all && it <= kSpinF; ++it) {
+    for (unsigned it = 0; !all && it < g.spin_limit; ++it) {
       all = true;
 #pragma unroll
       for (int i = 0; i < kPer; ++i) {
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
     __syncwarp();
     if (warp < 2 && warp * 32 + lane < n) {
       Word128 w = get128(words.gate + warp * 32 + lane);
-      for (unsigned it = 0; w.tag != tag && it <= kSpinF; ++it) w = get128(words.gate + warp * 32 + lane);
+      for (unsigned it = 1; w.tag != tag && it < g.spin_limit; ++it) w = get128(words.gate + warp * 32 + lane);
       ok = ok && w.tag == tag;
       s_fast[warp * 32 + lane] = w.b != 0u;
       s_rho[warp * 32 + lane] = __uint_as_float(w.a);
@@ -660,6 +660,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
     }
   }
   if (timed_out(ok)) return;
+  if (tid == 0) leave_launch(g.tickets);   // (that was the last wait)
   if (warp == 0) {
     int f = 0;
     for (int t0 = 0; t0 < n; t0 += 32) {
@@ -685,7 +686,6 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
     if (lane == 0) {
       s_fired[0] = f;
       if (leave_from && cta == 0) *g.n_fired = f;
-      if (cta == 0) *g.fused_call = tag;   // every CTA has read the counter: its norms are here
     }
   }
   __syncthreads();

@@ -17,7 +17,7 @@ constexpr int kStaticMaxD = 16384;
 constexpr int kMaxDevices = 64;
 
 // layout of the scratch array (bytes)
-constexpr size_t kOffCtrl = 0;     // call counter, status word
+constexpr size_t kOffCtrl = 0;     // ticket counter, status word
 constexpr size_t kOffRho = 256;
 constexpr size_t kOffWords = 512;  // exchange words
 constexpr size_t kStaticScratchBytes = 768 * 1024;   // fused_words_bytes of the largest call, checked below
@@ -97,13 +97,13 @@ extern "C" gsi_status_t gsi_forward_static(const void* const* W_host_array, cons
   g.area_B = kStaticMaxTokens;
   g.area_k = kStaticMaxK;
   g.area_d = kStaticMaxD;
-  unsigned* ctrl = reinterpret_cast<unsigned*>(base + kOffCtrl);
-  g.fused_call = ctrl;
-  g.status = reinterpret_cast<int*>(ctrl + 1);
+  g.tickets = reinterpret_cast<unsigned long long*>(base + kOffCtrl);
+  g.spin_limit = kFusedSpinLimit;
+  g.status = reinterpret_cast<int*>(base + kOffCtrl + 8);
   g.rho_scratch = reinterpret_cast<float*>(base + kOffRho);
   g.fused_words = reinterpret_cast<unsigned long long*>(base + kOffWords);
-  // The array keeps whatever the last call left; its exchange words carry that call's number,
-  // which is not this call's, so nothing has to be cleared.
+  // The array keeps whatever the last call left; its exchange words carry that call's tags,
+  // which are not this call's, so nothing has to be cleared.
 
   IoRef io{};
   io.x = x;

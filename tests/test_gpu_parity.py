@@ -130,6 +130,34 @@ def test_one_launch_calls_back_to_back_stream_their_own_residual(n):
     assert all(torch.equal(y, refs[i % 2]) for i, y in enumerate(outs))
 
 
+@pytest.mark.parametrize("n", [1, 6])
+def test_one_launch_wait_runs_out_and_the_next_calls_are_right(n):
+    """Failure detection without a fault: with a single poll per wait the exchanges between the CTAs
+    cannot complete, every CTA returns and the status word says so.  CTAs that begin after the others
+    have given up belong to the same launch all the same: with the default limit restored, forward
+    calls and basis extensions on the handle give the bits of an undisturbed one."""
+    g = G()
+    x, P, Ws = make_small(2056, 200, (1000, 64), 2 * n, seed=177 + n, outlier_every=2)
+    xs = [x[:n].cuda().contiguous(), x[n:].cuda().contiguous()]
+    inside = (P.double() @ torch.randn(200, dtype=torch.float64, generator=torch.Generator().manual_seed(5))).float().cuda()
+
+    def run(lay):
+        out = [t.clone() for xi in xs for t in lay.forward(xi)]
+        out += lay.extend_basis(inside, 0.5, torch.tensor([7], dtype=torch.int32, device="cuda"))
+        torch.cuda.synchronize()
+        return out
+    lays = [g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n) for _ in range(2)]
+    ref = run(lays[0])
+    assert lays[0].status() == 0 and ref[-2].item() == 0 and 0 < int(ref[1].sum()) + int(ref[4].sum())
+    for _ in range(5):
+        lays[1].set_spin_limit(1)
+        run(lays[1])
+        assert lays[1].status() == 5               # GSI_ERR_TIMEOUT, nothing hung
+        lays[1].set_spin_limit(0)                  # the default again
+        for _ in range(2):
+            assert all(torch.equal(a, b) for a, b in zip(ref, run(lays[1])))
+
+
 def test_config1_literal_batch1_all_tokens():
     st = S.config1()
     m = S.materialize_group(st, 0, 0, st.steps)
