@@ -176,7 +176,8 @@ gsi_status_t gsi_forward_host(gsi_handle_t h, const float* x_host, int n_tokens,
  * wants.  Here the scratch (the words its CTAs exchange) lives in a fixed array
  * inside the library: about 0.7 MB that every GPU which loads the library holds
  * until the process exits.  No device status word can be read back for this entry
- * point.
+ * point: a call in which a wait between its CTAs ran out (about a second) reports it by
+ * rho = NaN and gate = 1 for every token, and by NaN in the rows of y it did not finish.
  *
  * The caller passes everything else: W_host_array (HOST array of n_maps DEVICE
  * pointers, W_j [d_out_j][d] bf16), d_out (HOST array), P [d][k], and W_P, the
@@ -249,8 +250,9 @@ gsi_status_t gsi_get_status(gsi_handle_t h, int* device_status);
 /*
  * Polls a wait between the CTAs of one launch (gsi_forward*, gsi_extend_basis) may take before the
  * CTA gives up, records GSI_ERR_TIMEOUT in the status word and returns; 0 restores the default
- * (2^20, about a second).  After a time-out the outputs of that call are undefined and the status
- * word stays set; the calls that follow are not affected.  Applies from the next call (a captured
+ * (2^20, about a second).  After a time-out the status word stays set; that call's rho is NaN and its
+ * gate 1 for every token, and the rows of y it did not finish are NaN; the calls that follow are not
+ * affected.  Applies from the next call (a captured
  * call keeps the limit it was captured with).  A very small value makes the time-out path testable
  * without hanging anything.
  */

@@ -282,11 +282,10 @@ __device__ __forceinline__ void stream_w(const GroupParams& g, const IoRef& io, 
 // NB: eight-token blocks at a time in the projection.  kDirect: a build for calls of up to
 // kDirectTokens tokens (what the others need would cost it registers: 3 us at one token).  leave_from > 0: with that many gated tokens or
 // more W r is left to the tensor-core contraction that follows (r goes to g.r, the gated tokens to
-// g.fired).
+// g.fired).  False when a wait ran out (for every thread of the CTA).
 template <int NB, bool PF32, bool kDirect>
-__global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__ GroupParams g, const __grid_constant__ IoRef io,
-                                                         int n_tokens, int n_slabs,
-                                                         int leave_from) {
+__device__ __forceinline__ bool forward_fused(const GroupParams& g, const IoRef& io, int n_tokens, int n_slabs,
+                                              int leave_from) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ float2 s_unit[kSlots][GSI_MAX_TOKENS];    // ||r||^2, ||x||^2 of a 16-row unit of the basis
   __shared__ float2 s_run[GSI_MAX_TOKENS];             // ... of the units before
@@ -502,7 +501,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
                        op_store_pair(op + c * stride, 2 * (f - c * half), w.a, w.b, w.c);
                      }) && ok;
     }
-    if (timed_out(ok)) return;
+    if (timed_out(ok)) return false;
     // basis rows: a unit x eight tokens per warp.  The units' norms wait in shared memory and are
     // added in order by the warp that hands in last; it sends them off while the image rows run.
     for (int uc = 0; uc == 0 || uc < pt; uc += kSlots) {
@@ -659,7 +658,7 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
       fence_gpu();
     }
   }
-  if (timed_out(ok)) return;
+  if (timed_out(ok)) return false;
   if (tid == 0) leave_launch(g.tickets);   // (that was the last wait)
   if (warp == 0) {
     int f = 0;
@@ -689,12 +688,32 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
     }
   }
   __syncthreads();
-  if (s_fired[0] == 0 || (leave_from && s_fired[0] >= leave_from)) return;
+  if (s_fired[0] == 0 || (leave_from && s_fired[0] >= leave_from)) return true;
 
   // ---- C
   if (s_fired[0] <= 8) stream_w<1>(g, io, words.rb, s_fired, smem, o0, o1);
   else if (s_fired[0] <= 16) stream_w<2>(g, io, words.rb, s_fired, smem, o0, o1);
   else stream_w<4>(g, io, words.rb, s_fired, smem, o0, o1);
+  return true;
+}
+
+template <int NB, bool PF32, bool kDirect>
+__global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__ GroupParams g, const __grid_constant__ IoRef io,
+                                                         int n_tokens, int n_slabs,
+                                                         int leave_from) {
+  if (forward_fused<NB, PF32, kDirect>(g, io, n_tokens, n_slabs, leave_from)) return;
+  // The call's results must not pass for results (the allocation-free entry point has no status word
+  // to ask for): NaN in this CTA's rows of y, whose W r may be missing, and in every token's rho.
+  const float nan = __int_as_float(0x7fc00000);
+  const int cta = blockIdx.x, G = gridDim.x, slot = io_slot(io);
+  const int o0 = (int)((long long)g.O * cta / G), o1 = (int)((long long)g.O * (cta + 1) / G);
+  for (int t = 0; t < n_tokens; ++t)
+    for (int row = o0 + (int)threadIdx.x; row < o1; row += kT) io.y[(size_t)t * g.O + row] = nan;
+  for (int t = threadIdx.x; t < n_tokens; t += kT) {
+    io.gate[(long long)slot * io.log_step_stride + t] = 1;
+    (io.rho ? io.rho + (long long)slot * io.log_step_stride : g.rho_scratch)[t] = nan;
+  }
+  if (leave_from && cta == 0 && threadIdx.x == 0) *g.n_fired = 0;   // no list of another call for the contraction
 }
 
 template <int NB, bool PF32, bool kDirect>
