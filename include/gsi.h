@@ -113,7 +113,8 @@ const char* gsi_status_string(gsi_status_t s);
  * Cached image of Eq. (3.2) / Section 4.2 (built once per weight matrix, off the per-token path):
  *   W_P[a][j] = bf16_rne( sum_i W[a][i] * P[i][j] ),  fp32 accumulation.
  * W [o][d] bf16, P [d][k] of p_dtype, W_P_out [o][k] bf16; all device.
- * Enqueued on `stream`; no host synchronisation.
+ * Enqueued on `stream`; no host synchronisation.  A tile whose bounded wait (for its own copies, some
+ * seconds) ran out is NaN; gsi_create returns GSI_ERR_TIMEOUT in that case.
  */
 gsi_status_t gsi_build_image(const void* W, const void* P, int o, int d, int k,
                              gsi_dtype_t p_dtype, void* W_P_out, gsi_stream_t stream);

@@ -226,7 +226,7 @@ gsi_status_t gsi_build_image(const void* W, const void* P, int o, int d, int k,
   if (p_dtype != GSI_BF16 && p_dtype != GSI_F32) return GSI_ERR_INVALID_ARG;
   if (!aligned16(W) || !aligned16(P) || !aligned16(W_P_out)) return GSI_ERR_INVALID_ARG;
   if (o % 8 || d % 8 || k % 8) return GSI_ERR_UNSUPPORTED;
-  return launch_build_image(W, P, o, d, k, p_dtype == GSI_F32, W_P_out, stream) == cudaSuccess
+  return launch_build_image(W, P, o, d, k, p_dtype == GSI_F32, W_P_out, nullptr, stream) == cudaSuccess
              ? GSI_OK
              : GSI_ERR_CUDA;
 }
@@ -339,7 +339,7 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W, const void
   if (!dense) {
     for (int j = 0; j < desc->n_maps; ++j) {
       void* dst = h->ws + L.wp + (size_t)g.off[j] * desc->k * 2;
-      if (launch_build_image(W[j], P, desc->d_out[j], desc->d, desc->k, g.p_f32, dst, stream) !=
+      if (launch_build_image(W[j], P, desc->d_out[j], desc->d, desc->k, g.p_f32, dst, g.status, stream) !=
           cudaSuccess) {
         delete h;
         return GSI_ERR_CUDA;
@@ -352,9 +352,11 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W, const void
   }
   // A set-up call: return only when the images, max|P| and the cleared state are in
   // place, so the handle may be used from any stream afterwards.
-  if (cudaStreamSynchronize(stream) != cudaSuccess) {
+  int status = 0;
+  if (cudaMemcpyAsync(&status, g.status, sizeof status, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess || status != 0) {
     delete h;
-    return GSI_ERR_CUDA;
+    return status ? (gsi_status_t)status : GSI_ERR_CUDA;   // (an image with a tile that was given up)
   }
   *out = h;
   return GSI_OK;

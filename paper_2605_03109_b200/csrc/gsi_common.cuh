@@ -275,7 +275,8 @@ int front_proj_splits(int d, int k);
 int front_rows(int max_tokens);   // rows of the three-term operands
 // Kernel launches one generic forward of n_tokens tokens makes.
 int generic_launch_count(const GroupParams& g, int n_tokens, bool per_stage);
+// status (device, or null) is set when a tile had to be given up.
 cudaError_t launch_build_image(const void* W, const void* P, int o, int d, int k, bool p_f32,
-                               void* WP, cudaStream_t stream);
+                               void* WP, int* status, cudaStream_t st);
 
 }  // namespace gsi

@@ -24,7 +24,8 @@
 // One CTA per tile and share of the depth.  Narrow maps leave SMs idle, so a cluster of S CTAs may
 // split the depth: the partial tiles meet in distributed shared memory and are added in rank
 // order (reproducible).  Ragged edges are the tensor maps' zero fill plus guarded stores.
-// Every wait is bounded; a tile whose wait ran out is not written.
+// Every wait is bounded; a tile whose wait ran out is written as NaN, never as a wrong number, and the
+// status word, where the caller has one, says so.
 #include "gsi_umma.cuh"
 
 namespace gsi {
@@ -85,7 +86,7 @@ __device__ __forceinline__ void split3_pair(float a, float b, uint32_t (&t)[3]) 
 template <int kN, bool kF32>
 __global__ void __launch_bounds__(ICfg<kN, kF32>::kThreads, 1)
 k_image_tc(const __grid_constant__ ImageMaps tm, const float* __restrict__ Pf, int o, int d, int k, int splits,
-           uint16_t* __restrict__ WP) {
+           uint16_t* __restrict__ WP, int* status) {
   using C = ICfg<kN, kF32>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -253,6 +254,7 @@ k_image_tc(const __grid_constant__ ImageMaps tm, const float* __restrict__ Pf, i
   if (*reinterpret_cast<volatile int*>(s_fail)) mine = false;
   const bool done = __syncthreads_and(mine ? 1 : 0) != 0;
   if (!done && tid == 0) {   // copies issued but not consumed: a bounded time to land
+    if (status) atomicExch(status, (int)GSI_ERR_TIMEOUT);
     for (int s = 0; s < C::kStages && s < nloc; ++s) {
       const int last = ((nloc - 1 - s) / C::kStages) * C::kStages + s;
       (void)mbar_wait(&bar_full[s], (last / C::kStages) & 1, 1u << 16);
@@ -260,8 +262,12 @@ k_image_tc(const __grid_constant__ ImageMaps tm, const float* __restrict__ Pf, i
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
+  if (!done) {
+#pragma unroll
+    for (int e = 0; e < kHalf; ++e) sum[e] = __int_as_float(0x7fc00000);
+  }
   if (splits == 1) {
-    if (done && acc_warp && row < o) {
+    if (acc_warp && row < o) {
 #pragma unroll
       for (int c0 = 0; c0 < kHalf; c0 += 8)
         if (col0 + ch + c0 < k)
@@ -275,7 +281,7 @@ k_image_tc(const __grid_constant__ ImageMaps tm, const float* __restrict__ Pf, i
     float* part = reinterpret_cast<float*>(smem);
     if (acc_warp) {
 #pragma unroll
-      for (int e = 0; e < kHalf; ++e) part[(ch + e) * kTM + r] = done ? sum[e] : __int_as_float(0x7fc00000);   // (gave up: NaN, never a wrong number)
+      for (int e = 0; e < kHalf; ++e) part[(ch + e) * kTM + r] = sum[e];
     }
     cluster_sync();
     const int per = kN / 8 / splits * 8;   // columns of a rank: kN >= 64, splits <= 8
@@ -300,7 +306,7 @@ k_image_tc(const __grid_constant__ ImageMaps tm, const float* __restrict__ Pf, i
 }
 
 template <int kN, bool kF32>
-cudaError_t launch_n(const ImageMaps& tm, const void* P, int o, int d, int k, int splits, void* WP,
+cudaError_t launch_n(const ImageMaps& tm, const void* P, int o, int d, int k, int splits, void* WP, int* status,
                      cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_image_tc<kN, kF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        ICfg<kN, kF32>::kSmem);
@@ -317,13 +323,13 @@ cudaError_t launch_n(const ImageMaps& tm, const void* P, int o, int d, int k, in
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_image_tc<kN, kF32>, tm, static_cast<const float*>(kF32 ? P : nullptr), o, d, k,
-                            splits, static_cast<uint16_t*>(WP));
+                            splits, static_cast<uint16_t*>(WP), status);
 }
 
 }  // namespace
 
 cudaError_t launch_build_image(const void* W, const void* P, int o, int d, int k, bool p_f32, void* WP,
-                               cudaStream_t st) {
+                               int* status, cudaStream_t st) {
   ImageMaps tm;
   if (!encode_bf16_map(&tm.w, W, o, d, kTM)) return cudaErrorNotSupported;
   if (!p_f32 && !encode_bf16_map(&tm.p, P, d, k, kTK)) return cudaErrorNotSupported;
@@ -347,11 +353,11 @@ cudaError_t launch_build_image(const void* W, const void* P, int o, int d, int k
       }
     }
   }
-  if (p_f32) return launch_n<64, true>(tm, P, o, d, k, best_s, WP, st);
+  if (p_f32) return launch_n<64, true>(tm, P, o, d, k, best_s, WP, status, st);
   switch (best_n) {
-    case 64: return launch_n<64, false>(tm, P, o, d, k, best_s, WP, st);
-    case 128: return launch_n<128, false>(tm, P, o, d, k, best_s, WP, st);
-    default: return launch_n<256, false>(tm, P, o, d, k, best_s, WP, st);
+    case 64: return launch_n<64, false>(tm, P, o, d, k, best_s, WP, status, st);
+    case 128: return launch_n<128, false>(tm, P, o, d, k, best_s, WP, status, st);
+    default: return launch_n<256, false>(tm, P, o, d, k, best_s, WP, status, st);
   }
 }
 
