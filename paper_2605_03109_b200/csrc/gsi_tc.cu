@@ -10,12 +10,13 @@
 //   A (W tile, 128 x 64 bf16 per stage)   global -> shared by TMA in the 128-byte-swizzled
 //   B (R tile,   N x 64 bf16 per stage)   K-major layout tcgen05 reads
 //   D (128 lanes x N columns fp32)        tensor memory; tcgen05.mma, one issuing thread
-//   epilogue                              tcgen05.ld -> registers -> partial-sum buffer
+//   epilogue                              tcgen05.ld -> registers -> added to y (red.add.f32)
 //
-// Split-K over CTAs fills the machine for the narrow maps; partial sums are added
-// to y in a fixed order by a second small kernel, so results are reproducible.
-// Every wait is bounded; a timeout sets the status word, frees the tensor memory
-// and returns.
+// Split-K over CTAs fills the machine for the narrow maps.  The splits of a tile are a cluster
+// that adds them in a fixed order in distributed shared memory; those of a small map leave them
+// in memory for a second small kernel.  Either way results are reproducible.
+// Every wait is bounded; a timeout sets the status word, hands NaN on, frees the tensor
+// memory and returns.
 #include "gsi_umma.cuh"
 
 namespace gsi {
@@ -97,10 +98,13 @@ k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, 
     }
     __syncthreads();
   }
+  // A block whose contraction gave up hands on NaN: y (and what is kept of an earlier call's partial
+  // sums) must not pass for a result.
+  const float gave_up = __int_as_float(0x7fc00000);
+  if (!ok && threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
   if (kCluster && !skipped) {   // (the same for all blocks of the cluster)
     float* part = reinterpret_cast<float*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);   // [column][row]: the ring is consumed
-    if (!ok && threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
     const unsigned long long mask = s_mask;
     const int r = warp * 32 + lane;
     for (int c0 = 0; c0 < N; c0 += 16) {
@@ -109,7 +113,7 @@ k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, 
       tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
       tmem_ld_wait();
 #pragma unroll
-      for (int c = 0; c < 16; ++c) part[(c0 + c) * kTM + r] = __uint_as_float(v[c]);
+      for (int c = 0; c < 16; ++c) part[(c0 + c) * kTM + r] = ok ? __uint_as_float(v[c]) : gave_up;
     }
     cluster_sync();
 #pragma unroll 2
@@ -128,8 +132,6 @@ k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, 
     cluster_sync();   // nobody leaves while its sums are being read
   } else if (skipped) {
     // nothing to write
-  } else if (!ok) {
-    if (threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
   } else if (nloc > 0) {
     // warp w owns tensor-memory lanes 32w..32w+31 = rows row0+32w+lane; 16 columns per load
     // One split: the tile's rows belong to this block alone, and y holds the image product of
@@ -150,13 +152,13 @@ k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, 
           if ((mask >> (c0 + c)) & 1ull) {
             const int tok = mapped ? c0 + c : g.fired[c0 + c];
             asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(io.y + (size_t)tok * g.O + row),
-                         "f"(__uint_as_float(v[c]))
+                         "f"(ok ? __uint_as_float(v[c]) : gave_up)
                          : "memory");
           }
       } else {
 #pragma unroll
         for (int c = 0; c < 16; ++c)
-          if ((mask >> (c0 + c)) & 1ull) yp[(size_t)(c0 + c) * g.O] = __uint_as_float(v[c]);
+          if ((mask >> (c0 + c)) & 1ull) yp[(size_t)(c0 + c) * g.O] = ok ? __uint_as_float(v[c]) : gave_up;
       }
     }
   }
