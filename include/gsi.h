@@ -252,8 +252,9 @@ gsi_status_t gsi_get_status(gsi_handle_t h, int* device_status);
  * Polls a wait between the CTAs of one launch (gsi_forward*, gsi_extend_basis) may take before the
  * CTA gives up, records GSI_ERR_TIMEOUT in the status word and returns; 0 restores the default
  * (2^20, about a second).  After a time-out the status word stays set; that call's rho is NaN and its
- * gate 1 for every token, and the rows of y it did not finish are NaN; the calls that follow are not
- * affected.  Applies from the next call (a captured
+ * gate 1 for every token, and the rows of y it did not finish are NaN; an extension reports nothing appended
+ * and rho = NaN (unless it gave up behind the decision: basis and image are then undefined); the calls
+ * that follow are not affected.  Applies from the next call (a captured
  * call keeps the limit it was captured with).  A very small value makes the time-out path testable
  * without hanging anything.
  */

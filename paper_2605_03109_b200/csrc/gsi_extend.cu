@@ -83,6 +83,11 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
     return true;
   };
 
+  if (cta == 0 && tid == 0) {   // what a call that gives up leaves
+    if (a.appended_out) *a.appended_out = 0;
+    if (a.rho_out) *a.rho_out = __int_as_float(0x7fc00000);
+  }
+
   float inv = 0.f;
 #pragma unroll 1
   for (int pass = 1; pass <= 2; ++pass) {

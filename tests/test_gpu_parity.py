@@ -152,10 +152,13 @@ def test_one_launch_wait_runs_out_and_the_next_calls_are_right(n):
     assert lays[0].status() == 0 and ref[-2].item() == 0 and 0 < int(ref[1].sum()) + int(ref[4].sum())
     for _ in range(5):
         lays[1].set_spin_limit(1)
-        y, gate, rho, *_ = run(lays[1])
+        keep = [torch.full((1,), 1, dtype=torch.int32, device="cuda") for _ in range(64)]
+        del keep                                   # (what fresh memory may hold)
+        y, gate, rho, *_, appended, rho_x = run(lays[1])
         assert lays[1].status() == 5               # GSI_ERR_TIMEOUT, nothing hung
         # nothing that could pass for a result
         assert bool(torch.isnan(y).all()) and bool(torch.isnan(rho).all()) and bool((gate == 1).all())
+        assert appended.item() == 0 and bool(torch.isnan(rho_x).all())
         lays[1].set_spin_limit(0)                  # the default again
         for _ in range(2):
             assert all(torch.equal(a, b) for a, b in zip(ref, run(lays[1])))
