@@ -139,7 +139,8 @@ struct Area {
   Word128* gate;              // [token]: rho, fired
   Word128* cf;                // [token][k / 2]: two coefficients as three bf16 terms each
   unsigned char* rb;          // r as three bf16 terms, in operand order: [token][term_bytes(d)]
-  unsigned long long *ext_r, *ext_x2, *ext_r2;   // basis extension: [d], [slab], [pass][cta]
+  unsigned long long *ext_r, *ext_x2, *ext_r2;   // basis extension: [d], [slab], [cta] of pass 1
+  Word128* ext_r2d;           // ... [cta] of pass 2, a double each
 };
 // Operand bytes of one column: 192 for every 32 elements (zeros past the end).
 __host__ __device__ __forceinline__ int term_bytes(int n) { return (n + 31) / 32 * 192; }
@@ -152,7 +153,8 @@ __device__ __forceinline__ Area area_of(const GroupParams& g) {
   w.rb = reinterpret_cast<unsigned char*>(w.cf + (size_t)g.area_B * (g.area_k / 2));
   w.ext_x2 = reinterpret_cast<unsigned long long*>(w.rb + (size_t)g.area_B * term_bytes(g.area_d));
   w.ext_r2 = w.ext_x2 + kFusedMaxGrid;
-  w.ext_r = w.ext_r2 + 2 * kFusedMaxGrid;
+  w.ext_r2d = reinterpret_cast<Word128*>(w.ext_r2 + kFusedMaxGrid);
+  w.ext_r = w.ext_r2 + 3 * kFusedMaxGrid;
   return w;
 }
 

@@ -62,7 +62,7 @@ __device__ __forceinline__ bool stage(float* s, const float* x, const unsigned l
 template <int VPL, bool PF32>
 __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, int n_slabs) {
   __shared__ float s_v[kStage];
-  __shared__ float s_part[kW * kCols];
+  __shared__ __align__(8) float s_part[kW * kCols];
   __shared__ float s_c[1024];
   __shared__ float s_scale[16];
   __shared__ double s_norm[2];
@@ -91,8 +91,6 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
   float inv = 0.f;
 #pragma unroll 1
   for (int pass = 1; pass <= 2; ++pass) {
-    // (the first CTAs are done with pass 1, and at the words of pass 2, while a late one may still read)
-    unsigned long long* const r2_words = words.ext_r2 + (pass - 1) * kFusedMaxGrid;
     const unsigned tag = tag1 + (unsigned)(pass - 1);
     bool ok = true;
     // partial c of a slab of rows x 32 columns
@@ -160,6 +158,7 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
     if (give_up(ok)) return;
     // this CTA's rows of the residual
     float c8[VPL][8], sr = 0.f;
+    double sr2 = 0.0;   // pass 2: the column is divided by this norm, whatever the scale of x (squares of 1e-21 are not fp32 numbers)
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
 #pragma unroll
@@ -182,24 +181,50 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
         const float rv = (pass == 1 ? __ldg(a.x + row) : g.r[row]) - dot;   // (g.r: written here in pass 1)
         g.r[row] = rv;
         if (pass == 1) put(words.ext_r + row, rv, tag);
-        sr = fmaf(rv, rv, sr);
+        if (pass == 1) sr = fmaf(rv, rv, sr);
+        else sr2 = fma((double)rv, (double)rv, sr2);
       }
     }
-    sr = warp_sum(sr);
-    if (lane == 0) s_part[warp] = sr;
-    __syncthreads();
-    if (tid == 0) {
-      float s = 0.f;
+    // (each pass has norm words of its own: the first CTAs are done with pass 1, and at those of pass 2,
+    // while a late one may still read)
+    if (pass == 1) {
+      sr = warp_sum(sr);
+      if (lane == 0) s_part[warp] = sr;
+      __syncthreads();
+      if (tid == 0) {
+        float s = 0.f;
 #pragma unroll
-      for (int w = 0; w < kW; ++w) s += s_part[w];
-      put(r2_words + cta, s, tag);
+        for (int w = 0; w < kW; ++w) s += s_part[w];
+        put(words.ext_r2 + cta, s, tag);
+      }
+    } else {
+      double* s_part2 = reinterpret_cast<double*>(s_part);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sr2 += __shfl_xor_sync(0xffffffffu, sr2, o);
+      if (lane == 0) s_part2[warp] = sr2;
+      __syncthreads();
+      if (tid == 0) {
+        double s = 0.0;
+        for (int w = 0; w < kW; ++w) s += s_part2[w];
+        put128(words.ext_r2d + cta, (uint32_t)__double2loint(s), (uint32_t)__double2hiint(s), 0u, tag);
+      }
     }
-    if (warp < 3 - pass) {
+    if (pass == 2) {
+      if (warp == 0) {
+        double s = 0.0;
+        const int mine = G > lane ? (G - lane + 31) / 32 : 0;
+        ok = gather128([&](int u) { return words.ext_r2d + lane + 32 * u; }, mine, tag, g.spin_limit,
+                       [&](int, const Word128& w) { s += __hiloint2double((int)w.b, (int)w.a); });
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) s_norm[0] = s;
+      }
+    } else if (warp < 2) {
       // (First polls that arrive ahead of the words hold them up: all CTAs read the same few lines.  Asking
       // at once, this exchange took 1.7 or 2.7 to 4 us, by where the words lie in memory.)
       for (const long long t0 = clock64(); clock64() - t0 < kHoldOff;) {}
       double s = 0.0;
-      ok = warp ? warp_gather_sum(words.ext_x2, 1, n_slabs, tag, g.spin_limit, s) : warp_gather_sum(r2_words, 1, G, tag, g.spin_limit, s);
+      ok = warp ? warp_gather_sum(words.ext_x2, 1, n_slabs, tag, g.spin_limit, s) : warp_gather_sum(words.ext_r2, 1, G, tag, g.spin_limit, s);
       if (lane == 0) s_norm[warp] = s;
     }
     if (give_up(ok)) return;

@@ -739,7 +739,7 @@ cudaError_t launch_fused_p(const GroupParams& g, const IoRef& io, int n, int sla
 }  // namespace
 
 size_t fused_words_bytes(int d, int k, int max_tokens) {
-  return 8 * ((size_t)kFusedMaxGrid * (max_tokens * (kCols + 2) + 3) + (size_t)max_tokens * (k + 2) + d) +
+  return 8 * ((size_t)kFusedMaxGrid * (max_tokens * (kCols + 2) + 4) + (size_t)max_tokens * (k + 2) + d) +
          (size_t)max_tokens * term_bytes(d);
 }
 

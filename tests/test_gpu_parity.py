@@ -1356,6 +1356,27 @@ def test_extend_basis_passes_have_norm_words_of_their_own():
     assert words(2) - before[1] == slabs * k_cap + ctas
 
 
+@pytest.mark.parametrize("p_dtype", ["bf16", "f32"])
+def test_extend_basis_column_has_unit_length_at_any_scale_of_the_token(p_dtype):
+    """x and 2^-70 x (entries of 1e-21, whose squares are below the normal fp32 range) have the same
+    residual direction: scaling by a power of two commutes with every rounding, so the appended
+    columns are the same bits."""
+    g = G()
+    d, k_act, k_cap = 2064, 30, 64
+    x = torch.randn(d, generator=torch.Generator().manual_seed(781))
+    cols = []
+    for scale in (1.0, 2.0 ** -70):
+        q, P, Ws = _extend_case(d, k_act, k_cap, (64,), 780, p_dtype)
+        Pd = P.cuda()
+        lay = g.Layer([W.cuda() for W in Ws], Pd, 0.05, max_tokens=1)
+        appended, _ = lay.extend_basis((x * scale).cuda(), 0.05, torch.tensor([k_act], dtype=torch.int32, device="cuda"))
+        torch.cuda.synchronize()
+        assert lay.status() == 0 and appended.item() == 1
+        cols.append(Pd[:, k_act].clone())
+    assert abs(cols[0].double().norm().item() - 1.0) < 2.0 ** -8
+    assert torch.equal(*cols)
+
+
 def test_extend_basis_sequence_then_forward_sees_the_new_columns():
     """A stream of tokens, some in the span, some not: the GPU basis and the oracle's evolve
     independently from the same start and stay together (same decisions, same columns to
