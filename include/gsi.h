@@ -390,7 +390,8 @@ gsi_status_t gsi_stack_launches_per_step(gsi_stack_t s, int* n_out);
  * group order) are copied with a single transfer per direction.  From 3 MB of x and y on,
  * the step runs in segments of groups: the inputs of the next and the outputs of the
  * previous segment travel on streams of the stack's own while one segment runs (`stream`
- * waits for them; copies of neighbours are merged within a segment).
+ * waits for them; copies of neighbours are merged within a segment).  Host buffers of x and y may
+ * overlap: every x is read as it was at the call.
  */
 gsi_status_t gsi_stack_step_host(gsi_stack_t s, const float* const* x_host_array,
                                  float* const* y_host_array, unsigned char* gate_host,

@@ -1056,6 +1056,20 @@ gsi_status_t gsi_stack_step_host(gsi_stack_t s, const float* const* x_host, floa
     if (st != GSI_OK) return st;
     if (!ok(cudaEventRecord(s->ev_run[i], stream))) return GSI_ERR_CUDA;
   }
+  // A host buffer that is y of one segment and x of a later one must be read before it is written: no
+  // copy out starts before the last copy in then.  (Looked at here: the segments are on their way.)
+  auto overlap = [&]() -> bool {
+    for (int i = 0; i + 1 < n; ++i)
+      for (int a = unit_group(s, s->segment[i]); a < unit_group(s, s->segment[i + 1]); ++a) {
+        const uintptr_t y0 = (uintptr_t)y_host[a], y1 = y0 + (size_t)s->B * s->groups[a]->lay.O * 4;
+        for (int b = unit_group(s, s->segment[i + 1]); b < G; ++b) {
+          const uintptr_t x0 = (uintptr_t)x_host[b], x1 = x0 + (size_t)s->B * s->groups[b]->desc.d * 4;
+          if (x0 < y1 && y0 < x1) return true;
+        }
+      }
+    return false;
+  };
+  if (overlap() && !ok(cudaStreamWaitEvent(s->copy_out, s->ev_in[n - 1], 0))) return GSI_ERR_CUDA;
   for (int i = 0; i < n; ++i)   // (after all work is enqueued: a copy to pageable memory holds the host)
     if (!ok(cudaStreamWaitEvent(s->copy_out, s->ev_run[i], 0)) ||
         !copy_runs(false, unit_group(s, s->segment[i]), unit_group(s, s->segment[i + 1]), s->copy_out))

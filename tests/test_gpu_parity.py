@@ -413,6 +413,30 @@ def test_step_host_in_segments_matches_the_device_step(n_tokens, pinned):
             assert torch.equal(y.cpu().reshape(-1), yh)
 
 
+def test_step_host_reads_every_input_before_an_output_lands_on_it():
+    """The host buffer of the first group's y is also where the last group's x comes from: wide
+    inputs, so that the first segment is done long before the last one's inputs are in."""
+    g = G()
+    n_groups, d, k, o, B = 12, 8192, 128, 128, 64
+    q = S.gen_basis(d, k, 8300)
+    P = S.store_basis(q).cuda()
+    layers = [g.Layer([S.gen_weight(o, d, 8310 + i).cuda()], P, 0.05, max_tokens=B) for i in range(n_groups)]
+    stack = g.Stack(layers)
+    gen = torch.Generator().manual_seed(8301)
+    xs = [torch.randn((B, d), generator=gen).pin_memory() for _ in range(n_groups)]
+    stack.bind([torch.zeros((B, d), device="cuda") for _ in range(n_groups)], n_steps=1)
+    ys = [torch.empty(B * o).pin_memory() for _ in range(n_groups)]
+    gate = torch.empty((n_groups, B), dtype=torch.uint8).pin_memory()
+    stack.step_host(xs, ys, gate)
+    want = [y.clone() for y in ys]
+    for _ in range(3):
+        shared = xs[-1].clone().pin_memory()
+        stack.step_host(xs[:-1] + [shared], [shared.view(-1)[:B * o]] + ys[1:], gate)
+        assert stack.status() == 0 and bool(gate.all())
+        for y, w in zip([shared.view(-1)[:B * o]] + ys[1:], want):
+            assert torch.equal(y, w)
+
+
 def test_gptj_layer_full_size_sampled_rows():
     """One GPT-J-shaped layer at full size (k=256, eps=0.05), batch 1, in the
     launch configuration the benchmark uses; the oracle evaluates a sample of
