@@ -417,7 +417,7 @@ def test_step_host_reads_every_input_before_an_output_lands_on_it():
     """The host buffer of the first group's y is also where the last group's x comes from: wide
     inputs, so that the first segment is done long before the last one's inputs are in."""
     g = G()
-    n_groups, d, k, o, B = 12, 8192, 128, 128, 64
+    n_groups, d, k, o, B = 24, 16384, 128, 128, 64
     q = S.gen_basis(d, k, 8300)
     P = S.store_basis(q).cuda()
     layers = [g.Layer([S.gen_weight(o, d, 8310 + i).cuda()], P, 0.05, max_tokens=B) for i in range(n_groups)]
