@@ -895,7 +895,7 @@ static gsi_status_t stack_enqueue_range(gsi_stack_t s, int g0, int g1, bool firs
     io.log_step_stride = (long long)G * s->B;
     h->last_stream = stream;   // the joins below put all of the step's work in the caller's stream order
     return launch_generic_forward(h->gp, h->has_tm ? &h->tm : nullptr, io, s->B, st, nullptr,
-                                  chains ? &lane : nullptr, s->mode == 1) == cudaSuccess;
+                                  chains ? &lane : nullptr, true, s->mode == 1) == cudaSuccess;
   };
   for (int i = g0; i < g1; ++i) {
     if (chains && s->alternate) {

@@ -228,7 +228,7 @@ struct ResidualLane {
 
 cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, const IoRef& io,
                                    int n_tokens, cudaStream_t stream, int* n_launches,
-                                   ResidualLane* lane = nullptr, bool per_stage = false);
+                                   ResidualLane* lane = nullptr, bool in_stack = false, bool per_stage = false);
 cudaError_t launch_advance_step(int* step, cudaStream_t stream);
 // A whole call in one cooperative launch, any supported shape.  leave_from > 0: from that many
 // gated tokens on their W r is left to a contraction that follows (g.r, g.fired, *g.n_fired).

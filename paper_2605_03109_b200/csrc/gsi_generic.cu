@@ -396,8 +396,7 @@ int leave_to_contraction(const GroupParams& g, bool tc, int n_tokens) {
 
 cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, const IoRef& io,
                                    int n_tokens, cudaStream_t st, int* n_launches, ResidualLane* lane,
-                                   bool per_stage) {
-  const bool in_stack = lane != nullptr;
+                                   bool in_stack, bool per_stage) {
   int dummy = 0;
   if (!n_launches) n_launches = &dummy;
   int grid = (g.O + kWarps - 1) / kWarps;

@@ -986,6 +986,35 @@ def test_batched_residual_in_splits_and_clusters(d, k, d_out, n):
         compare_group(xs[s], P, Ws, 0.05, stack.ys[0].cpu().reshape(n, -1).numpy(), gate)
 
 
+@pytest.mark.parametrize("d,k,d_out,n,static,mode", [
+    (1024, 128, (512,), 8, True, 0), (1024, 128, (512,), 8, False, 0),   # tensor-core front end
+    (1024, 128, (512,), 8, True, 1), (1024, 72, (520,), 5, True, 1),     # ... and per-stage kernels
+    (1024, 72, (520,), 5, False, 0), (1024, 72, (520,), 5, True, 0),     # one launch
+    (4096, 64, (8192,), 40, False, 0),                                   # ... and a contraction behind it
+])
+def test_launches_per_step_counts_what_a_step_enqueues(d, k, d_out, n, static, mode):
+    """gsi_stack_launches_per_step against the kernel nodes of a captured step."""
+    from cuda.bindings import runtime as rt
+    g = G()
+    layers, xs = [], []
+    for i in range(2):
+        x, P, Ws = make_small(d, k, d_out, n, seed=9300 + i, outlier_every=2)
+        layers.append(g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n,
+                              flags=g.GSI_FLAG_STATIC_PROJECTION if static else 0))
+        xs.append(x.cuda())
+    stack = g.Stack(layers, mode=mode)
+    stack.bind(xs, n_steps=1)
+    stack.step()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        stack.step()
+    err, nodes, count = rt.cudaGraphGetNodes(rt.cudaGraph_t(graph.raw_cuda_graph()), 256)
+    assert int(err) == 0 and count < 256
+    kinds = [rt.cudaGraphNodeGetType(node)[1] for node in nodes[:count]]
+    assert kinds.count(rt.cudaGraphNodeType.cudaGraphNodeTypeKernel) == stack.launches_per_step()
+
+
 def test_persistent_nonfinite_token():
     g = G()
     x, P, Ws = make_small(256, 64, (64,), 3, seed=41)
