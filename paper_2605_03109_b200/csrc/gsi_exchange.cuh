@@ -160,8 +160,22 @@ __device__ __forceinline__ Area area_of(const GroupParams& g) {
 
 }  // namespace exchange
 
-// SMs of the current device, as CTAs of a cooperative launch; 0 on error.
+// CTAs of a cooperative launch: the SMs of the current context (a green context has fewer than its
+// device); 0 on error.
 int fused_grid();
+// launch(grid) with that many, or with fewer where the stream's SMs are fewer still: the kernels run on
+// any grid, and what the launches that waited for nobody took is taken.
+template <typename F>
+cudaError_t launch_resident(F&& launch) {
+  const int most = fused_grid();
+  if (!most) return cudaErrorInvalidDevice;
+  cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
+  for (int grid = most; grid >= 1 && e == cudaErrorCooperativeLaunchTooLarge; grid /= 2) {
+    e = launch(grid);
+    if (e == cudaErrorCooperativeLaunchTooLarge) (void)cudaGetLastError();
+  }
+  return e;
+}
 // Slabs of basis rows for the projection: slabs x column blocks over the grid, at least 32 rows each.
 int fused_slabs(int d, int k, int grid);
 

@@ -94,8 +94,8 @@ __global__ void __launch_bounds__(kT, 1) k_extend(GroupParams g, ExtendArgs a, i
     const unsigned tag = tag1 + (unsigned)(pass - 1);
     bool ok = true;
     // partial c of a slab of rows x 32 columns
-    if (cta < n_slabs * n_cb) {
-      const int slab = cta / n_cb, cb = cta % n_cb;
+    for (int part = cta; part < n_slabs * n_cb; part += G) {   // (a small grid may have fewer CTAs than column blocks)
+      const int slab = part / n_cb, cb = part % n_cb;
       const int r0 = (int)((long long)d * slab / n_slabs), r1 = (int)((long long)d * (slab + 1) / n_slabs);
       const int sub = lane >> 2, c = cb * kCols + (lane & 3) * 8;
       float acc[8], sx = 0.f;
@@ -340,12 +340,12 @@ cudaError_t launch_t(GroupParams g, ExtendArgs a, int slabs, int grid, cudaStrea
 }  // namespace
 
 cudaError_t launch_extend_basis(const GroupParams& g, const ExtendArgs& a, cudaStream_t st) {
-  const int grid = fused_grid();
-  if (!grid) return cudaErrorInvalidDevice;
-  const int slabs = fused_slabs(g.d, g.k, grid);
-  return g.k <= 256   ? launch_t<1>(g, a, slabs, grid, st)
-         : g.k <= 512 ? launch_t<2>(g, a, slabs, grid, st)
-                      : launch_t<4>(g, a, slabs, grid, st);
+  return launch_resident([&](int grid) -> cudaError_t {
+    const int slabs = fused_slabs(g.d, g.k, grid);
+    return g.k <= 256   ? launch_t<1>(g, a, slabs, grid, st)
+           : g.k <= 512 ? launch_t<2>(g, a, slabs, grid, st)
+                        : launch_t<4>(g, a, slabs, grid, st);
+  });
 }
 
 }  // namespace gsi

@@ -25,6 +25,8 @@
 // in an order that depends on the shape alone: results are reproducible, and a token's are the
 // same in a call of any size.
 // Every wait is bounded; a wait that gives up sets GSI_ERR_TIMEOUT and the CTA returns.
+#include <cuda.h>
+
 #include <type_traits>
 
 #include "gsi_exchange.cuh"
@@ -319,8 +321,10 @@ __device__ __forceinline__ bool forward_fused(const GroupParams& g, const IoRef&
 
   // ---- A: D[column of P][token] += P^T x over the slab; 256 rows staged at a time, 16 per warp
   const int n_cb = (k + kCols - 1) / kCols;
-  if (cta < n_slabs * n_cb) {
-    const int slab = cta / n_cb, cb = cta % n_cb;
+  // (a small grid may have fewer CTAs than column blocks; the direct build is not launched there: the loop costs it 0.7 us)
+  int part = cta;
+  if (part < n_slabs * n_cb) do {
+    const int slab = part / n_cb, cb = part % n_cb;
     const int r0 = (int)((long long)d * slab / n_slabs), r1 = (int)((long long)d * (slab + 1) / n_slabs);
     for (int tb = 0; tb < n; tb += kTok) {
       float acc[2][NB][4];
@@ -416,7 +420,8 @@ __device__ __forceinline__ bool forward_fused(const GroupParams& g, const IoRef&
       }
       __syncthreads();
     }
-  }
+    part += G;
+  } while (!kDirect && part < n_slabs * n_cb);
 
   // ---- x1.  Coefficient i (= token * k + column) summed over the slabs by Q adjacent lanes: each
   // adds kSegs / Q runs of slabs in order, the runs are added by a tree: the same sums for every Q
@@ -743,16 +748,43 @@ size_t fused_words_bytes(int d, int k, int max_tokens) {
          (size_t)max_tokens * term_bytes(d);
 }
 
+namespace {
+template <typename F>
+F driver_function(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess)
+    return nullptr;
+  return reinterpret_cast<F>(p);
+}
+}  // namespace
+
+// (The number of SMs is asked of a context once per thread: 0.3 us.  A context's id is never used again.)
 int fused_grid() {
-  static int sms_of[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  int grid = dev < 64 ? sms_of[dev] : 0;
-  if (!grid) {
-    if (cudaDeviceGetAttribute(&grid, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (dev < 64) sms_of[dev] = grid;
+  static const auto id_of = driver_function<CUresult (*)(CUcontext, unsigned long long*)>("cuCtxGetId");
+  static const auto resource_of =
+      driver_function<CUresult (*)(CUcontext, CUdevResource*, CUdevResourceType)>("cuCtxGetDevResource");
+  static const auto current = driver_function<CUresult (*)(CUcontext*)>("cuCtxGetCurrent");
+  static thread_local unsigned long long last_id = 0;
+  static thread_local int last_grid = 0;
+  int dev = 0, grid = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;   // (makes a context current)
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+  const bool known = id_of && resource_of && current && current(&ctx) == CUDA_SUCCESS && ctx &&
+                     id_of(ctx, &id) == CUDA_SUCCESS;
+  if (known && last_grid && id == last_id) return last_grid;
+  CUdevResource sm{};
+  if (known && resource_of(ctx, &sm, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && sm.sm.smCount > 0)
+    grid = (int)sm.sm.smCount;
+  else if (cudaDeviceGetAttribute(&grid, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  if (grid > kFusedMaxGrid) grid = kFusedMaxGrid;
+  if (known) {
+    last_id = id;
+    last_grid = grid;
   }
-  return grid > kFusedMaxGrid ? kFusedMaxGrid : grid;
+  return grid;
 }
 
 int fused_slabs(int d, int k, int grid) {
@@ -763,13 +795,14 @@ int fused_slabs(int d, int k, int grid) {
 
 cudaError_t launch_forward_fused(const GroupParams& g, const IoRef& io, int n_tokens, int leave_from,
                                  cudaStream_t st) {
-  const int grid = fused_grid();
-  if (!grid) return cudaErrorInvalidDevice;
-  const int slabs = fused_slabs(g.d, g.k, grid);
-  return n_tokens <= kDirectTokens ? launch_fused_p<1, true>(g, io, n_tokens, slabs, leave_from, grid, st)
-         : n_tokens <= 8           ? launch_fused_p<1, false>(g, io, n_tokens, slabs, leave_from, grid, st)
-         : n_tokens <= 16          ? launch_fused_p<2, false>(g, io, n_tokens, slabs, leave_from, grid, st)
-                                   : launch_fused_p<4, false>(g, io, n_tokens, slabs, leave_from, grid, st);
+  return launch_resident([&](int grid) -> cudaError_t {
+    const int slabs = fused_slabs(g.d, g.k, grid);
+    const bool direct = n_tokens <= kDirectTokens && grid * kCols >= g.k;
+    return direct            ? launch_fused_p<1, true>(g, io, n_tokens, slabs, leave_from, grid, st)
+           : n_tokens <= 8           ? launch_fused_p<1, false>(g, io, n_tokens, slabs, leave_from, grid, st)
+           : n_tokens <= 16          ? launch_fused_p<2, false>(g, io, n_tokens, slabs, leave_from, grid, st)
+                                     : launch_fused_p<4, false>(g, io, n_tokens, slabs, leave_from, grid, st);
+  });
 }
 
 }  // namespace gsi

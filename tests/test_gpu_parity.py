@@ -164,6 +164,45 @@ def test_one_launch_wait_runs_out_and_the_next_calls_are_right(n):
             assert all(torch.equal(a, b) for a, b in zip(ref, run(lays[1])))
 
 
+@pytest.mark.parametrize("d,k,d_out,n", [
+    (4096, 256, (1024, 512), 5), (2056, 1000, (264,), 2),   # more column blocks of c than CTAs
+    (16384, 40, (72,), 9),                                  # 64 units of basis rows per CTA
+])
+def test_one_launch_calls_in_a_context_with_few_sms(d, k, d_out, n):
+    """A green context of 16 SMs: the cooperative launches take the grid that it holds, captured or not."""
+    g = G()
+    from torch.cuda.green_contexts import GreenContext
+    x, P, Ws = make_small(d, k, d_out, n, seed=190 + n, outlier_every=2)
+    Pd, xd, Wd = P.cuda(), x.cuda(), [W.cuda() for W in Ws]
+    lay = g.Layer(Wd, Pd, 0.05, max_tokens=n)
+    img = torch.cat([g.gsi_build_image(W, Pd) for W in Wd])
+    inside = (P.double() @ torch.randn(k, dtype=torch.float64, generator=torch.Generator().manual_seed(5))).float().cuda()
+    ka = torch.tensor([k - 1], dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    outs = []
+    ctx = GreenContext.create(num_sms=16)
+    ctx.set_context()
+    try:
+        outs.append(lay.forward(xd))
+        if n <= 4 and k <= 512:
+            outs.append(g.gsi_forward_static(Wd, Pd, img, 0.05, xd))
+        appended, rho = lay.extend_basis(inside, 0.5, ka)
+        torch.cuda.synchronize()
+        y, gate, rho_c = (t.clone() for t in outs[0])
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            lay.forward(xd, y=y.zero_(), gate=gate, rho=rho_c)
+        graph.replay()
+        torch.cuda.synchronize()
+    finally:
+        ctx.pop_context()
+    outs += [(y, gate, rho_c), lay.forward(xd)]
+    torch.cuda.synchronize()
+    assert lay.status() == 0 and appended.item() == 0 and rho.item() < 0.05 and ka.item() == k - 1
+    for y, gate, rho in outs:
+        compare_group(x, P, Ws, 0.05, y.cpu().numpy(), gate.cpu().numpy(), rho.cpu().numpy())
+
+
 def test_config1_literal_batch1_all_tokens():
     st = S.config1()
     m = S.materialize_group(st, 0, 0, st.steps)
