@@ -42,6 +42,7 @@ constexpr int kTileRows = 16 * kW;     // rows of a basis slab (and of W) per pa
 constexpr int kPitch = 80;             // bytes between the staged 64-byte pieces: conflict-free ldmatrix
 constexpr int kDirectTokens = 2;       // calls of so few tokens gather the slabs' partials themselves
 constexpr int kDecideTokens = 4;       // calls of so few tokens decide the gates on every CTA
+constexpr int kGateHoldOff = 600;      // cycles before the first look at the decisions taken elsewhere
 constexpr int kSegs = 8;               // the slabs' partials are added in eight runs, these by a tree
 constexpr int kSlots = 16;             // 16-row units of the basis whose norms wait in shared memory
 // dynamic shared memory: operand terms (phase A: the slab), then partial sums
@@ -655,6 +656,8 @@ __device__ __forceinline__ bool forward_fused(const GroupParams& g, const IoRef&
     }
     __syncwarp();
     if (warp < 2 && warp * 32 + lane < n) {
+      // (a first look ahead of the words would hold up their writers: 21 tokens 26.6 -> 26.4 us)
+      for (const long long t0 = clock64(); clock64() - t0 < kGateHoldOff;) {}
       Word128 w = get128(words.gate + warp * 32 + lane);
       for (unsigned it = 1; w.tag != tag && it < g.spin_limit; ++it) w = get128(words.gate + warp * 32 + lane);
       ok = ok && w.tag == tag;
