@@ -20,11 +20,11 @@ namespace {
 
 using namespace umma;
 
-constexpr int kStages3 = 2;   // (blocks of 82 KB find a slot beside the W stream sooner: four stages left a step 2-7 % slower)
+// stages of the projection: in a stack, blocks of 82 KB, which find a slot beside the W streams sooner
+// (four stages left a step 2-7 % slower); in a call by itself there is nothing beside them
+constexpr int kStages3 = 2, kStages3Alone = 4;
 constexpr int kMaxN3 = 192;          // 3 terms x 64 tokens
 constexpr int kTmemCols3 = 256;      // power of two >= kMaxN3
-using Cfg3 = Cfg<kStages3, kMaxN3>;
-constexpr int kSmem3 = Cfg3::kSmem;
 // residual / image: K = k is short (four 64-wide blocks at k = 256).  Up to 32 tokens the B
 // operand is small enough for four stages with two blocks per SM, so every weight box of a
 // tile is requested before the wait on the previous kernel; beyond, two stages.
@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(256) k_split3_x(GroupParams g, IoRef io, int n
 }
 
 // c partials: cpart3[split][t][128*tile + lane row] over this split's share of d.
+template <bool kInStack>
 __global__ void __launch_bounds__(kThreads, 1)
 k_proj_tc(GroupParams g, const __grid_constant__ TmaMaps tm, int n_tokens) {
   extern __shared__ unsigned char smem_raw[];
@@ -106,8 +107,8 @@ k_proj_tc(GroupParams g, const __grid_constant__ TmaMaps tm, int n_tokens) {
   const int nkb = g.d / kTK;
   const int kb0 = (int)((long long)nkb * split / splits), kb1 = (int)((long long)nkb * (split + 1) / splits);
   uint32_t tmem;
-  const bool ok = tile_mma<kStages3, kMaxN3, kTmemCols3>(smem_raw, &tm.pt, tile * kTM, &tm.xb, 0,
-                                                         rows3(n_tokens), kb0, kb1 - kb0, &tmem);
+  const bool ok = tile_mma<kInStack ? kStages3 : kStages3Alone, kMaxN3, kTmemCols3, kInStack>(
+      smem_raw, &tm.pt, tile * kTM, &tm.xb, 0, rows3(n_tokens), kb0, kb1 - kb0, &tmem);
   if (!ok) {
     if (threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
   } else {
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(256) k_reduce_split3_c(GroupParams g, int n_to
 //                         r = x - P c -> bf16 rows of rb, the partial norms of the tile,
 //                         and in the block that finishes last the gate
 //   blocks [n_resid, ..)  tile of W_P, all tokens: y = W_P c
-template <int kStagesT, int kMaxRows, int kTmemColsT>
+template <int kStagesT, int kMaxRows, int kTmemColsT, bool kInStack>
 __global__ void __launch_bounds__(kThreads, 2)
 k_resid_image_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, int n_tokens, int rs) {
   extern __shared__ unsigned char smem_raw[];
@@ -198,7 +199,7 @@ k_resid_image_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, in
   bool ok = true;
   if (q_lo < q_hi) {   // block-uniform
     const int n_rows = min(48 * (q_hi - q_lo), rows3(n_tokens) - 48 * q_lo);
-    ok = tile_mma<kStagesT, kMaxRows, kTmemColsT>(smem_raw, image ? &tm.wp : &tm.p, tile * kTM, &tm.cb,
+    ok = tile_mma<kStagesT, kMaxRows, kTmemColsT, kInStack>(smem_raw, image ? &tm.wp : &tm.p, tile * kTM, &tm.cb,
                                                 48 * q_lo, n_rows, 0, g.k / kTK, &tmem);
     if (!ok && threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
     const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
@@ -283,14 +284,17 @@ cudaError_t launch_split3_x(const GroupParams& g, const IoRef& io, int n_tokens,
   return cudaGetLastError();
 }
 
-cudaError_t launch_front_tc(const GroupParams& g, const TmaMaps& tm, const IoRef& io, int n_tokens,
-                            cudaStream_t st, int* n_launches) {
+template <bool kInStack>
+static cudaError_t launch_front(const GroupParams& g, const TmaMaps& tm, const IoRef& io, int n_tokens,
+                                cudaStream_t st) {
+  constexpr int kSmem3 = Cfg<kInStack ? kStages3 : kStages3Alone, kMaxN3>::kSmem;
+  auto proj = k_proj_tc<kInStack>;
+  auto wide = k_resid_image_tc<kStagesRI, kMaxN3, kTmemCols3, kInStack>;
+  auto narrow = k_resid_image_tc<kStagesRIs, kMaxN3s, kTmemCols3s, kInStack>;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_proj_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem3)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(k_resid_image_tc<kStagesRI, kMaxN3, kTmemCols3>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRI)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(k_resid_image_tc<kStagesRIs, kMaxN3s, kTmemCols3s>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRIs)) != cudaSuccess)
+  if ((e = cudaFuncSetAttribute(proj, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem3)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRI)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRIs)) != cudaSuccess)
     return e;
   const bool small = term_rows(n_tokens) <= kMaxN3s;
   const int slots = (front_rows(n_tokens) + 2) / 3;   // token slots covering every operand row
@@ -301,18 +305,19 @@ cudaError_t launch_front_tc(const GroupParams& g, const TmaMaps& tm, const IoRef
   // k_split3_x was launched
   if ((e = launch_pdl(k_split3_x, dim3((g.d / 8 + 255) / 256, slots), dim3(256), 0, st, g, io, n_tokens)) !=
           cudaSuccess ||
-      (e = launch_pdl(k_proj_tc, dim3((g.k / kTM) * g.proj_splits), dim3(kThreads), kSmem3, st, g, tm,
-                      n_tokens)) != cudaSuccess ||
+      (e = launch_pdl(proj, dim3((g.k / kTM) * g.proj_splits), dim3(kThreads), kSmem3, st, g, tm, n_tokens)) !=
+          cudaSuccess ||
       (e = launch_pdl(k_reduce_split3_c, dim3(slots), dim3(256), 0, st, g, n_tokens)) != cudaSuccess ||
-      (e = small ? launch_pdl(k_resid_image_tc<kStagesRIs, kMaxN3s, kTmemCols3s>,
-                              dim3((g.d / kTM) * rs + g.O / kTM), dim3(kThreads), kSmemRIs, st, g, tm, io,
-                              n_tokens, rs)
-                 : launch_pdl(k_resid_image_tc<kStagesRI, kMaxN3, kTmemCols3>,
-                              dim3((g.d / kTM) * rs + g.O / kTM), dim3(kThreads), kSmemRI, st, g, tm, io,
-                              n_tokens, rs)) != cudaSuccess)
+      (e = launch_pdl(small ? narrow : wide, dim3((g.d / kTM) * rs + g.O / kTM), dim3(kThreads),
+                      small ? kSmemRIs : kSmemRI, st, g, tm, io, n_tokens, rs)) != cudaSuccess)
     return e;
-  if (n_launches) *n_launches += 4;
   return cudaGetLastError();
+}
+
+cudaError_t launch_front_tc(const GroupParams& g, const TmaMaps& tm, const IoRef& io, int n_tokens, bool in_stack,
+                            cudaStream_t st, int* n_launches) {
+  if (n_launches) *n_launches += 4;
+  return in_stack ? launch_front<true>(g, tm, io, n_tokens, st) : launch_front<false>(g, tm, io, n_tokens, st);
 }
 
 }  // namespace gsi

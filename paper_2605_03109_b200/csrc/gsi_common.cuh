@@ -254,14 +254,14 @@ cudaError_t launch_extend_basis(const GroupParams& g, const ExtendArgs& a, cudaS
 // mapped: rb holds every token's residual (row = token) and the fired list selects the
 // operand rows; otherwise a pack kernel first compacts the fired tokens of g.r into rb.
 cudaError_t launch_residual_gemm_tc(const GroupParams& g, const TmaMaps& tm, const IoRef& io,
-                                    int min_fired, bool mapped, int n_tokens,
+                                    int min_fired, bool mapped, bool in_stack, int n_tokens,
                                     cudaStream_t stream, int* n_launches);
 int tc_splits(int O, int d);
 int tc_launches(int O, int d);   // kernels of a contraction
 bool tc_eligible(const GroupParams& g);
 // Batched front end on the tensor cores: c, r, gate and y = W_P c for n_tokens tokens.
 cudaError_t launch_front_tc(const GroupParams& g, const TmaMaps& tm, const IoRef& io,
-                            int n_tokens, cudaStream_t stream, int* n_launches);
+                            int n_tokens, bool in_stack, cudaStream_t stream, int* n_launches);
 // Encodes the layer's tensor maps (front: also those of the batched front end).
 // False when the driver's encoder is unavailable or rejects a shape.
 bool build_tma_maps(const GroupParams& g, bool front, int max_tokens, TmaMaps* out);

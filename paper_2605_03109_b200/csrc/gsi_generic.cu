@@ -414,10 +414,10 @@ cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, cons
     const int leave = leave_to_contraction(g, tm != nullptr, n_tokens);
     if ((e = launch_forward_fused(g, io, n_tokens, leave, st)) != cudaSuccess) return e;
     *n_launches += 1;
-    return leave ? launch_residual_gemm_tc(g, *tm, io, leave, false, n_tokens, st, n_launches) : cudaSuccess;
+    return leave ? launch_residual_gemm_tc(g, *tm, io, leave, false, in_stack, n_tokens, st, n_launches) : cudaSuccess;
   }
   if (front) {
-    e = launch_front_tc(g, *tm, io, n_tokens, st, n_launches);
+    e = launch_front_tc(g, *tm, io, n_tokens, in_stack, st, n_launches);
   } else {
     e = dispatch_vpl(g, io, n_tokens, st, n_launches);
   }
@@ -433,13 +433,13 @@ cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, cons
         sr = lane->stream;
         lane->used = true;
       }
-      e = launch_residual_gemm_tc(g, *tm, io, 1, true, n_tokens, sr, n_launches);
+      e = launch_residual_gemm_tc(g, *tm, io, 1, true, in_stack, n_tokens, sr, n_launches);
       if (e != cudaSuccess) return e;
     } else {
       k_stream_gemv<false><<<grid, kThreads, 0, st>>>(g, io, n_tokens);
       *n_launches += 1;
       if (tm && g.tc_min_fired > 0) {
-        e = launch_residual_gemm_tc(g, *tm, io, g.tc_min_fired, false, n_tokens, st, n_launches);
+        e = launch_residual_gemm_tc(g, *tm, io, g.tc_min_fired, false, in_stack, n_tokens, st, n_launches);
         if (e != cudaSuccess) return e;
       }
     }

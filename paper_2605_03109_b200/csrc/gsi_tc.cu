@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256) k_pack_fired_bf16(GroupParams g, int min_
 //              of fired tokens are written out.
 // kCluster: the splits of a tile are a cluster; their sums meet in distributed shared memory, added
 // in split order by the ranks (a share of the columns each), and no partial sum goes to memory.
-template <bool kCluster>
+template <bool kCluster, bool kInStack>
 __global__ void __launch_bounds__(kThreadsTc, 2)
 k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, int min_fired, int splits,
                    int mapped, int n_tokens) {
@@ -82,8 +82,8 @@ k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, 
 
   uint32_t tmem;
   bool skipped = false;
-  const bool ok = tile_mma<kStages, kMaxN, kTmemCols>(smem_raw, &tm.w[j], row0 - g.off[j], &tm.rb, 0, N,
-                                                      kb0, nloc, &tmem, speculate ? g.n_fired : nullptr,
+  const bool ok = tile_mma<kStages, kMaxN, kTmemCols, kInStack>(smem_raw, &tm.w[j], row0 - g.off[j], &tm.rb, 0, N,
+                                                                kb0, nloc, &tmem, speculate ? g.n_fired : nullptr,
                                                       min_fired, &skipped);
   if (!skipped) {   // past the wait on the kernel before: the fired list is there
     if (threadIdx.x == 0) {
@@ -215,7 +215,7 @@ k_dense_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, int
   const int kb0 = (int)((long long)nkb * split / splits), kb1 = (int)((long long)nkb * (split + 1) / splits);
   const int N = (n_tokens + 15) & ~15;
   uint32_t tmem;
-  const bool ok = tile_mma<kStages, kMaxN, kTmemCols>(smem_raw, &tm.w[j], row0 - g.off[j], &tm.rb, 0, N,
+  const bool ok = tile_mma<kStages, kMaxN, kTmemCols, false>(smem_raw, &tm.w[j], row0 - g.off[j], &tm.rb, 0, N,
                                                       kb0, kb1 - kb0, &tmem);
   if (!ok) {
     if (threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
@@ -311,11 +311,12 @@ bool tc_eligible(const GroupParams& g) {
 }
 
 cudaError_t launch_residual_gemm_tc(const GroupParams& g, const TmaMaps& tm, const IoRef& io,
-                                    int min_fired, bool mapped, int n_tokens, cudaStream_t st,
-                                    int* n_launches) {
+                                    int min_fired, bool mapped, bool in_stack, int n_tokens,
+                                    cudaStream_t st, int* n_launches) {
   const int splits = tc_splits(g.O, g.d);
   const bool cluster = tc_cluster(g.O, g.d);
-  auto kernel = cluster ? k_residual_gemm_tc<true> : k_residual_gemm_tc<false>;
+  auto kernel = in_stack ? (cluster ? k_residual_gemm_tc<true, true> : k_residual_gemm_tc<false, true>)
+                         : (cluster ? k_residual_gemm_tc<true, false> : k_residual_gemm_tc<false, false>);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
   if (e != cudaSuccess) return e;
   if (!mapped) k_pack_fired_bf16<<<dim3((g.d + 2047) / 2048, kMaxN), 256, 0, st>>>(g, min_fired);

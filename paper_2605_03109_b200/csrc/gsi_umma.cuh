@@ -2,7 +2,7 @@
 // kernels: D[128 x N] (fp32, tensor memory) = A[128 x K] * B[N x K]^T with bf16
 // operands that are both K-major in global memory.
 //
-//   producer warp     TMA (cp.async.bulk.tensor, 128-byte swizzle, no multicast) brings a
+//   producer          TMA (cp.async.bulk.tensor, 128-byte swizzle, no multicast) brings a
 //                     stage = A box 128 rows x 64 K-elements + N/16 B boxes of 16 rows into
 //                     shared memory and signals the stage's "full" mbarrier by byte count
 //   MMA thread        waits "full", issues tcgen05.mma (accumulator in tensor memory),
@@ -140,7 +140,11 @@ __device__ __forceinline__ void tmem_ld_wait() {
 // run_count / run_min: if run_count is given, it is read after the wait on the previous
 // kernel and the contraction runs only if *run_count >= run_min; otherwise the weight boxes
 // already requested are allowed to land, *skipped is set and the function returns true.
-template <int kStages, int kBRows, int kTmemCols>
+// kLanes: the producer warp issues a stage with one lane per box (an issue takes about a hundred
+// cycles, a stage has up to thirteen), else one thread does, the weight box first.  With the kernels
+// of other groups beside it the former is faster (28 GPT-J layers, 64 tokens: 3257 -> 3215 us), in a
+// call by itself the latter (dense step of 8 layers, 64 tokens: 855.7 -> 853.8).
+template <int kStages, int kBRows, int kTmemCols, bool kLanes>
 __device__ __forceinline__ bool tile_mma(unsigned char* smem_raw, const CUtensorMap* map_a,
                                          int a_row0, const CUtensorMap* map_b, int b_row0, int N,
                                          int kb0, int nloc, uint32_t* tmem_out,
@@ -203,22 +207,41 @@ __device__ __forceinline__ bool tile_mma(unsigned char* smem_raw, const CUtensor
   }
 
   if (warp == 0) {
-    // producer: one lane per B box (an issue takes about a hundred cycles, a stage has up to twelve)
-    for (int i = 0; i < nloc; ++i) {
-      const int stage = i % kStages;
-      const uint32_t sa = s32(smem + stage * C::kStageBytes), sb = sa + kABytes;
-      const int x = (kb0 + i) * kTK;
-      if (i >= kStages && !__all_sync(0xffffffffu, mbar_wait(&bar_empty[stage], ((i / kStages) - 1) & 1))) {
-        if (lane == 0) *s_fail = 1;
-        break;
+    if constexpr (kLanes) {
+      for (int i = 0; i < nloc; ++i) {
+        const int stage = i % kStages;
+        const uint32_t sa = s32(smem + stage * C::kStageBytes), sb = sa + kABytes;
+        const int x = (kb0 + i) * kTK;
+        if (i >= kStages && !__all_sync(0xffffffffu, mbar_wait(&bar_empty[stage], ((i / kStages) - 1) & 1))) {
+          if (lane == 0) *s_fail = 1;
+          break;
+        }
+        if (lane == 0)   // (the first kStages blocks of A are on their way)
+          mbar_expect_tx(&bar_full[stage], i >= kStages ? stage_bytes : stage_bytes - (uint32_t)kABytes);
+        __syncwarp();
+        if (lane < N / kBBox)
+          tma_load_2d(sb + lane * (kBBox * kTK * 2), map_b, x, b_row0 + lane * kBBox, &bar_full[stage]);
+        else if (lane == N / kBBox && i >= kStages)
+          tma_load_2d(sa, map_a, x, a_row0, &bar_full[stage]);
       }
-      if (lane == 0)   // (the first kStages blocks of A are on their way)
-        mbar_expect_tx(&bar_full[stage], i >= kStages ? stage_bytes : stage_bytes - (uint32_t)kABytes);
-      __syncwarp();
-      if (lane < N / kBBox)
-        tma_load_2d(sb + lane * (kBBox * kTK * 2), map_b, x, b_row0 + lane * kBBox, &bar_full[stage]);
-      else if (lane == N / kBBox && i >= kStages)
-        tma_load_2d(sa, map_a, x, a_row0, &bar_full[stage]);
+    } else if (lane == 0) {
+      for (int i = 0; i < nloc; ++i) {
+        const int stage = i % kStages;
+        const uint32_t sa = s32(smem + stage * C::kStageBytes), sb = sa + kABytes;
+        const int x = (kb0 + i) * kTK;
+        if (i >= kStages) {
+          if (!mbar_wait(&bar_empty[stage], ((i / kStages) - 1) & 1)) {
+            *s_fail = 1;
+            break;
+          }
+          mbar_expect_tx(&bar_full[stage], stage_bytes);
+          tma_load_2d(sa, map_a, x, a_row0, &bar_full[stage]);
+        } else {
+          mbar_expect_tx(&bar_full[stage], stage_bytes - (uint32_t)kABytes);   // A is on its way
+        }
+        for (int j = 0; j < N / kBBox; ++j)
+          tma_load_2d(sb + j * (kBBox * kTK * 2), map_b, x, b_row0 + j * kBBox, &bar_full[stage]);
+      }
     }
     __syncwarp();
   } else if (warp == 1) {
