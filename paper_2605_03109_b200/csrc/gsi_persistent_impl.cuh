@@ -1544,10 +1544,11 @@ __device__ void consumer(const PersistParams& p, unsigned char* smem, Misc* misc
         const bool close = own;   // a grid barrier ends this stream
         if (!own) gw = next_stream();
         else gw = !mask_pp && plan[t + 1].kind == 2 && not_gated(t + 2) && not_gated(t + 3) ? &desc(t + 1) : nullptr;
-        if (gw) q = w_geometry(gw);
+        if (gw && !close) q = w_geometry(gw);
         w_finish(ws, smem, close || !gw || (ws.half && q.half));
         tr.mark(13);
         if (close && tid == 0) red_relaxed_u32(bar, 1u);
+        if (gw && close) q = w_geometry(gw);   // (under the grid barrier: 28 GPT-J layers, dense, 1.921 -> 1.893 ms)
         if (gw) w_load_in(q, src_of(gw), in);
         if (!close) continue;
         const uint32_t dword = gw ? desc_load(t + 4) : 0u;
