@@ -16,15 +16,17 @@
 //
 // What bounds it: a few MB and a chain of latencies; tcgen05 with its tensor-memory round trip
 // per 16-row unit would add to that chain.  Time per call, one after the other on a stream, against
-// the five launches of the per-stage kernels before: one token at 768 x 64 -> 3072 27.3 -> 15.8 us,
-// at 4096 x 256 -> 28672 41.7 -> 16.0 us; 21 tokens at 3000 x 200 -> 1576 84 -> 46 us (on CUDA-core
-// FMAs this kernel took 112 us there); 16 tokens, fp32 basis, 768 x 128 -> 2304 48.5 -> 23.7 us.
+// the five launches of the per-stage kernels before: one token at 768 x 64 -> 3072 27.3 -> 12.3 us
+// (of which the kernel 10.3; the rest is the caller's side), at 4096 x 256 -> 28672, nothing gated,
+// 43.0 -> 15.8 us; 21 tokens at 3000 x 200 -> 1576 90 -> 27 us; 16 tokens, fp32 basis, 768 x 128 ->
+// 2304 50 -> 21 us.
 //
 // The exchanges are words that carry the call's tag (gsi_exchange.cuh): a release / acquire
 // barrier would cost two L2 round trips and a fence where these cost one.  Every token's sums run
-// in an order that depends on the shape alone: results are reproducible, and a token's are the
-// same in a call of any size.
-// Every wait is bounded; a wait that gives up sets GSI_ERR_TIMEOUT and the CTA returns.
+// in an order that depends on the shape and the grid alone: results are reproducible, and a token's
+// are the same in a call of any size that runs here as a whole (not where W r is left to the
+// contraction, leave_from).
+// Every wait is bounded; a CTA whose wait ran out sets GSI_ERR_TIMEOUT, leaves NaN and returns.
 #include <cuda.h>
 
 #include <type_traits>
@@ -42,6 +44,8 @@ constexpr int kTileRows = 16 * kW;     // rows of a basis slab (and of W) per pa
 constexpr int kPitch = 80;             // bytes between the staged 64-byte pieces: conflict-free ldmatrix
 constexpr int kDirectTokens = 2;       // calls of so few tokens gather the slabs' partials themselves
 constexpr int kDecideTokens = 4;       // calls of so few tokens decide the gates on every CTA
+constexpr int kTermsHoldOff = 900;     // cycles before the first look at the coefficients added elsewhere
+constexpr int kTermsHoldOffFrom = 1024;   // ... in calls of so many coefficients
 constexpr int kGateHoldOff = 600;      // cycles before the first look at the decisions taken elsewhere
 constexpr int kSegs = 8;               // the slabs' partials are added in eight runs, these by a tree
 constexpr int kSlots = 16;             // 16-row units of the basis whose norms wait in shared memory
@@ -501,6 +505,10 @@ __device__ __forceinline__ bool forward_fused(const GroupParams& g, const IoRef&
         const int f = rot + u * kT;
         return f < all ? f : f - all;
       };
+      // (looks ahead of the words hold up the CTAs that still add theirs: 21 tokens 26.4 -> 24.6 us; three
+      // tokens at k = 64, whose words are few, would lose 0.7 of 14)
+      if (n * k >= kTermsHoldOffFrom)
+        for (const long long t0 = clock64(); clock64() - t0 < kTermsHoldOff;) {}
       ok = gather128([&](int u) { return words.cf + (size_t)tb * half + place(u); }, mine, tag, g.spin_limit,
                      [&](int u, const Word128& w) {
                        const int f = place(u), c = f / half;
