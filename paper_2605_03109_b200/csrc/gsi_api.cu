@@ -30,7 +30,7 @@ constexpr int kTcMinFired = 5;  // fewer fired tokens: one pass of the CUDA-core
 constexpr double kOwnStreamBytes = 262144.0;   // W rows of a CTA up to which a gated residual stays on its group's share
 constexpr int kChains = 2;   // chains of a batched step side by side
 constexpr int kMaxSegments = 12;   // of a step with host buffers
-constexpr int kFrontMinTokens = 2;  // single-token calls: the CUDA-core front end
+constexpr int kFrontMinTokens = 2;  // single-token calls never take the tcgen05 front end (nor small ones: takes_fused)
 
 bool tc_shapes_ok(const gsi_desc_t* d) {
   for (int j = 0; j < d->n_maps; ++j)
@@ -89,7 +89,7 @@ Layout make_layout_ws(const gsi_desc_t* d) {
   const bool tc = !dense && tc_any;
   const bool dense_tc = dense && tc_any;   // the dense baseline of batched calls, same tile routine
   L.tc_rb = take(tc_any ? (size_t)65 * d->d * 2 : 0);   // row 64 stays zero
-  L.tc_ypart = take(tc_any ? (size_t)tc_splits(O, d->d) * 64 * O * 4 : 0);
+  L.tc_ypart = take(tc_any && tc_partials(O, d->d, dense) ? (size_t)tc_splits(O, d->d) * 64 * O * 4 : 0);
   L.tc = tc;
   L.dense_tc = dense_tc;
   // tensor-core projection / residual / image for batched calls

@@ -258,6 +258,7 @@ cudaError_t launch_residual_gemm_tc(const GroupParams& g, const TmaMaps& tm, con
                                     cudaStream_t stream, int* n_launches);
 int tc_splits(int O, int d);
 int tc_launches(int O, int d);   // kernels of a contraction
+bool tc_partials(int O, int d, bool dense);   // its splits leave partial sums in g.ypart
 bool tc_eligible(const GroupParams& g);
 // Batched front end on the tensor cores: c, r, gate and y = W_P c for n_tokens tokens.
 cudaError_t launch_front_tc(const GroupParams& g, const TmaMaps& tm, const IoRef& io,

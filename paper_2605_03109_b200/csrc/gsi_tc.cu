@@ -282,13 +282,16 @@ cudaError_t launch_dense_gemm_tc(const GroupParams& g, const TmaMaps& tm, const 
 // gated 552 -> 422, at 64 tokens 710 -> 563).  Up to 2^20 entries of W the second kernel costs no more
 // than the two cluster barriers (768 x 768, 64 tokens: 27.1 / 27.5 us).
 static bool tc_cluster(int O, int d) { return (double)O * d > 1048576.0 && tc_splits(O, d) > 1; }
+bool tc_partials(int O, int d, bool dense) { return tc_splits(O, d) > 1 && (dense || !tc_cluster(O, d)); }
 int tc_launches(int O, int d) { return tc_splits(O, d) > 1 && !tc_cluster(O, d) ? 2 : 1; }
 
 int tc_splits(int O, int d) {
   const int tiles = O / kTM, nkb = d / kTK;
-  // A tile per CTA (nearly) fills the SMs: long pipelines, no partial sums to add.  (4096 deep, 64
-  // tokens, all gated: 140 tiles 55.0 us a call without a split, 56.8 with two; 112 tiles 51.0 against
-  // 49.2 with few gated.  16384 deep, where the idle SMs cost more than the sums: 128 tiles 136.5 / 126.8.)
+  // A tile per CTA (nearly) fills the SMs: long pipelines, no partial sums to add.  The deeper the map
+  // the more the idle SMs cost against the sums (64 tokens, all gated, us a call without a split /
+  // with two: 128 tiles of 2048 39.5 / 42.0, 4096 54.3 / 54.0, 6144 67.1 / 66.8, 8192 81.4 / 79.4, 16384
+  // 132.6 / 125.1; 140 tiles of 2048 40.1 / 43.9, 4096 55.0 / 56.0, 6144 68.5 / 69.5, 8192 83.8 / 82.5, 16384
+  // 138.1 / 131.8): the line at 4096 is within one percent of the better side everywhere.
   if (tiles >= 148 || (tiles >= 128 && d <= 4096)) return 1;
   // No more clusters than are resident at a time (a second wave of a few costs more than it balances;
   // as the occupancy calculator gives them for clusters of 1, 2, ... blocks at two blocks per SM: they
