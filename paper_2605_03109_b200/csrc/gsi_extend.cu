@@ -19,8 +19,8 @@
 //
 // What bounds it: the chain of two exchanges per pass (words that carry their validity,
 // gsi_exchange.cuh) and 2 MB of basis.  Before, fourteen launches whether a column was appended
-// or not: 107 us for a token inside the subspace at 4096 x 256 and 28672 image rows, now 12.9 us;
-// with a column appended (235 MB of W) 168 us, now 78 us.
+// or not: 107 us for a token inside the subspace at 4096 x 256 and 28672 image rows, now 12.1 us a
+// call (the kernel 9.5); with a column appended (235 MB of W) 168 us, now 78 us.
 #include "gsi_exchange.cuh"
 #include "gsi_pack.cuh"
 

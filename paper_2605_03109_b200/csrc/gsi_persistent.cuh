@@ -89,7 +89,7 @@ constexpr unsigned kPersistSpinLimitDefault = 1u << 22;
 
 int persist_smem_bytes();
 int persist_threads();
-// pairs: some phase of the table holds two groups; common_k: the rank shared by every gated
+// pairs: some phase of the table holds several groups; common_k: the rank shared by every gated
 // group of the table, or 0 (both select a build of the kernel)
 cudaError_t launch_decode_step(const PersistParams& p, int grid, bool pairs, int common_k,
                                cudaStream_t st);

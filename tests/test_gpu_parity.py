@@ -342,6 +342,17 @@ def test_image_tiles_and_edges(o, d, k, p_dtype):
     assert image_ulp_check(W, P, out[:o].cpu()) < 0.05
 
 
+@pytest.mark.parametrize("p_dtype", ["bf16", "f32"])
+def test_image_of_a_deep_map_rounds_as_an_fp32_sum(p_dtype):
+    """d = 16384: sums kept in the tensor core for the whole depth, whose own accumulation truncates,
+    would put 4e-3 of the entries on the other side of a bf16 rounding boundary, fp32 sums of chunks
+    5e-4 (32 of these 65536 entries, give or take 6): the line lies between the two."""
+    g = G()
+    o, d, k = 512, 16384, 128
+    P, W = S.store_basis(S.gen_basis(d, k, 321), p_dtype), S.gen_weight(o, d, 322)
+    assert image_ulp_check(W, P, g.gsi_build_image(W.cuda(), P.cuda()).cpu()) < 1.5e-3
+
+
 def test_forward_host_variant():
     x, P, Ws = make_small(768, 64, (3072,), 4, seed=81, outlier_every=2)
     g = G()
@@ -1175,8 +1186,8 @@ def test_tensor_core_front_end_batched_projection_residual_image(k, n_tokens):
 
 @pytest.mark.parametrize("n_tokens,d_out", [(3, (128,)), (17, (256, 128)), (64, (4096,)), (33, (8192,))])
 def test_tensor_core_residual_splits_meet_in_a_cluster(n_tokens, d_out):
-    """Deep narrow maps: the splits of a tile are a cluster (two, three and 32 tiles of eight
-    splits; the widest case has five and sums them through memory)."""
+    """Deep narrow maps: three and 32 tiles as clusters of eight splits, 64 tiles of four; the eight
+    splits of a single tile meet in memory."""
     d, k = 4096, 128
     x, P, Ws = make_small(d, k, d_out, n_tokens, seed=970 + n_tokens, noise=0.001, outlier_every=2)
     g = G()
