@@ -1,5 +1,6 @@
 // C ABI of the gated subspace layer: argument checking, workspace layout,
 // handle and stack bookkeeping, kernel sequencing.  No arithmetic lives here.
+#include <chrono>
 #include <algorithm>
 #include <new>
 #include <vector>
@@ -319,6 +320,7 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W, const void
     h->has_tm = true;
   }
 
+  const auto begin = std::chrono::steady_clock::now();
   if (cudaMemsetAsync(ctrl, 0, 256, stream) != cudaSuccess ||
       cudaMemsetAsync(h->ws + L.pk_acc, 0, L.total - L.pk_acc, stream) != cudaSuccess) {
     delete h;
@@ -352,9 +354,13 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W, const void
   }
   // A set-up call: return only when the images, max|P| and the cleared state are in
   // place, so the handle may be used from any stream afterwards.
+  // A wait of the image kernel that runs out takes 2^22 polls of twenty cycles at least, 43 ms: the
+  // status word (10 us to read) is looked at when the work took long enough to hold one.
   int status = 0;
-  if (cudaMemcpyAsync(&status, g.status, sizeof status, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
-      cudaStreamSynchronize(stream) != cudaSuccess || status != 0) {
+  if (cudaStreamSynchronize(stream) != cudaSuccess ||
+      (std::chrono::steady_clock::now() - begin > std::chrono::milliseconds(20) &&
+       cudaMemcpy(&status, g.status, sizeof status, cudaMemcpyDeviceToHost) != cudaSuccess) ||
+      status != 0) {
     delete h;
     return status ? (gsi_status_t)status : GSI_ERR_CUDA;   // (an image with a tile that was given up)
   }
