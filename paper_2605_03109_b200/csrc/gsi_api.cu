@@ -31,6 +31,11 @@ constexpr int kTcMinFired = 5;  // fewer fired tokens: one pass of the CUDA-core
 constexpr double kOwnStreamBytes = 262144.0;   // W rows of a CTA up to which a gated residual stays on its group's share
 constexpr int kChains = 2;   // chains of a batched step side by side
 constexpr int kMaxSegments = 12;   // of a step with host buffers
+// Batched stacks of fewer groups keep a chain of launches per group (one GPT-J layer, three groups, 64 tokens, a
+// tenth gated: 134 us against 152 in five launches; one GPT-2 layer, four groups, 60 against 45).
+constexpr int kWideMinGroups = 4;
+constexpr int kWideGemmSlots = 296;   // blocks of the contraction that are resident at a time
+constexpr int kWideBlocks = 592;   // projection blocks of a wide step: two waves of two per SM
 constexpr int kFrontMinTokens = 2;  // single-token calls never take the tcgen05 front end (nor small ones: takes_fused)
 
 bool tc_shapes_ok(const gsi_desc_t* d) {
@@ -178,6 +183,19 @@ struct gsi_stack {
   cudaStream_t copy_in = nullptr, copy_out = nullptr;
   cudaEvent_t ev_begin = nullptr, ev_in[kMaxSegments] = {}, ev_run[kMaxSegments] = {};
   cudaEvent_t ev_resid = nullptr, ev_front_fork = nullptr, ev_front_join = nullptr;
+  // batched steps in five launches over all groups (WideParams): the table, and for the whole step
+  // and for every segment the blocks before each group
+  struct WideRange {
+    int g0, g1;
+    const int *first, *order;   // device
+    int blocks[kWideStages];
+    int splits;                 // of the depth, in the contraction
+  };
+  char* wide_area;           // device, null when the workspace has no room for it
+  bool wide = false;
+  std::vector<WideRange> wide_ranges;
+  std::vector<WideGroup> wide_table;
+  std::vector<int> wide_ints;
   ~gsi_stack() {
     if (ev_fork) cudaEventDestroy(ev_fork);
     if (ev_join) cudaEventDestroy(ev_join);
@@ -479,11 +497,18 @@ gsi_status_t gsi_destroy(gsi_handle_t h) {
 }
 
 // ------------------------------------------------------------------ stack
-size_t gsi_stack_workspace_bytes(int n_groups) {
-  if (n_groups <= 0) return 0;
+static size_t stack_tables_bytes(int n_groups) {
   static_assert(sizeof(PersistGroup) <= 512, "group descriptor outgrew its slot");
   return align_up(256) + align_up((size_t)n_groups * 512) + align_up((size_t)n_groups * 8) +
          align_up((size_t)n_groups * 4);
+}
+static size_t wide_ints(int n_groups) {   // of the whole step and of the segments
+  return 2 * (kWideStages + 1) * (size_t)n_groups + kWideStages * (kMaxSegments + 1);
+}
+
+size_t gsi_stack_workspace_bytes(int n_groups) {
+  if (n_groups <= 0) return 0;
+  return stack_tables_bytes(n_groups) + align_up(n_groups * sizeof(WideGroup)) + align_up(4 * wide_ints(n_groups));
 }
 
 gsi_status_t gsi_stack_create(int n_groups, const gsi_handle_t* groups, void* workspace,
@@ -492,7 +517,7 @@ gsi_status_t gsi_stack_create(int n_groups, const gsi_handle_t* groups, void* wo
   *out = nullptr;
   if (n_groups <= 0 || !groups || !workspace) return GSI_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(workspace) % kAlign) return GSI_ERR_INVALID_ARG;
-  if (workspace_bytes < gsi_stack_workspace_bytes(n_groups)) return GSI_ERR_WORKSPACE;
+  if (workspace_bytes < stack_tables_bytes(n_groups)) return GSI_ERR_WORKSPACE;
   for (int i = 0; i < n_groups; ++i) {
     if (!groups[i]) return GSI_ERR_INVALID_ARG;
     if (groups[i]->desc.max_tokens != groups[0]->desc.max_tokens) return GSI_ERR_INVALID_ARG;
@@ -515,6 +540,8 @@ gsi_status_t gsi_stack_create(int n_groups, const gsi_handle_t* groups, void* wo
   s->dev_groups = reinterpret_cast<PersistGroup*>(static_cast<char*>(workspace) + 256);
   s->dev_phase_first = reinterpret_cast<int*>(static_cast<char*>(workspace) + align_up(256) +
                                               align_up((size_t)n_groups * 512) + align_up((size_t)n_groups * 8));
+  s->wide_area = workspace_bytes >= gsi_stack_workspace_bytes(n_groups)
+                     ? static_cast<char*>(workspace) + stack_tables_bytes(n_groups) : nullptr;
   s->spin_limit = kPersistSpinLimitDefault;
   s->mode = 0;
   s->trace = nullptr;
@@ -682,6 +709,100 @@ gsi_status_t gsi_stack_set_mode(gsi_stack_t s, int mode) {
 
 static bool plan_segments(gsi_stack* s);
 
+// Does every group of a batched stack take the tensor-core front end, and are there enough of them
+// to fill the launches of a wide step?
+static bool wide_eligible(const gsi_stack* s) {
+  const int G = (int)s->groups.size();
+  if (s->persistent || s->mode != 0 || !s->wide_area || G < kWideMinGroups || G > kWideMaxGroups) return false;
+  for (const gsi_layer* h : s->groups)
+    if (!h->has_tm || !h->lay.front || s->B < h->gp.front_min_tokens || (h->desc.flags & GSI_FLAG_DENSE)) return false;
+  return true;
+}
+
+// The table of a wide step and the blocks of its launches, for the whole step and for every segment.
+static bool plan_wide(gsi_stack* s, cudaStream_t stream) {
+  const int G = (int)s->groups.size();
+  long long kblocks = 0, tiles = 0;
+  for (const gsi_layer* h : s->groups) {
+    kblocks += (long long)(h->desc.d / umma::kTK) * (h->desc.k / umma::kTM);
+    tiles += (h->desc.d + h->lay.O) / umma::kTM;
+  }
+  const int per_split = (int)std::max(4ll, (kblocks + kWideBlocks - 1) / kWideBlocks);
+  s->wide_table.assign(G, WideGroup{});
+  for (int i = 0; i < G; ++i) {
+    gsi_layer* h = s->groups[i];
+    WideGroup& w = s->wide_table[i];
+    w.tm = h->tm;
+    w.g = h->gp;
+    const int nkb = h->desc.d / umma::kTK, dt = h->desc.d / umma::kTM, nq = (s->B + 15) / 16;
+    w.g.proj_splits = std::max(1, std::min(h->gp.proj_splits, (nkb + per_split - 1) / per_split));
+    // a residual tile in ranges of tokens only where its kernel would leave SMs idle
+    w.rs = std::min(nq, tiles >= kWideBlocks ? 1 : dt <= 37 ? 4 : dt <= 148 ? 2 : 1);
+    w.io = IoRef{s->io[i].x, s->io[i].y, s->gate_log + (size_t)i * s->B,
+                 s->rho_log ? s->rho_log + (size_t)i * s->B : nullptr, s->step, s->n_steps,
+                 (long long)s->B * h->desc.d, (long long)G * s->B};
+  }
+  char* ints_dev = s->wide_area + align_up(G * sizeof(WideGroup));
+  s->wide_ints.clear();
+  s->wide_ranges.clear();
+  auto add_range = [&](int g0, int g1) {
+    const int n = g1 - g0;
+    gsi_stack::WideRange r{g0, g1, nullptr, nullptr, {}, 1};
+    std::vector<int> order(n);
+    for (int i = 0; i < n; ++i) order[i] = i;
+    // the contraction: deep tiles, which take longest, first
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int a, int b) { return s->groups[g0 + a]->desc.d > s->groups[g0 + b]->desc.d; });
+    r.first = reinterpret_cast<const int*>(ints_dev) + s->wide_ints.size();
+    for (int stage = 0; stage < kWideStages; ++stage) {
+      int at = 0;
+      for (int i = 0; i < n; ++i) {
+        s->wide_ints.push_back(at);
+        const int gi = g0 + (stage == kWideGemm ? order[i] : i);
+        const WideGroup& w = s->wide_table[gi];
+        const int d = w.g.d, O = w.g.O;
+        at += stage == kWideSplit   ? wide_split_blocks(d, s->B)
+              : stage == kWideProj  ? w.g.k / umma::kTM * w.g.proj_splits
+              : stage == kWideResid ? d / umma::kTM * w.rs + O / umma::kTM
+              : (w.g.flags & GSI_FLAG_STATIC_PROJECTION) ? 0 : O / umma::kTM;
+      }
+      s->wide_ints.push_back(at);
+      r.blocks[stage] = at;
+    }
+    // So many splits that the deepest tile takes no longer than an even share of all, none below a
+    // depth of 2048 (64 tokens, a tenth gated: two GPT-J layers 237 us without, 227 with eight; 12 GPT-2
+    // layers, depth 3072, 151 without, 172 with two).
+    double work = 0.0, deepest = 0.0;
+    for (int i = 0; i < n; ++i) {
+      const GroupParams& g = s->wide_table[g0 + i].g;
+      work += (double)g.O / umma::kTM * g.d;
+      deepest = std::max(deepest, (double)g.d);
+    }
+    while (r.splits < 8 && deepest / r.splits > work / kWideGemmSlots && deepest / (2 * r.splits) >= 2048) r.splits *= 2;
+    r.order = reinterpret_cast<const int*>(ints_dev) + s->wide_ints.size();
+    s->wide_ints.insert(s->wide_ints.end(), order.begin(), order.end());
+    s->wide_ranges.push_back(r);
+  };
+  add_range(0, G);
+  for (size_t i = 0; s->segment.size() > 2 && i + 1 < s->segment.size(); ++i) add_range(s->segment[i], s->segment[i + 1]);
+  return cudaMemcpyAsync(s->wide_area, s->wide_table.data(), G * sizeof(WideGroup), cudaMemcpyHostToDevice, stream) ==
+             cudaSuccess &&
+         cudaMemcpyAsync(ints_dev, s->wide_ints.data(), s->wide_ints.size() * 4, cudaMemcpyHostToDevice, stream) ==
+             cudaSuccess;
+}
+
+static gsi_status_t wide_enqueue(gsi_stack* s, int g0, int g1, bool use_counter, cudaStream_t stream) {
+  for (const gsi_stack::WideRange& r : s->wide_ranges) {
+    if (r.g0 != g0 || r.g1 != g1) continue;
+    const WideParams p{reinterpret_cast<const WideGroup*>(s->wide_area) + g0, r.first, r.order, g1 - g0, use_counter ? 1 : 0};
+    for (int i = g0; i < g1; ++i) s->groups[i]->last_stream = stream;
+    if (launch_front_wide(p, r.blocks, s->B, stream) != cudaSuccess) return GSI_ERR_CUDA;
+    if (r.blocks[kWideGemm] && launch_gemm_wide(p, r.blocks[kWideGemm], r.splits, s->B, stream) != cudaSuccess) return GSI_ERR_CUDA;
+    return GSI_OK;
+  }
+  return GSI_ERR_CUDA;
+}
+
 gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps,
                             unsigned char* gate_log, float* rho_log, gsi_stream_t stream) {
   if (!s || !io || n_steps <= 0 || !gate_log) return GSI_ERR_INVALID_ARG;
@@ -709,7 +830,8 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
   if (!s->persistent)
     for (const gsi_layer* h : s->groups)
       if (h->desc.flags & GSI_FLAG_FP8_IMAGE) return GSI_ERR_UNSUPPORTED;
-  if (!s->persistent && !s->aux) {
+  s->wide = wide_eligible(s);
+  if (!s->persistent && !s->wide && !s->aux) {
     bool any = false;
     for (char c : s->pair_first) any = any || c;
     int least = 0, greatest = 0;
@@ -719,7 +841,7 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
                 cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess))
       return GSI_ERR_CUDA;
   }
-  if (!s->persistent && !s->ev_front_join) {
+  if (!s->persistent && !s->wide && !s->ev_front_join) {
     bool any = false;   // some group takes the tensor-core front end at this batch
     for (const gsi_layer* h : s->groups)
       any = any || (h->has_tm && h->gp.front_min_tokens > 0 && s->B >= h->gp.front_min_tokens &&
@@ -828,6 +950,7 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
       return GSI_ERR_CUDA;
   }
   if (!plan_segments(s)) return GSI_ERR_CUDA;
+  if (s->wide && !plan_wide(s, stream)) return GSI_ERR_CUDA;
   // A set-up call: the descriptor table and the cleared exchange state must be in
   // device memory before a step may be enqueued on ANY stream.
   if (cudaStreamSynchronize(stream) != cudaSuccess) return GSI_ERR_CUDA;
@@ -877,6 +1000,12 @@ static gsi_status_t stack_enqueue_range(gsi_stack_t s, int g0, int g1, bool firs
       p.advance = t == s->B - 1;
       if (launch_decode_step(p, s->grid, s->has_pairs, s->common_k, stream) != cudaSuccess) return GSI_ERR_CUDA;
     }
+    return GSI_OK;
+  }
+  if (s->wide) {
+    const gsi_status_t st = wide_enqueue(s, g0, g1, use_counter, stream);
+    if (st != GSI_OK) return st;
+    if (last && use_counter && launch_advance_step(s->step, stream) != cudaSuccess) return GSI_ERR_CUDA;
     return GSI_OK;
   }
   ResidualLane lane{stream, s->ev_resid, false};
@@ -988,6 +1117,10 @@ gsi_status_t gsi_stack_launches_per_step(gsi_stack_t s, int* n_out) {
   if (!s || !n_out || !s->bound) return GSI_ERR_INVALID_ARG;
   if (s->persistent) {
     *n_out = s->B;
+    return GSI_OK;
+  }
+  if (s->wide) {
+    *n_out = 4 + (s->wide_ranges[0].blocks[kWideGemm] ? 1 : 0) + 1;
     return GSI_OK;
   }
   int n = 0;

@@ -75,15 +75,13 @@ __device__ __forceinline__ void store_terms(const float (&v)[8], bool live, uint
   }
 }
 
-__global__ void __launch_bounds__(256) k_split3_x(GroupParams g, IoRef io, int n_tokens) {
-  // first kernel of the chain: wait first, so that nothing of the chain (its successors
-  // request weight tiles before their own waits) runs beside an earlier call's kernels
-  pdl_wait();   // xb may still be read by the previous call's projection
-  pdl_launch_dependents();
-  const int slot = blockIdx.y, n_rows = rows3(n_tokens);
+// Elements 8 i8 .. of token slot `slot`, i8 from `first` on in strides of `stride`.
+__device__ __forceinline__ void split3_body(const GroupParams& g, const IoRef& io, int n_tokens, int slot, int first,
+                                            int stride) {
+  const int n_rows = rows3(n_tokens);
   const bool live = slot < n_tokens;
   const float* x = io.x + (long long)io_slot(io) * io.x_step_stride + (size_t)slot * g.d;
-  for (int i8 = blockIdx.x * 256 + threadIdx.x; i8 < g.d / 8; i8 += gridDim.x * 256) {
+  for (int i8 = first; i8 < g.d / 8; i8 += stride) {
     float v[8] = {};
     if (live) {
       const float4 a = __ldg(reinterpret_cast<const float4*>(x) + 2 * i8);
@@ -95,15 +93,21 @@ __global__ void __launch_bounds__(256) k_split3_x(GroupParams g, IoRef io, int n
   }
 }
 
+__global__ void __launch_bounds__(256) k_split3_x(GroupParams g, IoRef io, int n_tokens) {
+  // first kernel of the chain: wait first, so that nothing of the chain (its successors
+  // request weight tiles before their own waits) runs beside an earlier call's kernels
+  pdl_wait();   // xb may still be read by the previous call's projection
+  pdl_launch_dependents();
+  split3_body(g, io, n_tokens, blockIdx.y, blockIdx.x * 256 + threadIdx.x, gridDim.x * 256);
+}
+
 // c partials: cpart3[split][t][128*tile + lane row] over this split's share of d.
 template <bool kInStack>
-__global__ void __launch_bounds__(kThreads, 1)
-k_proj_tc(GroupParams g, const __grid_constant__ TmaMaps tm, int n_tokens) {
-  extern __shared__ unsigned char smem_raw[];
-  pdl_launch_dependents();
+__device__ __forceinline__ void proj_body(unsigned char* smem_raw, const GroupParams& g, const TmaMaps& tm,
+                                          int n_tokens, int block) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int splits = g.proj_splits;
-  const int tile = blockIdx.x / splits, split = blockIdx.x % splits;
+  const int tile = block / splits, split = block % splits;
   const int nkb = g.d / kTK;
   const int kb0 = (int)((long long)nkb * split / splits), kb1 = (int)((long long)nkb * (split + 1) / splits);
   uint32_t tmem;
@@ -125,13 +129,19 @@ k_proj_tc(GroupParams g, const __grid_constant__ TmaMaps tm, int n_tokens) {
   tile_release<kTmemCols3>(tmem);
 }
 
+template <bool kInStack>
+__global__ void __launch_bounds__(kThreads, 1)
+k_proj_tc(GroupParams g, const __grid_constant__ TmaMaps tm, int n_tokens) {
+  extern __shared__ unsigned char smem_raw[];
+  pdl_launch_dependents();
+  proj_body<kInStack>(smem_raw, g, tm, n_tokens, blockIdx.x);
+}
+
 // c = sum of the split-K partials in split order; also its three bf16 terms.
 // One block per token slot, one coefficient per thread and pass.
-__global__ void __launch_bounds__(256) k_reduce_split3_c(GroupParams g, int n_tokens) {
-  const int slot = blockIdx.x, n_rows = rows3(n_tokens);
+__device__ __forceinline__ void reduce_body(const GroupParams& g, int n_tokens, int slot) {
+  const int n_rows = rows3(n_tokens);
   const bool live = slot < n_tokens;
-  pdl_launch_dependents();
-  pdl_wait();
   for (int j = threadIdx.x; j < g.k; j += 256) {
     float v = 0.f;
     if (live) {
@@ -163,6 +173,12 @@ __global__ void __launch_bounds__(256) k_reduce_split3_c(GroupParams g, int n_to
   }
 }
 
+__global__ void __launch_bounds__(256) k_reduce_split3_c(GroupParams g, int n_tokens) {
+  pdl_launch_dependents();
+  pdl_wait();
+  reduce_body(g, n_tokens, blockIdx.x);
+}
+
 // One launch for Algorithm 1 lines 2-5.  Every block contracts one 128-row tile against
 // the c terms of a range of 16-token groups (operand rows 48 q_lo .. 48 q_hi - 1):
 //   blocks [0, n_resid)   tile of P, one of rs token ranges (rs > 1 spreads the narrow
@@ -171,18 +187,16 @@ __global__ void __launch_bounds__(256) k_reduce_split3_c(GroupParams g, int n_to
 //                         and in the block that finishes last the gate
 //   blocks [n_resid, ..)  tile of W_P, all tokens: y = W_P c
 template <int kStagesT, int kMaxRows, int kTmemColsT, bool kInStack>
-__global__ void __launch_bounds__(kThreads, 2)
-k_resid_image_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, int n_tokens, int rs) {
-  extern __shared__ unsigned char smem_raw[];
+__device__ __forceinline__ void resid_image_body(unsigned char* smem_raw, const GroupParams& g, const TmaMaps& tm,
+                                                 const IoRef& io, int n_tokens, int rs, int block) {
   __shared__ float s_norm[kThreads / 32][GSI_MAX_TOKENS][2];
   __shared__ int s_last;
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nq = (n_tokens + 15) / 16;
   const int n_resid = (g.d / kTM) * rs;
-  const bool image = (int)blockIdx.x >= n_resid;
-  const int tile = image ? (int)blockIdx.x - n_resid : (int)blockIdx.x / rs;
-  const int part = image ? 0 : (int)blockIdx.x % rs;
+  const bool image = block >= n_resid;
+  const int tile = image ? block - n_resid : block / rs;
+  const int part = image ? 0 : block % rs;
   const int per = image ? nq : (nq + rs - 1) / rs;
   const int q_lo = min(part * per, nq), q_hi = min(q_lo + per, nq);
   const int row = tile * kTM + warp * 32 + lane;
@@ -244,6 +258,62 @@ k_resid_image_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, in
     }
   }
   decide_gate_last_block(g, io, slot, n_tokens, g.normpart3, g.d / kTM, (unsigned)n_resid, &s_last);
+}
+
+template <int kStagesT, int kMaxRows, int kTmemColsT, bool kInStack>
+__global__ void __launch_bounds__(kThreads, 2)
+k_resid_image_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, int n_tokens, int rs) {
+  extern __shared__ unsigned char smem_raw[];
+  pdl_launch_dependents();
+  resid_image_body<kStagesT, kMaxRows, kTmemColsT, kInStack>(smem_raw, g, tm, io, n_tokens, rs, blockIdx.x);
+}
+
+// ---- the same for all groups of a range of a stack in one launch each -------------------
+// (a block finds its group in the table; WideGroup)
+// A step in a chain of five launches per group is the latency of its chains and the tails of small
+// grids: 28 GPT-J layers, 64 tokens, a tenth gated, 477 launches 3.34 ms; the same kernels over all
+// groups, whose inputs are staged before the step, 2.68 ms (W r at the copy bandwidth); 12 GPT-2 layers,
+// k = 256, 636 -> 151 us.
+__global__ void __launch_bounds__(256) k_split3_x_wide(WideParams p, int n_tokens, int slots) {
+  pdl_wait();   // (first of the chain, as above)
+  pdl_launch_dependents();
+  int block;
+  const WideGroup& w = p.find(kWideSplit, &block);
+  const IoRef io = p.io_of(w);
+  split3_body(w.g, io, n_tokens, block % slots, block / slots * 256 + threadIdx.x, (w.g.d / 8 + 255) / 256 * 256);
+}
+
+__global__ void __launch_bounds__(kThreads, 1) k_proj_wide(WideParams p, int n_tokens) {
+  extern __shared__ unsigned char smem_raw[];
+  pdl_launch_dependents();
+  int block;
+  const WideGroup& w = p.find(kWideProj, &block);
+  if (threadIdx.x < 32) {
+    acquire_map(&w.tm.pt);
+    acquire_map(&w.tm.xb);
+  }
+  proj_body<true>(smem_raw, w.g, w.tm, n_tokens, block);
+}
+
+__global__ void __launch_bounds__(256) k_reduce_wide(WideParams p, int n_tokens, int slots) {
+  pdl_launch_dependents();
+  pdl_wait();
+  reduce_body(p.table[blockIdx.x / slots].g, n_tokens, blockIdx.x % slots);
+}
+
+template <int kStagesT, int kMaxRows, int kTmemColsT>
+__global__ void __launch_bounds__(kThreads, 2) k_resid_image_wide(WideParams p, int n_tokens) {
+  extern __shared__ unsigned char smem_raw[];
+  pdl_launch_dependents();
+  int block;
+  const WideGroup& w = p.find(kWideResid, &block);
+  if (threadIdx.x < 32) {
+    acquire_map(&w.tm.p);
+    acquire_map(&w.tm.wp);
+    acquire_map(&w.tm.cb);
+  }
+  const IoRef io = p.io_of(w);
+  resid_image_body<kStagesT, kMaxRows, kTmemColsT, true>(smem_raw, w.g, w.tm, io, n_tokens, w.rs, block);
 }
 
 // PT[j][i] = P[i][j], 32 x 32 tiles through shared memory.
@@ -318,6 +388,28 @@ cudaError_t launch_front_tc(const GroupParams& g, const TmaMaps& tm, const IoRef
                             cudaStream_t st, int* n_launches) {
   if (n_launches) *n_launches += 4;
   return in_stack ? launch_front<true>(g, tm, io, n_tokens, st) : launch_front<false>(g, tm, io, n_tokens, st);
+}
+
+int wide_split_blocks(int d, int n_tokens) { return (d / 8 + 255) / 256 * ((front_rows(n_tokens) + 2) / 3); }
+
+cudaError_t launch_front_wide(const WideParams& p, const int* blocks, int n_tokens, cudaStream_t st) {
+  constexpr int kSmem3 = Cfg<kStages3, kMaxN3>::kSmem;
+  auto wide = k_resid_image_wide<kStagesRI, kMaxN3, kTmemCols3>;
+  auto narrow = k_resid_image_wide<kStagesRIs, kMaxN3s, kTmemCols3s>;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_proj_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem3)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRI)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRIs)) != cudaSuccess)
+    return e;
+  const bool small = term_rows(n_tokens) <= kMaxN3s;
+  const int slots = (front_rows(n_tokens) + 2) / 3;
+  if ((e = launch_pdl(k_split3_x_wide, dim3(blocks[kWideSplit]), dim3(256), 0, st, p, n_tokens, slots)) != cudaSuccess ||
+      (e = launch_pdl(k_proj_wide, dim3(blocks[kWideProj]), dim3(kThreads), kSmem3, st, p, n_tokens)) != cudaSuccess ||
+      (e = launch_pdl(k_reduce_wide, dim3(p.n * slots), dim3(256), 0, st, p, n_tokens, slots)) != cudaSuccess ||
+      (e = launch_pdl(small ? narrow : wide, dim3(blocks[kWideResid]), dim3(kThreads), small ? kSmemRIs : kSmemRI, st,
+                      p, n_tokens)) != cudaSuccess)
+    return e;
+  return cudaGetLastError();
 }
 
 }  // namespace gsi

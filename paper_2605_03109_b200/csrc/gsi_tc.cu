@@ -52,14 +52,12 @@ __global__ void __launch_bounds__(256) k_pack_fired_bf16(GroupParams g, int min_
 // kCluster: the splits of a tile are a cluster; their sums meet in distributed shared memory, added
 // in split order by the ranks (a share of the columns each), and no partial sum goes to memory.
 template <bool kCluster, bool kInStack>
-__global__ void __launch_bounds__(kThreadsTc, 2)
-k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, int min_fired, int splits,
-                   int mapped, int n_tokens) {
-  pdl_launch_dependents();
+__device__ __forceinline__ void residual_gemm_body(unsigned char* smem_raw, const GroupParams& g, const TmaMaps& tm,
+                                                   const IoRef& io, int min_fired, int splits, int mapped,
+                                                   int n_tokens, int block, bool speculate) {
   // With many tokens per call some token is gated nearly always: the W tiles are then
   // requested before the fired list of the kernel before is known (mapped operand rows only:
   // their number does not depend on the list), and the block backs out if nobody fired.
-  const bool speculate = mapped && n_tokens >= kSpeculateTokens;
   int n_fired = 0;
   if (!speculate) {
     pdl_wait();   // the fired list comes from the kernel before
@@ -69,10 +67,9 @@ k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, 
   const int n_cols = mapped ? n_tokens : n_fired;
   const int N = (n_cols + 15) & ~15;          // 16..64
 
-  extern __shared__ unsigned char smem_raw[];
   __shared__ unsigned long long s_mask;       // columns to write out
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tile = blockIdx.x / splits, split = blockIdx.x % splits;
+  const int tile = block / splits, split = block % splits;
   const int row0 = tile * kTM;                 // first row of the concatenated maps
   int j = 0;
   while (j + 1 < g.n_maps && row0 >= g.off[j + 1]) ++j;   // a tile never straddles two maps
@@ -163,6 +160,32 @@ k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, 
     }
   }
   tile_release<kTmemCols>(tmem);
+}
+
+template <bool kCluster, bool kInStack>
+__global__ void __launch_bounds__(kThreadsTc, 2)
+k_residual_gemm_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, int min_fired, int splits,
+                   int mapped, int n_tokens) {
+  extern __shared__ unsigned char smem_raw[];
+  pdl_launch_dependents();
+  residual_gemm_body<kCluster, kInStack>(smem_raw, g, tm, io, min_fired, splits, mapped, n_tokens, blockIdx.x,
+                                         mapped && n_tokens >= kSpeculateTokens);
+}
+
+// W r of all groups of a range of a stack: a tile of 128 rows per block, or per cluster of `splits`
+// blocks over the depth.
+template <bool kCluster>
+__global__ void __launch_bounds__(kThreadsTc, 2) k_gemm_wide(WideParams p, int splits, int n_tokens) {
+  extern __shared__ unsigned char smem_raw[];
+  pdl_launch_dependents();
+  int block;
+  const WideGroup& w = p.find(kWideGemm, &block, splits);
+  if (threadIdx.x < 32) {
+    for (int j = 0; j < w.g.n_maps; ++j) acquire_map(&w.tm.w[j]);
+    acquire_map(&w.tm.rb);
+  }
+  const IoRef io = p.io_of(w);
+  residual_gemm_body<kCluster, true>(smem_raw, w.g, w.tm, io, 1, splits, 1, n_tokens, block, false);
 }
 
 // y[fired[n]][row] += sum over splits (fixed order); the partial sums of fired token n
@@ -344,6 +367,26 @@ cudaError_t launch_residual_gemm_tc(const GroupParams& g, const TmaMaps& tm, con
     return e;
   if (n_launches) *n_launches += (mapped ? 0 : 1) + tc_launches(g.O, g.d);
   return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_wide(const WideParams& p, int tiles, int splits, int n_tokens, cudaStream_t st) {
+  auto kernel = splits > 1 ? k_gemm_wide<true> : k_gemm_wide<false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(tiles * splits);
+  cfg.blockDim = dim3(kThreadsTc);
+  cfg.dynamicSmemBytes = kTcSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = splits;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = splits > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, p, splits, n_tokens);
 }
 
 }  // namespace gsi

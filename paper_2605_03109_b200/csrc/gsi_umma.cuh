@@ -329,4 +329,51 @@ struct alignas(64) TmaMaps {
   CUtensorMap rb;                // residuals  [65][d]     (B operand)
 };
 
+// A batched step in five launches: every kernel of the chain over all groups of the stack at once
+// (their inputs are staged before the step), a block finding its group by a table in device memory.
+enum { kWideSplit, kWideProj, kWideResid, kWideGemm, kWideStages };
+constexpr int kWideMaxGroups = 1024;   // two steps of thirty-two in the search
+
+struct alignas(64) WideGroup {
+  TmaMaps tm;
+  GroupParams g;
+  IoRef io;
+  int rs;      // token ranges per residual tile
+};
+
+// Makes a tensor map that the host wrote to device memory usable by this thread's copies.
+__device__ __forceinline__ void acquire_map(const CUtensorMap* m) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(m) : "memory");
+}
+
+struct WideParams {
+  const WideGroup* table;   // the range's groups
+  const int* first;         // [kWideStages][n + 1] blocks before each of them
+  const int* order;         // [n]: the order in which the contraction takes them
+  int n;
+  int use_counter;
+
+  __device__ __forceinline__ IoRef io_of(const WideGroup& w) const {
+    IoRef io = w.io;
+    if (!use_counter) io.step = nullptr;
+    return io;
+  }
+  // The group that this block belongs to in a stage, and its index there.  Every warp for itself.
+  // `parts` adjacent blocks share a place in the table.
+  __device__ __forceinline__ const WideGroup& find(int stage, int* block, int parts = 1) const {
+    const int* f = first + stage * (n + 1);
+    const int lane = threadIdx.x & 31, b = blockIdx.x / parts, step = (n + 31) / 32;
+    const unsigned m = __ballot_sync(0xffffffffu, lane * step < n && __ldg(f + min(lane * step, n)) <= b);
+    const int lo = (__popc(m) - 1) * step;
+    const int v = lane < step && lo + lane < n ? __ldg(f + lo + lane) : 0x7fffffff;
+    const unsigned q = __ballot_sync(0xffffffffu, v <= b);
+    const int i = __popc(q) - 1;
+    *block = blockIdx.x - parts * __shfl_sync(0xffffffffu, v, i);
+    return table[stage == kWideGemm ? __ldg(order + lo + i) : lo + i];
+  }
+};
+int wide_split_blocks(int d, int n_tokens);
+cudaError_t launch_front_wide(const WideParams& p, const int* blocks, int n_tokens, cudaStream_t st);
+cudaError_t launch_gemm_wide(const WideParams& p, int tiles, int splits, int n_tokens, cudaStream_t st);
+
 }  // namespace gsi

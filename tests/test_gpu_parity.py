@@ -1735,3 +1735,49 @@ def test_persistent_opt_layer_full_size_sampled_rows(k):
     assert stack.is_persistent() and stack.launches_per_step() == 1
     rates = [s["gate_rate"] for s in stats]
     assert 0.0 < np.mean(rates) < 1.0   # sigma scale 1.0 puts the median rho on eps: both paths occur
+
+
+@pytest.mark.parametrize("n_tokens,shapes,static", [
+    (3, ((256, 128, (128,)), (384, 128, (256, 128)), (1024, 256, (384,)), (8192, 128, (128,))), False),   # splits of W r
+    (16, ((384, 128, (640,)), (2048, 512, (128,)), (256, 128, (128, 128, 128)), (512, 384, (1152,))), False),
+    (33, ((768, 256, (256, 128)),) * 5, False),                 # beyond the narrow build of the residual kernel
+    (64, tuple((128 * (2 + i % 3), 128, (128,)) for i in range(70)), False),   # three groups per lane of the search
+    (8, ((256, 128, (128,)), (384, 128, (256,)), (512, 128, (128,)), (256, 128, (128,))), True),   # no contraction at all
+])
+def test_batched_step_over_all_groups_at_once(n_tokens, shapes, static):
+    """Batched stacks of four groups and more run every kernel of the chain once over all groups: steps
+    and graph replays against the oracle, a group whose tokens all lie inside its subspace among them; the
+    launches are those that gsi_stack_launches_per_step states.  (k < d and noise enough that rho is 5e-3 at
+    least: an fp32 sum is off by some 2^-24 of x, and rho has to agree to 2e-5 of itself.)"""
+    from cuda.bindings import runtime as rt
+    g = G()
+    groups = [make_small(d, k, d_out, 2 * n_tokens, seed=9500 + 7 * i, noise=0.005, outlier_every=0 if i == 1 else 3)
+              for i, (d, k, d_out) in enumerate(shapes)]
+    layers = [g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n_tokens,
+                      flags=g.GSI_FLAG_STATIC_PROJECTION if static else 0) for _, P, Ws in groups]
+    stack = g.Stack(layers)
+    stack.bind([x.cuda() for x, _, _ in groups], n_steps=2)
+    assert not stack.is_persistent() and stack.launches_per_step() == (5 if static else 6)
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        stack.step()
+    err, nodes, count = rt.cudaGraphGetNodes(rt.cudaGraph_t(graph.raw_cuda_graph()), 256)
+    kinds = [rt.cudaGraphNodeGetType(node)[1] for node in nodes[:count]]
+    assert kinds.count(rt.cudaGraphNodeType.cudaGraphNodeTypeKernel) == stack.launches_per_step()
+    graph.instantiate()
+    stack.seek(0)
+    for step in range(4):
+        stack.step() if step < 2 else graph.replay()
+        torch.cuda.synchronize()
+        assert stack.status() == 0
+        at = step % 2 * n_tokens
+        gates = stack.gate_log[step % 2].cpu().numpy()
+        assert gates[1].max() == 0 and gates[0].max() == 1
+        for i, (x, P, Ws) in enumerate(groups):
+            y = stack.ys[i].cpu().reshape(n_tokens, -1).numpy()
+            if static:
+                ref = np.concatenate([(x[at:at + n_tokens].double() @ P.double() @ (W.double() @ P.double()).T).numpy()
+                                      for W in Ws], axis=1)
+                assert np.max(np.abs(y - ref)) <= 1e-2 * np.max(np.abs(ref))
+            else:
+                compare_group(x[at:at + n_tokens], P, Ws, 0.05, y, gates[i], stack.rho_log[step % 2, i].cpu().numpy())
