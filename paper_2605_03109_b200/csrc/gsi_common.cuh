@@ -234,6 +234,10 @@ cudaError_t launch_advance_step(int* step, cudaStream_t stream);
 // gated tokens on their W r is left to a contraction that follows (g.r, g.fired, *g.n_fired).
 cudaError_t launch_forward_fused(const GroupParams& g, const IoRef& io, int n_tokens, int leave_from,
                                  cudaStream_t stream);
+// The same as clusters that need no word between them (gsi_cluster.cu); false when the call has to
+// take the cooperative launch (its basis does not fit sixteen SMs, or the context holds no cluster).
+bool launch_forward_cluster(const GroupParams& g, const IoRef& io, int n_tokens, int leave_from, cudaStream_t stream,
+                            cudaError_t* e);
 size_t fused_words_bytes(int d, int k, int max_tokens);
 // Online basis extension by one vector (see gsi_extend_basis).
 struct ExtendArgs {

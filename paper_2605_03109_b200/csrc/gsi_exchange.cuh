@@ -160,6 +160,8 @@ __device__ __forceinline__ Area area_of(const GroupParams& g) {
 
 }  // namespace exchange
 
+// Id of the current context, which is never used again; 0 when it cannot be told.
+unsigned long long context_id();
 // CTAs of a cooperative launch: the SMs of the current context (a green context has fewer than its
 // device); 0 on error.
 int fused_grid();

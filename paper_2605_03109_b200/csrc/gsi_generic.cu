@@ -412,7 +412,8 @@ cudaError_t launch_generic_forward(const GroupParams& g, const TmaMaps* tm, cons
   const bool front = tm && g.front_min_tokens > 0 && n_tokens >= g.front_min_tokens;
   if (!per_stage && takes_fused(g, front, n_tokens, in_stack)) {
     const int leave = leave_to_contraction(g, tm != nullptr, n_tokens);
-    if ((e = launch_forward_fused(g, io, n_tokens, leave, st)) != cudaSuccess) return e;
+    if (!launch_forward_cluster(g, io, n_tokens, leave, st, &e)) e = launch_forward_fused(g, io, n_tokens, leave, st);
+    if (e != cudaSuccess) return e;
     *n_launches += 1;
     return leave ? launch_residual_gemm_tc(g, *tm, io, leave, false, in_stack, n_tokens, st, n_launches) : cudaSuccess;
   }

@@ -112,5 +112,7 @@ extern "C" gsi_status_t gsi_forward_static(const void* const* W_host_array, cons
   io.rho = rho_out;
   io.step = nullptr;
   io.n_steps = 1;
-  return launch_forward_fused(g, io, n_tokens, 0, stream) == cudaSuccess ? GSI_OK : GSI_ERR_CUDA;
+  cudaError_t e;
+  if (!launch_forward_cluster(g, io, n_tokens, 0, stream, &e)) e = launch_forward_fused(g, io, n_tokens, 0, stream);
+  return e == cudaSuccess ? GSI_OK : GSI_ERR_CUDA;
 }

@@ -1781,3 +1781,29 @@ def test_batched_step_over_all_groups_at_once(n_tokens, shapes, static):
                 assert np.max(np.abs(y - ref)) <= 1e-2 * np.max(np.abs(ref))
             else:
                 compare_group(x[at:at + n_tokens], P, Ws, 0.05, y, gates[i], stack.rho_log[step % 2, i].cpu().numpy())
+
+
+@pytest.mark.parametrize("d,k,d_out,n,p_dtype,every", [
+    (8, 8, (8,), 2, "bf16", 1),                        # CTAs without rows, a cluster of one image unit
+    (1000, 120, (12000, 4992), 32, "bf16", 1),         # W r in several batches
+    (4088, 248, (4096, 2056), 1, "bf16", 2),           # a handle for one token: sixteen slabs of 130 KB
+    (1000, 200, (1000, 504, 72), 13, "f32", 2),        # three terms of the basis, odd rows and tokens
+    (520, 512, (1040,), 9, "bf16", 4),                 # 32 column tiles of c, two token blocks
+    (1288, 440, (4000,), 16, "bf16", 1),               # two passes over the tokens
+    (776, 96, (24,), 32, "bf16", 3),                   # every token block in use, one cluster
+])
+def test_cluster_forward_edges(d, k, d_out, n, p_dtype, every):
+    """Calls whose basis fits a cluster: the corners of its rows, token blocks and batches, against the
+    oracle, and the same bits from call to call with another call's input in between."""
+    g = G()
+    x, P, Ws = make_small(d, k, d_out, 2 * n, seed=9700 + d, noise=0.005, p_dtype=p_dtype, outlier_every=every)
+    lay = g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n)
+    xs = [x[:n].cuda().contiguous(), x[n:].cuda().contiguous()]
+    refs = [[t.clone() for t in lay.forward(xi)] for xi in xs]
+    outs = [lay.forward(xs[i % 2]) for i in range(20)]
+    torch.cuda.synchronize()
+    assert lay.status() == 0
+    for i, (y, gate, rho) in enumerate(refs):
+        compare_group(x[i * n:(i + 1) * n], P, Ws, 0.05, y.cpu().numpy(), gate.cpu().numpy())
+    for i, out in enumerate(outs):
+        assert all(torch.equal(a, b) or (torch.isnan(a) & torch.isnan(b)).all() for a, b in zip(out, refs[i % 2]))
