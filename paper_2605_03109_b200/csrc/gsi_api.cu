@@ -9,6 +9,7 @@
 #include "gsi_common.cuh"
 #include "gsi_umma.cuh"
 #include "gsi_persistent.cuh"
+#include "gsi_flat.cuh"
 
 using namespace gsi;
 
@@ -34,6 +35,13 @@ constexpr int kMaxSegments = 12;   // of a step with host buffers
 // Batched stacks of fewer groups keep a chain of launches per group (one GPT-J layer, three groups, 64 tokens, a
 // tenth gated: 134 us against 152 in five launches; one GPT-2 layer, four groups, 60 against 45).
 constexpr int kWideMinGroups = 4;
+// Single-token stacks that step in three launches (gsi_flat.cu) instead of the persistent kernel: groups enough
+// for their phases to add up, images that are small per group, bases that stay in the L2 (us a step,
+// persistent / three launches: 12 GPT-2 layers, k = 128, 70 % gated 124 / 53, k = 512 103 / 62; two layers, eight
+// groups, 41 / 32, 1 % gated 24.7 / 25.9; 12 OPT layers, k = 128, images of 2.4 MB, 158 / 148; three GPT-J
+// layers, k = 128, 3.1 MB, 46.9 / 48.6, k = 256, 6.3 MB, 76.6 / 80.7).
+constexpr int kFlatMinGroups = 8;
+constexpr double kFlatBasisBytes = 96.0e6, kFlatImageBytes = 3.0e6;
 constexpr int kWideGemmSlots = 296;   // blocks of the contraction that are resident at a time
 constexpr int kWideBlocks = 592;   // projection blocks of a wide step: two waves of two per SM
 constexpr int kFrontMinTokens = 2;  // single-token calls never take the tcgen05 front end (nor small ones: takes_fused)
@@ -196,6 +204,10 @@ struct gsi_stack {
   std::vector<WideRange> wide_ranges;
   std::vector<WideGroup> wide_table;
   std::vector<int> wide_ints;
+  // single-token steps of small groups in three launches (gsi_flat.cu): table and shares in the same area
+  bool flat = false;
+  int flat_grid = 0, flat_k = 0;
+  FlatParams flat_params;
   ~gsi_stack() {
     if (ev_fork) cudaEventDestroy(ev_fork);
     if (ev_join) cudaEventDestroy(ev_join);
@@ -502,8 +514,10 @@ static size_t stack_tables_bytes(int n_groups) {
   return align_up(256) + align_up((size_t)n_groups * 512) + align_up((size_t)n_groups * 8) +
          align_up((size_t)n_groups * 4);
 }
-static size_t wide_ints(int n_groups) {   // of the whole step and of the segments
-  return 2 * (kWideStages + 1) * (size_t)n_groups + kWideStages * (kMaxSegments + 1);
+static size_t wide_ints(int n_groups) {   // of the whole step and of the segments, or of a flat step
+  const size_t wide = 2 * (kWideStages + 1) * (size_t)n_groups + kWideStages * (kMaxSegments + 1);
+  const size_t flat = 14 * (size_t)n_groups + 7 * kFlatMaxGrid + 8;   // shares and their norms, groups, first shares
+  return wide > flat ? wide : flat;
 }
 
 size_t gsi_stack_workspace_bytes(int n_groups) {
@@ -709,11 +723,89 @@ gsi_status_t gsi_stack_set_mode(gsi_stack_t s, int mode) {
 
 static bool plan_segments(gsi_stack* s);
 
+// A step of one token in three launches over all groups?  The persistent kernel takes 3.5 us and more
+// per phase; the three launches read the bases twice, the second time from the L2.
+static bool flat_eligible(const gsi_stack* s, int grid) {
+  const int G = (int)s->groups.size();
+  if (s->mode != 0 || s->B != 1 || !s->wide_area || grid <= 0 || grid > kFlatMaxGrid || G < kFlatMinGroups ||
+      G > kFlatMaxGroups)
+    return false;
+  double basis = 0.0, image = 0.0;
+  for (const gsi_layer* h : s->groups) {
+    const gsi_desc_t& d = h->desc;
+    if ((d.flags & (GSI_FLAG_DENSE | GSI_FLAG_FP8_IMAGE)) || h->gp.p_f32 || d.d > kFlatMaxD) return false;
+    basis += 2.0 * d.d * d.k;
+    image += 2.0 * h->lay.O * d.k;
+  }
+  return basis <= kFlatBasisBytes && image / G <= kFlatImageBytes;
+}
+
+// The rows of all bases in even shares: CTA c has rows of cost [c, c + 1) / grid of the total, in units of
+// 16 rows.  False when a basis would have too many shares.
+static bool plan_flat(gsi_stack* s, int grid, cudaStream_t stream) {
+  const int G = (int)s->groups.size();
+  std::vector<int> first(1, 0), slots(G, 0);
+  std::vector<FlatShare> shares;
+  double total = 0.0, at = 0.0;
+  for (const gsi_layer* h : s->groups) total += (double)((h->desc.d + 15) / 16) * h->desc.k;
+  const double each = total / grid;
+  int gi = 0, unit = 0;
+  for (int c = 0; c < grid; ++c) {
+    const double end = c + 1 == grid ? total : each * (c + 1);
+    while (gi < G) {
+      const int units = (s->groups[gi]->desc.d + 15) / 16, k = s->groups[gi]->desc.k;
+      int n = c + 1 == grid ? units - unit : (int)((end - at) / k + 0.5);
+      n = std::min(n, units - unit);
+      if (n <= 0) break;
+      shares.push_back({gi, unit * 16, (unit + n) * 16, slots[gi]++});
+      at += (double)n * k;
+      unit += n;
+      if (unit < units) break;
+      ++gi;
+      unit = 0;
+    }
+    first.push_back((int)shares.size());
+  }
+  for (int n : slots)
+    if (n > kFlatMaxSlots) return false;
+  s->wide_table.assign(G, WideGroup{});
+  s->flat_k = 0;
+  for (int i = 0; i < G; ++i) {
+    WideGroup& w = s->wide_table[i];
+    w.g = s->groups[i]->gp;
+    w.io = IoRef{s->io[i].x, s->io[i].y, s->gate_log + i, s->rho_log ? s->rho_log + i : nullptr, s->step, s->n_steps,
+                 (long long)w.g.d, (long long)G};
+    s->flat_k = std::max(s->flat_k, w.g.k);
+  }
+  // (groups first: their records are read as 16-byte words)
+  s->wide_ints.clear();
+  for (int i = 0, at_share = 0; i < G; at_share += slots[i++]) {
+    const GroupParams& g = s->wide_table[i].g;
+    const FlatGroup f{at_share, slots[i], g.O, g.k, g.d, g.eps, g.flags, 0};
+    const int* words = reinterpret_cast<const int*>(&f);
+    s->wide_ints.insert(s->wide_ints.end(), words, words + sizeof f / 4);
+  }
+  const size_t at_shares = s->wide_ints.size();
+  for (const FlatShare& f : shares) s->wide_ints.insert(s->wide_ints.end(), {f.group, f.r0, f.r1, f.slot});
+  const size_t at_norms = s->wide_ints.size(), at_first = at_norms + 2 * shares.size();
+  s->wide_ints.resize(at_first, 0);
+  s->wide_ints.insert(s->wide_ints.end(), first.begin(), first.end());
+  int* ints = reinterpret_cast<int*>(s->wide_area + align_up(G * sizeof(WideGroup)));
+  s->flat_grid = grid;
+  s->flat_params = FlatParams{reinterpret_cast<const WideGroup*>(s->wide_area), ints + at_first,
+                              reinterpret_cast<const FlatShare*>(ints + at_shares), reinterpret_cast<const FlatGroup*>(ints),
+                              reinterpret_cast<float2*>(ints + at_norms), G, 0, s->step, s->step + 4};
+  return cudaMemsetAsync(s->step + 4, 0, sizeof(int), stream) == cudaSuccess &&
+         cudaMemcpyAsync(s->wide_area, s->wide_table.data(), G * sizeof(WideGroup), cudaMemcpyHostToDevice, stream) ==
+             cudaSuccess &&
+         cudaMemcpyAsync(ints, s->wide_ints.data(), s->wide_ints.size() * 4, cudaMemcpyHostToDevice, stream) == cudaSuccess;
+}
+
 // Does every group of a batched stack take the tensor-core front end, and are there enough of them
 // to fill the launches of a wide step?
 static bool wide_eligible(const gsi_stack* s) {
   const int G = (int)s->groups.size();
-  if (s->persistent || s->mode != 0 || !s->wide_area || G < kWideMinGroups || G > kWideMaxGroups) return false;
+  if (s->persistent || s->flat || s->mode != 0 || !s->wide_area || G < kWideMinGroups || G > kWideMaxGroups) return false;
   for (const gsi_layer* h : s->groups)
     if (!h->has_tm || !h->lay.front || s->B < h->gp.front_min_tokens || (h->desc.flags & GSI_FLAG_DENSE)) return false;
   return true;
@@ -816,7 +908,7 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
   s->rho_log = rho_log;
   s->last_stream = stream;
 
-  s->persistent = false;
+  s->persistent = s->flat = false;
   if (s->mode != 1) {
     int dev = 0, sms = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -824,14 +916,15 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess)
       return GSI_ERR_CUDA;
     s->grid = sms;
-    s->persistent = coop && persistent_eligible(s, sms);
+    s->flat = flat_eligible(s, sms) && plan_flat(s, sms, stream);
+    s->persistent = !s->flat && coop && persistent_eligible(s, sms);
     if (s->mode == 2 && !s->persistent) return GSI_ERR_UNSUPPORTED;
   }
   if (!s->persistent)
     for (const gsi_layer* h : s->groups)
       if (h->desc.flags & GSI_FLAG_FP8_IMAGE) return GSI_ERR_UNSUPPORTED;
   s->wide = wide_eligible(s);
-  if (!s->persistent && !s->wide && !s->aux) {
+  if (!s->persistent && !s->flat && !s->wide && !s->aux) {
     bool any = false;
     for (char c : s->pair_first) any = any || c;
     int least = 0, greatest = 0;
@@ -841,7 +934,7 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io, int n_steps
                 cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess))
       return GSI_ERR_CUDA;
   }
-  if (!s->persistent && !s->wide && !s->ev_front_join) {
+  if (!s->persistent && !s->flat && !s->wide && !s->ev_front_join) {
     bool any = false;   // some group takes the tensor-core front end at this batch
     for (const gsi_layer* h : s->groups)
       any = any || (h->has_tm && h->gp.front_min_tokens > 0 && s->B >= h->gp.front_min_tokens &&
@@ -1002,6 +1095,12 @@ static gsi_status_t stack_enqueue_range(gsi_stack_t s, int g0, int g1, bool firs
     }
     return GSI_OK;
   }
+  if (s->flat) {   // (one segment)
+    FlatParams p = s->flat_params;
+    p.use_counter = use_counter ? 1 : 0;
+    for (gsi_layer* h : s->groups) h->last_stream = stream;
+    return launch_flat_step(p, s->flat_grid, s->flat_k, stream) == cudaSuccess ? GSI_OK : GSI_ERR_CUDA;
+  }
   if (s->wide) {
     const gsi_status_t st = wide_enqueue(s, g0, g1, use_counter, stream);
     if (st != GSI_OK) return st;
@@ -1088,7 +1187,7 @@ static bool plan_segments(gsi_stack* s) {
   // 729 in two); the chains of batched steps go on from segment to segment without a gap: 3 MB
   // each (8 GPT-J layers: 821 us at 8 tokens and 1968 at 64, where the step alone takes 1200 and the
   // copies as long; in one piece, before the alternating chains, 1076 and 3359).
-  int n = s->persistent ? (s->B == 1 && total >= 3.0e6 ? 2 : 1) : (int)(total / 3.0e6);
+  int n = s->flat ? 1 : s->persistent ? (s->B == 1 && total >= 3.0e6 ? 2 : 1) : (int)(total / 3.0e6);
   n = std::max(1, std::min(n, std::min(units, kMaxSegments)));
   s->segment.assign(1, 0);
   double at = 0.0;
@@ -1117,6 +1216,10 @@ gsi_status_t gsi_stack_launches_per_step(gsi_stack_t s, int* n_out) {
   if (!s || !n_out || !s->bound) return GSI_ERR_INVALID_ARG;
   if (s->persistent) {
     *n_out = s->B;
+    return GSI_OK;
+  }
+  if (s->flat) {
+    *n_out = 3;
     return GSI_OK;
   }
   if (s->wide) {

@@ -1807,3 +1807,58 @@ def test_cluster_forward_edges(d, k, d_out, n, p_dtype, every):
         compare_group(x[i * n:(i + 1) * n], P, Ws, 0.05, y.cpu().numpy(), gate.cpu().numpy())
     for i, out in enumerate(outs):
         assert all(torch.equal(a, b) or (torch.isnan(a) & torch.isnan(b)).all() for a, b in zip(out, refs[i % 2]))
+
+
+@pytest.mark.parametrize("shapes,static", [
+    (((768, 128, (2304,)), (768, 128, (768,)), (768, 128, (3072,)), (3072, 128, (768,))) * 2, False),
+    (((264, 8, (8,)), (1000, 200, (504, 72)), (2056, 1000, (24,)), (16384, 40, (40,)), (520, 512, (1032,)),
+      (1032, 256, (8, 1040)), (4104, 512, (72,)), (16, 8, (16,)), (3000, 64, (600,))), False),
+    (((256, 64, (72,)),) * 300, False),                       # more groups than CTAs
+    (((512, 128, (256, 128)),) * 8, True),
+])
+def test_single_token_steps_over_all_groups_at_once(shapes, static):
+    """Stacks of many small groups step one token in three launches: steps, graph replays and host steps
+    against the oracle, with tokens inside the subspace, far outside it, zero and not finite; the launches
+    are those that gsi_stack_launches_per_step states."""
+    from cuda.bindings import runtime as rt
+    g = G()
+    n_steps = 3
+    groups = [make_small(d, k, d_out, n_steps, seed=9900 + i, noise=0.004, outlier_every=2 if i % 3 else 0)
+              for i, (d, k, d_out) in enumerate(shapes)]
+    groups[1][0][2] = 0.0
+    groups[2][0][1, 3] = float("inf")
+    layers = [g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=1,
+                      flags=g.GSI_FLAG_STATIC_PROJECTION if static else 0) for _, P, Ws in groups]
+    stack = g.Stack(layers)
+    xs = [x.cuda().contiguous() for x, _, _ in groups]
+    stack.bind(xs, n_steps=n_steps)
+    assert not stack.is_persistent() and stack.launches_per_step() == 3
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        stack.step()
+    err, nodes, count = rt.cudaGraphGetNodes(rt.cudaGraph_t(graph.raw_cuda_graph()), 256)
+    kinds = [rt.cudaGraphNodeGetType(node)[1] for node in nodes[:count]]
+    assert kinds.count(rt.cudaGraphNodeType.cudaGraphNodeTypeKernel) == 3
+    graph.instantiate()
+    stack.seek(0)
+    first = []
+    for step in range(2 * n_steps):
+        stack.step() if step < n_steps else graph.replay()
+        torch.cuda.synchronize()
+        assert stack.status() == 0
+        if step >= n_steps:   # the same bits again
+            assert all(torch.equal(a.nan_to_num(7.0), b.nan_to_num(7.0)) for a, b in zip(first[step - n_steps], stack.ys))
+            continue
+        first.append([y.clone() for y in stack.ys])
+        gates = stack.gate_log[step].cpu().numpy()
+        for i, (x, P, Ws) in enumerate(groups):
+            y = stack.ys[i].cpu().reshape(1, -1).numpy()
+            if not np.isfinite(x[step].numpy()).all():
+                assert gates[i, 0] == 1 and np.isnan(y).any()
+                continue
+            compare_group(x[step:step + 1], P, Ws, 0.05, y, gates[i], None, static=static)
+    ys = [torch.empty(sum(s[2])) for s in shapes]
+    gate = torch.empty((len(shapes), 1), dtype=torch.uint8)
+    stack.step_host([x[:1].contiguous() for x, _, _ in groups], ys, gate)
+    assert all(torch.equal(a.cpu().reshape(-1), b) for a, b in zip(first[0], ys))
+    assert torch.equal(gate, stack.gate_log[0].cpu())
