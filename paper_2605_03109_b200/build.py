@@ -1,4 +1,4 @@
-"""Build the CUDA library in-tree with nvcc for sm_100a."""
+"""Build the CUDA library in-tree with nvcc for sm_100a, and the extension module of the calls (g++)."""
 from __future__ import annotations
 
 import glob
@@ -81,6 +81,40 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+# The extension module of the calls (torch_calls.cpp): beside the library, built for this torch and Python.
+CALLS_SRC = os.path.join(CSRC, "torch_calls.cpp")
+CALLS = os.path.join(HERE, "_torch_calls.so")
+
+
+def _calls_command(out: str) -> list[str]:
+    import sysconfig
+    import torch
+    base = os.path.join(os.path.dirname(torch.__file__))
+    inc = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], "/usr/local/cuda/include", os.path.join(ROOT, "include")]
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-DTORCH_EXTENSION_NAME=_torch_calls",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *[f"-I{d}" for d in inc], CALLS_SRC,
+            "-o", out, "-L" + os.path.join(base, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+
+
+def build_calls(force: bool = False) -> str:
+    import hashlib
+    import torch
+    h = hashlib.sha256(" ".join(_calls_command("-")).encode() + torch.__version__.encode())
+    for p in (CALLS_SRC, os.path.join(ROOT, "include", "gsi.h")):
+        h.update(open(p, "rb").read())
+    digest, stamp = h.hexdigest(), CALLS + ".srchash"
+    if not force and os.path.exists(CALLS) and os.path.exists(stamp) and open(stamp).read().strip() == digest:
+        return CALLS
+    tmp = CALLS + f".tmp{os.getpid()}"
+    subprocess.check_call(_calls_command(tmp))
+    os.replace(tmp, CALLS)
+    with open(stamp, "w") as f:
+        f.write(digest)
+    return CALLS
+
+
 if __name__ == "__main__":
     import sys
+    build_calls("--force" in sys.argv)
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))

@@ -20,7 +20,7 @@
 // cluster reads the basis (from the L2, but for one), and seven clusters of sixteen leave 36 of 148
 // SMs idle; W r makes up for that with 128 KB in flight per SM (5.5 TB/s where the cooperative launch,
 // by loads into registers, reaches 4.7).  Kernel times in a captured graph, cooperative launch -> this: one
-// token at 768 x 64 -> 3072 10.3 -> 5.3 us, 4096 x 256 -> 28672 13.5 -> 13.8 (gated 64 -> 58); 16 tokens, fp32
+// token at 768 x 64 -> 3072 10.3 -> 5.3 us, 4096 x 256 -> 28672 13.5 -> 13.1 (gated 64 -> 57); 16 tokens, fp32
 // basis, 768 x 128 -> 2304 19 -> 10.3.
 //
 // Every wait is bounded; a CTA whose wait ran out sets GSI_ERR_TIMEOUT, leaves NaN, and stays until
@@ -39,7 +39,9 @@ using namespace mma16;
 constexpr int kC = 16;                  // CTAs of a cluster
 constexpr int kT = 512, kW = kT / 32;
 constexpr int kSmemCluster = 225 * 1024;
-constexpr int kDirectValues = 512;      // coefficients up to which every CTA adds the partials itself
+// Coefficients up to which every CTA adds all partials itself: one exchange, but sixteen times the words
+// (one token, in a graph: k = 64 5.2 us either way, k = 256 13.8 us, as two exchanges 13.1).
+constexpr int kDirectValues = 128;
 constexpr int kMostColumns = 512;
 constexpr int kMostPlane = 24576;       // bytes of a term of an fp32 basis per CTA
 constexpr int kMaxBatches = 4096;       // of W r: more than any call makes (bounds the stay of a CTA that gave up)
