@@ -201,6 +201,7 @@ struct gsi_stack {
   };
   char* wide_area;           // device, null when the workspace has no room for it
   bool wide = false;
+  int wide_k = 0;            // the largest rank
   std::vector<WideRange> wide_ranges;
   std::vector<WideGroup> wide_table;
   std::vector<int> wide_ints;
@@ -814,10 +815,11 @@ static bool wide_eligible(const gsi_stack* s) {
 // The table of a wide step and the blocks of its launches, for the whole step and for every segment.
 static bool plan_wide(gsi_stack* s, cudaStream_t stream) {
   const int G = (int)s->groups.size();
-  long long kblocks = 0, tiles = 0;
+  long long kblocks = 0;
+  s->wide_k = 0;
   for (const gsi_layer* h : s->groups) {
     kblocks += (long long)(h->desc.d / umma::kTK) * (h->desc.k / umma::kTM);
-    tiles += (h->desc.d + h->lay.O) / umma::kTM;
+    s->wide_k = std::max(s->wide_k, h->desc.k);
   }
   const int per_split = (int)std::max(4ll, (kblocks + kWideBlocks - 1) / kWideBlocks);
   s->wide_table.assign(G, WideGroup{});
@@ -826,10 +828,8 @@ static bool plan_wide(gsi_stack* s, cudaStream_t stream) {
     WideGroup& w = s->wide_table[i];
     w.tm = h->tm;
     w.g = h->gp;
-    const int nkb = h->desc.d / umma::kTK, dt = h->desc.d / umma::kTM, nq = (s->B + 15) / 16;
+    const int nkb = h->desc.d / umma::kTK;
     w.g.proj_splits = std::max(1, std::min(h->gp.proj_splits, (nkb + per_split - 1) / per_split));
-    // a residual tile in ranges of tokens only where its kernel would leave SMs idle
-    w.rs = std::min(nq, tiles >= kWideBlocks ? 1 : dt <= 37 ? 4 : dt <= 148 ? 2 : 1);
     w.io = IoRef{s->io[i].x, s->io[i].y, s->gate_log + (size_t)i * s->B,
                  s->rho_log ? s->rho_log + (size_t)i * s->B : nullptr, s->step, s->n_steps,
                  (long long)s->B * h->desc.d, (long long)G * s->B};
@@ -855,7 +855,7 @@ static bool plan_wide(gsi_stack* s, cudaStream_t stream) {
         const int d = w.g.d, O = w.g.O;
         at += stage == kWideSplit   ? wide_split_blocks(d, s->B)
               : stage == kWideProj  ? w.g.k / umma::kTM * w.g.proj_splits
-              : stage == kWideResid ? d / umma::kTM * w.rs + O / umma::kTM
+              : stage == kWideResid ? (d + O) / umma::kTM
               : (w.g.flags & GSI_FLAG_STATIC_PROJECTION) ? 0 : O / umma::kTM;
       }
       s->wide_ints.push_back(at);
@@ -886,9 +886,10 @@ static bool plan_wide(gsi_stack* s, cudaStream_t stream) {
 static gsi_status_t wide_enqueue(gsi_stack* s, int g0, int g1, bool use_counter, cudaStream_t stream) {
   for (const gsi_stack::WideRange& r : s->wide_ranges) {
     if (r.g0 != g0 || r.g1 != g1) continue;
-    const WideParams p{reinterpret_cast<const WideGroup*>(s->wide_area) + g0, r.first, r.order, g1 - g0, use_counter ? 1 : 0};
+    const WideParams p{reinterpret_cast<const WideGroup*>(s->wide_area) + g0, r.first, r.order, g1 - g0, use_counter ? 1 : 0,
+                       wide_term_bytes(s->wide_k, s->B)};
     for (int i = g0; i < g1; ++i) s->groups[i]->last_stream = stream;
-    if (launch_front_wide(p, r.blocks, s->B, stream) != cudaSuccess) return GSI_ERR_CUDA;
+    if (launch_front_wide(p, r.blocks, s->B, s->grid, stream) != cudaSuccess) return GSI_ERR_CUDA;
     if (r.blocks[kWideGemm] && launch_gemm_wide(p, r.blocks[kWideGemm], r.splits, s->B, stream) != cudaSuccess) return GSI_ERR_CUDA;
     return GSI_OK;
   }

@@ -179,6 +179,22 @@ __global__ void __launch_bounds__(256) k_reduce_split3_c(GroupParams g, int n_to
   reduce_body(g, n_tokens, blockIdx.x);
 }
 
+// Lane l's result: the sum of v[l] over the lanes.  Every step halves the values and pairs the lanes:
+// 31 shuffles for all 32 sums, where one after the other they take 160.
+__device__ __forceinline__ float sum32_over_lanes(float (&v)[32]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float give = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  return v[0];
+}
+
 // One launch for Algorithm 1 lines 2-5.  Every block contracts one 128-row tile against
 // the c terms of a range of 16-token groups (operand rows 48 q_lo .. 48 q_hi - 1):
 //   blocks [0, n_resid)   tile of P, one of rs token ranges (rs > 1 spreads the narrow
@@ -231,18 +247,19 @@ __device__ __forceinline__ void resid_image_body(unsigned char* smem_raw, const 
       for (int tt = 0; tt < 16; ++tt)
         xn[tt] = (q + 1 < q_hi && 16 * (q + 1) + tt < n_tokens) ? __ldg(x + (size_t)(16 * (q + 1) + tt) * g.d)
                                                                  : 0.f;
+      float sq[32];   // ||r||^2 of the sixteen tokens, then ||x||^2
 #pragma unroll
       for (int tt = 0; tt < 16; ++tt) {
         const int t = 16 * q + tt;
         const float rv = xv[tt] - s[tt];
         if (t < n_tokens) g.rb[(size_t)t * g.d + row] = bf16_bits(rv);
-        const float a = warp_sum(rv * rv), b = warp_sum(xv[tt] * xv[tt]);
-        if (lane == 0 && t < n_tokens) {
-          s_norm[warp][t][0] = a;
-          s_norm[warp][t][1] = b;
-        }
+        sq[tt] = rv * rv;
+        sq[16 + tt] = xv[tt] * xv[tt];
         xv[tt] = xn[tt];
       }
+      const float sum = sum32_over_lanes(sq);
+      const int t = 16 * q + (lane & 15);
+      if (t < n_tokens) s_norm[warp][t][lane >> 4] = sum;
     }
     tile_release<kTmemColsT>(tmem);
   }
@@ -301,19 +318,262 @@ __global__ void __launch_bounds__(256) k_reduce_wide(WideParams p, int n_tokens,
   reduce_body(p.table[blockIdx.x / slots].g, n_tokens, blockIdx.x % slots);
 }
 
-template <int kStagesT, int kMaxRows, int kTmemColsT>
-__global__ void __launch_bounds__(kThreads, 2) k_resid_image_wide(WideParams p, int n_tokens) {
+// Residual and image tiles of all groups, persistent: a CTA takes an even share of the tiles, in
+// order, and with it the terms of c of few groups, which it keeps in shared memory while weight tiles
+// stream through the ring (112 KB and more in flight).  Two accumulators: while four warps take one to
+// r, norms and y, the next tile is contracted into the other.
+//   warp 0 asks for the weight tiles (ahead of the wait on the kernel before), warp 1 for the terms, and
+//   issues the contractions; warps 2-5 and 6-9 take the accumulators in turn.
+// As a block per tile each lived 12 us (search, tensor maps, tensor memory, one round trip of the copies,
+// epilogue) for 64 KB of weights: eight GPT-J layers at 8 tokens 162 -> 76 us, at 64 173 -> 167 (there the
+// epilogue is what bounds it: 64 columns per row to store, and to add up for the residual).
+constexpr int kThreadsW = 320, kSmemW = 220 * 1024, kBarBytesW = 512, kMostStagesW = 13;
+constexpr int kTermBytesW = 100 * 1024;   // shared memory for the terms of c at most
+constexpr int kTmemColsW = 512;
+
+__global__ void __launch_bounds__(kThreadsW, 1) k_resid_image_wide(WideParams p, int n_tiles, int n_tokens) {
   extern __shared__ unsigned char smem_raw[];
+  __shared__ float s_norm[2][4][GSI_MAX_TOKENS][2];
+  __shared__ unsigned char s_gate[2][GSI_MAX_TOKENS];
+  __shared__ int s_last[2], s_fail, s_issued, s_terms;
   pdl_launch_dependents();
-  int block;
-  const WideGroup& w = p.find(kWideResid, &block);
-  if (threadIdx.x < 32) {
-    acquire_map(&w.tm.p);
-    acquire_map(&w.tm.wp);
-    acquire_map(&w.tm.cb);
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kSmemW - 1024 - kBarBytesW);
+  uint64_t *full = bars, *empty = bars + kMostStagesW, *tfull = empty + kMostStagesW, *tempty = tfull + 2,
+           *terms = tempty + 2, *read = terms + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(read + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nq = (n_tokens + 15) / 16, rows_all = rows3(n_tokens);
+  unsigned char* s_terms_at = smem;
+  unsigned char* s_ring = smem + p.term_bytes;
+  const int stages = min(kMostStagesW, (kSmemW - 1024 - kBarBytesW - p.term_bytes) / kABytes);
+  if (tid == 0) {
+    for (int s = 0; s < kMostStagesW; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int e = 0; e < 2; ++e) {
+      mbar_init(&tfull[e], 1);
+      mbar_init(&tempty[e], 128);
+    }
+    mbar_init(terms, 1);
+    mbar_init(read, 1);
+    s_fail = s_issued = s_terms = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  const IoRef io = p.io_of(w);
-  resid_image_body<kStagesT, kMaxRows, kTmemColsT, true>(smem_raw, w.g, w.tm, io, n_tokens, w.rs, block);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(tmem_slot)), "r"(kTmemColsW) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+
+  // This CTA's tiles, group by group, in passes over the tokens whose terms fit; every role goes through
+  // the same list.  `tile` is called with (group, tile of the group, first 16-token block, last), `open`
+  // and `close` around each pass; they return false to give up.
+  const int t0 = (int)((long long)n_tiles * blockIdx.x / gridDim.x), t1 = (int)((long long)n_tiles * (blockIdx.x + 1) / gridDim.x);
+  auto walk = [&](auto&& open, auto&& tile, auto&& close) {
+    const int* first = p.first + kWideResid * (p.n + 1);
+    int gi = 0;
+    for (int b = p.n; b - gi > 1;) {   // the last group that begins at or before tile t0
+      const int m = (gi + b) / 2;
+      if (first[m] <= t0) gi = m;
+      else b = m;
+    }
+    for (; gi < p.n && first[gi] < t1; ++gi) {
+      const int a = max(0, t0 - first[gi]), b = min(t1, first[gi + 1]) - first[gi];
+      if (a >= b) continue;
+      const WideGroup& w = p.table[gi];
+      const int per = max(1, p.term_bytes / (48 * w.g.k * 2));   // 16-token blocks of a pass
+      for (int q0 = 0; q0 < nq; q0 += per) {
+        const int q1 = min(nq, q0 + per);
+        if (!open(w, q0, q1)) return;
+        for (int t = a; t < b; ++t)
+          if (!tile(w, t, q0, q1)) return;
+        if (!close()) return;
+      }
+    }
+  };
+  auto nothing = [] { return true; };
+
+  if (warp == 0) {
+    if (lane == 0) {   // weight tiles
+      int n = 0;
+      const WideGroup* last = nullptr;
+      walk([](const WideGroup&, int, int) { return true; },
+           [&](const WideGroup& w, int t, int, int) {
+             if (&w != last) {
+               acquire_map(&w.tm.p);
+               acquire_map(&w.tm.wp);
+               last = &w;
+             }
+             const int dt = w.g.d / kTM;
+             const CUtensorMap* map = t < dt ? &w.tm.p : &w.tm.wp;
+             const int row = (t < dt ? t : t - dt) * kTM;
+             for (int kb = 0; kb < w.g.k / kTK; ++kb, ++n) {
+               const int s = n % stages;
+               if (n >= stages && !mbar_wait(&empty[s], ((n / stages) - 1) & 1)) {
+                 s_fail = 1;
+                 return false;
+               }
+               mbar_expect_tx(&full[s], (uint32_t)kABytes);
+               tma_load_2d(s32(s_ring + s * kABytes), map, kb * kTK, row, &full[s]);
+               s_issued = n + 1;
+             }
+             return true;
+           },
+           nothing);
+    }
+    __syncwarp();
+    pdl_wait();
+  } else if (warp == 1) {
+    pdl_wait();
+    int n = 0, n_tile = 0, n_pass = 0;
+    bool ok = true;   // (the same for the whole warp)
+    walk(
+        [&](const WideGroup& w, int q0, int q1) {   // the terms of c of the pass, a lane per box
+          const int N = min(48 * (q1 - q0), rows_all - 48 * q0), boxes = N / kBBox, all = w.g.k / kTK * boxes;
+          acquire_map(&w.tm.cb);
+          if (n_pass > 0) ok = __all_sync(0xffffffffu, mbar_wait(read, (n_pass - 1) & 1));   // those before are read
+          if (!ok) return false;
+          if (lane == 0) mbar_expect_tx(terms, (uint32_t)(all * kBBox * kTK * 2));
+          if (lane == 0) s_terms = n_pass + 1;
+          __syncwarp();
+          for (int i = lane; i < all; i += 32) {
+            const int kb = i / boxes, r = i - kb * boxes;
+            tma_load_2d(s32(s_terms_at) + (kb * N + r * kBBox) * (kTK * 2), &w.tm.cb, kb * kTK, 48 * q0 + r * kBBox, terms);
+          }
+          ok = __all_sync(0xffffffffu, mbar_wait(terms, n_pass & 1));
+          ++n_pass;
+          return ok;
+        },
+        [&](const WideGroup& w, int, int q0, int q1) {
+          const int N = min(48 * (q1 - q0), rows_all - 48 * q0), e = n_tile & 1;
+          if (lane == 0) {
+            const uint32_t idesc = instr_desc(kTM, N);
+            if (n_tile >= 2) ok = mbar_wait(&tempty[e], ((n_tile >> 1) - 1) & 1, kSpin * 8);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int kb = 0; ok && kb < w.g.k / kTK; ++kb) {
+              const int s = (n + kb) % stages;
+              ok = mbar_wait(&full[s], ((n + kb) / stages) & 1);
+              if (!ok) break;
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              const uint32_t a0 = s32(s_ring + s * kABytes), b0 = s32(s_terms_at) + kb * N * (kTK * 2);
+#pragma unroll
+              for (int k = 0; k < kTK / 16; ++k)
+                umma_bf16(tmem + e * 256, smem_desc_sw128(a0 + k * 32), smem_desc_sw128(b0 + k * 32), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+              umma_commit(&empty[s]);
+            }
+            if (ok) umma_commit(&tfull[e]);
+          }
+          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+          n += w.g.k / kTK;
+          ++n_tile;
+          return ok;
+        },
+        [&] {
+          if (lane == 0) umma_commit(read);
+          __syncwarp();
+          return true;
+        });
+    if (!ok && lane == 0) s_fail = 1;
+  } else {
+    pdl_wait();
+    const int e = (warp - 2) >> 2, quarter = warp & 3, tid4 = quarter * 32 + lane;
+    const uint32_t tl = tmem + e * 256 + ((uint32_t)(quarter * 32) << 16);
+    auto sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(1 + e) : "memory"); };
+    int n_tile = 0;
+    bool ok = true;   // after a wait that ran out: NaN, and every arrival that others count on
+    walk([](const WideGroup&, int, int) { return true; },
+         [&](const WideGroup& w, int tile, int q0, int q1) {
+           if ((n_tile & 1) != e) {
+             ++n_tile;
+             return true;
+           }
+           const GroupParams& g = w.g;
+           // (in registers: the table lies in memory that the stores below could reach, for all the compiler knows)
+           const int d = g.d, O = g.O, dt = d / kTM;
+           uint16_t* rb = g.rb;
+           const bool image = tile >= dt;
+           const int row = (image ? tile - dt : tile) * kTM + quarter * 32 + lane;
+           const IoRef io = p.io_of(w);
+           const int slot = io_slot(io);
+           float* y = io.y;
+           const float* x = io.x + (long long)slot * io.x_step_stride + row;
+           float xv[16];
+           if (!image)
+#pragma unroll
+             for (int tt = 0; tt < 16; ++tt)
+               xv[tt] = 16 * q0 + tt < n_tokens ? __ldg(x + (size_t)(16 * q0 + tt) * d) : 0.f;
+           if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&tfull[e], (n_tile >> 1) & 1, kSpin * 8));
+           if (!ok && lane == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
+           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+           for (int q = q0; q < q1; ++q) {
+             float s[16];
+             if (ok) {
+               sum3_tokens16(tl, q - q0, s);
+             } else {
+#pragma unroll
+               for (int tt = 0; tt < 16; ++tt) s[tt] = __int_as_float(0x7fc00000);
+             }
+             if (q + 1 == q1) {   // the accumulator is read
+               asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+               mbar_arrive(&tempty[e]);
+             }
+             if (image) {
+#pragma unroll
+               for (int tt = 0; tt < 16; ++tt)
+                 if (16 * q + tt < n_tokens) y[(size_t)(16 * q + tt) * O + row] = s[tt];
+               continue;
+             }
+             float xn[16], sq[32];
+#pragma unroll
+             for (int tt = 0; tt < 16; ++tt)
+               xn[tt] = (q + 1 < q1 && 16 * (q + 1) + tt < n_tokens) ? __ldg(x + (size_t)(16 * (q + 1) + tt) * d) : 0.f;
+#pragma unroll
+             for (int tt = 0; tt < 16; ++tt) {
+               const int t = 16 * q + tt;
+               const float rv = xv[tt] - s[tt];
+               if (t < n_tokens) rb[(size_t)t * d + row] = bf16_bits(rv);
+               sq[tt] = rv * rv;
+               sq[16 + tt] = xv[tt] * xv[tt];
+               xv[tt] = xn[tt];
+             }
+             const float sum = sum32_over_lanes(sq);
+             const int t = 16 * q + (lane & 15);
+             if (t < n_tokens) s_norm[e][quarter][t][lane >> 4] = sum;
+           }
+           ++n_tile;
+           if (image) return true;
+           sync();
+           for (int i = tid4; i < 32 * (q1 - q0); i += 128) {
+             const int t = 16 * q0 + (i >> 1), h = i & 1;
+             if (t < n_tokens) {
+               float sum = 0.f;
+#pragma unroll
+               for (int c = 0; c < 4; ++c) sum += s_norm[e][c][t][h];
+               g.normpart3[((size_t)tile * g.B + t) * 2 + h] = sum;
+             }
+           }
+           const int per = max(1, p.term_bytes / (48 * g.k * 2)), passes = (nq + per - 1) / per;
+           decide_gate_last(g, io, slot, n_tokens, g.normpart3, dt, (unsigned)(dt * passes), &s_last[e], s_gate[e], tid4, 128, sync);
+           sync();   // (s_last and s_norm are read)
+           return true;
+         },
+         nothing);
+    if (!ok) s_fail = 1;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (s_fail && tid == 0) {   // copies that were asked for: a bounded time to land before the block exits
+    for (int i = max(0, s_issued - stages); i < s_issued; ++i) (void)mbar_wait(&full[i % stages], (i / stages) & 1, 1u << 16);
+    if (s_terms > 0) (void)mbar_wait(terms, (s_terms - 1) & 1, 1u << 16);
+  }
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemColsW) : "memory");
 }
 
 // PT[j][i] = P[i][j], 32 x 32 tiles through shared memory.
@@ -392,22 +652,25 @@ cudaError_t launch_front_tc(const GroupParams& g, const TmaMaps& tm, const IoRef
 
 int wide_split_blocks(int d, int n_tokens) { return (d / 8 + 255) / 256 * ((front_rows(n_tokens) + 2) / 3); }
 
-cudaError_t launch_front_wide(const WideParams& p, const int* blocks, int n_tokens, cudaStream_t st) {
+int wide_term_bytes(int most_k, int n_tokens) {
+  const int nq = (n_tokens + 15) / 16, one = 48 * most_k * 2;
+  int q = kTermBytesW / one;
+  q = q < 1 ? 1 : q > nq ? nq : q;
+  return (q * one + 1023) / 1024 * 1024;
+}
+
+cudaError_t launch_front_wide(const WideParams& p, const int* blocks, int n_tokens, int grid, cudaStream_t st) {
   constexpr int kSmem3 = Cfg<kStages3, kMaxN3>::kSmem;
-  auto wide = k_resid_image_wide<kStagesRI, kMaxN3, kTmemCols3>;
-  auto narrow = k_resid_image_wide<kStagesRIs, kMaxN3s, kTmemCols3s>;
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(k_proj_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem3)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRI)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRIs)) != cudaSuccess)
+      (e = cudaFuncSetAttribute(k_resid_image_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemW)) != cudaSuccess)
     return e;
-  const bool small = term_rows(n_tokens) <= kMaxN3s;
-  const int slots = (front_rows(n_tokens) + 2) / 3;
+  const int slots = (front_rows(n_tokens) + 2) / 3, tiles = blocks[kWideResid];
   if ((e = launch_pdl(k_split3_x_wide, dim3(blocks[kWideSplit]), dim3(256), 0, st, p, n_tokens, slots)) != cudaSuccess ||
       (e = launch_pdl(k_proj_wide, dim3(blocks[kWideProj]), dim3(kThreads), kSmem3, st, p, n_tokens)) != cudaSuccess ||
       (e = launch_pdl(k_reduce_wide, dim3(p.n * slots), dim3(256), 0, st, p, n_tokens, slots)) != cudaSuccess ||
-      (e = launch_pdl(small ? narrow : wide, dim3(blocks[kWideResid]), dim3(kThreads), small ? kSmemRIs : kSmemRI, st,
-                      p, n_tokens)) != cudaSuccess)
+      (e = launch_pdl(k_resid_image_wide, dim3(tiles < grid ? tiles : grid), dim3(kThreadsW), kSmemW, st, p, tiles, n_tokens)) !=
+          cudaSuccess)
     return e;
   return cudaGetLastError();
 }

@@ -129,32 +129,32 @@ constexpr unsigned kFusedSpinLimit = 1u << 20;   // default: about a second
 
 // The block that arrives last (of n_blocks) sums the per-part norm partials in part
 // order in double precision, writes gate / rho (Eq. (3.3)) and the ascending list of
-// fired tokens, and rearms the arrival counter.  Every thread of every block calls it
-// after its partials are written; s_last is a shared-memory word.
-__device__ __forceinline__ void decide_gate_last_block(const GroupParams& g, const IoRef& io,
-                                                       int slot, int n_tokens,
-                                                       const float* normpart, int n_parts,
-                                                       unsigned n_blocks, int* s_last) {
+// fired tokens, and rearms the arrival counter.  Every thread of every block (or of the n_threads of
+// a block that `sync` holds together, thread `tid` of them) calls it after its partials are written;
+// s_last is a shared-memory word, s_gate holds the decisions for the list of gated tokens.
+template <typename Sync>
+__device__ __forceinline__ void decide_gate_last(const GroupParams& g, const IoRef& io, int slot, int n_tokens,
+                                                 const float* normpart, int n_parts, unsigned n_blocks, int* s_last,
+                                                 unsigned char* s_gate, int tid, int n_threads, Sync&& sync) {
   __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  sync();
+  if (tid == 0) {
     const unsigned prev = atomicAdd(g.counter, 1u);
     *s_last = (prev == n_blocks - 1);
   }
-  __syncthreads();
+  sync();
   if (!*s_last) return;
   __threadfence();
-  __shared__ unsigned char s_gate[GSI_MAX_TOKENS];   // the decisions, for the list of gated tokens
   unsigned char* gate = io.gate + (long long)slot * io.log_step_stride;
   float* rho = io.rho ? io.rho + (long long)slot * io.log_step_stride : g.rho_scratch;
   // L adjacent lanes share a token: each sums a contiguous range of parts in order (loads
   // issued thirty-two parts at a time), then the L sums are combined by a butterfly, so the
   // result depends on n_tokens and the block size only through L and is reproducible.
   int L = 1;
-  while (2 * L <= 32 && 2 * L * n_tokens <= (int)blockDim.x) L *= 2;
-  const int per_pass = blockDim.x / L;
+  while (2 * L <= 32 && 2 * L * n_tokens <= n_threads) L *= 2;
+  const int per_pass = n_threads / L;
   for (int t0 = 0; t0 < n_tokens; t0 += per_pass) {   // block-uniform trip count
-    const int t = t0 + (int)threadIdx.x / L, l = (int)threadIdx.x % L;
+    const int t = t0 + tid / L, l = tid % L;
     const bool live = t < n_tokens;
     const int p0 = (int)((long long)n_parts * l / L), p1 = (int)((long long)n_parts * (l + 1) / L);
     double sr = 0.0, sx = 0.0;
@@ -184,8 +184,8 @@ __device__ __forceinline__ void decide_gate_last_block(const GroupParams& g, con
       rho[t] = (float)(nr / nx);
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  sync();
+  if (tid == 0) {
     int n = 0;
     if (!(g.flags & GSI_FLAG_STATIC_PROJECTION)) {
       for (int t = 0; t < n_tokens; ++t)
@@ -194,6 +194,13 @@ __device__ __forceinline__ void decide_gate_last_block(const GroupParams& g, con
     *g.n_fired = n;
     *g.counter = 0u;
   }
+}
+__device__ __forceinline__ void decide_gate_last_block(const GroupParams& g, const IoRef& io, int slot, int n_tokens,
+                                                       const float* normpart, int n_parts, unsigned n_blocks,
+                                                       int* s_last) {
+  __shared__ unsigned char s_gate[GSI_MAX_TOKENS];
+  decide_gate_last(g, io, slot, n_tokens, normpart, n_parts, n_blocks, s_last, s_gate, (int)threadIdx.x, (int)blockDim.x,
+                   [] { __syncthreads(); });
 }
 
 // Launch that lets the kernel start before its predecessor in the stream has finished

@@ -338,7 +338,6 @@ struct alignas(64) WideGroup {
   TmaMaps tm;
   GroupParams g;
   IoRef io;
-  int rs;      // token ranges per residual tile
 };
 
 // Makes a tensor map that the host wrote to device memory usable by this thread's copies.
@@ -352,6 +351,7 @@ struct WideParams {
   const int* order;         // [n]: the order in which the contraction takes them
   int n;
   int use_counter;
+  int term_bytes;           // shared memory for terms of c in the residual / image kernel (a multiple of 1024)
 
   __device__ __forceinline__ IoRef io_of(const WideGroup& w) const {
     IoRef io = w.io;
@@ -373,7 +373,8 @@ struct WideParams {
   }
 };
 int wide_split_blocks(int d, int n_tokens);
-cudaError_t launch_front_wide(const WideParams& p, const int* blocks, int n_tokens, cudaStream_t st);
+int wide_term_bytes(int most_k, int n_tokens);
+cudaError_t launch_front_wide(const WideParams& p, const int* blocks, int n_tokens, int grid, cudaStream_t st);
 cudaError_t launch_gemm_wide(const WideParams& p, int tiles, int splits, int n_tokens, cudaStream_t st);
 
 }  // namespace gsi
