@@ -150,9 +150,11 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W_host_array,
  * sum d_out * d is 2^25 or more, d a multiple of 64 and every d_out of 128.
  * Results of a given call are reproducible bit for bit.
  * Enqueues on `stream` and returns; n_tokens = 0 is a no-op.
- * The calls that do not take that route (as do gsi_forward_static and gsi_extend_basis) run as one
+ * The calls that do not take that route (as does gsi_forward_static) run as one launch: of clusters of
+ * sixteen CTAs that hold the whole basis in shared memory (225 KB each; no CTA waits for another
+ * cluster) where the basis fits and the tokens are few, otherwise, like gsi_extend_basis, as a
  * cooperative launch with a CTA on every SM of the current context: beside a long kernel of another
- * stream they begin when every SM has room for 512 threads (and, but for the extension, 160 KB of
+ * stream the latter begin when every SM has room for 512 threads (and, but for the extension, 160 KB of
  * shared memory); a program whose other kernels never leave that room takes a stack in mode 1.
  */
 gsi_status_t gsi_forward(gsi_handle_t h, const float* x, float* y,
