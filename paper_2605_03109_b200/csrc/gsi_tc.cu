@@ -50,7 +50,9 @@ __global__ void __launch_bounds__(256) k_pack_fired_bf16(GroupParams g, int min_
 // mapped == 1: B rows are all n_tokens tokens of the call (row = token); only the columns
 //              of fired tokens are written out.
 // kCluster: the splits of a tile are a cluster; their sums meet in distributed shared memory, added
-// in split order by the ranks (a share of the columns each), and no partial sum goes to memory.
+// in split order by the ranks (a share of the columns each), and no partial sum goes to memory.  A launch
+// over many groups has one number of splits for all of them: a rank that a shallow group leaves without
+// a block of the depth (its tensor memory was never written) hands on zeros.
 template <bool kCluster, bool kInStack>
 __device__ __forceinline__ void residual_gemm_body(unsigned char* smem_raw, const GroupParams& g, const TmaMaps& tm,
                                                    const IoRef& io, int min_fired, int splits, int mapped,
@@ -110,7 +112,7 @@ __device__ __forceinline__ void residual_gemm_body(unsigned char* smem_raw, cons
       tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
       tmem_ld_wait();
 #pragma unroll
-      for (int c = 0; c < 16; ++c) part[(c0 + c) * kTM + r] = ok ? __uint_as_float(v[c]) : gave_up;
+      for (int c = 0; c < 16; ++c) part[(c0 + c) * kTM + r] = !ok ? gave_up : nloc > 0 ? __uint_as_float(v[c]) : 0.f;
     }
     cluster_sync();
 #pragma unroll 2

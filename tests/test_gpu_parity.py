@@ -1783,6 +1783,31 @@ def test_batched_step_over_all_groups_at_once(n_tokens, shapes, static):
                 compare_group(x[at:at + n_tokens], P, Ws, 0.05, y, gates[i], stack.rho_log[step % 2, i].cpu().numpy())
 
 
+@pytest.mark.parametrize("n_tokens,widths,splits", [
+    (8, (128, 256, 1024, 8192), 4),      # two blocks of the depth on four ranks
+    (33, (256, 256, 384, 16384), 8),     # four, and six, on eight
+    (64, (128, 128, 128, 128, 16384), 8),
+])
+def test_batched_step_of_depths_with_fewer_blocks_than_splits(n_tokens, widths, splits):
+    """The contraction of W r over all groups splits every depth by the deepest one's number: the ranks that a
+    shallow group leaves without a block add nothing to y.  Every token is gated (eps = 0), in every group."""
+    assert min(widths) // 64 < splits
+    g = G()
+    groups = [make_small(d, 128, (128,), n_tokens, seed=9600 + 7 * i + n_tokens, outlier_every=1)
+              for i, d in enumerate(widths)]
+    layers = [g.Layer([W.cuda() for W in Ws], P.cuda(), 0.0, max_tokens=n_tokens) for _, P, Ws in groups]
+    stack = g.Stack(layers)
+    stack.bind([x.cuda() for x, _, _ in groups])
+    assert stack.launches_per_step() == 6
+    for _ in range(2):
+        stack.step()
+        torch.cuda.synchronize()
+        assert stack.status() == 0 and bool((stack.gate_log == 1).all())
+        for i, (x, P, Ws) in enumerate(groups):
+            compare_group(x, P, Ws, 0.0, stack.ys[i].cpu().reshape(n_tokens, -1).numpy(),
+                          stack.gate_log[0, i].cpu().numpy())
+
+
 @pytest.mark.parametrize("d,k,d_out,n,p_dtype,every", [
     (8, 8, (8,), 2, "bf16", 1),                        # CTAs without rows, a cluster of one image unit
     (1000, 120, (12000, 4992), 32, "bf16", 1),         # W r in several batches
