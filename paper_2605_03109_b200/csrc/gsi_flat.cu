@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(kT, 1) k_flat_residual(FlatParams p) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_launch_dependents();
   const int i0 = p.first[blockIdx.x], i1 = p.first[blockIdx.x + 1];
+  if (i0 == i1) return;   // no share (its index may lie past the list): fewer units of rows than CTAs
   FlatShare sh = p.shares[i0];
   int n = p.groups[sh.group].slots;
   pdl_wait();

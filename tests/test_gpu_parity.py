@@ -1887,3 +1887,27 @@ def test_single_token_steps_over_all_groups_at_once(shapes, static):
     stack.step_host([x[:1].contiguous() for x, _, _ in groups], ys, gate)
     assert all(torch.equal(a.cpu().reshape(-1), b) for a, b in zip(first[0], ys))
     assert torch.equal(gate, stack.gate_log[0].cpu())
+
+
+@pytest.mark.parametrize("shapes", [
+    ((128, 64, (72,)),) * 8, ((64, 64, (8, 40)),) * 8, ((8, 8, (8,)),) * 8, ((64, 24, (16,)),) * 16,
+    ((256, 16, (24,)),) * 7 + ((1024, 1024, (40,)),),
+])
+def test_single_token_steps_of_fewer_basis_rows_than_the_ctas_can_share(shapes):
+    """Steps over all groups at once where CTAs, the last one among them, have no rows of any basis: more steps
+    than one (the words behind the list of shares are zeros in the first) against the oracle."""
+    g = G()
+    n_steps = 3
+    groups = [make_small(d, k, d_out, n_steps, seed=9950 + i, noise=0.01, outlier_every=2 if i % 2 else 0)
+              for i, (d, k, d_out) in enumerate(shapes)]
+    layers = [g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=1) for _, P, Ws in groups]
+    stack = g.Stack(layers)
+    stack.bind([x.cuda().contiguous() for x, _, _ in groups], n_steps=n_steps)
+    assert not stack.is_persistent() and stack.launches_per_step() == 3
+    for step in range(2 * n_steps):
+        stack.step()
+        torch.cuda.synchronize()
+        assert stack.status() == 0
+        gates = stack.gate_log[step % n_steps].cpu().numpy()
+        for i, (x, P, Ws) in enumerate(groups):
+            compare_group(x[step % n_steps][None], P, Ws, 0.05, stack.ys[i].cpu().reshape(1, -1).numpy(), gates[i])
