@@ -23,8 +23,8 @@
 // token at 768 x 64 -> 3072 10.3 -> 5.3 us, 4096 x 256 -> 28672 13.5 -> 13.1 (gated 64 -> 57); 16 tokens, fp32
 // basis, 768 x 128 -> 2304 19 -> 10.3.
 //
-// Every wait is bounded; a CTA whose wait ran out sets GSI_ERR_TIMEOUT, leaves NaN, and stays until
-// its peers are gone.
+// Every wait is bounded; a CTA whose wait ran out goes no further, sets GSI_ERR_TIMEOUT, leaves NaN, and
+// stays until its peers are gone.
 #include <cuda.h>
 
 #include "gsi_mma.cuh"
@@ -183,7 +183,8 @@ template <int kSlots>
 __device__ __forceinline__ void wait_slot() {   // all but the last kSlots - 1 groups
   asm volatile("cp.async.wait_group %0;" ::"n"(kSlots - 1) : "memory");
 }
-// y += W r for the fired tokens, 8 NB at a time.  False when a wait ran out.
+// y += W r for the fired tokens, 8 NB at a time.  False when a wait ran out (for every thread of the CTA):
+// the batches from there on are left out, what the peers wait for among them, which stop in turn.
 template <int NB>
 __device__ __forceinline__ bool stream_w(const GroupParams& g, const IoRef& io, const ClusterPlan& pl, const Cta& me,
                                          const int* s_fired, unsigned char* smem, uint64_t* s_bar) {
@@ -249,7 +250,6 @@ __device__ __forceinline__ bool stream_w(const GroupParams& g, const IoRef& io, 
 #pragma unroll 1
   for (int i = 0; i < n_ring - 1; ++i) issue();
   int slot_out = 0;
-  bool ok = true;
 #pragma unroll 1
   for (int b = 0; b <= batches; ++b) {
     if (b < batches) {
@@ -330,13 +330,14 @@ __device__ __forceinline__ bool stream_w(const GroupParams& g, const IoRef& io, 
     }
     if (b > 0) {   // the batch before: this CTA's units
       const int a = b - 1, f0 = a / per_pass * 8 * NB, NC = tokens_of(a), first = a % per_pass * batch_units;
-      const bool here = arrived(&s_bar[a & 1], (a >> 1) & 1, g.spin_limit);
-      ok = ok && here;
-      const float gave_up = __int_as_float(0x7fc00000);
+      // (a barrier whose words have not come may not be armed again: they would count towards another batch)
+      if (__syncthreads_or(!arrived(&s_bar[a & 1], (a >> 1) & 1, g.spin_limit))) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        return false;
+      }
       for (int i = tid; i < own_slots(a) * NC * 4; i += kT) {
         const int q = i & 3, sc = i >> 2, slot = sc / NC, c = sc - slot * NC;
-        float4 v = sum_ranks(reinterpret_cast<const float4*>(smem + part + ((a & 1) * slots + slot) * one) + c * 4 + q, NC * 4);
-        if (!here) v = make_float4(gave_up, gave_up, gave_up, gave_up);
+        const float4 v = sum_ranks(reinterpret_cast<const float4*>(smem + part + ((a & 1) * slots + slot) * one) + c * 4 + q, NC * 4);
         const int row = (me.u0 + first + slot * kC + me.rank) * 16 + q * 4;
         if (row < g.O) {
           float4* y = reinterpret_cast<float4*>(io.y + (size_t)s_fired[1 + f0 + c] * g.O + row);
@@ -348,7 +349,7 @@ __device__ __forceinline__ bool stream_w(const GroupParams& g, const IoRef& io, 
       if (a + 2 < batches) cluster_arrive();
     }
   }
-  return ok;
+  return true;
 }
 
 // Everything up to the gate.  False when a wait ran out (for every thread of the CTA); s_fired: the
@@ -718,8 +719,7 @@ k_forward_cluster(const __grid_constant__ GroupParams g, const __grid_constant__
     if (f > 16 && fits(min(f, 32))) ok = stream_w<4>(g, io, pl, me, s_fired, smem, s_bar + 3);
     else if (f > 8 && fits(min(f, 16))) ok = stream_w<2>(g, io, pl, me, s_fired, smem, s_bar + 3);
     else ok = stream_w<1>(g, io, pl, me, s_fired, smem, s_bar + 3);
-    if (!ok && threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
-    return;
+    if (ok) return;   // (likewise)
   }
   if (threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
   // The call's results must not pass for results: NaN in this CTA's rows of y and in every token's rho.
@@ -735,8 +735,10 @@ k_forward_cluster(const __grid_constant__ GroupParams g, const __grid_constant__
     (io.rho ? io.rho + (long long)slot * io.log_step_stride : g.rho_scratch)[t] = nan;
   }
   if (leave_from && blockIdx.x == 0 && threadIdx.x == 0) *g.n_fired = 0;
+  __syncthreads();
   // Peers may still send to this CTA: it stays until they have left (an exited thread counts as
-  // arrived, one that goes on with W r arrives once per batch), and for the words then in flight.
+  // arrived, one that goes on with W r arrives once per batch), and for the words then in flight (ten
+  // microseconds; they take under one).
 #pragma unroll 1
   for (int i = 0; i < kMaxBatches; ++i) {
     cluster_arrive();

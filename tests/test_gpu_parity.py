@@ -164,6 +164,58 @@ def test_one_launch_wait_runs_out_and_the_next_calls_are_right(n):
             assert all(torch.equal(a, b) for a, b in zip(ref, run(lays[1])))
 
 
+def captured_clusters(call):
+    """CTAs of a cluster (1 where a launch has none) of every kernel that `call` enqueues, from a captured graph."""
+    from cuda.bindings import runtime as rt
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    err, nodes, count = rt.cudaGraphGetNodes(rt.cudaGraph_t(graph.raw_cuda_graph()), 256)
+    out = []
+    for node in nodes[:count]:
+        if rt.cudaGraphNodeGetType(node)[1] == rt.cudaGraphNodeType.cudaGraphNodeTypeKernel:
+            err, value = rt.cudaGraphKernelNodeGetAttribute(
+                node, rt.cudaLaunchAttributeID.cudaLaunchAttributeClusterDimension)
+            assert err == rt.cudaError_t.cudaSuccess
+            out.append(max(1, int(value.clusterDim.x)))
+    return out
+
+
+@pytest.mark.parametrize("d,k,d_out,n", [
+    (16, 16, (20000,), 32),               # one CTA of a cluster has all the rows, the others wait for its sums; many batches
+    (1000, 120, (12000, 4992), 32),       # several batches
+    (4088, 248, (4096, 2056), 1),         # one
+    (1512, 72, (1000, 64), 9),
+])
+def test_cluster_call_that_gives_up_anywhere(d, k, d_out, n):
+    """Limits of a few polls (a microsecond each): the waits of a call run out in the front, in W r or not at
+    all.  The call returns; the status word tells which it was; what it left in y is the undisturbed call's
+    value or NaN; and the next calls give the bits of an undisturbed handle."""
+    g = G()
+    x, P, Ws = make_small(d, k, d_out, n, seed=277 + n, outlier_every=1)
+    xd, Wd, Pd = x.cuda(), [W.cuda() for W in Ws], P.cuda()
+    lay = g.Layer(Wd, Pd, 0.0, max_tokens=n)
+    ref = [t.clone() for t in lay.forward(xd)]
+    assert captured_clusters(lambda: lay.forward(xd)) == [16]
+    torch.cuda.synchronize()
+    assert lay.status() == 0 and bool((ref[1] == 1).all())
+    seen = set()
+    for limit in (1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 24, 32, 1, 2, 3):
+        lay = g.Layer(Wd, Pd, 0.0, max_tokens=n)
+        lay.set_spin_limit(limit)
+        y, gate, rho = lay.forward(xd)
+        torch.cuda.synchronize()
+        seen.add(lay.status())
+        assert lay.status() in (0, 5)              # GSI_OK, GSI_ERR_TIMEOUT
+        missing = torch.isnan(y)
+        assert bool(missing.any()) == (lay.status() == 5)
+        assert torch.equal(y[~missing], ref[0][~missing])
+        lay.set_spin_limit(0)                      # the default again
+        for _ in range(2):
+            assert all(torch.equal(a, b) for a, b in zip(ref, lay.forward(xd)))
+    assert 5 in seen
+
+
 @pytest.mark.parametrize("d,k,d_out,n", [
     (4096, 256, (1024, 512), 5), (2056, 1000, (264,), 2),   # more column blocks of c than CTAs
     (16384, 40, (72,), 9),                                  # 64 units of basis rows per CTA
