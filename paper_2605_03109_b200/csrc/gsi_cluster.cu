@@ -712,39 +712,43 @@ k_forward_cluster(const __grid_constant__ GroupParams g, const __grid_constant__
   bool ok = front<NB, PF32>(g, io, pl, me, n_tokens, leave_from, smem, s_fired, s_bar);
   if (ok) {
     const int f = s_fired[0];
-    if (f == 0) return;   // (all that its peers sent to this CTA has arrived)
+    if (f == 0) {   // (all that its peers sent to this CTA has arrived)
+      if (threadIdx.x == 0) exchange::leave_launch(g.tickets);
+      return;
+    }
     // as many tokens at a time as there are and as the first part of shared memory holds
     const int op = op_stride(pl.steps);
     auto fits = [&](int NC) { return NC * op + ring_bytes(kShallowSlots) + 2 * NC * 1024 <= pl.front_bytes; };
     if (f > 16 && fits(min(f, 32))) ok = stream_w<4>(g, io, pl, me, s_fired, smem, s_bar + 3);
     else if (f > 8 && fits(min(f, 16))) ok = stream_w<2>(g, io, pl, me, s_fired, smem, s_bar + 3);
     else ok = stream_w<1>(g, io, pl, me, s_fired, smem, s_bar + 3);
-    if (ok) return;   // (likewise)
+    if (ok) {   // (likewise)
+      if (threadIdx.x == 0) exchange::leave_launch(g.tickets);
+      return;
+    }
   }
   if (threadIdx.x == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
   // The call's results must not pass for results: NaN in this CTA's rows of y and in every token's rho.
   const float nan = __int_as_float(0x7fc00000);
-  const int slot = io_slot(io);
   for (int t = 0; t < n_tokens; ++t)
     for (int i = threadIdx.x; i < 16 * me.n_units; i += kT) {
       const int row = me.u0 * 16 + i;
       if ((i >> 4) % kC == me.rank && row < g.O) io.y[(size_t)t * g.O + row] = nan;
     }
-  for (int t = threadIdx.x; t < n_tokens; t += kT) {
-    io.gate[(long long)slot * io.log_step_stride + t] = 1;
-    (io.rho ? io.rho + (long long)slot * io.log_step_stride : g.rho_scratch)[t] = nan;
-  }
   if (leave_from && blockIdx.x == 0 && threadIdx.x == 0) *g.n_fired = 0;
   __syncthreads();
   // Peers may still send to this CTA: it stays until they have left (an exited thread counts as
-  // arrived, one that goes on with W r arrives once per batch), and for the words then in flight (ten
-  // microseconds; they take under one).
+  // arrived, one that goes on with W r arrives once per batch), and for the words then in flight.
+  // Meanwhile block 0, of this cluster or another, leaves.
+  bool told = blockIdx.x == 0;
 #pragma unroll 1
-  for (int i = 0; i < kMaxBatches; ++i) {
+  for (int i = 0; i < kMaxBatches || (!told && i < exchange::kReportPolls); ++i) {
     cluster_arrive();
     cluster_wait();
+    if (!told) told = __syncthreads_or(threadIdx.x == 0 && exchange::block0_left(g.tickets));
   }
-  for (const long long t0 = clock64(); clock64() - t0 < 20000;) {}
+  exchange::let_land();
+  exchange::report_give_up(g, io, n_tokens);
 }
 
 // Clusters that the current context (for this stream) holds at a time; 0: none, or it cannot be told.

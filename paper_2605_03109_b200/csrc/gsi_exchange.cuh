@@ -115,8 +115,8 @@ __device__ __forceinline__ bool warp_gather_sum(const unsigned long long* p, siz
 // its multiple of kTickets changes when the last one leaves: they all read the same launch number
 // whenever they begin, whatever the size of the grid, and a launch whose waits ran out, in part
 // before its last CTA had begun, shares no tag with the next.
-constexpr unsigned kTickets = 256;
-static_assert(kFusedMaxGrid <= (int)kTickets, "one at least for block 0");
+constexpr unsigned kTickets = 1024;
+static_assert(2 * kFusedMaxGrid <= (int)kTickets, "more for block 0 than for all others");
 __device__ __forceinline__ unsigned first_tag(const unsigned long long* counter) {
   return (unsigned)(*counter / kTickets) * 4u + 1u;
 }
@@ -124,6 +124,30 @@ __device__ __forceinline__ void leave_launch(unsigned long long* counter) {   //
   asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(counter),
                "l"(blockIdx.x == 0 ? (unsigned long long)(kTickets - (gridDim.x - 1)) : 1ull)
                : "memory");
+}
+// Gates and rho of a forward call are block 0's to write, but a CTA that gave up writes its report over
+// them, and that has to stay.  Block 0 leaves behind what it wrote; the CTA waits, itself not yet gone,
+// until block 0 has left, and for what block 0 wrote before to land (kLanding cycles, ten microseconds; a
+// release by block 0 would order the two, at 0.2 to 0.3 us in every call: 13.58 -> 13.84, 12.86 -> 13.15).
+constexpr int kReportPolls = 1 << 20;   // about a second
+constexpr int kLanding = 20000;
+__device__ __forceinline__ bool block0_left(const unsigned long long* counter) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(counter) : "memory");
+  return v % kTickets >= kTickets / 2;
+}
+__device__ __forceinline__ void let_land() {
+  for (const long long t0 = clock64(); clock64() - t0 < kLanding;) {}
+}
+// What a call that gave up leaves instead of gates and rho; every thread of the CTA, which leaves.
+__device__ __forceinline__ void report_give_up(const GroupParams& g, const IoRef& io, int n_tokens) {
+  const long long at = (long long)io_slot(io) * io.log_step_stride;
+  for (int t = threadIdx.x; t < n_tokens; t += blockDim.x) {
+    io.gate[at + t] = 1;
+    (io.rho ? io.rho + at : g.rho_scratch)[t] = __int_as_float(0x7fc00000);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) leave_launch(g.tickets);
 }
 
 // The exchange area of a handle (or of the allocation-free entry point).  A location holds words

@@ -322,7 +322,6 @@ __device__ __forceinline__ bool forward_fused(const GroupParams& g, const IoRef&
   auto timed_out = [&](bool good) -> bool {   // the same answer for every thread
     if (!__syncthreads_or(!good)) return false;
     if (tid == 0) atomicExch(g.status, (int)GSI_ERR_TIMEOUT);
-    if (tid == 0) leave_launch(g.tickets);
     return true;
   };
   if constexpr (!kDirect) {
@@ -538,7 +537,7 @@ __device__ __forceinline__ bool forward_fused(const GroupParams& g, const IoRef&
     }
   }
   if (timed_out(ok)) return false;
-  if (tid == 0) leave_launch(g.tickets);   // (that was the last wait)
+  if (tid == 0 && cta > 0) leave_launch(g.tickets);   // (that was the last wait)
   if (warp == 0) {
     int f = 0;
     for (int t0 = 0; t0 < n; t0 += 32) {
@@ -567,6 +566,7 @@ __device__ __forceinline__ bool forward_fused(const GroupParams& g, const IoRef&
     }
   }
   __syncthreads();
+  if (tid == 0 && cta == 0) leave_launch(g.tickets);   // (behind the gates and rho)
   if (s_fired[0] == 0 || (leave_from && s_fired[0] >= leave_from)) return true;
 
   // ---- C
@@ -584,15 +584,16 @@ __global__ void __launch_bounds__(kT, 1) k_forward_fused(const __grid_constant__
   // The call's results must not pass for results (the allocation-free entry point has no status word
   // to ask for): NaN in this CTA's rows of y, whose W r may be missing, and in every token's rho.
   const float nan = __int_as_float(0x7fc00000);
-  const int cta = blockIdx.x, G = gridDim.x, slot = io_slot(io);
+  const int cta = blockIdx.x, G = gridDim.x;
   const int o0 = (int)((long long)g.O * cta / G), o1 = (int)((long long)g.O * (cta + 1) / G);
   for (int t = 0; t < n_tokens; ++t)
     for (int row = o0 + (int)threadIdx.x; row < o1; row += kT) io.y[(size_t)t * g.O + row] = nan;
-  for (int t = threadIdx.x; t < n_tokens; t += kT) {
-    io.gate[(long long)slot * io.log_step_stride + t] = 1;
-    (io.rho ? io.rho + (long long)slot * io.log_step_stride : g.rho_scratch)[t] = nan;
-  }
   if (leave_from && cta == 0 && threadIdx.x == 0) *g.n_fired = 0;   // no list of another call for the contraction
+  if (cta > 0 && threadIdx.x == 0)
+    for (int i = 0; i < kReportPolls && !block0_left(g.tickets); ++i) {}
+  __syncthreads();
+  let_land();
+  report_give_up(g, io, n_tokens);
 }
 
 template <int NB, bool PF32, bool kDirect>
