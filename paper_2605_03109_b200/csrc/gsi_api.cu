@@ -1,6 +1,7 @@
 // C ABI of the gated subspace layer: argument checking, workspace layout,
 // handle and stack bookkeeping, kernel sequencing.  No arithmetic lives here.
 #include <chrono>
+#include <cmath>
 #include <algorithm>
 #include <new>
 #include <vector>
@@ -1171,6 +1172,22 @@ static int unit_group(const gsi_stack* s, int u) {
   return u < s->n_phases ? s->host_phase_first[u] : (int)s->groups.size();
 }
 
+// Segments of a batched step in launches over all groups.  A further segment costs the tails of five
+// launches, some 40 us, and spares a part of the first copy in and the last one out; where the copies of
+// one direction take longer than the step it costs nothing until it outgrows what they hide.  (us a step, a tenth
+// gated, by segments: 12 GPT-2 layers at 24 tokens 2 311, 4 324, 12 621; at 64 3 634, 5 582, 12 780; eight GPT-J
+// layers at 8 1 693, 3 582, 12 865; at 24 1 1437, 3 941, 5 965, 12 1179; at 64 3 2022, 8 1832, 12 1847.)
+static int wide_segments(const gsi_stack* s) {
+  double in = 0.0, out = 0.0, run = 0.0;   // us: copies at 20 per MB, the step as measured at 33 to 64 tokens
+  for (const gsi_layer* h : s->groups) {
+    in += 80e-6 * s->B * h->desc.d;
+    out += 80e-6 * s->B * h->lay.O;
+    run += 2.0 + 2.0 * h->lay.O * h->desc.d / 4.2e6;
+  }
+  if (in + out < 100.0) return 1;   // (two GPT-J layers at 8 tokens, 79 us of copies: 217, in two 227; 24 layers at 3, 350: 1047, 930)
+  return (int)std::max(0.6 + std::sqrt((in + out) / 40.0), (std::max(in, out) - run) / 45.0);
+}
+
 // Cuts a step with host buffers into segments of about equal bytes, and makes the streams and
 // events that overlap them.
 static bool plan_segments(gsi_stack* s) {
@@ -1185,16 +1202,15 @@ static bool plan_segments(gsi_stack* s) {
   for (int u = 0; u < units; ++u) total += bytes(u);
   // A copy of 1 MB takes 20 us.  A further launch of the persistent kernel costs about that (its
   // opening and closing ticks), so two halves from 3 MB on (28 GPT-J groups: 776 us in one piece,
-  // 729 in two); the chains of batched steps go on from segment to segment without a gap: 3 MB
-  // each (8 GPT-J layers: 821 us at 8 tokens and 1968 at 64, where the step alone takes 1200 and the
-  // copies as long; in one piece, before the alternating chains, 1076 and 3359).
+  // 729 in two); the chains of batched steps go on from segment to segment without a gap: 3 MB each.
   int n = s->flat ? 1 : s->persistent ? (s->B == 1 && total >= 3.0e6 ? 2 : 1) : (int)(total / 3.0e6);
+  if (s->wide) n = wide_segments(s);
   n = std::max(1, std::min(n, std::min(units, kMaxSegments)));
   s->segment.assign(1, 0);
   double at = 0.0;
   for (int u = 0; u < units && (int)s->segment.size() < n; ++u) {
     at += bytes(u);
-    const bool inside_pair = !s->persistent && s->pair_first[u];
+    const bool inside_pair = !s->persistent && !s->wide && s->pair_first[u];   // (a pair shares streams)
     if (at >= total * s->segment.size() / n && !inside_pair && u + 1 < units) s->segment.push_back(u + 1);
   }
   s->segment.push_back(units);
