@@ -478,6 +478,8 @@ __global__ void __launch_bounds__(kThreadsW, 1) k_resid_image_wide(WideParams p,
           __syncwarp();
           return true;
         });
+    // (no arrival is on its way to the barrier when the block leaves)
+    if (ok && n_pass > 0) ok = __all_sync(0xffffffffu, mbar_wait(read, (n_pass - 1) & 1));
     if (!ok && lane == 0) s_fail = 1;
   } else {
     pdl_wait();
