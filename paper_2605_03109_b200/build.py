@@ -86,24 +86,36 @@ CALLS_SRC = os.path.join(CSRC, "torch_calls.cpp")
 CALLS = os.path.join(HERE, "_torch_calls.so")
 
 
+def _calls_flags() -> list[str]:
+    import torch
+    return ["-O2", "-std=c++17", "-fPIC", "-shared", "-DTORCH_EXTENSION_NAME=_torch_calls",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+
+
 def _calls_command(out: str) -> list[str]:
     import sysconfig
     import torch
     base = os.path.join(os.path.dirname(torch.__file__))
     inc = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
            sysconfig.get_paths()["include"], "/usr/local/cuda/include", os.path.join(ROOT, "include")]
-    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-DTORCH_EXTENSION_NAME=_torch_calls",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *[f"-I{d}" for d in inc], CALLS_SRC,
-            "-o", out, "-L" + os.path.join(base, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    return ["g++", *[f"-I{d}" for d in inc], CALLS_SRC, "-o", out, "-L" + os.path.join(base, "lib"), *_calls_flags()]
+
+
+def _calls_hash() -> str:
+    """What the module was built from and for: the sources, the flags, this torch and this Python's binary
+    interface.  No path: the module is built once and used where the tree is copied to."""
+    import hashlib
+    import sysconfig
+    import torch
+    h = hashlib.sha256(" ".join([*_calls_flags(), torch.__version__, sysconfig.get_config_var("SOABI")]).encode())
+    for p in (CALLS_SRC, os.path.join(ROOT, "include", "gsi.h")):
+        h.update(open(p, "rb").read())
+    return h.hexdigest()
 
 
 def build_calls(force: bool = False) -> str:
-    import hashlib
-    import torch
-    h = hashlib.sha256(" ".join(_calls_command("-")).encode() + torch.__version__.encode())
-    for p in (CALLS_SRC, os.path.join(ROOT, "include", "gsi.h")):
-        h.update(open(p, "rb").read())
-    digest, stamp = h.hexdigest(), CALLS + ".srchash"
+    digest, stamp = _calls_hash(), CALLS + ".srchash"
     if not force and os.path.exists(CALLS) and os.path.exists(stamp) and open(stamp).read().strip() == digest:
         return CALLS
     tmp = CALLS + f".tmp{os.getpid()}"

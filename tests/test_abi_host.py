@@ -82,3 +82,23 @@ def test_null_and_misaligned_arguments_are_rejected_on_the_host():
     assert lib.gsi_stack_set_spin_limit(None, 1) == INVALID
     assert lib.gsi_extend_basis(None, 4096, 0.05, 4096, None, None, None) == INVALID
     assert lib.gsi_get_status(None, None) == INVALID
+
+
+def test_a_copy_of_the_tree_is_current_where_it_is_copied_to(tmp_path):
+    """Library and extension module are built once and travel with the tree: what decides whether they are
+    current (sources, flags, versions) does not depend on where it lies."""
+    import importlib.util
+    import shutil
+    from paper_2605_03109_b200 import build
+    shutil.copytree(os.path.join(ROOT, "include"), tmp_path / "include")
+    shutil.copytree(os.path.join(ROOT, "paper_2605_03109_b200", "csrc"), tmp_path / "paper_2605_03109_b200" / "csrc")
+    there = tmp_path / "paper_2605_03109_b200" / "build.py"
+    shutil.copy(build.__file__, there)
+    spec = importlib.util.spec_from_file_location("build_there", there)
+    copy = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(copy)
+    assert copy.CALLS_SRC != build.CALLS_SRC
+    assert copy._source_hash() == build._source_hash() and copy._calls_hash() == build._calls_hash()
+    with open(copy.CALLS_SRC, "a") as f:
+        f.write("// another source\n")
+    assert copy._calls_hash() != build._calls_hash()
