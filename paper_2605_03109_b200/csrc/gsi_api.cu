@@ -38,9 +38,10 @@ constexpr int kMaxSegments = 12;   // of a step with host buffers
 constexpr int kWideMinGroups = 4;
 // Single-token stacks that step in three launches (gsi_flat.cu) instead of the persistent kernel: groups enough
 // for their phases to add up, images that are small per group, bases that stay in the L2 (us a step,
-// persistent / three launches: 12 GPT-2 layers, k = 128, 70 % gated 124 / 53, k = 512 103 / 62; two layers, eight
-// groups, 41 / 32, 1 % gated 24.7 / 25.9; 12 OPT layers, k = 128, images of 2.4 MB, 158 / 148; three GPT-J
-// layers, k = 128, 3.1 MB, 46.9 / 48.6, k = 256, 6.3 MB, 76.6 / 80.7).
+// persistent / three launches: 12 GPT-2 layers, k = 128, 70 % gated 120 / 51, k = 512 126 / 70; two layers, eight
+// groups, 39.5 / 29.8, 1 % gated 23.0 / 22.7; OPT layers, k = 128, images of 2.4 MB, a tenth gated, two 42.6 / 38.0, 12
+// 160 / 147; k = 256, 4.9 MB, six layers 99 / 102, 1 % gated 71 / 73.  Between the two lines lie GPT-J layers at k = 128,
+// 3.1 MB, three 57.9 / 52.6, 14 165 / 154).
 constexpr int kFlatMinGroups = 8;
 constexpr double kFlatBasisBytes = 96.0e6, kFlatImageBytes = 3.0e6;
 constexpr int kWideGemmSlots = 296;   // blocks of the contraction that are resident at a time
@@ -796,7 +797,7 @@ static bool plan_flat(gsi_stack* s, int grid, cudaStream_t stream) {
   s->flat_grid = grid;
   s->flat_params = FlatParams{reinterpret_cast<const WideGroup*>(s->wide_area), ints + at_first,
                               reinterpret_cast<const FlatShare*>(ints + at_shares), reinterpret_cast<const FlatGroup*>(ints),
-                              reinterpret_cast<float2*>(ints + at_norms), G, 0, s->step, s->step + 4};
+                              reinterpret_cast<float2*>(ints + at_norms), G, (int)shares.size(), 0, s->step, s->step + 4};
   return cudaMemsetAsync(s->step + 4, 0, sizeof(int), stream) == cudaSuccess &&
          cudaMemcpyAsync(s->wide_area, s->wide_table.data(), G * sizeof(WideGroup), cudaMemcpyHostToDevice, stream) ==
              cudaSuccess &&

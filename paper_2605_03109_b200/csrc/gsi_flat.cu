@@ -10,8 +10,10 @@
 // (gsi_persistent_impl.cuh) goes through a stack phase by phase, 3.5 us each whatever a phase carries; with
 // small groups that is most of the step.  Here a step is three passes at the speed of the memory
 // system; the price is that the bases are read twice, so they have to fit the L2.  12 GPT-2 layers,
-// k = 128, 70 % gated: 124 -> 53 us, of which the launches take 8, 10 and 36 (140 MB of images and W; held
-// up by the decisions at its start and by rows of 1.5 to 6 KB, W flows at 4.5 TB/s).
+// k = 128, 70 % gated: 120 -> 51 us; by themselves the launches take 8, 10 and 37 (140 MB of images and W; held
+// up by the decisions at its start and by rows of 1.5 to 6 KB, W flows at 4.5 TB/s).  What a CTA needs of the
+// tables, and the first rows of the basis in the second launch, are read ahead of the wait on the launch before:
+// 4 us a step in small stacks (two GPT-2 layers, 1 % gated, 26.8 -> 22.7; the persistent kernel takes 23.0).
 //
 // All sums run in an order that depends on the shapes and the grid alone.
 #include "gsi_flat.cuh"
@@ -49,29 +51,63 @@ struct Lanes {
   }
 };
 
+// What the first two kernels need of a group, in registers: read ahead of the wait on the kernel before.
+struct Rows {
+  const uint4* P;
+  float *cpart, *c, *r;
+  IoRef io;
+  int k, d, r0, r1, slot, slots;
+  __device__ __forceinline__ Rows(const FlatParams& p, int i) {
+    const FlatShare sh = p.shares[i];
+    const WideGroup& w = p.table[sh.group];
+    P = static_cast<const uint4*>(w.g.P);
+    cpart = w.g.cpart;
+    c = w.g.c;
+    r = w.g.r;
+    k = w.g.k;
+    d = w.g.d;
+    io = io_of(w, p.use_counter);
+    slots = p.groups[sh.group].slots;
+    slot = sh.slot;
+    r0 = sh.r0;
+    r1 = min(d, sh.r1);
+  }
+  __device__ __forceinline__ const float* x() const {
+    return io.x + (io.step ? (long long)(__ldcg(io.step) % io.n_steps) * io.x_step_stride : 0);
+  }
+};
 template <int VPL>
-__device__ __forceinline__ void project(const GroupParams& g, const float* x, int r0, int r1, int slot, float* s_sum) {
-  constexpr int U = VPL == 1 ? 8 : VPL == 2 ? 4 : 2;   // rows in flight per lane
+__device__ constexpr int in_flight() { return VPL == 1 ? 8 : VPL == 2 ? 4 : 2; }   // rows per lane
+// Rows base, base + stride, ... of the basis, and their x.
+template <int VPL, int U>
+__device__ __forceinline__ void load_rows(const Rows& g, const float* x, const Lanes& L, int base, uint4 (&q)[U][VPL],
+                                          float (&xv)[U]) {
+  const int KV = g.k / 8, stride = kW * L.rpp;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int row = base + u * stride;
+    xv[u] = row < g.r1 ? __ldcg(x + row) : 0.f;
+#pragma unroll
+    for (int v = 0; v < VPL; ++v)
+      q[u][v] = row < g.r1 && L.cl + v * 32 < KV ? __ldg(g.P + (size_t)row * KV + L.cl + v * 32) : make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
+template <int VPL>
+__device__ __forceinline__ void project(const Rows& g, float* s_sum) {
+  constexpr int U = in_flight<VPL>();
   const int KV = g.k / 8, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Lanes L(KV);
-  const uint4* P = static_cast<const uint4*>(g.P);
+  const float* x = g.x();
   float acc[VPL][8];
 #pragma unroll
   for (int v = 0; v < VPL; ++v)
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[v][e] = 0.f;
-  const int stride = kW * L.rpp;
-  for (int base = r0 + warp * L.rpp + L.sub; base < r1; base += U * stride) {
+  for (int base = g.r0 + warp * L.rpp + L.sub; base < g.r1; base += U * kW * L.rpp) {
     uint4 p[U][VPL];
     float xv[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int row = base + u * stride;
-      xv[u] = row < r1 ? __ldg(x + row) : 0.f;
-#pragma unroll
-      for (int v = 0; v < VPL; ++v)
-        p[u][v] = row < r1 && L.cl + v * 32 < KV ? __ldg(P + (size_t)row * KV + L.cl + v * 32) : make_uint4(0u, 0u, 0u, 0u);
-    }
+    load_rows<VPL, U>(g, x, L, base, p, xv);
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -100,52 +136,60 @@ __device__ __forceinline__ void project(const GroupParams& g, const float* x, in
     float s = 0.f;
 #pragma unroll
     for (int w = 0; w < kW; ++w) s += s_sum[w * g.k + j];
-    g.cpart[(size_t)slot * g.k + j] = s;
+    g.cpart[(size_t)g.slot * g.k + j] = s;
   }
 }
 
 __global__ void __launch_bounds__(kT, 1) k_flat_project(FlatParams p) {
   extern __shared__ __align__(16) float s_sum[];   // [warp][k]
   const int i0 = p.first[blockIdx.x], i1 = p.first[blockIdx.x + 1];   // (written when the stack is bound)
-  pdl_wait();   // first of the chain: nothing of it runs beside an earlier step
+  Rows g(p, min(i0, p.n_shares - 1));
+  // First of the chain: nothing of it runs beside an earlier step, whose outputs and step the other two
+  // may so take for granted ahead of their own waits.
+  pdl_wait();
   pdl_launch_dependents();
   for (int i = i0; i < i1; ++i) {
-    const FlatShare sh = p.shares[i];
-    const WideGroup& w = p.table[sh.group];
-    const IoRef io = io_of(w, p.use_counter);
-    const float* x = io.x + (long long)io_slot(io) * io.x_step_stride;
-    const int r1 = min(w.g.d, sh.r1);
-    if (w.g.k <= 256) project<1>(w.g, x, sh.r0, r1, sh.slot, s_sum);
-    else if (w.g.k <= 512) project<2>(w.g, x, sh.r0, r1, sh.slot, s_sum);
-    else project<kMaxVec>(w.g, x, sh.r0, r1, sh.slot, s_sum);
+    if (i > i0) g = Rows(p, i);
+    if (g.k <= 256) project<1>(g, s_sum);
+    else if (g.k <= 512) project<2>(g, s_sum);
+    else project<kMaxVec>(g, s_sum);
   }
 }
 
+// r and the norms of a share's rows; the first rows are on their way while c comes together.
 template <int VPL>
-__device__ __forceinline__ void residual(const GroupParams& g, const float* x, int r0, int r1, const float* s_c, float& sr,
-                                         float& sx) {
-  constexpr int U = VPL == 1 ? 8 : VPL == 2 ? 4 : 2;
-  const int KV = g.k / 8, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void residual(const Rows& g, bool wait, float* s_c, float& sr, float& sx) {
+  constexpr int U = in_flight<VPL>();
+  const int KV = g.k / 8, tid = threadIdx.x, warp = tid >> 5;
   const Lanes L(KV);
-  const uint4* P = static_cast<const uint4*>(g.P);
+  const float* x = g.x();
+  const int stride = kW * L.rpp;
+  int base = g.r0 + warp * L.rpp;
+  uint4 q[U][VPL];
+  float xv[U], dot[U];
+  load_rows<VPL, U>(g, x, L, base + L.sub, q, xv);
+  if (wait) pdl_wait();
+  __syncthreads();   // c of the share before is read
+  for (int j = tid; j < g.k; j += kT) {   // the partials in slot order, eight in flight
+    float s = 0.f;
+    for (int q0 = 0; q0 < g.slots; q0 += 8) {
+      float v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = q0 + e < g.slots ? __ldcg(g.cpart + (size_t)(q0 + e) * g.k + j) : 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s += v[e];
+    }
+    s_c[j] = s;
+    if (g.slot == 0) g.c[j] = s;
+  }
+  __syncthreads();
   float4 c[VPL][2];
 #pragma unroll
   for (int v = 0; v < VPL; ++v)
 #pragma unroll
     for (int h = 0; h < 2; ++h)
       c[v][h] = L.cl + v * 32 < KV ? reinterpret_cast<const float4*>(s_c)[(L.cl + v * 32) * 2 + h] : make_float4(0.f, 0.f, 0.f, 0.f);
-  const int stride = kW * L.rpp;
-  for (int base = r0 + warp * L.rpp; base < r1; base += U * stride) {   // (warp-uniform)
-    uint4 q[U][VPL];
-    float xv[U], dot[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int row = base + L.sub + u * stride;
-      xv[u] = row < r1 ? __ldg(x + row) : 0.f;
-#pragma unroll
-      for (int v = 0; v < VPL; ++v)
-        q[u][v] = row < r1 && L.cl + v * 32 < KV ? __ldg(P + (size_t)row * KV + L.cl + v * 32) : make_uint4(0u, 0u, 0u, 0u);
-    }
+  while (base < g.r1) {   // (warp-uniform)
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       dot[u] = 0.f;
@@ -158,13 +202,15 @@ __device__ __forceinline__ void residual(const GroupParams& g, const float* x, i
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int row = base + L.sub + u * stride;
-      if (row < r1 && L.cl == 0) {
+      if (row < g.r1 && L.cl == 0) {
         const float rv = xv[u] - dot[u];
         g.r[row] = rv;
         sr = fmaf(rv, rv, sr);
         sx = fmaf(xv[u], xv[u], sx);
       }
     }
+    base += U * stride;
+    if (base < g.r1) load_rows<VPL, U>(g, x, L, base + L.sub, q, xv);
   }
 }
 
@@ -174,38 +220,12 @@ __global__ void __launch_bounds__(kT, 1) k_flat_residual(FlatParams p) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_launch_dependents();
   const int i0 = p.first[blockIdx.x], i1 = p.first[blockIdx.x + 1];
-  if (i0 == i1) return;   // no share (its index may lie past the list): fewer units of rows than CTAs
-  FlatShare sh = p.shares[i0];
-  int n = p.groups[sh.group].slots;
-  pdl_wait();
-  for (int i = i0; i < i1; ++i) {
-    if (i > i0) {
-      sh = p.shares[i];
-      n = p.groups[sh.group].slots;
-    }
-    const WideGroup& w = p.table[sh.group];
-    const GroupParams& g = w.g;
-    const IoRef io = io_of(w, p.use_counter);
-    const float* x = io.x + (long long)io_slot(io) * io.x_step_stride;
-    __syncthreads();
-    for (int j = tid; j < g.k; j += kT) {   // the partials in slot order, eight in flight
-      float s = 0.f;
-      for (int q0 = 0; q0 < n; q0 += 8) {
-        float v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = q0 + e < n ? __ldcg(g.cpart + (size_t)(q0 + e) * g.k + j) : 0.f;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) s += v[e];
-      }
-      s_c[j] = s;
-      if (sh.slot == 0) g.c[j] = s;
-    }
-    __syncthreads();
+  for (int i = i0; i < i1; ++i) {   // (a CTA without a share: its index may lie past the list)
+    const Rows g(p, i);
     float sr = 0.f, sx = 0.f;
-    const int r1 = min(g.d, sh.r1);
-    if (g.k <= 256) residual<1>(g, x, sh.r0, r1, s_c, sr, sx);
-    else if (g.k <= 512) residual<2>(g, x, sh.r0, r1, s_c, sr, sx);
-    else residual<kMaxVec>(g, x, sh.r0, r1, s_c, sr, sx);
+    if (g.k <= 256) residual<1>(g, i == i0, s_c, sr, sx);
+    else if (g.k <= 512) residual<2>(g, i == i0, s_c, sr, sx);
+    else residual<kMaxVec>(g, i == i0, s_c, sr, sx);
     sr = warp_sum(sr);
     sx = warp_sum(sx);
     if (lane == 0) s_norm[warp] = make_float2(sr, sx);

@@ -30,7 +30,7 @@ struct FlatParams {
   const FlatShare* shares;
   const FlatGroup* groups;   // [n]
   float2* norms;             // [shares]: ||r||^2 and ||x||^2 of their rows
-  int n;
+  int n, n_shares;
   int use_counter;
   int* step;                 // moved on by the last launch if use_counter
   int* arrived;              // its CTAs that have read it
