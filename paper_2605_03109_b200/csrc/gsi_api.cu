@@ -40,7 +40,7 @@ constexpr int kWideMinGroups = 4;
 // for their phases to add up, images that are small per group, bases that stay in the L2 (us a step,
 // persistent / three launches: 12 GPT-2 layers, k = 128, 70 % gated 120 / 51, k = 512 126 / 70; two layers, eight
 // groups, 39.5 / 29.8, 1 % gated 23.0 / 22.7; OPT layers, k = 128, images of 2.4 MB, a tenth gated, two 42.6 / 38.0, 12
-// 160 / 147; k = 256, 4.9 MB, six layers 99 / 102, 1 % gated 71 / 73.  Between the two lines lie GPT-J layers at k = 128,
+// 160 / 147; k = 256, 4.7 MB, six layers 99 / 102, 1 % gated 71 / 73.  Between the two lines lie GPT-J layers at k = 128,
 // 3.1 MB, three 57.9 / 52.6, 14 165 / 154).
 constexpr int kFlatMinGroups = 8;
 constexpr double kFlatBasisBytes = 96.0e6, kFlatImageBytes = 3.0e6;
