@@ -817,24 +817,24 @@ bool launch_t(const GroupParams& g, const IoRef& io, int n, int leave, cudaStrea
   return true;
 }
 
-// Which calls run here.  The shape has to fit with any number of tokens, so that a token's result
-// does not depend on the tokens it travels with (handles for one or two tokens: with those).  Every
-// cluster does all of the contractions with P, which the cooperative launch shares out: up to 16 tokens
-// that pays as far as (tokens rounded up to 8) d k <= 1.2e7, beyond up to 4.5e6.  A tenth gated, us per call,
+// Which calls run here.  The shape has to fit with any number of tokens of the handle's (handles for one
+// or two tokens: with those).  Every cluster does all of the contractions with P, which the cooperative launch
+// shares out: up to 16 tokens that pays as far as (tokens rounded up to 8) d k <= 1.2e7, beyond up to 4.5e6.  A tenth gated, us per call,
 // cooperative launch / this: 3000 x 200 -> 1576 at 8 tokens 15.1 / 10.7, 16 17.3 / 15.7, 24 24.3 / 25.3, 32 24.7 / 32.2;
 // 4000 x 200 -> 1000 at 8 15.9 / 12.0, 16 16.9 / 17.4; 8000 x 104 -> 1000 at 8 17.0 / 12.4, 16 18.6 / 20.4; 1000 x 400 ->
 // 2000 at 16 22.3 / 19.0, 24 24.1 / 26.5; 304 x 296 -> 600 at 32 22.8 / 19.9; 760 x 128 -> 2304, fp32 basis, at 32 24.4 / 17.9; 1000 x 72 -> 4000 at 48
-// 25.7 / 21.8, 64 28.0 / 28.0.
+// 25.7 / 21.8, 64 28.0 / 28.0.  Nine to 16 tokens have to fit in one pass (1800 x 400 -> 3000 at 16 19.5 / 22.0, 1408 x 504 -> 3000
+// at 12 23.3 / 26.0, -> 64 18.7 / 20.1; but 1288 x 440 -> 64 at 16 20.6 / 19.6).  Where the rows outnumber the width by far,
+// twenty to forty times, a quarter gated, the 112 SMs of seven clusters are behind: 520 x 512 -> 16000 at 8 24.3 / 24.2, 16 27.0 /
+// 32.6, but 20.7 / 20.6 with 1 % gated, at 4 16.7 / 11.4; 768 x 64 -> 20480 at 32 33.1 / 38.0.
 template <bool PF32>
 bool launch_p(const GroupParams& g, const IoRef& io, int n, int leave, cudaStream_t st, cudaError_t* e) {
   ClusterPlan pl;
   if (g.k > kMostColumns) return false;
   if ((double)((n + 7) / 8 * 8) * g.d * g.k > (n <= 16 ? 1.2e7 : 4.5e6)) return false;
   if (g.B > 2 && !make_plan<1, PF32>(g.d, g.k, GSI_MAX_TOKENS, &pl)) return false;
-  // (as many tokens at a time as the shared memory holds)
   if (n > 16 && launch_t<4, PF32>(g, io, n, leave, st, e)) return true;
-  if (n > 8 && launch_t<2, PF32>(g, io, n, leave, st, e)) return true;
-  return launch_t<1, PF32>(g, io, n, leave, st, e);
+  return n > 8 ? launch_t<2, PF32>(g, io, n, leave, st, e) : launch_t<1, PF32>(g, io, n, leave, st, e);
 }
 
 }  // namespace

@@ -1867,16 +1867,20 @@ def test_batched_step_of_depths_with_fewer_blocks_than_splits(n_tokens, widths, 
                           stack.gate_log[0, i].cpu().numpy())
 
 
-@pytest.mark.parametrize("d,k,d_out,n,p_dtype,every", [
-    (8, 8, (8,), 2, "bf16", 1),                        # CTAs without rows, a cluster of one image unit
-    (1000, 120, (12000, 4992), 32, "bf16", 1),         # W r in several batches
-    (4088, 248, (4096, 2056), 1, "bf16", 2),           # a handle for one token: sixteen slabs of 130 KB
-    (1000, 200, (1000, 504, 72), 13, "f32", 2),        # three terms of the basis, odd rows and tokens
-    (520, 512, (1040,), 9, "bf16", 4),                 # 32 column tiles of c, two token blocks
-    (1288, 440, (4000,), 16, "bf16", 1),               # two passes over the tokens
-    (776, 96, (24,), 32, "bf16", 3),                   # every token block in use, one cluster
+@pytest.mark.parametrize("d,k,d_out,n,p_dtype,every,cluster", [
+    (8, 8, (8,), 2, "bf16", 1, 16),                    # CTAs without rows, a cluster of one image unit
+    (1000, 120, (12000, 4992), 32, "bf16", 1, 16),     # W r in several batches
+    (4088, 248, (4096, 2056), 1, "bf16", 2, 16),       # a handle for one token: sixteen slabs of 130 KB
+    (1000, 184, (1000, 504, 72), 13, "f32", 2, 16),    # three terms of the basis, odd rows and tokens
+    (1000, 200, (1000, 504, 72), 13, "f32", 2, 1),     # ... of which three do not fit: the cooperative launch
+    (520, 512, (1040,), 9, "bf16", 4, 16),             # 32 column tiles of c, two token blocks
+    (360, 360, (4000,), 32, "bf16", 1, 16),            # two passes over the tokens
+    (280, 280, (72, 496), 32, "f32", 2, 16),           # ... with an fp32 basis
+    (1288, 440, (4000,), 15, "bf16", 1, 16),           # the most tokens that fit in one pass
+    (1288, 440, (4000,), 16, "bf16", 1, 1),            # more
+    (776, 96, (24,), 32, "bf16", 3, 16),               # every token block in use, one cluster
 ])
-def test_cluster_forward_edges(d, k, d_out, n, p_dtype, every):
+def test_cluster_forward_edges(d, k, d_out, n, p_dtype, every, cluster):
     """Calls whose basis fits a cluster: the corners of its rows, token blocks and batches, against the
     oracle, and the same bits from call to call with another call's input in between."""
     g = G()
@@ -1884,6 +1888,7 @@ def test_cluster_forward_edges(d, k, d_out, n, p_dtype, every):
     lay = g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=n)
     xs = [x[:n].cuda().contiguous(), x[n:].cuda().contiguous()]
     refs = [[t.clone() for t in lay.forward(xi)] for xi in xs]
+    assert captured_clusters(lambda: lay.forward(xs[0])) == [cluster]
     outs = [lay.forward(xs[i % 2]) for i in range(20)]
     torch.cuda.synchronize()
     assert lay.status() == 0
