@@ -1975,3 +1975,51 @@ def test_single_token_steps_of_fewer_basis_rows_than_the_ctas_can_share(shapes):
         gates = stack.gate_log[step % n_steps].cpu().numpy()
         for i, (x, P, Ws) in enumerate(groups):
             compare_group(x[step % n_steps][None], P, Ws, 0.05, stack.ys[i].cpu().reshape(1, -1).numpy(), gates[i])
+
+
+def test_calls_refuse_and_accept_what_their_arguments_say():
+    """The calls that go through the extension module: inputs that are no contiguous float32 tensors on the
+    device, a counter that is not one int32 on it, and objects that are no tensors or streams are refused
+    before anything is launched; a stream may be given as an object or as its handle, outputs by the caller."""
+    g = G()
+    x, P, Ws = make_small(256, 64, (72, 40), 2, seed=9990, outlier_every=2)
+    xd, Pd, Wd = x.cuda(), P.cuda(), [W.cuda() for W in Ws]
+    lay = g.Layer(Wd, Pd, 0.05, max_tokens=2)
+    y, gate, rho = lay.forward(xd)
+    ka = torch.tensor([64], dtype=torch.int32, device="cuda")
+    strided = torch.stack([xd, xd], dim=2)[:, :, 0]
+    assert not strided.is_contiguous()
+    for bad in (x, xd.double(), xd.half(), strided):
+        with pytest.raises(AssertionError):
+            lay.forward(bad)
+    for bad in (x[0], xd[0].double(), torch.stack([xd[0], xd[0]], dim=1)[:, 0], xd[:, 0]):   # (the last: not d elements)
+        with pytest.raises(AssertionError):
+            lay.extend_basis(bad, 0.5, ka)
+    for bad in (ka.cpu(), ka.long(), torch.zeros(2, dtype=torch.int32, device="cuda")):
+        with pytest.raises(AssertionError):
+            lay.extend_basis(xd[0].contiguous(), 0.5, bad)
+    for bad in (None, x.numpy(), [1.0]):
+        with pytest.raises((TypeError, AttributeError)):
+            lay.forward(bad)
+    with pytest.raises((TypeError, ValueError)):
+        lay.forward(xd, stream="a stream")
+    with pytest.raises(g.GsiError):
+        lay.forward(torch.cat([xd, xd]))                         # more tokens than the handle takes
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    out = [torch.empty_like(t) for t in (y, gate, rho)]
+    for stream in (s, s.cuda_stream, None):
+        for t in out:
+            t.zero_()
+        torch.cuda.synchronize()
+        got = lay.forward(xd, *out, stream=stream)
+        torch.cuda.synchronize()
+        assert all(a is b for a, b in zip(got, out)) and all(torch.equal(a, b) for a, b in zip(got, (y, gate, rho)))
+    with torch.cuda.stream(s):
+        again = lay.forward(xd)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(again, (y, gate, rho)))
+    closed = g.Layer(Wd, Pd, 0.05, max_tokens=2)
+    closed.close()
+    with pytest.raises(g.GsiError):
+        closed.forward(xd)
