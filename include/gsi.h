@@ -142,7 +142,9 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W_host_array,
  * max_tokens tokens (gsi_forward_n).  x [n][d] fp32; y [n][sum d_out] fp32;
  * gate_mask_out [n] bytes (1 = slow path, W r added); rho_out [n] fp32 or NULL.
  * Each token is processed independently of the others in the call (Algorithm 1
- * is per token); its rounding can depend on the size of the call: calls of 2 or
+ * is per token); its rounding can depend on the size of the call.  Which kernel sums,
+ * and in which order, follows from the sizes of the handle and the number of tokens (calls as
+ * clusters, below, or as one cooperative launch).  Calls of 2 or
  * more tokens (bf16 basis; k, d and every d_out multiples of 128) beyond 32 tokens
  * or n * d * sum d_out = 2^27 (in a stack always) sum in another order and add W r
  * from r rounded to bf16 (|dy| <= 3e-3 max|y|); with other
@@ -153,9 +155,10 @@ gsi_status_t gsi_create(const gsi_desc_t* desc, const void* const* W_host_array,
  * The calls that do not take that route (as does gsi_forward_static) run as one launch: of clusters of
  * sixteen CTAs that hold the whole basis in shared memory (225 KB each; no CTA waits for another
  * cluster) where the basis fits and the tokens are few, otherwise, like gsi_extend_basis, as a
- * cooperative launch with a CTA on every SM of the current context: beside a long kernel of another
- * stream the latter begin when every SM has room for 512 threads (and, but for the extension, 160 KB of
- * shared memory); a program whose other kernels never leave that room takes a stack in mode 1.
+ * cooperative launch with a CTA on every SM of the current context.  Beside a long kernel of another
+ * stream the former begin when sixteen SMs that can form a cluster have room for 512 threads and 225 KB of
+ * shared memory each, the latter when every SM has room for 512 threads (and, but for the extension, 160 KB
+ * of shared memory); a program whose other kernels never leave that room takes a stack in mode 1.
  */
 gsi_status_t gsi_forward(gsi_handle_t h, const float* x, float* y,
                          unsigned char* gate_mask_out, gsi_stream_t stream);
@@ -279,9 +282,10 @@ gsi_status_t gsi_destroy(gsi_handle_t h);
  * image, gated residual) is Algorithm 1, but consecutive groups overlap: a
  * group's gate may be settled, and its W r added, while later groups already
  * project their inputs (the persistent kernel reads a group's x two phases
- * ahead, projects it one phase ahead and settles a gate one phase later;
- * batched stacks run the gated residual contraction of a group beside the
- * kernels of the groups after it).
+ * ahead, projects it one phase ahead and settles a gate one phase later; steps in
+ * launches over all groups, gsi_stack_set_mode, take every stage of the chain for all
+ * groups at once; batched stacks that step in chains run the gated residual
+ * contraction of a group beside the kernels of the groups after it).
  * Every y, gate byte and rho of a step is final when the step's work has
  * completed in the order of `stream`, not earlier.
  * ------------------------------------------------------------------------ */
@@ -292,7 +296,9 @@ typedef struct {
 } gsi_stack_io_t;
 
 /* Bytes of extra device workspace the stack itself needs (step counter,
- * barrier words, per-group parameter table). */
+ * barrier words, per-group parameter table, tables of steps over all groups).
+ * gsi_stack_create also takes a workspace without room for the last; such a
+ * stack never steps in launches over all groups. */
 size_t gsi_stack_workspace_bytes(int n_groups);
 
 /* groups_host_array: HOST array of n_groups handles in execution order; all
@@ -321,26 +327,37 @@ gsi_status_t gsi_stack_bind(gsi_stack_t s, const gsi_stack_io_t* io_host_array,
 /*
  * Declares that groups first_group and first_group + 1 do not read each other's
  * outputs (two branches of one block: in GPT-J the attention output projection
- * and the MLP down projection).  In the per-stage and batched kernels the
+ * and the MLP down projection).  Where a step is a chain of launches per group (mode 1,
+ * and stacks that qualify for none of the other forms, gsi_stack_set_mode) the
  * second group of a pair is then enqueued on a stream of the stack's own, forked
  * from and joined to the caller's stream by events, so the two chains of
  * launches run side by side (and a stream capture records a fork and a join).
- * Off by default; a group belongs to at most one pair.  The persistent kernel
- * needs no declaration: a step's inputs are given, so it puts consecutive groups
- * into one phase itself.  Takes effect at the next gsi_stack_bind.
+ * Off by default; a group belongs to at most one pair.  The other forms
+ * need no declaration and take no notice of it: a step's inputs are given, so the
+ * persistent kernel puts consecutive groups into one phase itself, and launches over
+ * all groups hold them all.  Takes effect at the next gsi_stack_bind.
  */
 gsi_status_t gsi_stack_set_concurrent(gsi_stack_t s, int first_group, int enable);
 
 /*
  * Execution mode, taken at the next gsi_stack_bind:
- *   0 (default)  the persistent kernel, one launch per token of the step, when
- *                every group qualifies (one or two tokens per step, no dense
+ *   0 (default)  the first of these that the stack qualifies for:
+ *                three launches over all groups: one token per step, 8 to 512 groups with
+ *                images of 3 MB on average at most and bases of 96 MB in all, every basis
+ *                bf16, no dense group, no FP8 image, d <= 16384;
+ *                the persistent kernel, one launch per token of the step: one or
+ *                two tokens per step, no dense
  *                group in a two-token stack, bf16 basis with k in
  *                {64,128,256,512}, d a multiple of 16, rows that fit the
- *                per-CTA buffers), else the per-stage / batched kernels;
+ *                per-CTA buffers;
+ *                five launches over all groups: two or more tokens per step, 4 to 1024
+ *                groups, none dense, all with a bf16 basis and k, d and every d_out
+ *                multiples of 128;
+ *                a chain of launches per group (the per-stage and batched kernels);
  *   1            always the per-stage kernels;
  *   2            the persistent launch or GSI_ERR_UNSUPPORTED from bind.
- * Both modes compute the same layer; they differ in reduction order only.
+ * All forms compute the same layer; they differ in reduction order, and batched forms add
+ * W r from r rounded to bf16 (gsi_forward).  gsi_stack_launches_per_step tells them apart.
  */
 gsi_status_t gsi_stack_set_mode(gsi_stack_t s, int mode);
 
@@ -351,6 +368,7 @@ gsi_status_t gsi_stack_set_mode(gsi_stack_t s, int mode);
  * restores the default (2^22, about a second).  Waits inside a CTA (its own
  * copies in flight) keep their own, larger limit.  Applies from the next step.
  * A very small value makes the time-out path testable without hanging anything.
+ * The other forms of a step have no waits between CTAs that it could limit.
  */
 gsi_status_t gsi_stack_set_spin_limit(gsi_stack_t s, unsigned polls);
 
@@ -358,7 +376,8 @@ gsi_status_t gsi_stack_set_spin_limit(gsi_stack_t s, unsigned polls);
 gsi_status_t gsi_stack_is_persistent(gsi_stack_t s, int* out);
 
 /*
- * Tracing.  `cycles` is a DEVICE array [n_CTAs][GSI_TRACE_SECTIONS] of 64-bit
+ * Tracing, of the persistent kernel only (gsi_stack_is_persistent; mode 2 asks for it).
+ * `cycles` is a DEVICE array [n_CTAs][GSI_TRACE_SECTIONS] of 64-bit
  * counters (n_CTAs = SM count; NULL switches tracing off).  While set, thread 0
  * of every CTA of the persistent launch adds the SM cycles it spends in each
  * section of the per-phase pipeline:
@@ -393,7 +412,8 @@ gsi_status_t gsi_stack_launches_per_step(gsi_stack_t s, int* n_out);
  * HOST pointers ([max_tokens][d] and [max_tokens][sum d_out]); pinned memory
  * makes the copies asynchronous.  gate_host [n_groups][max_tokens].  Groups whose
  * host buffers AND device buffers are adjacent in memory (carved out of one arena, in
- * group order) are copied with a single transfer per direction.  From 3 MB of x and y on,
+ * group order) are copied with a single transfer per direction.  From 3 MB of x and y on
+ * (5 MB in launches over all groups; never in three launches),
  * the step runs in segments of groups: the inputs of the next and the outputs of the
  * previous segment travel on streams of the stack's own while one segment runs (`stream`
  * waits for them; copies of neighbours are merged within a segment).  Host buffers of x and y may

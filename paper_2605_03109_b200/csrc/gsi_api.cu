@@ -34,7 +34,8 @@ constexpr double kOwnStreamBytes = 262144.0;   // W rows of a CTA up to which a 
 constexpr int kChains = 2;   // chains of a batched step side by side
 constexpr int kMaxSegments = 12;   // of a step with host buffers
 // Batched stacks of fewer groups keep a chain of launches per group (one GPT-J layer, three groups, 64 tokens, a
-// tenth gated: 134 us against 152 in five launches; one GPT-2 layer, four groups, 60 against 45).
+// tenth gated: 134 us against 152 in five launches; four groups, one GPT-2 layer 60 against 45, one OPT layer at 8
+// tokens 123 against 117, at 33 139 against 143, but 117 against 104 with 1 % gated).
 constexpr int kWideMinGroups = 4;
 // Single-token stacks that step in three launches (gsi_flat.cu) instead of the persistent kernel: groups enough
 // for their phases to add up, images that are small per group, bases that stay in the L2 (us a step,

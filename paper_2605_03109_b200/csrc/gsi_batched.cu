@@ -289,8 +289,8 @@ k_resid_image_tc(GroupParams g, const __grid_constant__ TmaMaps tm, IoRef io, in
 // (a block finds its group in the table; WideGroup)
 // A step in a chain of five launches per group is the latency of its chains and the tails of small
 // grids: 28 GPT-J layers, 64 tokens, a tenth gated, 477 launches 3.34 ms; the same kernels over all
-// groups, whose inputs are staged before the step, 2.68 ms (W r at the copy bandwidth); 12 GPT-2 layers,
-// k = 256, 636 -> 151 us.
+// groups, whose inputs are staged before the step, 2.58 ms, with the persistent one below 2.49 (W r at the copy
+// bandwidth); 12 GPT-2 layers, k = 256, 636 -> 153 -> 137 us.
 __global__ void __launch_bounds__(256) k_split3_x_wide(WideParams p, int n_tokens, int slots) {
   pdl_wait();   // (first of the chain, as above)
   pdl_launch_dependents();
@@ -325,8 +325,8 @@ __global__ void __launch_bounds__(256) k_reduce_wide(WideParams p, int n_tokens,
 //   warp 0 asks for the weight tiles (ahead of the wait on the kernel before), warp 1 for the terms, and
 //   issues the contractions; warps 2-5 and 6-9 take the accumulators in turn.
 // As a block per tile each lived 12 us (search, tensor maps, tensor memory, one round trip of the copies,
-// epilogue) for 64 KB of weights: eight GPT-J layers at 8 tokens 162 -> 76 us, at 64 173 -> 167 (there the
-// epilogue is what bounds it: 64 columns per row to store, and to add up for the residual).
+// epilogue) for 64 KB of weights: eight GPT-J layers at 8 tokens 175 -> 77 us (the step 463 -> 370), at 64 193 -> 167
+// (760 -> 741; there the epilogue is what bounds it: 64 columns per row to store, and to add up for the residual).
 constexpr int kThreadsW = 320, kSmemW = 220 * 1024, kBarBytesW = 512, kMostStagesW = 13;
 constexpr int kTermBytesW = 100 * 1024;   // shared memory for the terms of c at most
 constexpr int kTmemColsW = 512;

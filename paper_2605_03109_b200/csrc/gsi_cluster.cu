@@ -16,7 +16,7 @@
 //
 // What bounds it: a chain of latencies.  An exchange through the L2 between the CTAs of a
 // cooperative grid costs 2 us (gsi_fused.cu), one between the CTAs of a cluster 0.4, and nothing is
-// kept between calls: no tags, no scratch, no order between streams.  The price is that every
+// kept between calls but the count of the launches (for the report of a CTA that gave up).  The price is that every
 // cluster reads the basis (from the L2, but for one), and seven clusters of sixteen leave 36 of 148
 // SMs idle; W r makes up for that with 128 KB in flight per SM (5.5 TB/s where the cooperative launch,
 // by loads into registers, reaches 4.7).  Kernel times in a captured graph, cooperative launch -> this: one
