@@ -1977,6 +1977,37 @@ def test_single_token_steps_of_fewer_basis_rows_than_the_ctas_can_share(shapes):
             compare_group(x[step % n_steps][None], P, Ws, 0.05, stack.ys[i].cpu().reshape(1, -1).numpy(), gates[i])
 
 
+def test_single_token_steps_read_the_inputs_written_just_before_them():
+    """Steps over all groups whose inputs a kernel writes right before each of them, without a pause: launches
+    that begin ahead of their wait on the one before read this step's x, and write r of this step."""
+    g = G()
+    shapes = ((768, 128, (2304,)), (768, 128, (768,)), (768, 128, (3072,)), (3072, 128, (768,))) * 2
+    groups = [make_small(d, k, d_out, 2, seed=9970 + i, noise=0.004, outlier_every=2) for i, (d, k, d_out) in enumerate(shapes)]
+    layers = [g.Layer([W.cuda() for W in Ws], P.cuda(), 0.05, max_tokens=1) for _, P, Ws in groups]
+    stack = g.Stack(layers)
+    src = [[x[j:j + 1].cuda().contiguous() for x, _, _ in groups] for j in range(2)]
+    xs = [torch.empty_like(x) for x in src[0]]
+    stack.bind(xs)
+    assert stack.launches_per_step() == 3
+
+    def step(j):
+        for x, new in zip(xs, src[j]):
+            x.copy_(new)
+        stack.step()
+        return [y.clone() for y in stack.ys] + [stack.gate_log.clone(), stack.rho_log.clone()]
+    refs = []
+    for j in range(2):
+        torch.cuda.synchronize()
+        refs.append(step(j))
+        torch.cuda.synchronize()
+        for i, (x, P, Ws) in enumerate(groups):
+            compare_group(x[j:j + 1], P, Ws, 0.05, refs[j][i].cpu().reshape(1, -1).numpy(), refs[j][-2][0, i].cpu().numpy())
+    outs = [step(i % 2) for i in range(60)]
+    torch.cuda.synchronize()
+    assert stack.status() == 0
+    assert all(torch.equal(a, b) for i, out in enumerate(outs) for a, b in zip(out, refs[i % 2]))
+
+
 def test_calls_refuse_and_accept_what_their_arguments_say():
     """The calls that go through the extension module: inputs that are no contiguous float32 tensors on the
     device, a counter that is not one int32 on it, and objects that are no tensors or streams are refused
